@@ -268,7 +268,7 @@ chicle_status_t chicle_get_info(const chicle_glm_t *h, int64_t *round, int32_t *
  * sized and frozen at start-up, a thread that holds a lock the allocator also wants, or a process whose device
  * memory is handed out by another component. chicle_partition allocates its sort workspace and the K x dim update
  * buffers; this call allocates nothing, on the host or on the device: no cudaMalloc, cudaFree, or framework
- * allocator. Its workspace (about 3.2 MB) is a static device array that every GPU loading this library holds until
+ * allocator. Its workspace (1 MB) is a static device array that every GPU loading this library holds until
  * the process ends.
  *   device, cuda_stream   where to run; the work is enqueued on the stream and the call does not synchronise.
  *   n_coord, K, seed      as in chicle_partition: 1 <= K <= n_coord <= CHICLE_NOALLOC_MAX_COORDS. A larger n_coord

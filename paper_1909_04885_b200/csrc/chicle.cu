@@ -368,19 +368,18 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
     bool fresh = false;
     if (!h->owner) {
         fresh = true;
-        SortWorkspace w;
+        OrderWorkspace w;
+        // (buckets: at most one per started 512 coordinates of every partition, whatever K is later)
+        const size_t nbk = (size_t)order_buckets(n) + 1, ntmp = (size_t)(n <= CHICLE_NOALLOC_MAX_COORDS ? 2 * n : n);
         bool ok = alloc_into(h, owner, (size_t)n) && alloc_into(h, members, (size_t)n) && alloc_into(h, perm, (size_t)n) &&
-                  alloc_into(h, w.keys[0], (size_t)n) && alloc_into(h, w.keys[1], (size_t)n) &&
-                  alloc_into(h, w.vals[0], (size_t)n) && alloc_into(h, w.vals[1], (size_t)n) &&
-                  alloc_into(h, w.hist, sort_hist_entries(n)) && alloc_into(h, w.scan_sums, sort_scan_tiles(n) + 1);
+                  alloc_into(h, w.tmp, ntmp) && alloc_into(h, w.bowner, nbk) &&
+                  alloc_into(h, w.table, sort_hist_entries(n)) && alloc_into(h, w.scan_sums, sort_scan_tiles(n) + 1);
         if (!ok) {
             dev_free(h, owner); dev_free(h, members); dev_free(h, perm);
-            dev_free(h, w.keys[0]); dev_free(h, w.keys[1]); dev_free(h, w.vals[0]); dev_free(h, w.vals[1]);
-            dev_free(h, w.hist); dev_free(h, w.scan_sums);
+            dev_free(h, w.tmp); dev_free(h, w.bowner); dev_free(h, w.table); dev_free(h, w.scan_sums);
             return fail(h, CHICLE_ERR_OOM, "device allocation failed (partition workspaces)");
         }
-        w.capacity = n;
-        h->sortws = w;
+        h->ord = w;
     }
     float *U = h->U;
     int64_t *part_off = h->part_off;
@@ -395,14 +394,17 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
         if (e != cudaSuccess) return fail_cuda(h, e, "stream synchronise");
         float *newU = nullptr;
         int64_t *new_off = nullptr;
-        int64_t *new_hoff = new (std::nothrow) int64_t[(size_t)K + 1];
+        int64_t *new_hoff = new (std::nothrow) int64_t[2 * (size_t)K + 2];
+        uint32_t *new_bk = nullptr;
+        const size_t nbk = (size_t)order_buckets(n) + (size_t)K + 1; // buckets of the visiting orders, at most
         // release the old update workspace first: at the large configurations two of them do not fit
         dev_free(h, h->U);
         h->U = nullptr;
-        bool ok = new_hoff && alloc_into(h, newU, (size_t)K * (size_t)h->dim) && alloc_into(h, new_off, 2 * (size_t)K + 2); // K+1 offsets, then K step budgets
+        bool ok = new_hoff && alloc_into(h, newU, (size_t)K * (size_t)h->dim) && alloc_into(h, new_off, 3 * (size_t)K + 2) && // K+1 offsets, K+1 bucket offsets, K step budgets
+                  alloc_into(h, new_bk, 3 * nbk + 1);
         if (!ok) {
             delete[] new_hoff;
-            dev_free(h, newU); dev_free(h, new_off);
+            dev_free(h, newU); dev_free(h, new_off); dev_free(h, new_bk);
             h->K = 0; // the old workspace is gone: a new partition call is required
             if (fresh) { h->owner = owner; h->members = members; h->perm = perm; h->perm_epochs = 1; }
             return fail(h, CHICLE_ERR_OOM, "device allocation failed (K x dim update workspace)");
@@ -410,6 +412,11 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
         dev_free(h, h->part_off);
         delete[] h->h_part_off;
         U = newU; part_off = new_off; h_off = new_hoff;
+        dev_free(h, h->ord.cursor);
+        h->ord.cursor = new_bk;
+        h->ord.nbm = new_bk + nbk;
+        h->ord.start = new_bk + 2 * nbk;
+        (void)cudaMemsetAsync(new_bk, 0, nbk * sizeof(uint32_t), h->stream);
         // the look-ahead solver's per-round records (their number depends on K); without them the blocked solver runs
         dev_free(h, h->la_rec); dev_free(h, h->la_dir); dev_free(h, h->la_cursor); dev_free(h, h->la_blk_base); dev_free(h, h->la_slice);
         h->la_rec = nullptr; h->la_dir = nullptr; h->la_cursor = nullptr; h->la_blk_base = nullptr; h->la_slice = nullptr;
@@ -432,16 +439,25 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
     }
     if (fresh) { h->owner = owner; h->members = members; h->perm = perm; h->perm_epochs = 1; }
     h->U = U; h->part_off = part_off; h->h_part_off = h_off;
-    h->d_steps = part_off + K + 1;
+    h->bucket_off = part_off + K + 1;
+    h->d_steps = part_off + 2 * ((size_t)K + 1);
     h->U_rows = K;
     const int64_t base = n / K, extra = n % K;
     h_off[0] = 0;
     for (int32_t k = 1; k <= K; ++k) h_off[k] = sizes ? h_off[k - 1] + sizes[k - 1] : (int64_t)k * base + (k < extra ? k : extra);
     h->min_nk = n;
-    for (int32_t k = 0; k < K; ++k) h->min_nk = h_off[k + 1] - h_off[k] < h->min_nk ? h_off[k + 1] - h_off[k] : h->min_nk;
+    h->max_nk = 0;
+    h_off[K + 1] = 0;
+    for (int32_t k = 0; k < K; ++k) {
+        const int64_t nk = h_off[k + 1] - h_off[k];
+        h->min_nk = nk < h->min_nk ? nk : h->min_nk;
+        h->max_nk = nk > h->max_nk ? nk : h->max_nk;
+        h_off[K + 2 + k] = h_off[K + 1 + k] + order_buckets(nk);
+    }
+    h->n_buckets = h_off[2 * K + 1];
     h->K = K;
     h->seed = seed;
-    e = cudaMemcpyAsync(part_off, h_off, ((size_t)K + 1) * 8, cudaMemcpyHostToDevice, h->stream);
+    e = cudaMemcpyAsync(part_off, h_off, 2 * ((size_t)K + 1) * 8, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(U, 0, (size_t)K * (size_t)h->dim * 4, h->stream);
     int64_t *d_coff = nullptr;
     int32_t *d_ctask = nullptr;
@@ -525,18 +541,18 @@ static chicle_status_t round_impl(chicle_glm_t *h, int64_t H, const int64_t *hos
     }
     cudaStream_t s = h->stream;
     if (stats) (void)cudaEventRecord(h->ev[0], s);
-    e = launch_permutation(*h, h->round, epochs);
+    if (host_steps) {
+        // a pageable source: the runtime has taken its copy of the K words when the call returns
+        e = cudaMemcpyAsync(h->d_steps, host_steps, (size_t)h->K * sizeof(int64_t), cudaMemcpyHostToDevice, s);
+        if (e != cudaSuccess) return fail_cuda(h, e, "step budgets to the device");
+    }
+    e = launch_permutation(*h, h->round, epochs, H, host_steps ? h->d_steps : nullptr);
     if (e != cudaSuccess) return fail_cuda(h, e, "visiting-order kernels");
     if (stats) (void)cudaEventRecord(h->ev[1], s);
     int variant = 0;
     h->time_prepare = stats != nullptr;
     h->solver_launches = 0;
-    if (host_steps) {
-        // a pageable source: the runtime has taken its copy of the K words when the call returns
-        e = cudaMemcpyAsync(h->d_steps, host_steps, (size_t)h->K * sizeof(int64_t), cudaMemcpyHostToDevice, s);
-        if (e != cudaSuccess) return fail_cuda(h, e, "step budgets to the device");
-        h->round_steps = host_steps;
-    }
+    h->round_steps = host_steps;
     if (!host_steps || budget_total > 0) e = launch_local_solver(*h, H, sigma_prime, &variant);
     else if (stats) (void)cudaEventRecord(h->ev[4], s); // nobody steps this round
     h->round_steps = nullptr;
@@ -566,7 +582,7 @@ static chicle_status_t round_impl(chicle_glm_t *h, int64_t H, const int64_t *hos
         r.solver_slices = variant >= 4 ? h->la_last_slices : 0;
         r.cluster_ctas = variant == 4 ? (1 << h->la_logC) : 1;
         r.solver_launches = steps > 0 ? (h->solver_launches > 0 ? h->solver_launches : 1) : 0;
-        r.order_launches = (int32_t)(epochs * (22 + 5 * (h->K <= 256 ? 1 : 2)));
+        r.order_launches = h->order_launches;
         *stats = r;
         if (logging)
             fprintf(stderr, "[chicle] round %lld: K=%d steps=%lld solver=%d slices=%d ctas/partition=%d launches=%d; ms: orders %.3f, "
@@ -703,7 +719,7 @@ chicle_status_t chicle_get_permutation(chicle_glm_t *h, int64_t round, int32_t k
     const int64_t nk = h->h_part_off[k + 1] - h->h_part_off[k];
     if (!host_out || len != nk) return fail(h, CHICLE_ERR_INVALID_ARG, "chicle_get_permutation: bad out or len");
     cudaError_t e = cudaSetDevice(h->device);
-    if (e == cudaSuccess) e = launch_permutation(*h, round, 1); // scratch use of the order buffer: rounds rebuild it
+    if (e == cudaSuccess) e = launch_permutation(*h, round, 1, 0, nullptr); // scratch use of the order buffer: rounds rebuild it
     if (e == cudaSuccess && nk > 0)
         e = cudaMemcpyAsync(host_out, h->perm + h->h_part_off[k], (size_t)nk * 4, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);

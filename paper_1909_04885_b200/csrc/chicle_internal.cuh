@@ -46,14 +46,17 @@ constexpr int kSortThreads = 256;
 constexpr int kSortItems = 16;
 constexpr int kSortTile = kSortThreads * kSortItems;  // elements per block and pass
 
-struct SortWorkspace {
-    uint64_t *keys[2] = {nullptr, nullptr};
-    int32_t *vals[2] = {nullptr, nullptr};
-    uint32_t *hist = nullptr;      // 256 * nblk digit-major counters
+// Workspace of the partition and of the visiting orders (see partition.cu).
+struct OrderWorkspace {
+    uint32_t *cursor = nullptr;    // per bucket: its elements, then the running place in it; zero between calls
+    uint32_t *start = nullptr;     // per bucket (+ 1): its first position
+    uint32_t *nbm = nullptr;       // per bucket: buckets of its segment, 0: not needed in order
+    int32_t *bowner = nullptr;     // per bucket: the partition that all of it falls to, or -1
+    int32_t *tmp = nullptr;        // ids by bucket
+    uint32_t *table = nullptr;     // 256 counters per tile
     uint32_t *scan_sums = nullptr; // one per scan tile
-    int64_t capacity = 0;          // elements
-    int nblk = 0;
 };
+int64_t order_buckets(int64_t nk); // buckets of a segment of nk elements
 
 size_t sort_hist_entries(int64_t n);
 size_t sort_scan_tiles(int64_t n);
@@ -101,9 +104,11 @@ struct Glm {
     int32_t *owner = nullptr;   // n_coord
     int32_t *members = nullptr; // n_coord, grouped by partition, ascending id inside
     int64_t *part_off = nullptr; // K+1 (device)
-    int64_t *h_part_off = nullptr; // K+1 (host)
-    int64_t min_nk = 0;            // smallest partition
-    int64_t *d_steps = nullptr;    // K (device, behind part_off): the step budgets of a round that gives each partition its own
+    int64_t *h_part_off = nullptr; // K+1 (host), then the K+1 of bucket_off
+    int64_t min_nk = 0, max_nk = 0; // smallest and largest partition
+    int64_t *bucket_off = nullptr; // K+1 (device, behind part_off): first bucket of each partition's visiting order
+    int64_t n_buckets = 0;
+    int64_t *d_steps = nullptr;    // K (device, behind bucket_off): the step budgets of a round that gives each partition its own
     const int64_t *round_steps = nullptr; // the same on the host while such a round is being enqueued, else nullptr
     int32_t *perm = nullptr;    // epochs * n_coord
     int64_t perm_epochs = 0;
@@ -132,7 +137,8 @@ struct Glm {
     cudaEvent_t *la_ev_done = nullptr; // per slice: its chain launch is done (its region is free)
     bool time_prepare = false; // record ev[4] between the prepare and the chain kernel (round statistics asked for)
 
-    SortWorkspace sortws;
+    OrderWorkspace ord;
+    int order_launches = 0;        // kernels launched for the last visiting orders
     double *gap_partials = nullptr; // gap kernel partial sums
     int gap_blocks = 0;
     double *gap_out = nullptr;      // 8 doubles on the device
@@ -152,7 +158,8 @@ cudaError_t launch_validate(Glm &g, bool values = true, bool rest = true); // th
 cudaError_t launch_sqnorm(Glm &g);
 cudaError_t launch_partition(Glm &g, int32_t K, uint64_t seed);           // fills owner, members
 cudaError_t launch_partition_chunks(Glm &g, int32_t K, int64_t C, const int64_t *chunk_off, const int32_t *chunk_task); // device arrays
-cudaError_t launch_permutation(Glm &g, int64_t round, int64_t epochs);    // fills perm[epochs * n_coord]
+cudaError_t launch_permutation(Glm &g, int64_t round, int64_t epochs, int64_t H, const int64_t *steps); // fills perm[epochs * n_coord]
+                                                                          // as far as a round of H steps (or the device's K budgets) walks
 cudaError_t launch_local_solver(Glm &g, int64_t H, float sigma_prime, int *variant);
 cudaError_t launch_reduce(Glm &g);                                        // v += sum_k U_k ; U = 0 ; resid
 cudaError_t launch_sum_updates(Glm &g, float *delta);                     // delta = sum_k U_k ; U = 0 (v untouched)
