@@ -319,8 +319,10 @@ chicle_status_t chicle_glm_create(const chicle_matrix_t *X, const float *labels,
     }
     e = launch_sqnorm(*h);
     if (e == cudaSuccess) e = launch_refresh_resid(*h);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_status, h->d_status + kStatusMaxNorm, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return bail_cuda(e, "preprocessing kernels");
+    std::memcpy(&h->max_sqnorm, h->h_status, sizeof(float));
     *out = h;
     return CHICLE_OK;
 }

@@ -20,6 +20,8 @@ enum : uint32_t {
     ST_BOUNDS = 1u << 5,           // a -DCHICLE_DEBUG_BOUNDS build: an index that a kernel loaded lay outside its array
 };
 
+constexpr int kStatusMaxNorm = 8; // the word of the status buffer where the largest squared norm is found
+
 // A -DCHICLE_DEBUG_BOUNDS build checks every index that the solvers and the gap kernels load from memory (visiting
 // order entries, row extents, entry ids, record directory entries, record sizes) before it is used as an address.
 // A failed check sets ST_BOUNDS in the status word and the access is skipped (the value is replaced by a harmless
@@ -88,6 +90,7 @@ struct Glm {
     float *values = nullptr;
     float *labels = nullptr; // per example
     float *sqnorm = nullptr; // per coordinate
+    float max_sqnorm = 0.f;  // the largest of them
     float *alpha = nullptr;  // per coordinate: signed dual variable, or w for ridge
     float *v = nullptr;      // shared vector, dim
     float *resid = nullptr;  // ridge only: v - y, refreshed by the reduction kernel
@@ -127,6 +130,8 @@ struct Glm {
     int la_depth = 2;                // blocks the dot products are taken ahead of the recurrence (2: with cross Gram matrices)
     bool la_overlap = true;          // prepare kernels beside the chain kernels (side stream) or alternating with them
     int32_t la_nzcap = 0, la_hotc = 0; // non-zeros per worker record; entry ids per CTA kept in shared memory
+    int32_t la_tab_bins = 0;         // logistic: bins per coordinate of the step's tables (0: none)
+    size_t la_tab_off = 0;           // where they lie in a region
     size_t la_smem = 0;              // dynamic shared memory of the chain kernel
     int la_last_slices = 0;          // slices of the last round
     int solver_launches = 0;         // kernels the local solvers launched in the round being enqueued

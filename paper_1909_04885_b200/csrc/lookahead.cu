@@ -55,18 +55,19 @@ constexpr int kIdBits = 26;        // entry ids of a staged non-zero (problems w
 constexpr uint32_t kIdMask = (1u << kIdBits) - 1u;
 constexpr int kChainThreads = 512;
 constexpr int kSubSlots = 4;       // worker records in shared memory: blocks b .. b + 3
-constexpr int kHeadSlots = 3;      // recurrence records in shared memory
+constexpr int kHeadSlots = 2;      // recurrence records (and tables of the logistic step, see tab_map) in shared memory
 // Worker warps: all but the warps that share warp 0's scheduler (warp ids 0, 4, 8, 12), which stay out of its way.
 constexpr int kWorkWarps = 12;
 constexpr int kWorkThreads = kWorkWarps * 32;
 constexpr int kBarWork = 1;        // named barrier of the worker warps
+constexpr int kFeedWarp = 4;       // in CTA 0: fetches the recurrence records and writes the new states (see the kernel)
 
 // Per-step constants for the recurrence warp (see coordinate_step for p0 .. p3).
 struct alignas(16) CHdr {
     int32_t coord;
     float p0, p1, p2, p3;
     float A, B; // the recurrence's state starts at A + B * (dot product against the older model) (+ the cross terms)
-    float lq;   // logistic: log of p2
+    float lq;   // logistic: log of p2; with tables: tab_map's `off`
 };
 static_assert(sizeof(CHdr) == 32, "header size");
 
@@ -125,6 +126,8 @@ struct LookParams {
     int64_t n_blocks;
     int64_t drop_block;          // test aid: this block's records are left unpublished (-1: none)
     int64_t nnz;                 // entries of the matrix (what a coordinate's extent is checked against in a debug build)
+    int32_t tab_bins;            // logistic: bins per coordinate of the tables (0: the root is solved on the chain)
+    unsigned long long tab_off;  // the tables start here in the region, one per block
     int32_t model_in;            // the round's first chain launch: row k of the update workspace holds U_k and is turned
                                  // into the local model w = v + sigma' U_k in place
     int32_t model_out;           // the round's last chain launch: the row is turned back into U_k. Between a round's
@@ -255,6 +258,124 @@ template <int LOSS> __device__ __forceinline__ float recurrence_map(float s, flo
     return logistic_root(s, p2, lq);
 }
 
+// ---- The logistic step from tables. a(c) = sigmoid(root of z + q sigmoid(z) = c) is a function of the state c alone once
+// the coordinate's q is known, and q does not depend on the model: the prepare kernel tabulates a(c) for each of a
+// block's coordinates as Taylor polynomials of degree 7, and a step of the chain is a look-up and a polynomial instead of
+// a root search (two exponentials, two divisions and two reciprocals one behind the other: 510 cycles, now about 90).
+// a(c) is analytic but for branch points at c0 +- i pi (where 1 + q a (1 - a) = 0) and their mirror images at q - c0, and
+// a(q - c) = 1 - a(c), so u = min(c, q - c) is expanded about nodes whose distance grows like the distance to c0: with
+// x = (u - c0) / 3, four bins per octave of 1 + |x| on either side of c0. Beyond x = -7 (a below 1e-9) the last value
+// serves. In an fp32 emulation against the exact root the largest error of a is 1.6e-7 over q from 0 to 45 000, where
+// the two Halley steps of logistic_root leave 5.9e-7.
+constexpr int kTabNeg = 12;                // bins below c0: three octaves
+constexpr float kTabScale = 3.0f;
+constexpr float kTabInv = 1.0f / kTabScale;
+constexpr float kTabXmin = -6.99999f;      // (1 + |x| stays inside the third octave)
+__host__ __device__ constexpr uint32_t tab_bytes(int bins) { return (uint32_t)(kLB * bins) * 32u; }
+// Largest q whose bins fit (u - c0 <= q / 2 - c0 and -c0 <= log(1 + q) + 1): 32 bins have five octaves above c0, 64 thirteen.
+inline float tab_max_q(int bins) { return bins >= 64 ? 40000.0f : (bins >= 32 ? 160.0f : -1.0f); }
+
+__device__ __forceinline__ float tab_center(float q)
+{
+    const float rt = sqrtf(fmaf(q, q, 4.0f * q));
+    const float E = 2.0f / (2.0f + q + rt);
+    return logf(E) - (q > 1e-12f ? 2.0f * q / (q + rt) : 0.0f);
+}
+// What the chain adds to -|c - q / 2| / 3 to get x (kept inside the table whatever q is).
+__device__ __forceinline__ float tab_offset(float q, int bins)
+{
+    const float top = (float)(1 << ((bins - kTabNeg) >> 2));
+    return fminf((0.5f * q - tab_center(q)) * kTabInv, top * 0.999999f - 1.0f);
+}
+// Bin i of a coordinate's table: the coefficients of a(c0 + sgn * 3 * (|x|)) in |x| - (the bin's centre).
+__device__ __forceinline__ void tab_bin(float q, float log_q, int bins, int i, float4 &lo, float4 &hi)
+{
+    const int npos = bins - kTabNeg;
+    const bool neg = i >= npos;
+    const int n = neg ? i - npos : i;
+    const float yc = (float)(1 << (n >> 2)) * (1.0f + ((float)(n & 3) + 0.5f) * 0.25f);
+    const float step = neg ? -kTabScale : kTabScale;
+    float c = fmaf(step, yc - 1.0f, tab_center(q));
+    const bool flip = c > 0.5f * q;
+    if (flip) c = q - c;
+    // the root as in logistic_root, with a third Halley step (the coefficients inherit its error)
+    const float kappa = log_q + c;
+    float z = kappa <= 0.0f ? fminf(c, 0.0f) : fminf(c - (kappa - __logf(1.0f + kappa)), 0.0f);
+#pragma unroll
+    for (int it = 0; it < kRootIters + 1; ++it) {
+        const float e = __expf(z);
+        const float s = 1.0f + e, qe = q * e;
+        const float A = fmaf(z - c, s, qe), B = fmaf(s, s, qe), C = qe * (1.0f - e);
+        z = fminf(z - __fdividef(2.0f * A * B * s, fmaf(2.0f * B, B, -A * C)), 0.0f);
+    }
+    const float e = expf(z);
+    // a' = p / (1 + q p) with p = a (1 - a): Taylor coefficients a_k of a, p_k of p, y_k of a' one after the other
+    float a[8], p[8], y[7];
+    a[0] = e / (1.0f + e);
+    p[0] = a[0] * (1.0f - a[0]);
+    const float r = 1.0f / fmaf(q, p[0], 1.0f);
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+        float acc = 0.0f;
+#pragma unroll
+        for (int m = 1; m <= k; ++m) acc = fmaf(p[m], y[k - m], acc);
+        y[k] = fmaf(-q, acc, p[k]) * r;
+        a[k + 1] = y[k] * (1.0f / (float)(k + 1));
+        float sq = 0.0f;
+#pragma unroll
+        for (int m = 0; m <= k + 1; ++m) sq = fmaf(a[m], a[k + 1 - m], sq);
+        p[k + 1] = a[k + 1] - sq;
+    }
+    if (flip) { // a(q - c) = 1 - a(c)
+        a[0] = 1.0f - a[0];
+        a[2] = -a[2];
+        a[4] = -a[4];
+        a[6] = -a[6];
+    }
+    float w = step;
+#pragma unroll
+    for (int k = 1; k < 8; ++k) {
+        a[k] *= w;
+        w *= step;
+    }
+    lo = make_float4(a[0], a[1], a[2], a[3]);
+    hi = make_float4(a[4], a[5], a[6], a[7]);
+}
+// A block's table (all threads of the CTA; hdr: its coordinates' constants).
+__device__ __forceinline__ void write_table(const LookParams &P, int64_t bid, const CHdr *hdr, int threads)
+{
+    float4 *out = reinterpret_cast<float4 *>(P.rec + P.tab_off + (size_t)bid * tab_bytes(P.tab_bins));
+    const int bins = P.tab_bins, lg = bins >= 64 ? 6 : 5;
+    for (int i = threadIdx.x; i < kLB << lg; i += threads) {
+        const float q = hdr[i >> lg].p2;
+        float4 lo, hi;
+        tab_bin(q, q > 0.0f ? __logf(q) : -CUDART_INF_F, bins, i & (bins - 1), lo, hi);
+        out[2 * i] = lo;
+        out[2 * i + 1] = hi;
+    }
+}
+// a(c) from the table. h = q / 2; `row`: where the coordinate's table would have a bin of exponent 0; `on`: whether this
+// lane's result is wanted (the other lanes keep off the shared-memory pipe).
+__device__ __forceinline__ float tab_map(float c, float h, float off, uint32_t row, uint32_t neg, bool on, float4 &lo, float4 &hi)
+{
+    const float d = c - h;
+    const float x = fmaxf(fmaf(-fabsf(d), kTabInv, off), kTabXmin);
+    const float ax = fabsf(x), y = 1.0f + ax;
+    const uint32_t bits = __float_as_uint(y);
+    const float dl = ax - (__uint_as_float((bits & 0xffe00000u) | 0x00100000u) - 1.0f);
+    const uint32_t at = ((bits & 0xffe00000u) >> 16) + (x < 0.0f ? row + neg : row); // 32 bytes a bin
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %9, 0;\n\t"
+                 "@q ld.shared.v4.f32 {%0, %1, %2, %3}, [%8];\n\t@q ld.shared.v4.f32 {%4, %5, %6, %7}, [%8 + 16];\n\t}"
+                 : "+f"(lo.x), "+f"(lo.y), "+f"(lo.z), "+f"(lo.w), "+f"(hi.x), "+f"(hi.y), "+f"(hi.z), "+f"(hi.w)
+                 : "r"(at), "r"((uint32_t)on));
+    const float d2 = dl * dl, d4 = d2 * d2;
+    const float p01 = fmaf(lo.y, dl, lo.x), p23 = fmaf(lo.w, dl, lo.z), p45 = fmaf(hi.y, dl, hi.x), p67 = fmaf(hi.w, dl, hi.z);
+    const float v = fmaf(fmaf(p67, d2, p45), d4, fmaf(p23, d2, p01));
+    // (a state that is not finite gives a result that is not, as the root search would)
+    const float bias = fmaf(0.0f, c, d > 0.0f ? 1.0f : 0.0f);
+    return fmaf(v, d > 0.0f ? -1.0f : 1.0f, bias);
+}
+
 // The most frequent ids (ids are frequency-ranked) are in most of a block's coordinates. Their part of the Gram
 // matrices is taken from dense 32 x kHD tiles; only the other entries are walked through the table. Table slot: the id itself below kHD, a hashed slot above.
 constexpr int kHD = 32;
@@ -332,6 +453,7 @@ __device__ __forceinline__ void prepare_block(const LookParams &P, const int64_t
             int32_t c = P.S.perm[off + b * kLB + lane];
             checked_extent(P, c, rs, n);
             hd = make_hdr<LOSS>(P.S, c);
+            if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) hd.lq = tab_offset(hd.p2, P.tab_bins);
         }
         sh.hdr[lane] = hd;
         sh.rs[lane] = rs;
@@ -542,6 +664,7 @@ __device__ __forceinline__ void prepare_block(const LookParams &P, const int64_t
         for (int i = tid; i < kLB * kLB; i += THREADS) out.X[i] = 0.0f;
         return;
     }
+    if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) write_table(P, bid, sh.hdr, THREADS);
     // ---- the workers' record heads, shared-id tables and list starts
     if (tid < C) {
         SubHead &h = *reinterpret_cast<SubHead *>(P.rec + sh.sub_off[tid]);
@@ -813,15 +936,23 @@ __global__ void __launch_bounds__(THREADS) k_lookahead_prepare(const LookParams 
 
 // Short dense rows: every row has every id, so the lists are implicit: constants, Gram triangle, cross Gram matrix
 // and the rows themselves (one worker record: the model lives in one CTA).
+// All 64 visiting-order entries first, then all headers (a lane per coordinate) and all rows with every load of a thread
+// issued before the first is used: three round trips to memory per block. (A warp per row, headers by its first lane, was
+// a chain of 24 of them: 72 000 cycles per block at 28 entries per row, with the tables.)
 constexpr int kPreThreads = 256;
+constexpr int kPreDensePerSm = 4;
 struct PreDenseShared {
-    float row[2 * kLB][kCapL + 1]; // this block's rows, then the next block's
     CHdr hdr[kLB];
-    float gsc[kLB], ys[kLB], as[kLB], gscn[kLB];
+    float gsc[2 * kLB], ys[kLB], as[kLB];
+    int32_t coord[2 * kLB];
+    float T[kLB][2 * kLB + 1];       // scaled Gram entries: row l, this block's columns, then the next block's
     unsigned long long offset;
-    uint32_t bytes;
     int32_t walk;
+    alignas(16) float row[1];        // 64 rows of row_stride(dim) floats: this block's, then the next block's
 };
+// 16-byte pieces of consecutive rows lie on different banks
+__host__ __device__ constexpr int row_stride(int dim) { return (((dim + 3) / 4) | 1) * 4; }
+inline size_t pre_dense_bytes(int dim) { return sizeof(PreDenseShared) + 2 * kLB * (size_t)row_stride(dim) * sizeof(float); }
 
 template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const LookParams &P, const int64_t bid, PreDenseShared &sh)
 {
@@ -836,9 +967,14 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
     const int cnt = (int)((steps - b * kLB) < kLB ? (steps - b * kLB) : kLB);
     const int64_t left = steps - (b + 1) * kLB;
     const int ncnt = (left <= 0 || P.depth < 2) ? 0 : (left < kLB ? (int)left : kLB);
-    const int dim = (int)P.S.dim;
+    const int dim = (int)P.S.dim, stride = row_stride(dim);
     ChainHead &out = *reinterpret_cast<ChainHead *>(P.rec + (size_t)bid * sizeof(ChainHead));
-    if (tid == 0) {
+    if (tid < 2 * kLB) {
+        const bool on = tid < kLB ? tid < cnt : tid - kLB < ncnt;
+        int32_t c = on ? P.S.perm[off + b * kLB + tid] : -1; // (the next block's entries follow)
+        if (on && !CHICLE_IN_BOUNDS(P.S.status, c >= 0 && (int64_t)c < P.S.n_coord)) c = 0;
+        sh.coord[tid] = c;
+    } else if (tid == 2 * kLB) {
         const uint32_t bytes = sub_bytes(cnt * dim, 0, true);
         unsigned long long at = atomicAdd(P.cursor, (unsigned long long)bytes);
         BlkDir d;
@@ -869,48 +1005,108 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
         h.n = cnt * dim; h.T = 0; h.cnt = cnt; h.flags = 0;
     }
     if (!walk && tid < kLB + 8) reinterpret_cast<SubHead *>(rec)->roff[tid] = (uint16_t)((tid < cnt ? tid : cnt) * dim);
-    for (int j = warp; j < 2 * kLB; j += NW) {
-        const bool next = j >= kLB;
-        const int jj = next ? j - kLB : j;
-        const bool on = jj < (next ? ncnt : cnt);
-        int32_t c = 0;
-        if (on) c = P.S.perm[off + (b + (next ? 1 : 0)) * kLB + jj];
-        if (!CHICLE_IN_BOUNDS(P.S.status, c >= 0 && (int64_t)c < P.S.n_coord)) c = 0;
-        const int64_t rs = (int64_t)c * dim;
-        for (int e = lane; e < dim; e += 32) {
-            const float x = on ? P.S.values[rs + e] : 0.0f;
-            sh.row[j][e] = x;
-            if (on && !next && !walk) val_g[jj * dim + e] = x;
+    // ---- rows: a warp takes eight of the 64, in 16-byte pieces where rows start on such boundaries
+    constexpr int RPW = 2 * kLB / NW;
+    if ((dim & 3) == 0) {
+        const int nv = dim >> 2;
+        const int lpr = nv <= 8 ? 8 : (nv <= 16 ? 16 : 32); // lanes per row
+        const int sub = lane & (lpr - 1), per = 32 / lpr;   // rows per turn
+        float4 v[RPW];
+#pragma unroll
+        for (int u = 0; u < RPW; ++u) {
+            const int j = warp * RPW + u * per + lane / lpr;
+            v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (u * per < RPW && sub < nv && sh.coord[j] >= 0) v[u] = reinterpret_cast<const float4 *>(P.S.values + (int64_t)sh.coord[j] * dim)[sub];
         }
-        if (lane == 0) {
-            CHdr hd{0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            if (on) hd = make_hdr<LOSS>(P.S, c);
-            const float gs = on ? gram_scale<LOSS>(hd, P.S.sigma, P.S.inv_n) : 0.0f;
-            if (next) sh.gscn[jj] = gs;
-            else {
-                sh.hdr[jj] = hd;
-                sh.gsc[jj] = gs;
-                sh.ys[jj] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 1.0f : hd.p3;
-                sh.as[jj] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : hd.p1;
+#pragma unroll
+        for (int u = 0; u < RPW; ++u) {
+            const int j = warp * RPW + u * per + lane / lpr;
+            if (u * per < RPW && sub < nv) {
+                reinterpret_cast<float4 *>(sh.row + j * stride)[sub] = v[u];
+                if (j < cnt && !walk) reinterpret_cast<float4 *>(val_g + j * dim)[sub] = v[u];
+            }
+        }
+    } else {
+        for (int e0 = 0; e0 < 4 * ((dim + 3) / 4); e0 += 32) {
+            const int e = e0 + lane;
+            float v[RPW];
+#pragma unroll
+            for (int u = 0; u < RPW; ++u) {
+                const int j = warp * RPW + u;
+                v[u] = e < dim && sh.coord[j] >= 0 ? P.S.values[(int64_t)sh.coord[j] * dim + e] : 0.0f;
+            }
+#pragma unroll
+            for (int u = 0; u < RPW; ++u) {
+                const int j = warp * RPW + u;
+                if (e < 4 * ((dim + 3) / 4)) sh.row[j * stride + e] = v[u]; // (padded with zeros to a multiple of four)
+                if (e < dim && j < cnt && !walk) val_g[j * dim + e] = v[u];
             }
         }
     }
+    // ---- headers: warp 0 this block's coordinates, warp 1 the next block's
+    if (warp < 2) {
+        const int32_t c = sh.coord[warp * kLB + lane];
+        CHdr hd{0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (c >= 0) {
+            hd = make_hdr<LOSS>(P.S, c);
+            if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) hd.lq = tab_offset(hd.p2, P.tab_bins);
+        }
+        sh.gsc[warp * kLB + lane] = c >= 0 ? gram_scale<LOSS>(hd, P.S.sigma, P.S.inv_n) : 0.0f;
+        if (warp == 0) {
+            sh.hdr[lane] = hd;
+            sh.ys[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 1.0f : hd.p3;
+            sh.as[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : hd.p1;
+        }
+    }
     __syncthreads();
-    // a warp per column j; lane l has x_j . x_l: first inside the block (l < j), then from this block to the next
-    for (int j = warp; j < 2 * kLB; j += NW) {
-        const bool next = j >= kLB;
-        const int jj = next ? j - kLB : j;
-        float acc = 0.0f;
-        if (!walk && (next ? lane < cnt : lane < jj))
-            for (int e = 0; e < dim; ++e) acc = fmaf(sh.row[j][e], sh.row[lane][e], acc);
-        acc *= (next ? sh.gscn[jj] : sh.gsc[jj]) * sh.ys[lane];
-        (next ? out.X : out.G)[lane * kLB + jj] = acc;
-        float q0 = acc * sh.as[lane];
+    if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins && !walk) write_table(P, bid, sh.hdr, kPreThreads);
+    // ---- x_l . x_j for this block's l and the 64 columns j: a thread has l = lp, lp + 16 and j = jq, jq + 16, .. (every
+    //      sum over the entries in ascending order)
+    {
+        const int jq = tid & 15, lp = tid >> 4;
+        float acc[2][4];
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[a][c] = 0.0f;
+        if (!walk) {
+            const float *rl = sh.row + lp * stride, *rj = sh.row + jq * stride;
+            for (int e = 0; e < dim; e += 4) {
+                float4 xl[2], xj[4];
+#pragma unroll
+                for (int a = 0; a < 2; ++a) xl[a] = *reinterpret_cast<const float4 *>(rl + 16 * a * stride + e);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) xj[c] = *reinterpret_cast<const float4 *>(rj + 16 * c * stride + e);
+#pragma unroll
+                for (int a = 0; a < 2; ++a)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        acc[a][c] = fmaf(xj[c].x, xl[a].x, acc[a][c]);
+                        acc[a][c] = fmaf(xj[c].y, xl[a].y, acc[a][c]);
+                        acc[a][c] = fmaf(xj[c].z, xl[a].z, acc[a][c]);
+                        acc[a][c] = fmaf(xj[c].w, xl[a].w, acc[a][c]);
+                    }
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int l = lp + 16 * a, j = jq + 16 * c;
+                const bool on = c < 2 ? l < j : l < cnt; // inside the block: earlier coordinates only
+                const float v = on ? acc[a][c] * (sh.gsc[j] * sh.ys[l]) : 0.0f;
+                sh.T[l][j] = v;
+                (c < 2 ? out.G : out.X)[l * kLB + (j & (kLB - 1))] = v;
+            }
+    }
+    __syncthreads();
+    for (int j = warp; j < 2 * kLB; j += NW) { // what the states at round start contribute
+        float q0 = sh.T[lane][j] * sh.as[lane];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) q0 += __shfl_xor_sync(0xffffffffu, q0, o);
         if (lane == 0) {
-            if (next) out.q0n[jj] = q0;
-            else sh.hdr[jj].A -= q0;
+            if (j >= kLB) out.q0n[j - kLB] = q0;
+            else sh.hdr[j].A -= q0;
         }
     }
     __syncthreads();
@@ -918,7 +1114,7 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
 }
 
 // (blocks blockIdx.x, blockIdx.x + gridDim.x, ...: see k_lookahead_prepare)
-template <int LOSS> __global__ void __launch_bounds__(kPreThreads) k_lookahead_prepare_dense(const LookParams P)
+template <int LOSS> __global__ void __launch_bounds__(kPreThreads, kPreDensePerSm) k_lookahead_prepare_dense(const LookParams P)
 {
     extern __shared__ __align__(16) unsigned char smem_pre[];
     PreDenseShared &sh = *reinterpret_cast<PreDenseShared *>(smem_pre);
@@ -1053,21 +1249,23 @@ struct alignas(16) ChainCtl {
     uint64_t ackbar;               // CTA 0: every CTA has applied all updates (before a block is walked in place)
     alignas(16) float pbuf[2][kMaxC][kLB];
     alignas(16) float dbuf[2][kLB];
+    alignas(16) float sbuf[2][kLB]; // CTA 0: the block's new states (arrive with its deltas)
     float sink[32]; // where a lane's stores go that have no target
     int abort_flag;
     int done; // the CTA's workers are through (the warps with no role sleep until then)
 };
 
-// Shared-memory layout of the chain kernel (sizes fixed at launch): control, recurrence records, worker records,
-// products, the CTA's part of the model.
+// Shared-memory layout of the chain kernel (sizes fixed at launch): control, recurrence records, logistic tables,
+// worker records, products, the CTA's part of the model.
 struct ChainLayout {
-    uint32_t heads, subs, sub_stride, prod, w, total;
+    uint32_t heads, tabs, subs, sub_stride, prod, w, total;
 };
-__host__ __device__ inline ChainLayout chain_layout(int nzcap, int hotc, bool dense, int dim)
+__host__ __device__ inline ChainLayout chain_layout(int nzcap, int hotc, bool dense, int dim, int tab_bins)
 {
     ChainLayout L;
     L.heads = (uint32_t)((sizeof(ChainCtl) + 127) & ~(size_t)127);
-    L.subs = L.heads + kHeadSlots * (uint32_t)sizeof(ChainHead);
+    L.tabs = L.heads + kHeadSlots * (uint32_t)sizeof(ChainHead);
+    L.subs = L.tabs + kHeadSlots * tab_bytes(tab_bins);
     L.sub_stride = dense ? sub_bytes(kLB * dim, 0, true) : sub_bytes(nzcap, nzcap / 2, false);
     L.prod = L.subs + kSubSlots * L.sub_stride;
     L.w = L.prod + 4u * (uint32_t)(dense ? kLB : nzcap);
@@ -1075,7 +1273,7 @@ __host__ __device__ inline ChainLayout chain_layout(int nzcap, int hotc, bool de
     return L;
 }
 
-template <int LOSS, bool DENSE>
+template <int LOSS, bool DENSE, bool TAB>
 __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const LookParams P)
 {
     extern __shared__ __align__(128) unsigned char smem_chain[];
@@ -1084,7 +1282,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     const uint32_t crank = cluster_ctarank();
     const int k = (int)(blockIdx.x >> logC);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const ChainLayout L = chain_layout(P.nzcap, P.hotc, DENSE, (int)S.dim);
+    const ChainLayout L = chain_layout(P.nzcap, P.hotc, DENSE, (int)S.dim, TAB ? P.tab_bins : 0);
     ChainCtl &ctl = *reinterpret_cast<ChainCtl *>(smem_chain);
     float *W = reinterpret_cast<float *>(smem_chain + L.w);
     float *prod = reinterpret_cast<float *>(smem_chain + L.prod);
@@ -1092,7 +1290,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
 
     const int64_t nk = S.part_off[k + 1] - S.part_off[k];
     const int64_t steps = steps_of(P, k, nk);
-    const int64_t nb = (steps + kLB - 1) / kLB;
+    const int nb = (int)((steps + kLB - 1) / kLB); // (32-bit counters: 64-bit ones cost the chain hundreds of cycles a block)
     const int64_t bid0 = P.blk_base[k];
     float *Uk = S.U + (size_t)k * (size_t)S.dim;
     const float sigma = S.sigma;
@@ -1101,6 +1299,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     const uint32_t hot_total = (uint32_t)(hot_all < S.dim ? hot_all : S.dim);
     const int hot_mine = hot_total > crank ? (int)((hot_total - crank + C - 1) >> logC) : 0;
 
+    const uint32_t d_bytes = crank == 0 ? 2u * kLB * 4u : (uint32_t)kLB * 4u; // what a block's deltas (CTA 0: and states) bring
     if (tid == 0) {
         ctl.abort_flag = 0;
         ctl.done = 0;
@@ -1115,7 +1314,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         // armed for the first two blocks before anybody can send
         for (int i = 0; i < 2; ++i) {
             mbar_arrive_expect_tx(smem_u32(&ctl.pbar[i]), (uint32_t)(C * kLB * 4));
-            mbar_arrive_expect_tx(smem_u32(&ctl.dbar[i]), (uint32_t)(kLB * 4));
+            mbar_arrive_expect_tx(smem_u32(&ctl.dbar[i]), d_bytes);
         }
     }
     for (int l = tid; l < hot_mine; l += kChainThreads) {
@@ -1138,15 +1337,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     if (is_chain && nb > 0) {
         // ============================== the recurrence warp =====================================================
         const int q = lane & 7, rep = lane >> 3;
-        auto head_at = [&](int64_t blk) { return reinterpret_cast<const ChainHead *>(smem_chain + L.heads + (size_t)(blk % kHeadSlots) * sizeof(ChainHead)); };
-        auto issue_head = [&](int64_t blk) {
-            const bool on = blk < nb && lane == 0;
-            const int64_t at = blk < nb ? blk : nb - 1;
-            const uint32_t bar = smem_u32(&ctl.headfull[at % kHeadSlots]);
-            mbar_arrive_expect_tx_if(bar, (uint32_t)sizeof(ChainHead), on);
-            bulk_g2s_if(smem_u32(head_at(at)), P.rec + (size_t)(bid0 + at) * sizeof(ChainHead), (uint32_t)sizeof(ChainHead), bar, on);
-        };
-        for (int i = 0; i < kHeadSlots; ++i) issue_head(i);
+        const uint32_t tab_neg = TAB ? (uint32_t)(P.tab_bins - kTabNeg) * 32u : 0u;
         // where the deltas go: the copy `rep` of lane q sends the lane's four values to CTAs rep and rep + 4
         uint32_t d_dst[2], d_bar[2];
 #pragma unroll
@@ -1155,14 +1346,17 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             d_dst[i] = mapa_u32(smem_u32(&ctl.dbuf[0][4 * q]), c);
             d_bar[i] = mapa_u32(smem_u32(&ctl.dbar[0]), c);
         }
+        const uint32_t s_dst = smem_u32(&ctl.sbuf[0][4 * q]), s_bar = smem_u32(&ctl.dbar[0]); // (this CTA's own)
         float xs[4] = {0.f, 0.f, 0.f, 0.f}; // what the block before contributes to this block's states
-        int64_t fp = 0, sc = 0;            // staged blocks and walked blocks so far
+        int fp = 0, sc = 0;                // staged blocks and walked blocks so far
 #ifdef CHICLE_LA_TIMING
         long long tw = 0, tr = 0, te = 0, t0 = clock64(), t1 = 0;
 #endif
-        for (int64_t b = 0; b < nb; ++b) {
-            if (!mbar_wait_cluster(smem_u32(&ctl.headfull[b % kHeadSlots]), (uint32_t)(b / kHeadSlots) & 1u, abort_flag, S.status)) { aborted = true; break; }
-            const ChainHead &H = *head_at(b);
+#pragma unroll 1
+        for (int b = 0; b < nb; ++b) {
+            const int slot = b & (kHeadSlots - 1);
+            if (!mbar_wait_cluster(smem_u32(&ctl.headfull[slot]), (uint32_t)(b / kHeadSlots) & 1u, abort_flag, S.status)) { aborted = true; break; }
+            const ChainHead &H = *reinterpret_cast<const ChainHead *>(smem_chain + L.heads + (size_t)slot * sizeof(ChainHead));
             const int cnt = H.cnt;
             const uint32_t par = (uint32_t)(b & 1);
             if (H.flags & 1) {
@@ -1214,6 +1408,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
                     st_async_f32x4_if(d_dst[i] + par * (uint32_t)(kLB * 4), 0.f, 0.f, 0.f, 0.f, d_bar[i] + par * 8u, rep + 4 * i < C);
+                st_async_f32x4_if(s_dst + par * (uint32_t)(kLB * 4), 0.f, 0.f, 0.f, 0.f, s_bar + par * 8u, rep == 0);
                 xs[0] = xs[1] = xs[2] = xs[3] = 0.0f;
             } else {
                 // ---- four coordinates at a time. Lane q (and its copies q + 8, q + 16, q + 24, which compute the
@@ -1221,14 +1416,26 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 //      by itself, the four results are handed round, and every lane adds what they mean for its own
                 //      four, in this block and in the next.
                 float hp1[4], hp2[4], hp3[4], hlq[4], s[4], mine[4];
-                int32_t hcoord[4];
                 float hA[4], hB[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const CHdr &h = H.hdr[4 * q + i];
-                    hcoord[i] = h.coord; hp1[i] = h.p1; hp2[i] = h.p2; hp3[i] = h.p3; hlq[i] = h.lq; hA[i] = h.A; hB[i] = h.B;
+                    hp1[i] = h.p1; hp2[i] = h.p2; hp3[i] = h.p3; hlq[i] = h.lq; hA[i] = h.A; hB[i] = h.B;
                     mine[i] = 0.0f;
                 }
+                // with tables: half of q, and where each coordinate's table would have exponent 0
+                uint32_t row[4];
+                if (TAB) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        hp2[i] *= 0.5f;
+                        row[i] = smem_u32(smem_chain + L.tabs) + (uint32_t)slot * tab_bytes(P.tab_bins) + (uint32_t)((4 * q + i) * P.tab_bins) * 32u - (127u << 2) * 32u;
+                    }
+                }
+                float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo; // (the lanes whose result nobody wants keep what is there)
+                auto step_map = [&](float st, int i, bool on) {
+                    return TAB ? tab_map(st, hp2[i], hlq[i], row[i], tab_neg, on, lo, hi) : recurrence_map<LOSS>(st, hp2[i], hlq[i]);
+                };
                 const float4 q0n = *reinterpret_cast<const float4 *>(&H.q0n[4 * q]);
                 if (!mbar_wait_cluster(smem_u32(&ctl.pbar[fp & 1]), (uint32_t)(fp >> 1) & 1u, abort_flag, S.status)) { aborted = true; break; }
                 LA_T(tw);
@@ -1243,7 +1450,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 xs[0] = -q0n.x; xs[1] = -q0n.y; xs[2] = -q0n.z; xs[3] = -q0n.w;
                 const float4 *G4 = reinterpret_cast<const float4 *>(H.G); // G4[l * 8 + q]: row l, columns 4q .. 4q + 3
                 const float4 *X4 = reinterpret_cast<const float4 *>(H.X);
-#pragma unroll
+                // (with tables a loop: unrolled, the code outgrows the instruction cache and its fetches set the pace)
+#pragma unroll (TAB ? 1 : kLB / 4)
                 for (int g = 0; g < kLB / 4; ++g) {
                     float4 blk[4], nxt[4];
 #pragma unroll
@@ -1254,13 +1462,13 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                     // inside the group (the numbers matter on the lanes with q == g, where blk holds the group's own
                     // triangle; the others run the same instructions on copies)
                     float o[4];
-                    o[0] = recurrence_map<LOSS>(s[0], hp2[0], hlq[0]);
+                    o[0] = step_map(s[0], 0, q == g);
                     const float t1 = fmaf(o[0], blk[0].y, s[1]);
-                    o[1] = recurrence_map<LOSS>(t1, hp2[1], hlq[1]);
+                    o[1] = step_map(t1, 1, q == g);
                     const float t2 = fmaf(o[1], blk[1].z, fmaf(o[0], blk[0].z, s[2]));
-                    o[2] = recurrence_map<LOSS>(t2, hp2[2], hlq[2]);
+                    o[2] = step_map(t2, 2, q == g);
                     const float t3 = fmaf(o[2], blk[2].w, fmaf(o[1], blk[1].w, fmaf(o[0], blk[0].w, s[3])));
-                    o[3] = recurrence_map<LOSS>(t3, hp2[3], hlq[3]);
+                    o[3] = step_map(t3, 3, q == g);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) mine[i] = q == g ? o[i] : mine[i];
                     float og[4];
@@ -1280,40 +1488,41 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                     }
                 }
                 LA_T(tr);
-                float dl[4];
+                if (TAB) { // (not kept in registers over the steps)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const CHdr &h = H.hdr[4 * q + i];
+                        hp1[i] = h.p1; hp3[i] = h.p3;
+                    }
+                }
+                float dl[4], st[4];
+                bool odd = false; // a step that is not finite
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const int j = 4 * q + i;
-                    float my_delta = 0.0f;
-                    if (j < cnt) {
-                        float my_state;
-                        if (LOSS == CHICLE_LOSS_RIDGE_PRIMAL) {
-                            my_delta = mine[i];
-                            my_state = hp1[i] + mine[i];
-                        } else {
-                            my_delta = hp3[i] * (mine[i] - hp1[i]);
-                            my_state = hp3[i] * mine[i];
-                        }
-                        if (!(fabsf(my_delta) <= CUDART_MAX_NORMAL_F)) {
-                            atomicOr(S.status, ST_NONFINITE_STEP);
-                            my_delta = 0.0f;
-                            my_state = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? hp1[i] : hp3[i] * hp1[i];
-                        }
-                        if (CHICLE_IN_BOUNDS(S.status, hcoord[i] >= 0 && (int64_t)hcoord[i] < S.n_coord))
-                            S.alpha[hcoord[i]] = my_state; // (the four copies of a lane store the same value)
+                    const bool in = 4 * q + i < cnt;
+                    if (LOSS == CHICLE_LOSS_RIDGE_PRIMAL) {
+                        dl[i] = mine[i];
+                        st[i] = hp1[i] + mine[i];
+                    } else {
+                        dl[i] = hp3[i] * (mine[i] - hp1[i]);
+                        st[i] = hp3[i] * mine[i];
                     }
-                    dl[i] = my_delta;
+                    const bool fine = fabsf(dl[i]) <= CUDART_MAX_NORMAL_F;
+                    odd |= in && !fine;
+                    if (!fine) st[i] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? hp1[i] : hp3[i] * hp1[i];
+                    if (!in || !fine) dl[i] = 0.0f;
                 }
                 // armed for block fp + 2 before the deltas go out (its dot products are sent only after they arrive)
                 mbar_arrive_expect_tx_if(smem_u32(&ctl.pbar[fp & 1]), (uint32_t)(C * kLB * 4), lane == 0);
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
                     st_async_f32x4_if(d_dst[i] + par * (uint32_t)(kLB * 4), dl[0], dl[1], dl[2], dl[3], d_bar[i] + par * 8u, rep + 4 * i < C);
+                st_async_f32x4_if(s_dst + par * (uint32_t)(kLB * 4), st[0], st[1], st[2], st[3], s_bar + par * 8u, rep == 0);
                 ++fp;
+                if (__any_sync(0xffffffffu, odd) && lane == 0) atomicOr(S.status, ST_NONFINITE_STEP);
                 LA_T(te);
             }
             __syncwarp();
-            issue_head(b + kHeadSlots);
         }
 #ifdef CHICLE_LA_TIMING
         if (blockIdx.x == 0 && lane == 0) {
@@ -1322,6 +1531,33 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         }
 #endif
     }
+    if (crank == 0 && warp == kFeedWarp && nb > 0) {
+        // ============================== the feeder: what the recurrence warp need not do itself =====================
+        // When a block's deltas have arrived here, the recurrence warp is done with the block's head: its new states go
+        // to global memory and the head (and table) two blocks on into its slot. (The recurrence warp waits for that
+        // head before it sends deltas on this barrier again, so the feeder never misses a phase.)
+        const uint32_t tab_len = TAB ? tab_bytes(P.tab_bins) : 0u;
+        const uint32_t heads0 = smem_u32(smem_chain + L.heads), tabs0 = smem_u32(smem_chain + L.tabs);
+        auto issue_head = [&](int blk, int slot) {
+            const bool on = blk < nb && lane == 0;
+            const uint32_t bar = smem_u32(&ctl.headfull[slot]);
+            const size_t at = (size_t)(bid0 + (blk < nb ? blk : nb - 1));
+            mbar_arrive_expect_tx_if(bar, (uint32_t)sizeof(ChainHead) + tab_len, on);
+            bulk_g2s_if(heads0 + (uint32_t)slot * (uint32_t)sizeof(ChainHead), P.rec + at * sizeof(ChainHead), (uint32_t)sizeof(ChainHead), bar, on);
+            if (TAB) bulk_g2s_if(tabs0 + (uint32_t)slot * tab_len, P.rec + P.tab_off + at * tab_len, tab_len, bar, on);
+        };
+        for (int i = 0; i < kHeadSlots; ++i) issue_head(i, i);
+#pragma unroll 1
+        for (int b = 0; b < nb; ++b) {
+            const int slot = b & (kHeadSlots - 1);
+            if (!mbar_wait_cluster(smem_u32(&ctl.dbar[b & 1]), (uint32_t)(b >> 1) & 1u, abort_flag, S.status)) break;
+            const ChainHead &H = *reinterpret_cast<const ChainHead *>(smem_chain + L.heads + (size_t)slot * sizeof(ChainHead));
+            const int32_t c = H.hdr[lane].coord;
+            if (lane < H.cnt && !(H.flags & 1) && CHICLE_IN_BOUNDS(S.status, c >= 0 && (int64_t)c < S.n_coord)) S.alpha[c] = ctl.sbuf[b & 1][lane];
+            __syncwarp();
+            issue_head(b + kHeadSlots, slot);
+        }
+    }
     if (is_worker && nb > 0) {
         // ============================== the worker warps ========================================================
         const int wt = (warp - 1 - (warp >> 2)) * 32 + lane; // 0 .. kWorkThreads - 1
@@ -1329,17 +1565,17 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         const uint32_t p_buf0 = mapa_u32(smem_u32(&ctl.pbuf[0][crank][0]), 0u);
         const uint32_t ack_bar = mapa_u32(smem_u32(&ctl.ackbar), 0u);
         const int dim = (int)S.dim;
-        auto sub_at = [&](int64_t blk) { return smem_chain + L.subs + (size_t)(blk & (kSubSlots - 1)) * L.sub_stride; };
+        auto sub_at = [&](int blk) { return smem_chain + L.subs + (size_t)(blk & (kSubSlots - 1)) * L.sub_stride; };
         // The directory entry of a block is loaded a block ahead of its use (an unconditional load from a clamped
         // address, so that nothing has to wait for it at the point of issue).
-        auto load_dir = [&](int64_t blk, uint32_t (&d)[4]) {
-            const int64_t at = blk < nb ? blk : nb - 1;
+        auto load_dir = [&](int blk, uint32_t (&d)[4]) {
+            const int at = blk < nb ? blk : nb - 1;
             asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
                          : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
                          : "l"(P.dirS + (((bid0 + at) << logC) + crank))
                          : "memory");
         };
-        auto issue_sub = [&](int64_t blk, const uint32_t (&d)[4]) {
+        auto issue_sub = [&](int blk, const uint32_t (&d)[4]) {
             const uint32_t bar = smem_u32(&ctl.subfull[blk & (kSubSlots - 1)]);
             // (the slot is only ever written by the copy engine and read by loads that are done by now)
             const unsigned long long offset = ((unsigned long long)d[1] << 32) | d[0];
@@ -1364,14 +1600,14 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             load_dir(2, d); issue_sub(2, d); sl2 = nb > 2 && (d[3] & 1u) != 0u;
             load_dir(3, d); issue_sub(3, d); sl3 = nb > 3 && (d[3] & 1u) != 0u;
         }
-        int64_t fg = 0; // staged blocks whose dot products have been sent
+        int fg = 0; // staged blocks whose dot products have been sent
         bool failed = false; // this warp gave up a wait (voted on at the next barrier)
 #ifdef CHICLE_LA_TIMING
         long long wd = 0, ws = 0, wg = 0, ws1 = 0, wg0 = 0, wg1 = 0, t0 = clock64(), t1 = 0;
 #endif
 
         // Block x's dot products against the model as it is now (this CTA's part), sent to CTA 0.
-        auto take_dots = [&](int64_t x) -> bool {
+        auto take_dots = [&](int x) -> bool {
             // Every warp waits for the record by itself (a barrier costs more than 200 cycles); a warp whose wait runs out
             // skips the work and says so at the next barrier's vote, so that all warps still meet there.
             bool ok = mbar_wait_cluster(smem_u32(&ctl.subfull[x & (kSubSlots - 1)]), (uint32_t)(x >> 2) & 1u, abort_flag, S.status);
@@ -1488,7 +1724,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         if (depth == 2) { sl2 = sl0; sl3 = sl1; sl0 = false; sl1 = false; } // flags of blocks b .. b + 3 for b = -2
         else { sl3 = sl2; sl2 = sl1; sl1 = sl0; sl0 = false; }              // ... for b = -1
 #pragma unroll 1
-        for (int64_t b = -depth; b < nb && !aborted; ++b) {
+        for (int b = -depth; b < nb && !aborted; ++b) {
             uint32_t dn[4];
             load_dir(b + kSubSlots, dn);
             const uint32_t par = (uint32_t)(b & 1);
@@ -1645,7 +1881,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 work_bar();
             }
             if (b >= 0) {
-                mbar_arrive_expect_tx_if(smem_u32(&ctl.dbar[par]), (uint32_t)(kLB * 4), wt == 0); // for block b + 2
+                mbar_arrive_expect_tx_if(smem_u32(&ctl.dbar[par]), d_bytes, wt == 0); // for block b + 2
                 issue_sub(b + kSubSlots, dn); // block b's slot is free
             }
             LA_T(ws);
@@ -1712,9 +1948,9 @@ __global__ void k_block_bases_slices(const int64_t *__restrict__ slice, int32_t 
     out[K] = run;
 }
 
-template <int LOSS, bool DENSE> cudaError_t launch_chain(Glm &g, const LookParams &P)
+template <int LOSS, bool DENSE, bool TAB> cudaError_t launch_chain(Glm &g, const LookParams &P)
 {
-    auto kern = k_lookahead_chain<LOSS, DENSE>;
+    auto kern = k_lookahead_chain<LOSS, DENSE, TAB>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.la_smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -1773,12 +2009,13 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
     const int chain_sms = g.K << g.la_logC;
     const unsigned free_sms = (unsigned)(g.sm_count > chain_sms ? g.sm_count - chain_sms : 1);
     if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) {
-        const unsigned per_sm = 4;
+        const unsigned per_sm = kPreDensePerSm;
+        const size_t smem = pre_dense_bytes((int)g.dim);
         const unsigned grid = stream == g.stream || nb < free_sms * per_sm ? nb : free_sms * per_sm;
         auto pre = k_lookahead_prepare_dense<LOSS>;
-        cudaError_t e = cudaFuncSetAttribute(pre, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PreDenseShared));
+        cudaError_t e = cudaFuncSetAttribute(pre, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        pre<<<grid, kPreThreads, sizeof(PreDenseShared), stream>>>(P);
+        pre<<<grid, kPreThreads, smem, stream>>>(P);
         return cudaGetLastError();
     }
     cudaError_t e;
@@ -1808,8 +2045,10 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
 
 template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P)
 {
-    if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) return launch_chain<LOSS, true>(g, P);
-    return launch_chain<LOSS, false>(g, P);
+    constexpr bool tables = LOSS == CHICLE_LOSS_LOGISTIC_DUAL;
+    const bool dense = g.fmt == CHICLE_FMT_DENSE_ROWMAJOR;
+    if (tables && P.tab_bins) return dense ? launch_chain<LOSS, true, tables>(g, P) : launch_chain<LOSS, false, tables>(g, P);
+    return dense ? launch_chain<LOSS, true, false>(g, P) : launch_chain<LOSS, false, false>(g, P);
 }
 
 // A round's launches, slice after slice (consecutive pieces of every partition's walk). The first slice's prepare
@@ -1902,6 +2141,17 @@ void lookahead_plan(Glm &g, int32_t K)
         if (env && (env[0] == '0' || env[0] == '1') && env[1] == 0) g.la_overlap = env[0] == '1';
     }
     const size_t budget = (size_t)(g.max_smem_optin > 0 ? g.max_smem_optin : 227 * 1024);
+    // logistic tables: as many bins as the largest q = sigma' |x|^2 / (lambda n) at sigma' = K needs (a round with a larger
+    // sigma' solves the roots on the chain), if two blocks' tables fit beside the rest
+    g.la_tab_bins = 0;
+    if (g.loss == CHICLE_LOSS_LOGISTIC_DUAL) {
+        const float q_max = (float)K * g.max_sqnorm / (g.lambda * (float)g.n_examples);
+        for (int bins = 64; bins >= 32; bins >>= 1)
+            if (q_max <= tab_max_q(bins)) g.la_tab_bins = bins;
+        if (dense && chain_layout(0, (int)g.dim, true, (int)g.dim, g.la_tab_bins).total > budget) g.la_tab_bins = 0;
+        const char *env = getenv("CHICLE_LA_TABLES"); // 0: none (tests)
+        if (env && env[0] == '0') g.la_tab_bins = 0;
+    }
     if (dense) {
         g.la_nzcap = 0;
         g.la_hotc = (int32_t)g.dim;
@@ -1910,13 +2160,13 @@ void lookahead_plan(Glm &g, int32_t K)
         g.la_hotc = 0;
     } else {
         g.la_nzcap = logC == 0 ? 2048 : (logC == 1 ? 1536 : 1024);
-        const ChainLayout L0 = chain_layout(g.la_nzcap, 0, false, (int)g.dim);
+        const ChainLayout L0 = chain_layout(g.la_nzcap, 0, false, (int)g.dim, g.la_tab_bins);
         int64_t hotc = ((int64_t)budget - (int64_t)L0.total - 64) / 4;
         hotc = hotc < 0 ? 0 : (hotc / 32) * 32;
         const int64_t need = (g.dim + ((int64_t)1 << logC) - 1) >> logC; // per CTA for the whole model
         g.la_hotc = (int32_t)(hotc < need ? hotc : (need + 31) / 32 * 32);
     }
-    g.la_smem = chain_layout(g.la_nzcap, g.la_hotc, dense, (int)g.dim).total;
+    g.la_smem = chain_layout(g.la_nzcap, g.la_hotc, dense, (int)g.dim, g.la_tab_bins).total;
 
     // slices: at most a sixteenth of the walk, but at least 256 blocks per partition; three regions
     const int64_t n = g.n_coord;
@@ -1947,8 +2197,10 @@ void lookahead_plan(Glm &g, int32_t K)
         pool = (size_t)part + (size_t)region_blocks * C * 128 + 4096;
     }
     const size_t heads = ((size_t)region_blocks * sizeof(ChainHead) + 255) & ~(size_t)255;
-    g.la_pool_off = heads;
-    g.la_region_bytes = (heads + pool + 255) & ~(size_t)255;
+    const size_t tabs = (size_t)region_blocks * tab_bytes(g.la_tab_bins);
+    g.la_tab_off = heads;
+    g.la_pool_off = heads + tabs;
+    g.la_region_bytes = (heads + tabs + pool + 255) & ~(size_t)255;
     g.la_dir_bytes = (size_t)g.la_regions * (size_t)region_blocks * C * sizeof(BlkDir);
 }
 
@@ -2034,6 +2286,7 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const char *drop = getenv("CHICLE_TEST_DROP_RECORD"); // test aid: leave one block's records unpublished
     const size_t C = (size_t)1 << g.la_logC;
+    const bool tables = g.la_tab_bins > 0 && S.sigma * g.max_sqnorm <= tab_max_q(g.la_tab_bins) * S.lam_n;
     std::vector<LookParams> P((size_t)Sn);
     for (int s = 0; s < Sn; ++s) {
         const int r = s % g.la_regions;
@@ -2058,6 +2311,8 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
         p.n_blocks = blocks[(size_t)s];
         p.drop_block = (drop && s == 0) ? atoll(drop) : -1;
         p.nnz = g.nnz;
+        p.tab_bins = tables ? g.la_tab_bins : 0;
+        p.tab_off = g.la_tab_off;
         p.model_in = s == 0 ? 1 : 0;
         p.model_out = s == Sn - 1 ? 1 : 0;
     }

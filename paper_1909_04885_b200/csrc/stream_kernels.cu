@@ -59,10 +59,11 @@ __global__ void k_validate_structure(const int64_t *__restrict__ indptr, const i
 // ---------------------------------------------------------------------------------------- squared norms
 __global__ void __launch_bounds__(kThreads)
 k_sqnorm(const int64_t *__restrict__ indptr, const float *__restrict__ values, int64_t n_coord, int64_t dim,
-         float *__restrict__ out)
+         float *__restrict__ out, uint32_t *__restrict__ largest /* bits of the largest norm, 0 before the call */)
 {
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * kWarpsPerBlock;
+    float most = 0.0f;
     for (int64_t c = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5); c < n_coord; c += nw) {
         const int64_t b = indptr ? indptr[c] : c * dim;
         const int64_t e = indptr ? indptr[c + 1] : b + dim;
@@ -73,7 +74,9 @@ k_sqnorm(const int64_t *__restrict__ indptr, const float *__restrict__ values, i
         }
         s = warp_sum_d(s);
         if (lane == 0) out[c] = (float)s;
+        most = fmaxf(most, (float)s);
     }
+    if (lane == 0 && most > 0.0f) atomicMax(largest, __float_as_uint(most)); // (positive floats order like their bits)
 }
 
 // ---------------------------------------------------------------------------------------- aggregation (a5)
@@ -701,7 +704,7 @@ cudaError_t launch_validate(Glm &g, bool values, bool rest)
 cudaError_t launch_sqnorm(Glm &g)
 {
     const unsigned grid = (unsigned)g.sm_count * 8;
-    k_sqnorm<<<grid, kThreads, 0, g.stream>>>(g.indptr, g.values, g.n_coord, g.dim, g.sqnorm);
+    k_sqnorm<<<grid, kThreads, 0, g.stream>>>(g.indptr, g.values, g.n_coord, g.dim, g.sqnorm, g.d_status + kStatusMaxNorm);
     return cudaGetLastError();
 }
 
