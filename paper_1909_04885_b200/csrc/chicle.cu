@@ -582,7 +582,7 @@ static chicle_status_t round_impl(chicle_glm_t *h, int64_t H, const int64_t *hos
         r.solver_variant = variant;
         if (variant >= 4) (void)cudaEventElapsedTime(&r.ms_prepare, h->ev[1], h->ev[4]);
         r.solver_slices = variant >= 4 ? h->la_last_slices : 0;
-        r.cluster_ctas = variant == 4 ? (1 << h->la_logC) : 1;
+        r.cluster_ctas = variant >= 4 ? (1 << h->la_logC) : 1;
         r.solver_launches = steps > 0 ? (h->solver_launches > 0 ? h->solver_launches : 1) : 0;
         r.order_launches = h->order_launches;
         *stats = r;

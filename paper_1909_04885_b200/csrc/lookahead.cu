@@ -50,7 +50,8 @@ namespace {
 
 constexpr int kLB = 32;            // steps per block
 constexpr int kMaxC = 8;           // CTAs per cluster at most (the portable limit)
-constexpr int kCapL = 128;         // longest dense coordinate
+constexpr int kDenseSlice = 384;   // columns of a dense row that one CTA of a cluster can take (a worker thread each)
+constexpr int kDenseEasy = 128;    // and what it takes where the cluster may be larger
 constexpr int kIdBits = 26;        // entry ids of a staged non-zero (problems with more ids take the blocked solver)
 constexpr uint32_t kIdMask = (1u << kIdBits) - 1u;
 constexpr int kChainThreads = 512;
@@ -87,7 +88,7 @@ static_assert(sizeof(ChainHead) % 16 == 0, "bulk copy size");
 // the coordinate's place in the block above them, the top bit marks an id that several coordinates of the block
 // have), ids[T] u32 (those shared ids), cpos[n] u16 (for a non-zero with a shared id: its place in the id's list;
 // the lists lie one after the other, each in ascending coordinate order), off[T + 1] u16 (where each list starts).
-// Dense: val[cnt * dim].
+// Dense: val[cnt][slice of the row, padded to a multiple of four].
 struct alignas(16) SubHead {
     int32_t n;     // non-zeros of the block that fall to this CTA
     int32_t T;     // shared ids among them
@@ -946,13 +947,18 @@ struct PreDenseShared {
     float gsc[2 * kLB], ys[kLB], as[kLB];
     int32_t coord[2 * kLB];
     float T[kLB][2 * kLB + 1];       // scaled Gram entries: row l, this block's columns, then the next block's
-    unsigned long long offset;
     int32_t walk;
-    alignas(16) float row[1];        // 64 rows of row_stride(dim) floats: this block's, then the next block's
+    unsigned long long sub_off[kMaxC];
+    alignas(16) float row[1];        // 64 rows of row_stride(columns at a time) floats: this block's, then the next block's
 };
+// Rows go through shared memory this many columns at a time (four CTAs per SM either way).
+constexpr int kDenseCols = 128;
 // 16-byte pieces of consecutive rows lie on different banks
-__host__ __device__ constexpr int row_stride(int dim) { return (((dim + 3) / 4) | 1) * 4; }
-inline size_t pre_dense_bytes(int dim) { return sizeof(PreDenseShared) + 2 * kLB * (size_t)row_stride(dim) * sizeof(float); }
+__host__ __device__ constexpr int row_stride(int cols) { return (((cols + 3) / 4) | 1) * 4; }
+inline size_t pre_dense_bytes(int dim)
+{
+    return sizeof(PreDenseShared) + 2 * kLB * (size_t)row_stride(dim < kDenseCols ? dim : kDenseCols) * sizeof(float);
+}
 
 template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const LookParams &P, const int64_t bid, PreDenseShared &sh)
 {
@@ -967,7 +973,8 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
     const int cnt = (int)((steps - b * kLB) < kLB ? (steps - b * kLB) : kLB);
     const int64_t left = steps - (b + 1) * kLB;
     const int ncnt = (left <= 0 || P.depth < 2) ? 0 : (left < kLB ? (int)left : kLB);
-    const int dim = (int)P.S.dim, stride = row_stride(dim);
+    const int dim = (int)P.S.dim, C = 1 << P.logC, slice = P.hotc, stride = row_stride(dim < kDenseCols ? dim : kDenseCols);
+    auto cols_of = [&](int c) { return dim - c * slice < slice ? (dim > c * slice ? dim - c * slice : 0) : slice; }; // of a CTA
     ChainHead &out = *reinterpret_cast<ChainHead *>(P.rec + (size_t)bid * sizeof(ChainHead));
     if (tid < 2 * kLB) {
         const bool on = tid < kLB ? tid < cnt : tid - kLB < ncnt;
@@ -975,73 +982,35 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
         if (on && !CHICLE_IN_BOUNDS(P.S.status, c >= 0 && (int64_t)c < P.S.n_coord)) c = 0;
         sh.coord[tid] = c;
     } else if (tid == 2 * kLB) {
-        const uint32_t bytes = sub_bytes(cnt * dim, 0, true);
-        unsigned long long at = atomicAdd(P.cursor, (unsigned long long)bytes);
-        BlkDir d;
-        if (at + bytes > P.pool_cap) { // no room: walked in place
-            d.offset = (unsigned long long)bid * sizeof(ChainHead);
-            d.bytes = 16u;
-            d.flags = 1u;
-            sh.walk = 1;
-        } else {
-            d.offset = P.pool_off + at;
-            d.bytes = bytes;
-            d.flags = 0u;
-            sh.walk = 0;
+        unsigned long long need = 0;
+        for (int c = 0; c < C; ++c) need += sub_bytes(cnt * ((cols_of(c) + 3) & ~3), 0, true);
+        unsigned long long at = atomicAdd(P.cursor, need);
+        sh.walk = at + need > P.pool_cap ? 1 : 0; // no room: walked in place
+        for (int c = 0; c < C; ++c) {
+            BlkDir d;
+            if (sh.walk) {
+                d.offset = (unsigned long long)bid * sizeof(ChainHead);
+                d.bytes = 16u;
+                d.flags = 1u;
+            } else {
+                d.offset = P.pool_off + at;
+                d.bytes = sub_bytes(cnt * ((cols_of(c) + 3) & ~3), 0, true);
+                d.flags = 0u;
+                at += d.bytes;
+            }
+            sh.sub_off[c] = d.offset;
+            if (bid == P.drop_block) d.bytes = 0u;
+            P.dirS[bid * C + c] = d;
         }
-        sh.offset = d.offset;
-        if (bid == P.drop_block) d.bytes = 0u;
-        P.dirS[bid] = d;
         out.cnt = cnt;
         out.flags = sh.walk;
         out.pad[0] = out.pad[1] = 0;
     }
     __syncthreads();
     const bool walk = sh.walk != 0;
-    unsigned char *rec = P.rec + sh.offset;
-    float *val_g = reinterpret_cast<float *>(rec + sizeof(SubHead));
-    if (!walk && tid == 0) {
-        SubHead &h = *reinterpret_cast<SubHead *>(rec);
-        h.n = cnt * dim; h.T = 0; h.cnt = cnt; h.flags = 0;
-    }
-    if (!walk && tid < kLB + 8) reinterpret_cast<SubHead *>(rec)->roff[tid] = (uint16_t)((tid < cnt ? tid : cnt) * dim);
-    // ---- rows: a warp takes eight of the 64, in 16-byte pieces where rows start on such boundaries
-    constexpr int RPW = 2 * kLB / NW;
-    if ((dim & 3) == 0) {
-        const int nv = dim >> 2;
-        const int lpr = nv <= 8 ? 8 : (nv <= 16 ? 16 : 32); // lanes per row
-        const int sub = lane & (lpr - 1), per = 32 / lpr;   // rows per turn
-        float4 v[RPW];
-#pragma unroll
-        for (int u = 0; u < RPW; ++u) {
-            const int j = warp * RPW + u * per + lane / lpr;
-            v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (u * per < RPW && sub < nv && sh.coord[j] >= 0) v[u] = reinterpret_cast<const float4 *>(P.S.values + (int64_t)sh.coord[j] * dim)[sub];
-        }
-#pragma unroll
-        for (int u = 0; u < RPW; ++u) {
-            const int j = warp * RPW + u * per + lane / lpr;
-            if (u * per < RPW && sub < nv) {
-                reinterpret_cast<float4 *>(sh.row + j * stride)[sub] = v[u];
-                if (j < cnt && !walk) reinterpret_cast<float4 *>(val_g + j * dim)[sub] = v[u];
-            }
-        }
-    } else {
-        for (int e0 = 0; e0 < 4 * ((dim + 3) / 4); e0 += 32) {
-            const int e = e0 + lane;
-            float v[RPW];
-#pragma unroll
-            for (int u = 0; u < RPW; ++u) {
-                const int j = warp * RPW + u;
-                v[u] = e < dim && sh.coord[j] >= 0 ? P.S.values[(int64_t)sh.coord[j] * dim + e] : 0.0f;
-            }
-#pragma unroll
-            for (int u = 0; u < RPW; ++u) {
-                const int j = warp * RPW + u;
-                if (e < 4 * ((dim + 3) / 4)) sh.row[j * stride + e] = v[u]; // (padded with zeros to a multiple of four)
-                if (e < dim && j < cnt && !walk) val_g[j * dim + e] = v[u];
-            }
-        }
+    if (!walk && tid < C) {
+        SubHead &h = *reinterpret_cast<SubHead *>(P.rec + sh.sub_off[tid]);
+        h.n = cnt * cols_of(tid); h.T = 0; h.cnt = cnt; h.flags = 0;
     }
     // ---- headers: warp 0 this block's coordinates, warp 1 the next block's
     if (warp < 2) {
@@ -1058,10 +1027,10 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
             sh.as[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : hd.p1;
         }
     }
-    __syncthreads();
-    if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins && !walk) write_table(P, bid, sh.hdr, kPreThreads);
     // ---- x_l . x_j for this block's l and the 64 columns j: a thread has l = lp, lp + 16 and j = jq, jq + 16, .. (every
-    //      sum over the entries in ascending order)
+    //      sum over the entries in ascending order). The rows pass through shared memory kDenseCols columns at a time, and
+    //      this block's go into the workers' records on the way.
+    constexpr int RPW = 2 * kLB / NW; // rows a warp loads
     {
         const int jq = tid & 15, lp = tid >> 4;
         float acc[2][4];
@@ -1069,23 +1038,71 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
         for (int a = 0; a < 2; ++a)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[a][c] = 0.0f;
-        if (!walk) {
-            const float *rl = sh.row + lp * stride, *rj = sh.row + jq * stride;
-            for (int e = 0; e < dim; e += 4) {
-                float4 xl[2], xj[4];
+        for (int e0 = 0; e0 < dim; e0 += kDenseCols) {
+            const int cols = dim - e0 < kDenseCols ? dim - e0 : kDenseCols, cols4 = (cols + 3) & ~3;
+            if (e0 > 0) __syncthreads(); // the chunk before has been read
+            if ((dim & 3) == 0) { // rows start on 16-byte boundaries (and so do slices)
+                const int nv = cols >> 2;
+                const int lpr = nv <= 8 ? 8 : (nv <= 16 ? 16 : 32); // lanes per row
+                const int sub = lane & (lpr - 1), per = 32 / lpr;   // rows per turn
+                float4 v[RPW];
 #pragma unroll
-                for (int a = 0; a < 2; ++a) xl[a] = *reinterpret_cast<const float4 *>(rl + 16 * a * stride + e);
+                for (int u = 0; u < RPW; ++u) {
+                    const int j = warp * RPW + u * per + lane / lpr;
+                    v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (u * per < RPW && sub < nv && sh.coord[j] >= 0)
+                        v[u] = reinterpret_cast<const float4 *>(P.S.values + (int64_t)sh.coord[j] * dim + e0)[sub];
+                }
+                const int e = e0 + 4 * sub, c = e / slice;
+                float *val_g = reinterpret_cast<float *>(P.rec + (walk || c >= C ? 0 : sh.sub_off[c]) + sizeof(SubHead));
+                const int st = (cols_of(c) + 3) & ~3;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) xj[c] = *reinterpret_cast<const float4 *>(rj + 16 * c * stride + e);
-#pragma unroll
-                for (int a = 0; a < 2; ++a)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        acc[a][c] = fmaf(xj[c].x, xl[a].x, acc[a][c]);
-                        acc[a][c] = fmaf(xj[c].y, xl[a].y, acc[a][c]);
-                        acc[a][c] = fmaf(xj[c].z, xl[a].z, acc[a][c]);
-                        acc[a][c] = fmaf(xj[c].w, xl[a].w, acc[a][c]);
+                for (int u = 0; u < RPW; ++u) {
+                    const int j = warp * RPW + u * per + lane / lpr;
+                    if (u * per < RPW && sub < nv) {
+                        reinterpret_cast<float4 *>(sh.row + j * stride)[sub] = v[u];
+                        if (j < cnt && !walk) *reinterpret_cast<float4 *>(val_g + j * st + (e - c * slice)) = v[u];
                     }
+                }
+            } else {
+                for (int f = lane; f < cols4; f += 32) {
+                    const int e = e0 + f, c = e / slice;
+                    float v[RPW];
+#pragma unroll
+                    for (int u = 0; u < RPW; ++u) {
+                        const int j = warp * RPW + u;
+                        v[u] = f < cols && sh.coord[j] >= 0 ? P.S.values[(int64_t)sh.coord[j] * dim + e] : 0.0f;
+                    }
+                    float *val_g = reinterpret_cast<float *>(P.rec + (walk || c >= C ? 0 : sh.sub_off[c]) + sizeof(SubHead));
+                    const int st = c < C ? (cols_of(c) + 3) & ~3 : 0;
+#pragma unroll
+                    for (int u = 0; u < RPW; ++u) {
+                        const int j = warp * RPW + u;
+                        sh.row[j * stride + f] = v[u];
+                        if (j < cnt && !walk && c < C && e - c * slice < st) val_g[j * st + (e - c * slice)] = v[u]; // (with the zero padding)
+                    }
+                }
+            }
+            __syncthreads();
+            if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins && !walk && e0 == 0) write_table(P, bid, sh.hdr, kPreThreads);
+            if (!walk) {
+                const float *rl = sh.row + lp * stride, *rj = sh.row + jq * stride;
+                for (int e = 0; e < cols; e += 4) {
+                    float4 xl[2], xj[4];
+#pragma unroll
+                    for (int a = 0; a < 2; ++a) xl[a] = *reinterpret_cast<const float4 *>(rl + 16 * a * stride + e);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) xj[c] = *reinterpret_cast<const float4 *>(rj + 16 * c * stride + e);
+#pragma unroll
+                    for (int a = 0; a < 2; ++a)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            acc[a][c] = fmaf(xj[c].x, xl[a].x, acc[a][c]);
+                            acc[a][c] = fmaf(xj[c].y, xl[a].y, acc[a][c]);
+                            acc[a][c] = fmaf(xj[c].z, xl[a].z, acc[a][c]);
+                            acc[a][c] = fmaf(xj[c].w, xl[a].w, acc[a][c]);
+                        }
+                }
             }
         }
 #pragma unroll
@@ -1260,20 +1277,20 @@ struct alignas(16) ChainCtl {
 struct ChainLayout {
     uint32_t heads, tabs, subs, sub_stride, prod, w, total;
 };
-__host__ __device__ inline ChainLayout chain_layout(int nzcap, int hotc, bool dense, int dim, int tab_bins)
+__host__ __device__ inline ChainLayout chain_layout(int nzcap, int hotc, bool dense, int tab_bins)
 {
     ChainLayout L;
     L.heads = (uint32_t)((sizeof(ChainCtl) + 127) & ~(size_t)127);
     L.tabs = L.heads + kHeadSlots * (uint32_t)sizeof(ChainHead);
     L.subs = L.tabs + kHeadSlots * tab_bytes(tab_bins);
-    L.sub_stride = dense ? sub_bytes(kLB * dim, 0, true) : sub_bytes(nzcap, nzcap / 2, false);
+    L.sub_stride = dense ? sub_bytes(kLB * hotc, 0, true) : sub_bytes(nzcap, nzcap / 2, false);
     L.prod = L.subs + kSubSlots * L.sub_stride;
     L.w = L.prod + 4u * (uint32_t)(dense ? kLB : nzcap);
     L.total = L.w + 4u * (uint32_t)(hotc > 0 ? hotc : 4);
     return L;
 }
 
-template <int LOSS, bool DENSE, bool TAB>
+template <int LOSS, bool DENSE, bool FLAT, bool TAB>
 __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const LookParams P)
 {
     extern __shared__ __align__(128) unsigned char smem_chain[];
@@ -1282,7 +1299,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     const uint32_t crank = cluster_ctarank();
     const int k = (int)(blockIdx.x >> logC);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const ChainLayout L = chain_layout(P.nzcap, P.hotc, DENSE, (int)S.dim, TAB ? P.tab_bins : 0);
+    const ChainLayout L = chain_layout(P.nzcap, P.hotc, DENSE, TAB ? P.tab_bins : 0);
     ChainCtl &ctl = *reinterpret_cast<ChainCtl *>(smem_chain);
     float *W = reinterpret_cast<float *>(smem_chain + L.w);
     float *prod = reinterpret_cast<float *>(smem_chain + L.prod);
@@ -1297,7 +1314,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     // entry ids below hot_total live in shared memory: id g in CTA g mod C at place g / C
     const int64_t hot_all = (int64_t)P.hotc << logC;
     const uint32_t hot_total = (uint32_t)(hot_all < S.dim ? hot_all : S.dim);
-    const int hot_mine = hot_total > crank ? (int)((hot_total - crank + C - 1) >> logC) : 0;
+    // (dense rows: consecutive columns to a CTA, hotc of them, a multiple of four)
+    const int slice0 = DENSE ? (int)crank * P.hotc : 0;
+    const int hot_mine = DENSE ? ((int)S.dim - slice0 < P.hotc ? ((int)S.dim > slice0 ? (int)S.dim - slice0 : 0) : P.hotc)
+                               : (hot_total > crank ? (int)((hot_total - crank + C - 1) >> logC) : 0);
 
     const uint32_t d_bytes = crank == 0 ? 2u * kLB * 4u : (uint32_t)kLB * 4u; // what a block's deltas (CTA 0: and states) bring
     if (tid == 0) {
@@ -1318,9 +1338,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         }
     }
     for (int l = tid; l < hot_mine; l += kChainThreads) {
-        const size_t g = ((size_t)l << logC) + crank;
+        const size_t g = DENSE ? (size_t)(slice0 + l) : ((size_t)l << logC) + crank;
         W[l] = P.model_in ? fmaf(sigma, Uk[g], S.vbase[g]) : Uk[g];
     }
+    if (DENSE && tid < 4 && hot_mine + tid < P.hotc) W[hot_mine + tid] = 0.0f; // (the padding of the last slice)
     // the ids beyond the part in shared memory that fall to this CTA (id mod C): the model in place
     const size_t cold0 = (size_t)hot_total + (((size_t)crank - (size_t)hot_total) & (size_t)(C - 1));
     if (P.model_in)
@@ -1366,6 +1387,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 fence_cluster(); // the other CTAs' updates of their parts of the model, made by ordinary stores
                 ++sc;
                 const uint32_t w_base = smem_u32(W);
+                auto w_at = [&](uint32_t g) { // where a model entry in shared memory lies
+                    const uint32_t c = DENSE ? g / (uint32_t)P.hotc : g & (uint32_t)(C - 1);
+                    return mapa_u32(w_base + 4u * (DENSE ? g - c * (uint32_t)P.hotc : g >> logC), c);
+                };
                 for (int j = 0; j < cnt; ++j) {
                     const CHdr h = H.hdr[j];
                     if (!CHICLE_IN_BOUNDS(S.status, h.coord >= 0 && (int64_t)h.coord < S.n_coord)) continue;
@@ -1378,7 +1403,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                     for (int e = lane; e < n; e += 32) {
                         uint32_t g = DENSE ? (uint32_t)e : (uint32_t)ix[e];
                         if (!CHICLE_IN_BOUNDS(S.status, (int64_t)g < S.dim)) g = 0u;
-                        const float ww = g < hot_total ? ld_cluster_f32(mapa_u32(w_base + 4u * (g >> logC), g & (uint32_t)(C - 1)))
+                        const float ww = g < hot_total ? ld_cluster_f32(w_at(g))
                                                        : __ldcg(Uk + g);
                         acc = fmaf(xv[e], ww, acc);
                     }
@@ -1394,7 +1419,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                             uint32_t g = DENSE ? (uint32_t)e : (uint32_t)ix[e];
                             if (!CHICLE_IN_BOUNDS(S.status, (int64_t)g < S.dim)) continue;
                             if (g < hot_total) {
-                                const uint32_t a = mapa_u32(w_base + 4u * (g >> logC), g & (uint32_t)(C - 1));
+                                const uint32_t a = w_at(g);
                                 st_cluster_f32(a, fmaf(sigma * delta, xv[e], ld_cluster_f32(a)));
                             } else Uk[g] = fmaf(sigma * delta, xv[e], __ldcg(Uk + g));
                         }
@@ -1450,8 +1475,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 xs[0] = -q0n.x; xs[1] = -q0n.y; xs[2] = -q0n.z; xs[3] = -q0n.w;
                 const float4 *G4 = reinterpret_cast<const float4 *>(H.G); // G4[l * 8 + q]: row l, columns 4q .. 4q + 3
                 const float4 *X4 = reinterpret_cast<const float4 *>(H.X);
-                // (with tables a loop: unrolled, the code outgrows the instruction cache and its fetches set the pace)
-#pragma unroll (TAB ? 1 : kLB / 4)
+                // (how far this is unrolled was measured: the code of the block loop has to stay near the instruction cache's
+                // size, or fetches set the pace of all roles. With tables not at all: 147 -> 119 cycles a step; sparse
+                // hinge twice: the recurrence 1 066 -> 1 290 cycles a block, the workers, who are the bound there, 4 610 -> 4 410)
+#pragma unroll (TAB ? 1 : (DENSE ? kLB / 4 : 2))
                 for (int g = 0; g < kLB / 4; ++g) {
                     float4 blk[4], nxt[4];
 #pragma unroll
@@ -1564,7 +1591,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         const uint32_t p_bar0 = mapa_u32(smem_u32(&ctl.pbar[0]), 0u);
         const uint32_t p_buf0 = mapa_u32(smem_u32(&ctl.pbuf[0][crank][0]), 0u);
         const uint32_t ack_bar = mapa_u32(smem_u32(&ctl.ackbar), 0u);
-        const int dim = (int)S.dim;
+        const int dstride = (hot_mine + 3) & ~3; // dense: floats per row of a record
         auto sub_at = [&](int blk) { return smem_chain + L.subs + (size_t)(blk & (kSubSlots - 1)) * L.sub_stride; };
         // The directory entry of a block is loaded a block ahead of its use (an unconditional load from a clamped
         // address, so that nothing has to wait for it at the point of issue).
@@ -1633,8 +1660,14 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 if (wt < kLB * 8) {
                     const int j = wt >> 3, qq = wt & 7;
                     float acc = 0.0f;
-                    if (j < h.cnt)
-                        for (int e = qq; e < dim; e += 8) acc = fmaf(val[j * dim + e], W[e], acc);
+                    if (j < h.cnt) {
+                        const float4 *v4 = reinterpret_cast<const float4 *>(val + j * dstride), *w4 = reinterpret_cast<const float4 *>(W);
+#pragma unroll 4
+                        for (int e = qq; e < dstride >> 2; e += 8) {
+                            const float4 a = v4[e], w = w4[e];
+                            acc = fmaf(a.x, w.x, acc); acc = fmaf(a.y, w.y, acc); acc = fmaf(a.z, w.z, acc); acc = fmaf(a.w, w.w, acc);
+                        }
+                    }
                     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
                     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
                     acc += __shfl_xor_sync(0xffffffffu, acc, 4);
@@ -1650,7 +1683,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 // Eight threads per coordinate, each its every eighth non-zero: the first two with all loads issued
                 // before anything is used. Ids below hot_total from shared memory; the others from row k of the
                 // update workspace (read at L2: the updates are made there by reductions) and from v.
-                if (wt < kLB * 8 && hot_total == 0u) {
+                if (FLAT && wt < kLB * 8) {
                     // (no id in shared memory: every gather goes to L2, eight per thread in flight)
                     const int j = wt >> 3, qq = wt & 7;
                     const int lo = h.roff[j] + qq, hi = h.roff[j + 1];
@@ -1672,7 +1705,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
                     acc += __shfl_xor_sync(0xffffffffu, acc, 4);
                     if (qq == 0) st_async_f32(p_buf0 + (slot * (uint32_t)(kMaxC * kLB) + (uint32_t)j) * 4u, acc, p_bar0 + slot * 8u);
-                } else if (wt < kLB * 8) {
+                } else if (!FLAT && wt < kLB * 8) {
                     const int j = wt >> 3, qq = wt & 7;
                     const int lo = h.roff[j] + qq, hi = h.roff[j + 1];
                     float x[2], hv[2], uu[2];
@@ -1748,11 +1781,11 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 const SubHead &h = *reinterpret_cast<const SubHead *>(rec);
                 const float *val = reinterpret_cast<const float *>(rec + sizeof(SubHead));
                 if (DENSE) {
-                    if (wt < dim) {
+                    if (wt < hot_mine) {
                         float sum = 0.0f;
                         const int cnt = h.cnt;
 #pragma unroll 8
-                        for (int j = 0; j < cnt; ++j) sum = fmaf(dl[j], val[j * dim + wt], sum);
+                        for (int j = 0; j < cnt; ++j) sum = fmaf(dl[j], val[j * dstride + wt], sum);
                         W[wt] = fmaf(sigma, sum, W[wt]);
                     }
                 } else {
@@ -1766,7 +1799,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                     //     their product delta_j * x at their place in the id's list. One store per non-zero, its
                     //     address chosen without a branch: the list place, the model word, or a word that nobody reads;
                     //     ids beyond the part in shared memory add to the workspace row instead.
-                    if (wt < kLB * 8 && hot_total == 0u) {
+                    if (FLAT && wt < kLB * 8) {
                         // (no id in shared memory: a list place or a reduction at L2, eight non-zeros per turn)
                         const int j = wt >> 3, qq = wt & 7;
                         const int lo = h.roff[j] + qq, hi = h.roff[j + 1];
@@ -1793,7 +1826,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                                 red_add_if(Uk + (far ? (m8[u] & kIdMask) : 0u), sigma * p8[u], far);
                             }
                         }
-                    } else if (wt < kLB * 8) {
+                    } else if (!FLAT && wt < kLB * 8) {
                         const int j = wt >> 3, qq = wt & 7;
                         const int lo = h.roff[j] + qq, hi = h.roff[j + 1];
                         const float d = dl[j];
@@ -1888,10 +1921,9 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             // dot products: of block b + 2 against the model as it is now; of block b + 1 first if block b was walked in
             // place (a block right behind a walked one starts from the model as the walk left it)
 #pragma unroll 1
-            for (int ahead = 1; ahead <= 2; ++ahead) {
+            for (int ahead = depth == 1 || sl0 ? 1 : 2; ahead <= depth; ++ahead) {
                 // (one block ahead: block b + 1 after block b's update, whatever block b was)
-                const bool due = depth == 1 ? (ahead == 1 && b + 1 < nb && !sl1)
-                                            : (ahead == 1 ? (sl0 && b + 1 < nb && !sl1) : (b + 2 < nb && !sl2 && !sl1));
+                const bool due = b + ahead < nb && !sl1 && (ahead == 1 || !sl2);
                 if (due && !take_dots(b + ahead)) { aborted = true; break; }
             }
             if (aborted) break;
@@ -1912,7 +1944,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         work_bar();
         const float inv_sigma = 1.0f / sigma;
         for (int l = wt; l < hot_mine; l += kWorkThreads) {
-            const size_t g = ((size_t)l << logC) + crank;
+            const size_t g = DENSE ? (size_t)(slice0 + l) : ((size_t)l << logC) + crank;
             Uk[g] = P.model_out ? (W[l] - S.vbase[g]) * inv_sigma : W[l];
         }
         if (P.model_out)
@@ -1948,9 +1980,9 @@ __global__ void k_block_bases_slices(const int64_t *__restrict__ slice, int32_t 
     out[K] = run;
 }
 
-template <int LOSS, bool DENSE, bool TAB> cudaError_t launch_chain(Glm &g, const LookParams &P)
+template <int LOSS, bool DENSE, bool FLAT, bool TAB> cudaError_t launch_chain(Glm &g, const LookParams &P)
 {
-    auto kern = k_lookahead_chain<LOSS, DENSE, TAB>;
+    auto kern = k_lookahead_chain<LOSS, DENSE, FLAT, TAB>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.la_smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -2046,9 +2078,11 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
 template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P)
 {
     constexpr bool tables = LOSS == CHICLE_LOSS_LOGISTIC_DUAL;
-    const bool dense = g.fmt == CHICLE_FMT_DENSE_ROWMAJOR;
-    if (tables && P.tab_bins) return dense ? launch_chain<LOSS, true, tables>(g, P) : launch_chain<LOSS, false, tables>(g, P);
-    return dense ? launch_chain<LOSS, true, false>(g, P) : launch_chain<LOSS, false, false>(g, P);
+    const bool flat = g.la_hotc == 0;
+    if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR)
+        return tables && P.tab_bins ? launch_chain<LOSS, true, false, tables>(g, P) : launch_chain<LOSS, true, false, false>(g, P);
+    if (tables && P.tab_bins) return flat ? launch_chain<LOSS, false, true, tables>(g, P) : launch_chain<LOSS, false, false, tables>(g, P);
+    return flat ? launch_chain<LOSS, false, true, false>(g, P) : launch_chain<LOSS, false, false, false>(g, P);
 }
 
 // A round's launches, slice after slice (consecutive pieces of every partition's walk). The first slice's prepare
@@ -2104,7 +2138,7 @@ template <int LOSS> cudaError_t launch_slices(Glm &g, std::vector<LookParams> &P
 
 } // namespace
 
-int lookahead_max_dense_dim() { return kCapL; }
+int lookahead_max_dense_dim() { return kMaxC * kDenseSlice; }
 int lookahead_max_slices() { return 64; }
 int64_t lookahead_max_dim() { return (int64_t)1 << kIdBits; }
 
@@ -2124,6 +2158,16 @@ void lookahead_plan(Glm &g, int32_t K)
             logC = want >= 8 ? 3 : (want >= 4 ? 2 : (want >= 2 ? 1 : 0));
             while (logC > 0 && ((int64_t)K << logC) > g.sm_count) --logC;
         }
+    }
+    int slice = (int)((g.dim + 3) & ~(int64_t)3); // dense: columns per CTA
+    if (dense) {
+        // Long rows are shared out over a cluster: slices of about 128 columns where the SMs allow it for all partitions at
+        // once, else as few CTAs as slices of 384 columns need (a worker thread per column, four blocks' slices in shared
+        // memory); the clusters then take turns.
+        auto cut = [&](int lg) { return (int)((((g.dim + (1 << lg) - 1) >> lg) + 3) & ~(int64_t)3); };
+        while (logC < 3 && cut(logC) > kDenseSlice) ++logC;
+        while (logC < 3 && cut(logC) > kDenseEasy && ((int64_t)K << (logC + 1)) <= g.sm_count) ++logC;
+        slice = cut(logC);
     }
     g.la_logC = logC;
     // Beside chains on at most half of the SMs the prepare kernels run on the side stream; otherwise they alternate with
@@ -2148,25 +2192,25 @@ void lookahead_plan(Glm &g, int32_t K)
         const float q_max = (float)K * g.max_sqnorm / (g.lambda * (float)g.n_examples);
         for (int bins = 64; bins >= 32; bins >>= 1)
             if (q_max <= tab_max_q(bins)) g.la_tab_bins = bins;
-        if (dense && chain_layout(0, (int)g.dim, true, (int)g.dim, g.la_tab_bins).total > budget) g.la_tab_bins = 0;
+        if (dense && chain_layout(0, slice, true, g.la_tab_bins).total > budget) g.la_tab_bins = 0;
         const char *env = getenv("CHICLE_LA_TABLES"); // 0: none (tests)
         if (env && env[0] == '0') g.la_tab_bins = 0;
     }
     if (dense) {
         g.la_nzcap = 0;
-        g.la_hotc = (int32_t)g.dim;
+        g.la_hotc = slice;
     } else if (!g.hot_variant) {
         g.la_nzcap = 3072;
         g.la_hotc = 0;
     } else {
         g.la_nzcap = logC == 0 ? 2048 : (logC == 1 ? 1536 : 1024);
-        const ChainLayout L0 = chain_layout(g.la_nzcap, 0, false, (int)g.dim, g.la_tab_bins);
+        const ChainLayout L0 = chain_layout(g.la_nzcap, 0, false, g.la_tab_bins);
         int64_t hotc = ((int64_t)budget - (int64_t)L0.total - 64) / 4;
         hotc = hotc < 0 ? 0 : (hotc / 32) * 32;
         const int64_t need = (g.dim + ((int64_t)1 << logC) - 1) >> logC; // per CTA for the whole model
         g.la_hotc = (int32_t)(hotc < need ? hotc : (need + 31) / 32 * 32);
     }
-    g.la_smem = chain_layout(g.la_nzcap, g.la_hotc, dense, (int)g.dim, g.la_tab_bins).total;
+    g.la_smem = chain_layout(g.la_nzcap, g.la_hotc, dense, g.la_tab_bins).total;
 
     // slices: at most a sixteenth of the walk, but at least 256 blocks per partition; three regions
     const int64_t n = g.n_coord;
@@ -2189,7 +2233,7 @@ void lookahead_plan(Glm &g, int32_t K)
     const double frac = whole ? 1.0 : (double)region_blocks / (double)(n / kLB + 1);
     const size_t C = (size_t)1 << logC;
     size_t pool;
-    if (dense) pool = (size_t)region_blocks * sub_bytes(kLB * (int)g.dim, 0, true);
+    if (dense) pool = (size_t)region_blocks * C * sub_bytes(kLB * slice, 0, true);
     else {
         const double all = 14.0 * (double)g.nnz;
         double part = whole ? all : 1.2 * frac * all + (double)(1 << 20);
