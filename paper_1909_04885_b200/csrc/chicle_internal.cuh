@@ -123,7 +123,7 @@ struct Glm {
     void *la_rec = nullptr;
     void *la_dir = nullptr;          // per region: cluster-size entries per block
     unsigned long long *la_cursor = nullptr; // [r]: bytes of region r's pool handed out; [8..]: timing scratch
-    size_t la_region_bytes = 0, la_pool_off = 0, la_dir_bytes = 0;
+    size_t la_region_bytes = 0, la_pool_off = 0, la_pool_piece = 0, la_dir_bytes = 0;
     int64_t la_region_blocks = 0;    // blocks a region has records for
     int la_regions = 0;
     int la_logC = 0;                 // log2 of the CTAs per partition (thread-block cluster)

@@ -118,6 +118,7 @@ struct LookParams {
     unsigned long long *timing;  // scratch words of a -DCHICLE_LA_TIMING build
     unsigned long long pool_off; // the pool of worker records starts here (the heads lie before it, one per block)
     unsigned long long pool_cap; // bytes of the pool
+    unsigned long long pool_piece; // what a CTA of the sparse prepare kernel takes of it at a time
     const int64_t *blk_base;     // K + 1: the first block of each partition in this launch's numbering of the blocks
     int32_t K, logC;
     int32_t depth;               // 2: a block's dot products are taken two blocks ahead and corrected with the cross
@@ -149,15 +150,6 @@ __device__ __forceinline__ int32_t checked_id(const LookParams &P, int32_t id)
 {
     return CHICLE_IN_BOUNDS(P.S.status, id >= 0 && (int64_t)id < P.S.dim) ? id : 0;
 }
-// (debug build) a visiting-order entry and the extent of its coordinate: an empty coordinate 0 if either is off
-__device__ __forceinline__ void checked_extent(const LookParams &P, int32_t &c, int64_t &rs, int32_t &n)
-{
-    if (!CHICLE_IN_BOUNDS(P.S.status, c >= 0 && (int64_t)c < P.S.n_coord)) c = 0;
-    rs = P.S.indptr[c];
-    const int64_t len = P.S.indptr[c + 1] - rs;
-    n = (int32_t)len;
-    if (!CHICLE_IN_BOUNDS(P.S.status, rs >= 0 && len >= 0 && len <= 0x7fffffff && rs + len <= P.nnz)) { rs = 0; n = 0; }
-}
 // The same search over a copy of blk_base in shared memory (a launch with at most kBaseStaged - 1 partitions; block
 // counts fit 32 bits): the dependent loads of the search cost 30 cycles each instead of an L2 round trip.
 constexpr int kBaseStaged = 260;
@@ -187,13 +179,11 @@ __device__ __forceinline__ void block_to_part(const LookParams &P, int64_t bid, 
 // The constants of coordinate c's scalar step (see coordinate_step), and the line A + B * dot that the recurrence's
 // state starts from (what the block's earlier coordinates contribute at their round-start states is taken off A
 // once the Gram triangle is known).
-template <int LOSS> __device__ __forceinline__ CHdr make_hdr(const SolverParams &P, int32_t c)
+template <int LOSS> __device__ __forceinline__ CHdr make_hdr_of(const SolverParams &P, int32_t c, float s, float al, float y)
 {
     CHdr hd;
     hd.coord = c;
     hd.lq = 0.0f;
-    const float s = P.sqnorm[c];
-    const float al = P.alpha[c];
     if (LOSS == CHICLE_LOSS_RIDGE_PRIMAL) {
         hd.p0 = P.inv_n;
         hd.p1 = al;
@@ -202,7 +192,6 @@ template <int LOSS> __device__ __forceinline__ CHdr make_hdr(const SolverParams 
         hd.A = P.lambda * al;
         hd.B = P.inv_n;
     } else {
-        const float y = P.labels[c];
         hd.p0 = y / P.lam_n;
         hd.p1 = y * al;
         hd.p3 = y;
@@ -220,6 +209,11 @@ template <int LOSS> __device__ __forceinline__ CHdr make_hdr(const SolverParams 
         }
     }
     return hd;
+}
+
+template <int LOSS> __device__ __forceinline__ CHdr make_hdr(const SolverParams &P, int32_t c)
+{
+    return make_hdr_of<LOSS>(P, c, P.sqnorm[c], P.alpha[c], LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : P.labels[c]);
 }
 
 // Loads that are issued only where `on` holds (0 elsewhere), with nothing waiting on them at the point of issue.
@@ -388,56 +382,306 @@ template <int HT> __device__ __forceinline__ uint32_t home_slot(int32_t id)
 template <int HT> __device__ __forceinline__ uint32_t next_slot(uint32_t p) { return p + 1 < (uint32_t)HT ? p + 1 : kHD; }
 
 // ------------------------------------------------------------------------------------------------ prepare
-template <int NZ, int HT, int THREADS> struct PreShared {
-    int32_t idx[NZ];     // the block's non-zeros, row after row (later: the membership mask of the non-zero's id)
-    float val[NZ];
-    uint16_t slot[NZ];   // table slot of each non-zero's id (later: where the id's list of values starts)
-    int32_t key[HT];     // id in a table slot, -1 = empty
-    uint32_t mask[HT];   // bit j: coordinate j of the block has this id
-    uint16_t soff[HT];   // start of the slot's list in lval
-    uint16_t coff[HT];   // a shared id: start of its list among the lists of its CTA's record
-    float lval[NZ];      // the values of the block's non-zeros, one list per id, each in ascending coordinate order
-    float G[kLB][kLB + 1];
-    float X[kLB][kLB + 1];
-    alignas(16) float Dc[kLB][kHDS]; // this block's entries with the kHD most frequent ids, dense
-    alignas(16) float Dn[kLB][kHDS]; // the next block's
+// A CTA takes a run of consecutive blocks, so that a block's rows are fetched once: they serve as the next block of the
+// one before (cross Gram matrix) and then as the block itself. All fetches are asynchronous copies into shared memory and
+// run ahead of their use: while block b is worked on, the rows of b + 1, the row extents and constants of b + 2 and the
+// visiting-order entries of b + 3 are under way. Passes over the block's non-zeros take them as one flat array (32 at a
+// time whatever the rows' lengths).
+// What bounds it is instruction issue and shared-memory latency; before (a CTA per block, each fetching its own rows and
+// its successor's in three dependent round trips) a block of 1 600 non-zeros took 63 000 cycles at three CTAs per SM.
+constexpr int kDirNew = 4; // (metadata slots: a power of two)
+
+// One block's coordinates as the kernel keeps them: constants of the steps and extents of the rows.
+struct PreBlock {
     CHdr hdr[kLB];
-    float q0n[kLB];
     int64_t rs[kLB];
     int32_t nnz[kLB];
-    int32_t roff[kLB + 1];
-    uint16_t rc[kLB + 1][kMaxC]; // non-zeros of coordinate j that fall to CTA c; then where they start in c's record
-    uint32_t cntTL[kMaxC], cntTL2[kMaxC], cntAll; // per CTA: shared ids (high half) and their list entries (low half); all list entries
+    int32_t roff[kLB + 1];            // where each coordinate's entries start in the flat array ([32] = all of them)
     float gsc[kLB], ys[kLB], as[kLB]; // per coordinate: its Gram scale, and what multiplies / enters from the earlier ones
-    float gscn[kLB];                  // the next block's coordinates: their Gram scales
-    int64_t nrs[kLB];
-    int32_t nnnz[kLB];
-    unsigned long long sub_off[kMaxC];
-    uint32_t sub_len[kMaxC];
-    int32_t subT[kMaxC];
-    int32_t ncls[kMaxC]; // the next block's non-zeros per CTA
-    int32_t total, slow, carry, ncnt;
-    int32_t base[kBaseStaged]; // blk_base of the first partitions, staged once per launch (see block_to_part_staged)
+    int32_t k, cnt, total, over;      // partition; over: more non-zeros than the arrays hold (total is 0 then): walked in place
 };
 
-// One block's records (all threads of the CTA; every return below is taken by all of them).
-template <int LOSS, int NZ, int HT, int THREADS>
-__device__ __forceinline__ void prepare_block(const LookParams &P, const int64_t bid, PreShared<NZ, HT, THREADS> &sh)
+template <int NZ, int HT, int THREADS> struct PreShared {
+    static constexpr int CH = NZ / 32;  // chunks of 32 entries
+    alignas(16) int32_t key[HT];        // id in a table slot, -1 = empty
+    alignas(16) uint32_t mask[HT];      // bit j: coordinate j of the block has this id
+    uint16_t soff[HT];                  // where the id's values are: an entry of val (one coordinate has it), or NZ + a place in lval
+    uint16_t coff[HT];                  // a shared id: start of its list among the lists of its CTA's record
+    int32_t idx[2][NZ];                 // the block's entries, and the next block's
+    float val[2][NZ];
+    float lval[NZ];                     // the values of shared ids, one list per id, each in ascending coordinate order
+    uint16_t slot[NZ];                  // table slot of each entry's id
+    uint16_t found[NZ];                 // the next block's entries: table slot of the id, 0xffff: this block does not have it
+    uint8_t row[2][NZ];                 // coordinate of each entry
+    uint32_t bal[2][CH + 1][kMaxC];     // per chunk and CTA: which of the entries fall to it
+    uint16_t pre[2][CH + 1][kMaxC];     // and how many before the chunk
+    float G[kLB][kLB + 1];              // scaled Gram entries: the triangle, then the cross Gram matrix
+    alignas(16) float D[2][kLB][kHDS];  // the entries with the kHD most frequent ids, dense
+    PreBlock blk[kDirNew];
+    int32_t coord[kDirNew][kLB];        // visiting-order entries
+    int64_t ip[2][kLB];                 // fetched for a block: row extents, squared norms, states, labels
+    float sq[kLB], al[kLB], lb[kLB];
+    uint16_t rc[kLB + 1][kMaxC];        // where coordinate j's entries start in CTA c's record
+    uint32_t cntTL[kMaxC], cntAll;      // per CTA: shared ids (high half) and their list entries (low half); all list entries
+    unsigned long long sub_off[kMaxC];
+    int32_t walk;
+    unsigned long long pool_at, pool_end; // what this CTA holds of the pool
+    float q0n[kLB];
+    int32_t base[kBaseStaged];          // blk_base, and first step and step count of each partition (see pre_locate)
+    int64_t off[kBaseStaged];
+    int32_t steps[kBaseStaged];
+};
+
+// Where block x of the launch lies: partition, first step in the visiting-order array, steps in the block.
+struct PrePlace {
+    int32_t k;
+    int64_t at;
+    int32_t cnt;
+};
+template <class Shared> __device__ __forceinline__ PrePlace pre_locate(const LookParams &P, const Shared &sh, int64_t x)
 {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    constexpr int NW = THREADS / 32;
-    const int C = 1 << P.logC;
+    PrePlace r;
     int k;
-    int64_t b;
-    if (P.K < kBaseStaged) block_to_part_staged(sh.base, P.K, bid, k, b);
-    else block_to_part(P, bid, k, b);
-    const int64_t nk = P.S.part_off[k + 1] - P.S.part_off[k];
-    const int64_t off = P.S.part_off[k] + (P.S.first_k ? P.S.first_k[k] : 0); // of this launch's first step in the order
-    const int64_t steps = steps_of(P, k, nk);
-    const int cnt = (int)((steps - b * kLB) < kLB ? (steps - b * kLB) : kLB);
-    const int64_t left = steps - (b + 1) * kLB; // steps behind this block
-    const int ncnt = (left <= 0 || P.depth < 2) ? 0 : (left < kLB ? (int)left : kLB);
-    ChainHead &out = *reinterpret_cast<ChainHead *>(P.rec + (size_t)bid * sizeof(ChainHead));
+    int64_t b, off, steps;
+    if (P.K < kBaseStaged) {
+        block_to_part_staged(sh.base, P.K, x, k, b);
+        off = sh.off[k];
+        steps = sh.steps[k];
+    } else {
+        block_to_part(P, x, k, b);
+        off = P.S.part_off[k] + (P.S.first_k ? P.S.first_k[k] : 0);
+        steps = steps_of(P, k, P.S.part_off[k + 1] - P.S.part_off[k]);
+    }
+    r.k = k;
+    r.at = off + b * kLB;
+    const int64_t left = steps - b * kLB;
+    r.cnt = (int32_t)(left < kLB ? left : kLB);
+    return r;
+}
+
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// The three stages of a block's fetches (a warp each; the caller waits for the copies and meets the other threads).
+template <class Shared> __device__ __forceinline__ void pre_fetch_order(const LookParams &P, Shared &sh, int64_t x)
+{
+    const int lane = threadIdx.x & 31;
+    const PrePlace pl = pre_locate(P, sh, x);
+    if (lane < pl.cnt) cp_async4(smem_u32(&sh.coord[x & (kDirNew - 1)][lane]), P.S.perm + pl.at + lane);
+    else sh.coord[x & (kDirNew - 1)][lane] = -1;
+    if (lane == 0) {
+        sh.blk[x & (kDirNew - 1)].cnt = pl.cnt;
+        sh.blk[x & (kDirNew - 1)].k = pl.k;
+    }
+}
+template <int LOSS, class Shared> __device__ __forceinline__ void pre_fetch_extents(const LookParams &P, Shared &sh, int64_t x)
+{
+    const int lane = threadIdx.x & 31;
+    int32_t c = sh.coord[x & (kDirNew - 1)][lane];
+    if (c >= 0 && !CHICLE_IN_BOUNDS(P.S.status, (int64_t)c < P.S.n_coord)) c = 0;
+    if (c < 0) return;
+    cp_async8(smem_u32(&sh.ip[0][lane]), P.S.indptr + c);
+    cp_async8(smem_u32(&sh.ip[1][lane]), P.S.indptr + c + 1);
+    cp_async4(smem_u32(&sh.sq[lane]), P.S.sqnorm + c);
+    cp_async4(smem_u32(&sh.al[lane]), P.S.alpha + c);
+    if (LOSS != CHICLE_LOSS_RIDGE_PRIMAL) cp_async4(smem_u32(&sh.lb[lane]), P.S.labels + c);
+}
+// (a warp: what was fetched for block x becomes its PreBlock)
+template <int LOSS, int NZ, int HT, class Shared> __device__ __forceinline__ void pre_make_block(const LookParams &P, Shared &sh, int64_t x)
+{
+    const int lane = threadIdx.x & 31;
+    PreBlock &B = sh.blk[x & (kDirNew - 1)];
+    int32_t c = sh.coord[x & (kDirNew - 1)][lane];
+    if (c >= 0 && !CHICLE_IN_BOUNDS(P.S.status, (int64_t)c < P.S.n_coord)) c = 0;
+    CHdr hd{0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    int64_t rs = 0;
+    int32_t n = 0;
+    if (c >= 0) {
+        rs = sh.ip[0][lane];
+        const int64_t len = sh.ip[1][lane] - rs;
+        n = (int32_t)len;
+        if (!CHICLE_IN_BOUNDS(P.S.status, rs >= 0 && len >= 0 && len <= 0x7fffffff && rs + len <= P.nnz)) { rs = 0; n = 0; }
+        hd = make_hdr_of<LOSS>(P.S, c, sh.sq[lane], sh.al[lane], LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : sh.lb[lane]);
+        if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) hd.lq = tab_offset(hd.p2, P.tab_bins);
+    }
+    B.hdr[lane] = hd;
+    B.rs[lane] = rs;
+    B.nnz[lane] = n;
+    B.gsc[lane] = c >= 0 ? gram_scale<LOSS>(hd, P.S.sigma, P.S.inv_n) : 0.0f;
+    B.ys[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 1.0f : hd.p3;
+    B.as[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : hd.p1;
+    constexpr int room = NZ < HT - kHD ? NZ : HT - kHD; // entries, and slots for their ids if none is shared
+    const int m = n < room + 1 ? n : room + 1; // (more than the arrays hold is all that matters of a longer one)
+    int incl = m;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const int tot = __shfl_sync(0xffffffffu, incl, 31);
+    const bool over = tot > room;
+    B.roff[lane] = over ? 0 : incl - m;
+    if (lane == 31) {
+        B.roff[kLB] = over ? 0 : incl;
+        B.total = over ? 0 : incl;
+        B.over = over ? 1 : 0;
+    }
+}
+// (all warps: the rows of a block into buffer `buf`; the caller waits)
+template <int NZ, int THREADS, class Shared> __device__ __forceinline__ void pre_fetch_rows(const LookParams &P, Shared &sh, int64_t x, int buf)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const PreBlock &B = sh.blk[x & (kDirNew - 1)];
+    if (B.over) return;
+    for (int j = warp; j < kLB; j += THREADS / 32) {
+        const int n = B.nnz[j], r0 = B.roff[j];
+        const int32_t *ix = P.S.indices + B.rs[j];
+        const float *xv = P.S.values + B.rs[j];
+        for (int e = lane; e < n; e += 32) {
+            cp_async4(smem_u32(&sh.idx[buf][r0 + e]), ix + e);
+            cp_async4(smem_u32(&sh.val[buf][r0 + e]), xv + e);
+            sh.row[buf][r0 + e] = (uint8_t)j;
+        }
+    }
+}
+// (all warps: which entries of a fetched block fall to which CTA, its dense tile, and, with PROBE, where the table of the
+// current block has their ids)
+template <int NZ, int HT, int THREADS, class Shared>
+__device__ __forceinline__ void pre_scan(const LookParams &P, Shared &sh, int total, int buf, int C, bool probe)
+{
+    const int lane = threadIdx.x & 31;
+    for (int e = threadIdx.x; (e & ~31) < total; e += THREADS) {
+        const bool on = e < total;
+        const int32_t id = on ? checked_id(P, sh.idx[buf][e]) : -1;
+        if (C > 1) {
+            uint32_t mine = 0u;
+            for (int c = 0; c < C; ++c) {
+                const uint32_t b = __ballot_sync(0xffffffffu, on && (id & (C - 1)) == c);
+                mine = lane == c ? b : mine;
+            }
+            if (lane < C) sh.bal[buf][e >> 5][lane] = mine;
+        } else {
+            const uint32_t b = __ballot_sync(0xffffffffu, on);
+            if (lane == 0) sh.bal[buf][e >> 5][0] = b;
+        }
+        if (on && id < kHD) sh.D[buf][sh.row[buf][e]][id] = sh.val[buf][e];
+        if (probe && on) {
+            uint32_t p = 0xffffu;
+            if (id >= kHD) {
+                uint32_t q = home_slot<HT>(id);
+                for (int t = 0; t < HT; ++t) {
+                    const int32_t seen = sh.key[q];
+                    if (seen == id) { p = q; break; }
+                    if (seen == -1) break;
+                    q = next_slot<HT>(q);
+                }
+            }
+            sh.found[e] = (uint16_t)p;
+        }
+    }
+}
+// (warp c: how many of the entries before each chunk fall to CTA c)
+template <class Shared> __device__ __forceinline__ void pre_prefix(Shared &sh, int total, int buf, int c)
+{
+    const int lane = threadIdx.x & 31;
+    const int nch = (total + 31) >> 5;
+    int run = 0;
+    for (int b = 0; b <= nch; b += 32) {
+        const int ch = b + lane;
+        const int x = ch < nch ? __popc(sh.bal[buf][ch][c]) : 0;
+        int incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (ch <= nch) sh.pre[buf][ch][c] = (uint16_t)(run + incl - x);
+        run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+}
+
+// Dot product of a coordinate's dense part (row j of `a`) with lane's row of `m`.
+__device__ __forceinline__ float pre_dense_dot(const float *a, const float *m)
+{
+    float acc = 0.0f;
+    const float4 *dj = reinterpret_cast<const float4 *>(a), *dm = reinterpret_cast<const float4 *>(m);
+#pragma unroll
+    for (int h = 0; h < kHD / 4; ++h) {
+        const float4 x = dj[h], y = dm[h];
+        acc = fmaf(x.x, y.x, acc); acc = fmaf(x.y, y.y, acc); acc = fmaf(x.z, y.z, acc); acc = fmaf(x.w, y.w, acc);
+    }
+    return acc;
+}
+// Adds what the entries marked in `todo` (lanes of this chunk) contribute: mask, list address and value handed round by
+// shuffles, two entries per turn, so that the second one's loads are under way while the first is added.
+__device__ __forceinline__ void pre_add_listed(uint32_t todo, uint32_t m_l, uint32_t at_l, float x_l, float &acc)
+{
+    const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
+    while (todo) {
+        const int src0 = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const bool two = todo != 0u;
+        const int src1 = two ? __ffs(todo) - 1 : src0;
+        todo &= todo - 1u;
+        const uint32_t m0 = __shfl_sync(0xffffffffu, m_l, src0), m1 = __shfl_sync(0xffffffffu, m_l, src1);
+        const uint32_t a0 = __shfl_sync(0xffffffffu, at_l, src0), a1 = __shfl_sync(0xffffffffu, at_l, src1);
+        const float x0 = __shfl_sync(0xffffffffu, x_l, src0), x1 = __shfl_sync(0xffffffffu, x_l, src1);
+        const bool on0 = (m0 >> lane) & 1u, on1 = two && ((m1 >> lane) & 1u);
+        const float v0 = lds_f32(a0 + (on0 ? 4u * (uint32_t)__popc(m0 & lt) : 0u)), v1 = lds_f32(a1 + (on1 ? 4u * (uint32_t)__popc(m1 & lt) : 0u));
+        acc = fmaf(x0, on0 ? v0 : 0.0f, acc);
+        acc = fmaf(x1, on1 ? v1 : 0.0f, acc);
+    }
+}
+
+template <int LOSS, int NZ, int HT, int THREADS, int PER_SM>
+__global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const LookParams P)
+{
+    extern __shared__ __align__(16) unsigned char smem_pre[];
+    using Shared = PreShared<NZ, HT, THREADS>;
+    Shared &sh = *reinterpret_cast<Shared *>(smem_pre);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int NW = THREADS / 32, EPT = NZ / THREADS;
+    static_assert(NZ % THREADS == 0 && NW >= 8, "entries per thread; a warp per CTA of the cluster");
+    const int C = 1 << P.logC;
+    const int64_t lo = P.n_blocks * (int64_t)blockIdx.x / gridDim.x, hi = P.n_blocks * ((int64_t)blockIdx.x + 1) / gridDim.x;
+    if (lo >= hi) return;
+    if (P.K < kBaseStaged)
+        for (int i = tid; i <= P.K; i += THREADS) {
+            sh.base[i] = (int32_t)P.blk_base[i];
+            if (i < P.K) {
+                sh.off[i] = P.S.part_off[i] + (P.S.first_k ? P.S.first_k[i] : 0);
+                sh.steps[i] = (int32_t)steps_of(P, i, P.S.part_off[i + 1] - P.S.part_off[i]);
+            }
+        }
+    for (int p = tid; p < HT; p += THREADS) { sh.key[p] = -1; sh.mask[p] = 0u; }
+    for (int p = tid; p < 2 * kLB * kHDS; p += THREADS) (&sh.D[0][0][0])[p] = 0.0f;
+    if (tid < kMaxC) sh.cntTL[tid] = 0u;
+    if (tid == 0) { sh.cntAll = 0u; sh.pool_at = sh.pool_end = 0ull; }
+    __syncthreads();
+    // blocks that are fetched: the run, and the one behind it where the last block has a cross Gram matrix with it
+    int64_t end = hi;
+    if (P.depth >= 2 && hi < P.n_blocks && pre_locate(P, sh, hi).k == pre_locate(P, sh, hi - 1).k) end = hi + 1;
+    if (warp < 3 && lo + warp < end) pre_fetch_order(P, sh, lo + warp);
+    cp_async_wait_all();
+    __syncthreads();
+    if (warp == 0)
+        for (int64_t x = lo; x < end && x < lo + 2; ++x) {
+            pre_fetch_extents<LOSS>(P, sh, x);
+            cp_async_wait_all();
+            __syncwarp();
+            pre_make_block<LOSS, NZ, HT>(P, sh, x);
+            __syncwarp();
+        }
+    __syncthreads();
+    pre_fetch_rows<NZ, THREADS>(P, sh, lo, (int)(lo & 1));
+    cp_async_wait_all();
+    __syncthreads();
+    pre_scan<NZ, HT, THREADS>(P, sh, sh.blk[lo & (kDirNew - 1)].total, (int)(lo & 1), C, false);
+    __syncthreads();
+    if (warp < C) pre_prefix(sh, sh.blk[lo & (kDirNew - 1)].total, (int)(lo & 1), warp);
+    __syncthreads();
 #ifdef CHICLE_LA_TIMING
     long long pt0 = clock64(), pt1 = 0;
 #define PRE_T(i) do { asm volatile("" ::: "memory"); pt1 = clock64(); if (tid == 0) atomicAdd(P.timing + 16 + (i), (unsigned long long)(pt1 - pt0)); pt0 = pt1; asm volatile("" ::: "memory"); } while (0)
@@ -445,493 +689,255 @@ __device__ __forceinline__ void prepare_block(const LookParams &P, const int64_t
 #define PRE_T(i) do { } while (0)
 #endif
 
-    // ---- headers: warp 0 this block's coordinates, warp 1 the next block's
-    if (warp == 0) {
-        CHdr hd{0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        int64_t rs = 0;
-        int32_t n = 0;
-        if (lane < cnt) {
-            int32_t c = P.S.perm[off + b * kLB + lane];
-            checked_extent(P, c, rs, n);
-            hd = make_hdr<LOSS>(P.S, c);
-            if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) hd.lq = tab_offset(hd.p2, P.tab_bins);
-        }
-        sh.hdr[lane] = hd;
-        sh.rs[lane] = rs;
-        sh.nnz[lane] = n;
-        sh.gsc[lane] = lane < cnt ? gram_scale<LOSS>(hd, P.S.sigma, P.S.inv_n) : 0.0f;
-        sh.ys[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 1.0f : hd.p3;
-        sh.as[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : hd.p1;
-        int incl = n;
+#pragma unroll 1
+    for (int64_t bid = lo; bid < hi; ++bid) {
+        const int cur = (int)(bid & 1), nxt = cur ^ 1;
+        PreBlock &B = sh.blk[bid & (kDirNew - 1)];
+        const PreBlock &N = sh.blk[(bid + 1) & (kDirNew - 1)];
+        const bool have_next = bid + 1 < end;
+        const int total = B.total, cnt = B.cnt;
+        ChainHead &out = *reinterpret_cast<ChainHead *>(P.rec + (size_t)bid * sizeof(ChainHead));
+        // ---- fetches for the blocks ahead
+        if (have_next) pre_fetch_rows<NZ, THREADS>(P, sh, bid + 1, nxt);
+        if (warp == NW - 1 && bid + 2 < end) pre_fetch_extents<LOSS>(P, sh, bid + 2);
+        if (warp == NW - 2 && bid + 3 < end) pre_fetch_order(P, sh, bid + 3);
+        for (int p = tid; p < kLB * kHDS; p += THREADS) (&sh.D[nxt][0][0])[p] = 0.0f;
+        // ---- every id into the table
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        const int tot = __shfl_sync(0xffffffffu, incl, 31);
-        const bool over = tot > NZ; // more non-zeros than this kernel's arrays hold: walked in place
-        sh.roff[lane] = over ? 0 : incl - n;
-        if (lane == 31) {
-            sh.roff[kLB] = over ? 0 : incl;
-            sh.total = over ? 0 : incl;
-            sh.slow = over ? 1 : 0;
-        }
-    } else if (warp == 1) {
-        CHdr hd{0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        int64_t rs = 0;
-        int32_t n = 0;
-        if (lane < ncnt) {
-            int32_t c = P.S.perm[off + (b + 1) * kLB + lane];
-            checked_extent(P, c, rs, n);
-            hd = make_hdr<LOSS>(P.S, c);
-        }
-        sh.nrs[lane] = rs;
-        sh.nnnz[lane] = n;
-        sh.gscn[lane] = lane < ncnt ? gram_scale<LOSS>(hd, P.S.sigma, P.S.inv_n) : 0.0f;
-        int tot = n;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-        if (lane == 0) {
-            sh.ncnt = ncnt;
-            sh.carry = (ncnt > 0 && tot <= NZ) ? 1 : 0; // (and both blocks must be staged: see below)
-        }
-    }
-    for (int p = tid; p < HT; p += THREADS) {
-        sh.key[p] = -1;
-        sh.mask[p] = 0u;
-    }
-    for (int p = tid; p < (kLB + 1) * kMaxC; p += THREADS) (&sh.rc[0][0])[p] = 0;
-    for (int p = tid; p < kLB * kHDS; p += THREADS) {
-        (&sh.Dc[0][0])[p] = 0.0f;
-        (&sh.Dn[0][0])[p] = 0.0f;
-    }
-    if (tid < kMaxC) { sh.ncls[tid] = 0; sh.cntTL[tid] = 0u; sh.cntTL2[tid] = 0u; }
-    if (tid == 0) sh.cntAll = 0u;
-    __syncthreads();
-    PRE_T(0);
-    const int total = sh.total;
-    const bool slow = sh.slow != 0;
-    const bool carry = !slow && sh.carry != 0;
-    if (!slow) {
-        // ---- the block's non-zeros into shared memory, every id into the table; how many fall to each CTA. The
-        //      first 128 entries of a coordinate are loaded before any is used.
-        //      The loads of a warp's next coordinate are issued before this one's entries are inserted.
-        int32_t ids_nx[4];
-        float vals_nx[4];
-        auto load4 = [&](int j, int32_t (&ids)[4], float (&vals)[4]) {
-            const int n = j < cnt ? sh.nnz[j] : 0;
-            const int64_t rs = j < cnt ? sh.rs[j] : 0;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int e = lane + 32 * c;
-                ids[c] = e < n ? checked_id(P, P.S.indices[rs + e]) : -1;
-                vals[c] = e < n ? P.S.values[rs + e] : 0.0f;
-            }
-        };
-        load4(warp, ids_nx, vals_nx);
-        for (int j = warp; j < cnt; j += NW) {
-            const int n = sh.nnz[j], r0 = sh.roff[j];
-            const int64_t rs = sh.rs[j];
-            int per_class[kMaxC];
-#pragma unroll
-            for (int c = 0; c < kMaxC; ++c) per_class[c] = 0;
-            int32_t ids4[4];
-            float vals4[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) { ids4[c] = ids_nx[c]; vals4[c] = vals_nx[c]; }
-            load4(j + NW, ids_nx, vals_nx);
-            auto take = [&](int e, int32_t id, float x) {
-                const bool on = id >= 0;
-                if (on) {
-                    sh.idx[r0 + e] = id;
-                    sh.val[r0 + e] = x;
-                    uint32_t p = home_slot<HT>(id);
-                    if (id < kHD) {
-                        sh.key[p] = id;
-                        sh.Dc[j][id] = x;
-                    } else {
-                        for (int probe = 0; probe < HT; ++probe) {
-                            int32_t seen = sh.key[p];
-                            if (seen == -1) {
-                                seen = atomicCAS(&sh.key[p], -1, id);
-                                if (seen == -1) break;
-                            }
-                            if (seen == id) break;
-                            p = next_slot<HT>(p);
-                        }
+        for (int i = 0; i < EPT; ++i) {
+            const int e = tid + i * THREADS;
+            if (e >= total) break;
+            const int32_t id = checked_id(P, sh.idx[cur][e]);
+            uint32_t p = home_slot<HT>(id);
+            if (id < kHD) sh.key[p] = id;
+            else
+                for (int t = 0; t < HT; ++t) {
+                    int32_t seen = sh.key[p];
+                    if (seen == -1) {
+                        seen = atomicCAS(&sh.key[p], -1, id);
+                        if (seen == -1) break;
                     }
-                    atomicOr(&sh.mask[p], 1u << j);
-                    sh.slot[r0 + e] = (uint16_t)p;
+                    if (seen == id) break;
+                    p = next_slot<HT>(p);
                 }
-#pragma unroll
-                for (int c = 0; c < kMaxC; ++c)
-                    if (c < C) per_class[c] += __popc(__ballot_sync(0xffffffffu, on && (id & (C - 1)) == c));
-            };
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (32 * c < n) take(lane + 32 * c, ids4[c], vals4[c]);
-            for (int e0 = 128; e0 < n; e0 += 32) {
-                const int e = e0 + lane;
-                take(e, e < n ? checked_id(P, P.S.indices[rs + e]) : -1, e < n ? P.S.values[rs + e] : 0.0f);
-            }
-            if (lane == 0) {
-#pragma unroll
-                for (int c = 0; c < kMaxC; ++c) sh.rc[j][c] = (uint16_t)per_class[c];
-            }
+            atomicOr(&sh.mask[p], 1u << sh.row[cur][e]);
+            sh.slot[e] = (uint16_t)p;
         }
-    }
-    __syncthreads();
-    PRE_T(1);
-    // ---- count the ids that more than one coordinate has, and their list entries, per CTA (shared-memory atomics:
-    //      ids in the high half, list entries in the low half; only the totals are needed before the records' places
-    //      are known)
-    if (!slow)
-        for (int p = tid; p < HT; p += THREADS) {
+        __syncthreads();
+        PRE_T(0);
+        // ---- the first coordinate that has an id numbers it: shared ids among their CTA's (ids in the high half of the
+        //      counter, list entries in the low half) and in lval. (The order of the numbers varies from run to run, which
+        //      moves records' contents about but changes no result: every id's own sum is taken in coordinate order, in a
+        //      shape that depends on the list's length alone.)
+        uint32_t tl[EPT];
+#pragma unroll
+        for (int i = 0; i < EPT; ++i) {
+            const int e = tid + i * THREADS;
+            tl[i] = 0xffffffffu;
+            if (e >= total) break;
+            const int p = sh.slot[e], j = sh.row[cur][e];
             const uint32_t m = sh.mask[p];
-            if (m & (m - 1u)) atomicAdd(&sh.cntTL[sh.key[p] & (C - 1)], (1u << 16) + (uint32_t)__popc(m));
+            if (m & ((1u << j) - 1u)) continue;
+            if (m & (m - 1u)) {
+                const uint32_t pc = (uint32_t)__popc(m);
+                tl[i] = atomicAdd(&sh.cntTL[sh.key[p] & (C - 1)], (1u << 16) + pc);
+                sh.coff[p] = (uint16_t)(tl[i] & 0xffffu);
+                sh.soff[p] = (uint16_t)(NZ + atomicAdd(&sh.cntAll, pc));
+            } else sh.soff[p] = (uint16_t)e;
         }
-    // where each coordinate's non-zeros start in each CTA's record (warp 0, lane = coordinate)
-    if (warp == 0 && !slow) {
-#pragma unroll
-        for (int c = 0; c < kMaxC; ++c) {
-            const int mine = sh.rc[lane][c];
-            int incl = mine;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
+        if (warp == NW - 3) { // where each coordinate's entries start in each CTA's record
+            for (int j = lane; j <= kLB; j += 32) {
+                const int s = B.roff[j], ch = s >> 5;
+                for (int c = 0; c < C; ++c)
+                    sh.rc[j][c] = (uint16_t)(sh.pre[cur][ch][c] + __popc(sh.bal[cur][ch][c] & ((1u << (s & 31)) - 1u)));
             }
-            sh.rc[lane][c] = (uint16_t)(incl - mine);
-            if (lane == 31) sh.rc[kLB][c] = (uint16_t)incl;
         }
-    }
-    __syncthreads();
-    PRE_T(2);
-    // ---- the records' places: the head has its own (one per block); the workers' records come from the pool. A
-    //      block that the pool has no room for is walked in place like one that is too long.
-    if (tid == 0) {
-        unsigned long long need = 0;
-        uint32_t len[kMaxC];
-#pragma unroll
-        for (int c = 0; c < kMaxC; ++c) {
-            len[c] = c < C ? sub_bytes(sh.rc[kLB][c], (int)(sh.cntTL[c] >> 16), false) : 0u;
-            need += len[c];
-        }
-        unsigned long long at = 0;
-        int sl = sh.slow;
-#pragma unroll
-        for (int c = 0; c < kMaxC; ++c)
-            if (c < C && sh.rc[kLB][c] > P.nzcap) sl = 1; // more of them fall to one CTA than its record holds
-        if (!sl) {
-            at = atomicAdd(P.cursor, need);
-            if (at + need > P.pool_cap) sl = 2;
-        }
-        sh.slow = sl;
-#pragma unroll
-        for (int c = 0; c < kMaxC; ++c) {
-            if (c >= C) continue;
-            BlkDir d;
-            if (sl) { // nothing to stage: the workers copy the first bytes of the head instead
-                d.offset = (unsigned long long)bid * sizeof(ChainHead);
-                d.bytes = 16u;
-                d.flags = 1u;
-            } else {
-                d.offset = P.pool_off + at;
-                d.bytes = len[c];
-                d.flags = 0u;
-                sh.sub_off[c] = d.offset;
-                sh.sub_len[c] = len[c];
-                sh.subT[c] = (int32_t)(sh.cntTL[c] >> 16);
-                at += len[c];
-            }
-            if (bid == P.drop_block) d.bytes = 0u;
-            P.dirS[bid * C + c] = d;
-        }
-    }
-    __syncthreads();
-    PRE_T(3);
-    const bool walk = sh.slow != 0; // (slow, or no room in the pool)
-    if (warp == 0 && lane == 0) {
-        out.cnt = cnt;
-        out.flags = walk ? 1 : 0;
-        out.pad[0] = out.pad[1] = 0;
-    }
-    if (walk) {
-        // the head carries the constants of the steps and nothing else; nothing is carried to the next block
-        if (warp == 0) {
-            out.hdr[lane] = sh.hdr[lane];
-            out.q0n[lane] = 0.0f;
-        }
-        for (int i = tid; i < kLB * kLB; i += THREADS) out.X[i] = 0.0f;
-        return;
-    }
-    if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) write_table(P, bid, sh.hdr, THREADS);
-    // ---- the workers' record heads, shared-id tables and list starts
-    if (tid < C) {
-        SubHead &h = *reinterpret_cast<SubHead *>(P.rec + sh.sub_off[tid]);
-        h.n = sh.rc[kLB][tid];
-        h.T = sh.subT[tid];
-        h.cnt = cnt;
-        h.flags = 0;
-    }
-    for (int i = tid; i < C * (kLB + 8); i += THREADS) {
-        const int c = i / (kLB + 8), j = i - c * (kLB + 8);
-        reinterpret_cast<SubHead *>(P.rec + sh.sub_off[c])->roff[j] = sh.rc[j < kLB ? j : kLB][c];
-    }
-    for (int p = tid; p < HT; p += THREADS) {
-        const uint32_t m = sh.mask[p];
-        if (m == 0u) continue;
-        // (numbered with atomics: the order varies from run to run, which moves records' contents about but changes no
-        // result: every id's own sum is taken in coordinate order, in a shape that depends on the list's length alone)
-        const uint32_t pc = (uint32_t)__popc(m);
-        sh.soff[p] = (uint16_t)atomicAdd(&sh.cntAll, pc);
-        if (m & (m - 1u)) {
-            const int32_t id = sh.key[p];
-            const int c = id & (C - 1);
-            const uint32_t r = atomicAdd(&sh.cntTL2[c], (1u << 16) + pc);
-            const uint32_t t = r >> 16, o = r & 0xffffu;
-            unsigned char *rec = P.rec + sh.sub_off[c];
-            const int n_c = sh.rc[kLB][c], T_c = sh.subT[c];
-            uint32_t *ids_g = reinterpret_cast<uint32_t *>(rec + sizeof(SubHead) + 8u * n_c);
-            uint16_t *off_g = reinterpret_cast<uint16_t *>(rec + sizeof(SubHead) + 8u * n_c + 4u * T_c + 2u * n_c);
-            ids_g[t] = (uint32_t)id;
-            off_g[t] = (uint16_t)o;
-            sh.coff[p] = (uint16_t)o;
-        }
-    }
-    if (tid < C) { // the end of the last list
-        unsigned char *rec = P.rec + sh.sub_off[tid];
-        const int n_c = sh.rc[kLB][tid], T_c = sh.subT[tid];
-        reinterpret_cast<uint16_t *>(rec + sizeof(SubHead) + 8u * n_c + 4u * T_c + 2u * n_c)[T_c] = (uint16_t)(sh.cntTL[tid] & 0xffffu);
-    }
-    __syncthreads();
-    PRE_T(4);
-    // ---- the non-zeros into the workers' records, row after row: place = start of (coordinate, CTA) + rank among
-    //      the coordinate's non-zeros of that CTA; a shared id's place in its list is the number of lower
-    //      coordinates that have the id
-    for (int j = warp; j < cnt; j += NW) {
-        const int n = sh.nnz[j], r0 = sh.roff[j];
-        int before[kMaxC];
-#pragma unroll
-        for (int c = 0; c < kMaxC; ++c) before[c] = sh.rc[j][c];
-        for (int e0 = 0; e0 < n; e0 += 32) {
-            const int e = e0 + lane;
-            const bool on = e < n;
-            const int32_t id = on ? sh.idx[r0 + e] : 0;
-            const int cls = id & (C - 1);
-            int place = 0;
+        __syncthreads();
+        PRE_T(1);
+        // ---- the records' places: the head has its own (one per block); the workers' records come from the pool, of which
+        //      a CTA takes a piece for several blocks at a time. A block that the pool has no room for is walked in place
+        //      like one that is too long.
+        if (tid == 0) {
+            unsigned long long need = 0;
+            int sl = B.over;
+            uint32_t len[kMaxC];
 #pragma unroll
             for (int c = 0; c < kMaxC; ++c) {
                 if (c >= C) continue;
-                const uint32_t bal = __ballot_sync(0xffffffffu, on && cls == c);
-                if (cls == c) place = before[c] + __popc(bal & ((1u << lane) - 1u));
-                before[c] += __popc(bal);
+                len[c] = sub_bytes(sh.rc[kLB][c], (int)(sh.cntTL[c] >> 16), false);
+                need += len[c];
+                if (sh.rc[kLB][c] > P.nzcap) sl = 1; // more of them fall to one CTA than its record holds
             }
-            if (!on) continue;
-            const int p = sh.slot[r0 + e];
-            const uint32_t m = sh.mask[p];
-            const bool shared_id = (m & (m - 1u)) != 0u;
-            const int lower = __popc(m & ((1u << j) - 1u));
-            const float x = sh.val[r0 + e];
-            sh.lval[sh.soff[p] + lower] = x;
-            unsigned char *rec = P.rec + sh.sub_off[cls];
-            const int n_c = sh.rc[kLB][cls], T_c = sh.subT[cls];
-            float *val_g = reinterpret_cast<float *>(rec + sizeof(SubHead));
-            uint32_t *meta_g = reinterpret_cast<uint32_t *>(rec + sizeof(SubHead) + 4u * n_c);
-            uint16_t *cpos_g = reinterpret_cast<uint16_t *>(rec + sizeof(SubHead) + 8u * n_c + 4u * T_c);
-            val_g[place] = x;
-            meta_g[place] = (uint32_t)id | ((uint32_t)j << kIdBits) | (shared_id ? 0x80000000u : 0u);
-            cpos_g[place] = shared_id ? (uint16_t)(sh.coff[p] + lower) : (uint16_t)0;
-            // for the Gram pass: the id itself is no longer needed, its mask and its list's start are (top bit: one of
-            // the ids that the dense tiles cover)
-            sh.idx[r0 + e] = (int32_t)m;
-            sh.slot[r0 + e] = (uint16_t)(sh.soff[p] | (id < kHD ? 0x8000 : 0));
+            if (!sl && sh.pool_at + need > sh.pool_end) {
+                const unsigned long long take = need > P.pool_piece ? need : P.pool_piece;
+                unsigned long long at = atomicAdd(P.cursor, take);
+                sh.pool_at = at;
+                sh.pool_end = at + take < P.pool_cap ? at + take : P.pool_cap;
+                if (at + need > P.pool_cap) { sl = 2; sh.pool_end = 0ull; }
+            }
+            sh.walk = sl;
+            unsigned long long at = sh.pool_at;
+#pragma unroll
+            for (int c = 0; c < kMaxC; ++c) {
+                if (c >= C) continue;
+                BlkDir d;
+                if (sl) { // nothing to stage: the workers copy the first bytes of the head instead
+                    d.offset = (unsigned long long)bid * sizeof(ChainHead);
+                    d.bytes = 16u;
+                    d.flags = 1u;
+                } else {
+                    d.offset = P.pool_off + at;
+                    d.bytes = len[c];
+                    d.flags = 0u;
+                    sh.sub_off[c] = d.offset;
+                    at += len[c];
+                }
+                if (bid == P.drop_block) d.bytes = 0u;
+                P.dirS[bid * C + c] = d;
+            }
+            if (!sl) sh.pool_at = at;
+            out.cnt = cnt;
+            out.flags = sl ? 1 : 0;
+            out.pad[0] = out.pad[1] = 0;
         }
-    }
-    __syncthreads();
-    PRE_T(5);
-    // ---- Gram triangle: a warp per coordinate j, lane l collects x_j . x_l over j's entries in ascending order. The
-    //      lanes first look at 32 entries at once and keep those whose id an earlier coordinate has too; only these
-    //      are then walked, their mask, list start and value handed round by shuffles.
-    for (int j = warp; j < kLB; j += NW) {
-        float acc = 0.0f;
-        if (j < cnt) {
-            const int n = sh.nnz[j], r0 = sh.roff[j];
-            const uint32_t below = (1u << j) - 1u, lt = (1u << lane) - 1u;
-            {
-                const float4 *dj = reinterpret_cast<const float4 *>(&sh.Dc[j][0]);
-                const float4 *dm = reinterpret_cast<const float4 *>(&sh.Dc[lane][0]);
-#pragma unroll
-                for (int h = 0; h < kHD / 4; ++h) {
-                    const float4 a = dj[h], b4 = dm[h];
-                    acc = fmaf(a.x, b4.x, acc); acc = fmaf(a.y, b4.y, acc); acc = fmaf(a.z, b4.z, acc); acc = fmaf(a.w, b4.w, acc);
-                }
-            }
-            for (int e0 = 0; e0 < n; e0 += 32) {
-                const int e = e0 + lane;
-                uint32_t m_l = 0u;
-                int so_l = 0;
-                float x_l = 0.0f;
-                if (e < n) {
-                    m_l = (uint32_t)sh.idx[r0 + e];
-                    so_l = sh.slot[r0 + e];
-                    x_l = sh.val[r0 + e];
-                }
-                uint32_t todo = __ballot_sync(0xffffffffu, (m_l & below) != 0u && !(so_l & 0x8000)); // (not the dense ones)
-                // two entries per turn, so that the second one's loads are under way while the first is added
-                while (todo) {
-                    const int src0 = __ffs(todo) - 1;
-                    todo &= todo - 1u;
-                    const bool two = todo != 0u;
-                    const int src1 = two ? __ffs(todo) - 1 : src0;
-                    todo &= todo - 1u;
-                    const uint32_t m0 = __shfl_sync(0xffffffffu, m_l, src0), m1 = __shfl_sync(0xffffffffu, m_l, src1);
-                    const int so0 = __shfl_sync(0xffffffffu, so_l, src0), so1 = __shfl_sync(0xffffffffu, so_l, src1);
-                    const float x0 = __shfl_sync(0xffffffffu, x_l, src0), x1 = __shfl_sync(0xffffffffu, x_l, src1);
-                    const bool on0 = (m0 >> lane) & 1u, on1 = two && ((m1 >> lane) & 1u);
-                    const float v0 = sh.lval[on0 ? so0 + __popc(m0 & lt) : 0], v1 = sh.lval[on1 ? so1 + __popc(m1 & lt) : 0];
-                    acc = fmaf(x0, on0 ? v0 : 0.0f, acc);
-                    acc = fmaf(x1, on1 ? v1 : 0.0f, acc);
-                }
-            }
-            if (lane >= j) acc = 0.0f;
-        }
-        acc *= sh.gsc[j] * sh.ys[lane];
-        sh.G[lane][j] = acc; // row l, column j
-        float q0 = acc * sh.as[lane];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) q0 += __shfl_xor_sync(0xffffffffu, q0, o);
-        if (lane == 0) sh.hdr[j].A -= q0;
-    }
-    PRE_T(6);
-    // ---- cross Gram matrix with the next block: a warp per coordinate j of the next block, whose non-zeros come
-    //      straight from the matrix and are looked up in this block's table; lane l collects x_j . x_l
-    //      (the first 128 entries of a warp's next coordinate are loaded while it works on the current one)
-    int32_t xids_nx[4];
-    float xvals_nx[4];
-    auto xload4 = [&](int j, int32_t (&ids)[4], float (&vals)[4]) {
-        const bool have = carry && j < sh.ncnt;
-        const int n = have ? sh.nnnz[j] : 0;
-        const int64_t rs = have ? sh.nrs[j] : 0;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int e = lane + 32 * c;
-            ids[c] = e < n ? checked_id(P, P.S.indices[rs + e]) : -1;
-            vals[c] = e < n ? P.S.values[rs + e] : 0.0f;
-        }
-    };
-    xload4(warp, xids_nx, xvals_nx);
-    for (int j = warp; j < kLB; j += NW) {
-        float acc = 0.0f;
-        int32_t ids4[4];
-        float vals4[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) { ids4[c] = xids_nx[c]; vals4[c] = xvals_nx[c]; }
-        xload4(j + NW, xids_nx, xvals_nx);
-        if (carry && j < sh.ncnt) {
-            const int n = sh.nnnz[j];
-            const int64_t rs = sh.nrs[j];
-            const uint32_t lt = (1u << lane) - 1u;
-            int per_class[kMaxC];
-#pragma unroll
-            for (int c = 0; c < kMaxC; ++c) per_class[c] = 0;
-            auto take = [&](int32_t id, float x_l) {
-                uint32_t m_l = 0u;
-                int so_l = 0;
-#pragma unroll
-                for (int c = 0; c < kMaxC; ++c)
-                    if (c < C) per_class[c] += __popc(__ballot_sync(0xffffffffu, id >= 0 && (id & (C - 1)) == c));
-                if (id >= 0 && id < kHD) sh.Dn[j][id] = x_l;
-                else if (id >= 0) {
-                    uint32_t p = home_slot<HT>(id);
-                    for (int probe = 0; probe < HT; ++probe) {
-                        const int32_t seen = sh.key[p];
-                        if (seen == id) { m_l = sh.mask[p]; so_l = sh.soff[p]; break; }
-                        if (seen == -1) break;
-                        p = next_slot<HT>(p);
-                    }
-                }
-                uint32_t todo = __ballot_sync(0xffffffffu, m_l != 0u);
-                while (todo) {
-                    const int src0 = __ffs(todo) - 1;
-                    todo &= todo - 1u;
-                    const bool two = todo != 0u;
-                    const int src1 = two ? __ffs(todo) - 1 : src0;
-                    todo &= todo - 1u;
-                    const uint32_t m0 = __shfl_sync(0xffffffffu, m_l, src0), m1 = __shfl_sync(0xffffffffu, m_l, src1);
-                    const int so0 = __shfl_sync(0xffffffffu, so_l, src0), so1 = __shfl_sync(0xffffffffu, so_l, src1);
-                    const float x0 = __shfl_sync(0xffffffffu, x_l, src0), x1 = __shfl_sync(0xffffffffu, x_l, src1);
-                    const bool on0 = (m0 >> lane) & 1u, on1 = two && ((m1 >> lane) & 1u);
-                    const float v0 = sh.lval[on0 ? so0 + __popc(m0 & lt) : 0], v1 = sh.lval[on1 ? so1 + __popc(m1 & lt) : 0];
-                    acc = fmaf(x0, on0 ? v0 : 0.0f, acc);
-                    acc = fmaf(x1, on1 ? v1 : 0.0f, acc);
-                }
-            };
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (32 * c < n) take(ids4[c], vals4[c]);
-            for (int e0 = 128; e0 < n; e0 += 32) {
-                const int e = e0 + lane;
-                take(e < n ? checked_id(P, P.S.indices[rs + e]) : -1, e < n ? P.S.values[rs + e] : 0.0f);
-            }
-            __syncwarp();
-            {
-                const float4 *dj = reinterpret_cast<const float4 *>(&sh.Dn[j][0]);
-                const float4 *dm = reinterpret_cast<const float4 *>(&sh.Dc[lane][0]);
-#pragma unroll
-                for (int h = 0; h < kHD / 4; ++h) {
-                    const float4 a = dj[h], b4 = dm[h];
-                    acc = fmaf(a.x, b4.x, acc); acc = fmaf(a.y, b4.y, acc); acc = fmaf(a.z, b4.z, acc); acc = fmaf(a.w, b4.w, acc);
-                }
-            }
-            if (lane >= cnt) acc = 0.0f;
-            if (lane == 0) {
-#pragma unroll
-                for (int c = 0; c < kMaxC; ++c)
-                    if (c < C && per_class[c]) atomicAdd(&sh.ncls[c], per_class[c]);
-            }
-        }
-        acc *= sh.gscn[j] * sh.ys[lane];
-        sh.X[lane][j] = acc; // row l (this block), column j (next block)
-        float q0 = acc * sh.as[lane];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) q0 += __shfl_xor_sync(0xffffffffu, q0, o);
-        if (lane == 0) sh.q0n[j] = q0;
-    }
-    __syncthreads();
-    PRE_T(7);
-    // (a next block that is walked in place because more of its non-zeros fall to one CTA than a record holds takes
-    // nothing over either)
-    bool keep = true;
-#pragma unroll
-    for (int c = 0; c < kMaxC; ++c)
-        if (c < C && sh.ncls[c] > P.nzcap) keep = false;
-    for (int i = tid; i < kLB * kLB; i += THREADS) {
-        out.G[i] = sh.G[i >> 5][i & 31];
-        out.X[i] = keep ? sh.X[i >> 5][i & 31] : 0.0f;
-    }
-    if (warp == 0) {
-        out.hdr[lane] = sh.hdr[lane];
-        out.q0n[lane] = keep ? sh.q0n[lane] : 0.0f;
-    }
-}
-
-// A CTA takes blocks blockIdx.x, blockIdx.x + gridDim.x, ...: one each when the grid has a CTA per block; a launch
-// beside the chain kernels gets a grid that fits the SMs they leave, so that it never has CTAs waiting for an SM (which
-// would take the SMs of a finished chain launch before the next chain launch's CTAs, which need a whole SM each).
-template <int LOSS, int NZ, int HT, int THREADS>
-__global__ void __launch_bounds__(THREADS) k_lookahead_prepare(const LookParams P)
-{
-    extern __shared__ __align__(16) unsigned char smem_pre[];
-    using Shared = PreShared<NZ, HT, THREADS>;
-    Shared &sh = *reinterpret_cast<Shared *>(smem_pre);
-    if (P.K < kBaseStaged) {
-        for (int i = threadIdx.x; i <= P.K; i += THREADS) sh.base[i] = (int32_t)P.blk_base[i];
         __syncthreads();
-    }
-    for (int64_t bid = blockIdx.x; bid < P.n_blocks; bid += gridDim.x) {
-        prepare_block<LOSS, NZ, HT, THREADS>(P, bid, sh);
-        __syncthreads(); // the shared arrays are reused by the next block
+        PRE_T(2);
+        const bool walk = sh.walk != 0;
+        const bool carry = have_next && !walk && !N.over && P.depth >= 2 && B.k == N.k;
+        if (!walk) {
+            if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) write_table(P, bid, B.hdr, THREADS);
+            // ---- the workers' record heads, and the entries, row after row: place = entries of that CTA before this one; a
+            //      shared id's place in its list is the number of lower coordinates that have the id
+            if (tid < C) {
+                SubHead &h = *reinterpret_cast<SubHead *>(P.rec + sh.sub_off[tid]);
+                const int n_c = sh.rc[kLB][tid], T_c = (int)(sh.cntTL[tid] >> 16);
+                h.n = n_c;
+                h.T = T_c;
+                h.cnt = cnt;
+                h.flags = 0;
+                // the end of the last list
+                reinterpret_cast<uint16_t *>(P.rec + sh.sub_off[tid] + sizeof(SubHead) + 10u * n_c + 4u * T_c)[T_c] = (uint16_t)(sh.cntTL[tid] & 0xffffu);
+            }
+            for (int i = tid; i < C * (kLB + 8); i += THREADS) {
+                const int c = i / (kLB + 8), j = i - c * (kLB + 8);
+                reinterpret_cast<SubHead *>(P.rec + sh.sub_off[c])->roff[j] = sh.rc[j < kLB ? j : kLB][c];
+            }
+#pragma unroll
+            for (int i = 0; i < EPT; ++i) {
+                const int e = tid + i * THREADS;
+                if (e >= total) break;
+                const int32_t id = checked_id(P, sh.idx[cur][e]);
+                const int cls = id & (C - 1), j = sh.row[cur][e], p = sh.slot[e];
+                const int place = sh.pre[cur][e >> 5][cls] + __popc(sh.bal[cur][e >> 5][cls] & ((1u << lane) - 1u));
+                const uint32_t m = sh.mask[p];
+                const bool shared_id = (m & (m - 1u)) != 0u;
+                const int lower = __popc(m & ((1u << j) - 1u));
+                const float x = sh.val[cur][e];
+                unsigned char *rec = P.rec + sh.sub_off[cls] + sizeof(SubHead);
+                const uint32_t n_c = sh.rc[kLB][cls], T_c = sh.cntTL[cls] >> 16;
+                reinterpret_cast<float *>(rec)[place] = x;
+                reinterpret_cast<uint32_t *>(rec + 4u * n_c)[place] = (uint32_t)id | ((uint32_t)j << kIdBits) | (shared_id ? 0x80000000u : 0u);
+                uint16_t *cpos_g = reinterpret_cast<uint16_t *>(rec + 8u * n_c + 4u * T_c);
+                cpos_g[place] = shared_id ? (uint16_t)(sh.coff[p] + lower) : (uint16_t)0;
+                if (shared_id) sh.lval[sh.soff[p] - NZ + lower] = x;
+                if (tl[i] != 0xffffffffu) {
+                    reinterpret_cast<uint32_t *>(rec + 8u * n_c)[tl[i] >> 16] = (uint32_t)id;
+                    (cpos_g + n_c)[tl[i] >> 16] = (uint16_t)(tl[i] & 0xffffu);
+                }
+            }
+        }
+        __syncthreads();
+        PRE_T(3);
+        // ---- Gram triangle: a warp per coordinate j, lane l collects x_j . x_l over j's entries in ascending order. The
+        //      lanes first look at 32 entries at once and keep those whose id an earlier coordinate has too; only these
+        //      are then walked.
+        if (!walk)
+            for (int j = warp; j < kLB; j += NW) {
+                float acc = 0.0f;
+                const int n = B.nnz[j], r0 = B.roff[j];
+                if (n) {
+                    const uint32_t below = (1u << j) - 1u;
+                    acc = pre_dense_dot(&sh.D[cur][j][0], &sh.D[cur][lane][0]);
+                    for (int e0 = 0; e0 < n; e0 += 32) {
+                        uint32_t m_l = 0u, at_l = 0u;
+                        float x_l = 0.0f;
+                        if (e0 + lane < n) {
+                            const int p = sh.slot[r0 + e0 + lane];
+                            if (p >= kHD) { // (the dense tile has the others)
+                                m_l = sh.mask[p];
+                                at_l = smem_u32(&sh.lval[0]) + 4u * (uint32_t)(sh.soff[p] - NZ);
+                                x_l = sh.val[cur][r0 + e0 + lane];
+                            }
+                        }
+                        pre_add_listed(__ballot_sync(0xffffffffu, (m_l & below) != 0u), m_l, at_l, x_l, acc);
+                    }
+                    if (lane >= j) acc = 0.0f;
+                }
+                acc *= B.gsc[j] * B.ys[lane];
+                sh.G[lane][j] = acc; // row l, column j
+                float q0 = acc * B.as[lane];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) q0 += __shfl_xor_sync(0xffffffffu, q0, o);
+                if (lane == 0) B.hdr[j].A -= q0;
+            }
+        cp_async_wait_all(); // the next block's rows, the extents after it, the order after that
+        __syncthreads();
+        PRE_T(4);
+        // ---- the head's Gram triangle and constants; the next block's entries looked up in this block's table
+        if (!walk)
+            for (int i = tid; i < kLB * kLB; i += THREADS) out.G[i] = sh.G[i >> 5][i & 31];
+        if (warp == 0) out.hdr[lane] = B.hdr[lane];
+        if (warp == NW - 1 && bid + 2 < end) pre_make_block<LOSS, NZ, HT>(P, sh, bid + 2);
+        if (have_next) pre_scan<NZ, HT, THREADS>(P, sh, N.total, nxt, C, carry);
+        __syncthreads();
+        PRE_T(5);
+        // ---- cross Gram matrix: a warp per coordinate j of the next block; lane l collects x_j . x_l
+        if (have_next && warp < C) pre_prefix(sh, N.total, nxt, warp);
+        if (carry)
+            for (int j = warp; j < kLB; j += NW) {
+                float acc = 0.0f;
+                const int n = N.nnz[j], r0 = N.roff[j];
+                if (n) {
+                    acc = pre_dense_dot(&sh.D[nxt][j][0], &sh.D[cur][lane][0]);
+                    for (int e0 = 0; e0 < n; e0 += 32) {
+                        uint32_t m_l = 0u, at_l = 0u;
+                        float x_l = 0.0f;
+                        if (e0 + lane < n) {
+                            const int p = sh.found[r0 + e0 + lane];
+                            if (p != 0xffff) {
+                                m_l = sh.mask[p];
+                                const int so = sh.soff[p];
+                                at_l = so < NZ ? smem_u32(&sh.val[cur][so]) : smem_u32(&sh.lval[so - NZ]);
+                                x_l = sh.val[nxt][r0 + e0 + lane];
+                            }
+                        }
+                        pre_add_listed(__ballot_sync(0xffffffffu, m_l != 0u), m_l, at_l, x_l, acc);
+                    }
+                    if (lane >= cnt) acc = 0.0f;
+                }
+                acc *= N.gsc[j] * B.ys[lane];
+                sh.G[lane][j] = acc; // row l (this block), column j (next block)
+                float q0 = acc * B.as[lane];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) q0 += __shfl_xor_sync(0xffffffffu, q0, o);
+                if (lane == 0) sh.q0n[j] = q0;
+            }
+        __syncthreads();
+        PRE_T(6);
+        // (a next block that is walked in place because more of its entries fall to one CTA than a record holds takes
+        // nothing over either)
+        bool keep = carry;
+        for (int c = 0; c < C && keep; ++c) keep = sh.pre[nxt][(N.total + 31) >> 5][c] <= P.nzcap;
+        for (int i = tid; i < kLB * kLB; i += THREADS) out.X[i] = keep ? sh.G[i >> 5][i & 31] : 0.0f;
+        if (tid < kLB) out.q0n[tid] = keep ? sh.q0n[tid] : 0.0f;
+        for (int p = tid; p < HT / 4; p += THREADS) {
+            reinterpret_cast<int4 *>(sh.key)[p] = make_int4(-1, -1, -1, -1);
+            reinterpret_cast<uint4 *>(sh.mask)[p] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        if (tid < kMaxC) sh.cntTL[tid] = 0u;
+        if (tid == 0) sh.cntAll = 0u;
+        __syncthreads();
+        PRE_T(7);
     }
 }
 
@@ -2013,13 +2019,15 @@ template <int LOSS, bool DENSE, bool FLAT, bool TAB> cudaError_t launch_chain(Gl
     return e;
 }
 
-template <int LOSS, int NZ, int HT, int THREADS> cudaError_t launch_prepare(const LookParams &P, unsigned nb, cudaStream_t stream)
+template <int LOSS, int NZ, int HT, int THREADS, int PER_SM> cudaError_t launch_prepare(const LookParams &P, unsigned sms, cudaStream_t stream)
 {
     using Shared = PreShared<NZ, HT, THREADS>;
-    auto pre = k_lookahead_prepare<LOSS, NZ, HT, THREADS>;
+    static_assert(PER_SM * (sizeof(Shared) + 1024) <= 228 * 1024, "CTAs per SM");
+    auto pre = k_lookahead_prepare<LOSS, NZ, HT, THREADS, PER_SM>;
     cudaError_t e = cudaFuncSetAttribute(pre, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
     if (e != cudaSuccess) return e;
-    pre<<<nb, THREADS, sizeof(Shared), stream>>>(P);
+    const unsigned nb = (unsigned)P.n_blocks;
+    pre<<<nb < sms * PER_SM ? nb : sms * PER_SM, THREADS, sizeof(Shared), stream>>>(P);
     return cudaGetLastError();
 }
 
@@ -2051,16 +2059,10 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
         return cudaGetLastError();
     }
     cudaError_t e;
-    if (small_prepare(g)) {
-        const unsigned grid = stream == g.stream || nb < free_sms * 3 ? nb : free_sms * 3;
-        e = launch_prepare<LOSS, kPreSmallNz, 2048, 256>(P, grid, stream);
-    } else if (mid_prepare(g)) {
-        const unsigned grid = stream == g.stream || nb < free_sms * 2 ? nb : free_sms * 2;
-        e = launch_prepare<LOSS, kPreMidNz, 4096, 512>(P, grid, stream);
-    } else {
-        const unsigned grid = stream == g.stream || nb < free_sms ? nb : free_sms;
-        e = launch_prepare<LOSS, 4096, 4096, 512>(P, grid, stream);
-    }
+    const unsigned sms = stream == g.stream ? (unsigned)g.sm_count : free_sms;
+    if (small_prepare(g)) e = launch_prepare<LOSS, kPreSmallNz, 2048, 512, 2>(P, sms, stream);
+    else if (mid_prepare(g)) e = launch_prepare<LOSS, kPreMidNz, 4096, 1024, 1>(P, sms, stream);
+    else e = launch_prepare<LOSS, 4096, 4096, 1024, 1>(P, sms, stream);
 #ifdef CHICLE_LA_TIMING
     if (e == cudaSuccess) {
         unsigned long long t[8] = {0};
@@ -2068,8 +2070,7 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
         (void)cudaMemcpy(t, P.timing + 16, sizeof(t), cudaMemcpyDeviceToHost);
         (void)cudaMemset(P.timing + 16, 0, sizeof(t));
         const double n = (double)nb;
-        fprintf(stderr, "lookahead prepare, cycles per block: headers %.0f, load + insert %.0f, count %.0f, place %.0f, number %.0f, "
-                "entries %.0f, gram %.0f, cross + write %.0f\n", t[0] / n, t[1] / n, t[2] / n, t[3] / n, t[4] / n, t[5] / n, t[6] / n, t[7] / n);
+        fprintf(stderr, "lookahead prepare, cycles per block: insert %.0f, number %.0f, place %.0f, entries %.0f, gram %.0f, scan %.0f, cross %.0f, write %.0f\n", t[0] / n, t[1] / n, t[2] / n, t[3] / n, t[4] / n, t[5] / n, t[6] / n, t[7] / n);
     }
 #endif
     return e;
@@ -2238,6 +2239,9 @@ void lookahead_plan(Glm &g, int32_t K)
         const double all = 14.0 * (double)g.nnz;
         double part = whole ? all : 1.2 * frac * all + (double)(1 << 20);
         if (part > all) part = all;
+        // (what the prepare kernel's CTAs hold in advance: a piece of about four blocks each)
+        g.la_pool_piece = ((size_t)(4.0 * 14.0 * 32.0 * (double)g.nnz / (double)g.n_coord) + 4096) & ~(size_t)255; // (records start on 16-byte boundaries)
+        part += (double)g.la_pool_piece * (double)(region_blocks < 2 * (int64_t)g.sm_count ? region_blocks : 2 * (int64_t)g.sm_count);
         pool = (size_t)part + (size_t)region_blocks * C * 128 + 4096;
     }
     const size_t heads = ((size_t)region_blocks * sizeof(ChainHead) + 255) & ~(size_t)255;
@@ -2346,6 +2350,7 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
         p.timing = g.la_cursor + 8;
         p.pool_off = g.la_pool_off;
         p.pool_cap = g.la_region_bytes - g.la_pool_off;
+        p.pool_piece = g.la_pool_piece;
         p.blk_base = g.la_blk_base + (size_t)s * ((size_t)K + 1);
         p.K = K;
         p.logC = g.la_logC;
