@@ -377,7 +377,7 @@ constexpr int kHD = 32;
 constexpr int kHDS = kHD + 4; // row stride of the tiles: 16-byte loads of consecutive rows fall on different banks
 template <int HT> __device__ __forceinline__ uint32_t home_slot(int32_t id)
 {
-    return id < kHD ? (uint32_t)id : kHD + (((uint32_t)id * 2654435761u) >> 16) % (uint32_t)(HT - kHD);
+    return id < kHD ? (uint32_t)id : kHD + __umulhi((uint32_t)id * 2654435761u, (uint32_t)(HT - kHD));
 }
 template <int HT> __device__ __forceinline__ uint32_t next_slot(uint32_t p) { return p + 1 < (uint32_t)HT ? p + 1 : kHD; }
 
@@ -549,36 +549,45 @@ template <int NZ, int THREADS, class Shared> __device__ __forceinline__ void pre
 // (all warps: which entries of a fetched block fall to which CTA, its dense tile, and, with PROBE, where the table of the
 // current block has their ids)
 template <int NZ, int HT, int THREADS, class Shared>
-__device__ __forceinline__ void pre_scan(const LookParams &P, Shared &sh, int total, int buf, int C, bool probe)
+__device__ __forceinline__ void pre_scan(const LookParams &P, Shared &sh, int total, int buf, bool probe)
 {
+    constexpr int EPT = NZ / THREADS;
     const int lane = threadIdx.x & 31;
-    for (int e = threadIdx.x; (e & ~31) < total; e += THREADS) {
-        const bool on = e < total;
-        const int32_t id = on ? checked_id(P, sh.idx[buf][e]) : -1;
-        if (C > 1) {
-            uint32_t mine = 0u;
-            for (int c = 0; c < C; ++c) {
-                const uint32_t b = __ballot_sync(0xffffffffu, on && (id & (C - 1)) == c);
-                mine = lane == c ? b : mine;
-            }
-            if (lane < C) sh.bal[buf][e >> 5][lane] = mine;
-        } else {
-            const uint32_t b = __ballot_sync(0xffffffffu, on);
-            if (lane == 0) sh.bal[buf][e >> 5][0] = b;
+    int32_t id[EPT], seen[EPT];
+    uint32_t p[EPT];
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) {
+        const int e = (int)threadIdx.x + i * THREADS;
+        id[i] = e < total ? checked_id(P, sh.idx[buf][e]) : -1;
+        p[i] = id[i] >= kHD ? home_slot<HT>(id[i]) : 0u;
+    }
+    if (probe) {
+#pragma unroll
+        for (int i = 0; i < EPT; ++i) seen[i] = sh.key[p[i]];
+    }
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) {
+        const int e = (int)threadIdx.x + i * THREADS;
+        if ((e & ~31) >= total) break; // (whole warps)
+        uint32_t mine = __ballot_sync(0xffffffffu, id[i] >= 0);
+        for (int bit = 0; bit < P.logC; ++bit) {
+            const uint32_t b = __ballot_sync(0xffffffffu, (id[i] >> bit) & 1);
+            mine &= (lane >> bit) & 1 ? b : ~b;
         }
-        if (on && id < kHD) sh.D[buf][sh.row[buf][e]][id] = sh.val[buf][e];
-        if (probe && on) {
-            uint32_t p = 0xffffu;
-            if (id >= kHD) {
-                uint32_t q = home_slot<HT>(id);
-                for (int t = 0; t < HT; ++t) {
-                    const int32_t seen = sh.key[q];
-                    if (seen == id) { p = q; break; }
-                    if (seen == -1) break;
-                    q = next_slot<HT>(q);
+        if (lane >> P.logC == 0) sh.bal[buf][e >> 5][lane] = mine; // lane c: the entries of CTA c
+        if (id[i] >= 0 && id[i] < kHD) sh.D[buf][sh.row[buf][e]][id[i]] = sh.val[buf][e];
+    }
+    if (probe) {
+#pragma unroll
+        for (int i = 0; i < EPT; ++i) {
+            const int e = (int)threadIdx.x + i * THREADS;
+            if (e >= total) break;
+            if (id[i] >= kHD)
+                for (int t = 0; t < HT && seen[i] != id[i] && seen[i] != -1; ++t) {
+                    p[i] = next_slot<HT>(p[i]);
+                    seen[i] = sh.key[p[i]];
                 }
-            }
-            sh.found[e] = (uint16_t)p;
+            sh.found[e] = id[i] >= kHD && seen[i] == id[i] ? (uint16_t)p[i] : (uint16_t)0xffffu;
         }
     }
 }
@@ -615,23 +624,25 @@ __device__ __forceinline__ float pre_dense_dot(const float *a, const float *m)
     return acc;
 }
 // Adds what the entries marked in `todo` (lanes of this chunk) contribute: mask, list address and value handed round by
-// shuffles, two entries per turn, so that the second one's loads are under way while the first is added.
+// shuffles, four entries per turn, so that their loads are under way together (the additions stay in ascending order).
 __device__ __forceinline__ void pre_add_listed(uint32_t todo, uint32_t m_l, uint32_t at_l, float x_l, float &acc)
 {
     const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
     while (todo) {
-        const int src0 = __ffs(todo) - 1;
-        todo &= todo - 1u;
-        const bool two = todo != 0u;
-        const int src1 = two ? __ffs(todo) - 1 : src0;
-        todo &= todo - 1u;
-        const uint32_t m0 = __shfl_sync(0xffffffffu, m_l, src0), m1 = __shfl_sync(0xffffffffu, m_l, src1);
-        const uint32_t a0 = __shfl_sync(0xffffffffu, at_l, src0), a1 = __shfl_sync(0xffffffffu, at_l, src1);
-        const float x0 = __shfl_sync(0xffffffffu, x_l, src0), x1 = __shfl_sync(0xffffffffu, x_l, src1);
-        const bool on0 = (m0 >> lane) & 1u, on1 = two && ((m1 >> lane) & 1u);
-        const float v0 = lds_f32(a0 + (on0 ? 4u * (uint32_t)__popc(m0 & lt) : 0u)), v1 = lds_f32(a1 + (on1 ? 4u * (uint32_t)__popc(m1 & lt) : 0u));
-        acc = fmaf(x0, on0 ? v0 : 0.0f, acc);
-        acc = fmaf(x1, on1 ? v1 : 0.0f, acc);
+        float v[4], x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool any = todo != 0u;
+            const int src = any ? __ffs(todo) - 1 : 0;
+            todo &= todo - 1u; // (0 stays 0)
+            const uint32_t m = __shfl_sync(0xffffffffu, m_l, src), at = __shfl_sync(0xffffffffu, at_l, src);
+            x[u] = __shfl_sync(0xffffffffu, x_l, src);
+            const bool on = any && ((m >> lane) & 1u);
+            v[u] = 0.0f;
+            if (on) v[u] = lds_f32(at + 4u * (uint32_t)__popc(m & lt));
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc = fmaf(x[u], v[u], acc);
     }
 }
 
@@ -678,7 +689,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
     pre_fetch_rows<NZ, THREADS>(P, sh, lo, (int)(lo & 1));
     cp_async_wait_all();
     __syncthreads();
-    pre_scan<NZ, HT, THREADS>(P, sh, sh.blk[lo & (kDirNew - 1)].total, (int)(lo & 1), C, false);
+    pre_scan<NZ, HT, THREADS>(P, sh, sh.blk[lo & (kDirNew - 1)].total, (int)(lo & 1), false);
     __syncthreads();
     if (warp < C) pre_prefix(sh, sh.blk[lo & (kDirNew - 1)].total, (int)(lo & 1), warp);
     __syncthreads();
@@ -703,25 +714,33 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         if (warp == NW - 2 && bid + 3 < end) pre_fetch_order(P, sh, bid + 3);
         for (int p = tid; p < kLB * kHDS; p += THREADS) (&sh.D[nxt][0][0])[p] = 0.0f;
         // ---- every id into the table
+        {
+            int32_t id[EPT], seen[EPT];
+            uint32_t p[EPT];
 #pragma unroll
-        for (int i = 0; i < EPT; ++i) {
-            const int e = tid + i * THREADS;
-            if (e >= total) break;
-            const int32_t id = checked_id(P, sh.idx[cur][e]);
-            uint32_t p = home_slot<HT>(id);
-            if (id < kHD) sh.key[p] = id;
-            else
-                for (int t = 0; t < HT; ++t) {
-                    int32_t seen = sh.key[p];
-                    if (seen == -1) {
-                        seen = atomicCAS(&sh.key[p], -1, id);
-                        if (seen == -1) break;
-                    }
-                    if (seen == id) break;
-                    p = next_slot<HT>(p);
+            for (int i = 0; i < EPT; ++i) {
+                const int e = tid + i * THREADS;
+                id[i] = e < total ? checked_id(P, sh.idx[cur][e]) : -1;
+                p[i] = home_slot<HT>(id[i] >= 0 ? id[i] : 0);
+            }
+#pragma unroll
+            for (int i = 0; i < EPT; ++i) { // (most find their place at the first try: a thread's tries are under way together)
+                seen[i] = -1;
+                if (id[i] >= kHD) seen[i] = atomicCAS(&sh.key[p[i]], -1, id[i]);
+                else if (id[i] >= 0) sh.key[p[i]] = id[i];
+            }
+#pragma unroll
+            for (int i = 0; i < EPT; ++i) {
+                const int e = tid + i * THREADS;
+                if (e >= total) break;
+                for (int t = 0; t < HT && seen[i] != -1 && seen[i] != id[i]; ++t) {
+                    p[i] = next_slot<HT>(p[i]);
+                    seen[i] = sh.key[p[i]];
+                    if (seen[i] == -1) seen[i] = atomicCAS(&sh.key[p[i]], -1, id[i]);
                 }
-            atomicOr(&sh.mask[p], 1u << sh.row[cur][e]);
-            sh.slot[e] = (uint16_t)p;
+                atomicOr(&sh.mask[p[i]], 1u << sh.row[cur][e]);
+                sh.slot[e] = (uint16_t)p[i];
+            }
         }
         __syncthreads();
         PRE_T(0);
@@ -730,20 +749,35 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         //      moves records' contents about but changes no result: every id's own sum is taken in coordinate order, in a
         //      shape that depends on the list's length alone.)
         uint32_t tl[EPT];
+        {
+            uint32_t p[EPT], m[EPT], ls[EPT];
+            int32_t id[EPT];
 #pragma unroll
-        for (int i = 0; i < EPT; ++i) {
-            const int e = tid + i * THREADS;
-            tl[i] = 0xffffffffu;
-            if (e >= total) break;
-            const int p = sh.slot[e], j = sh.row[cur][e];
-            const uint32_t m = sh.mask[p];
-            if (m & ((1u << j) - 1u)) continue;
-            if (m & (m - 1u)) {
-                const uint32_t pc = (uint32_t)__popc(m);
-                tl[i] = atomicAdd(&sh.cntTL[sh.key[p] & (C - 1)], (1u << 16) + pc);
-                sh.coff[p] = (uint16_t)(tl[i] & 0xffffu);
-                sh.soff[p] = (uint16_t)(NZ + atomicAdd(&sh.cntAll, pc));
-            } else sh.soff[p] = (uint16_t)e;
+            for (int i = 0; i < EPT; ++i) {
+                const int e = tid + i * THREADS;
+                p[i] = e < total ? sh.slot[e] : 0u;
+                id[i] = e < total ? checked_id(P, sh.idx[cur][e]) : 0;
+                const uint32_t all = e < total ? sh.mask[p[i]] : 0u;
+                m[i] = e < total && (all & ((1u << sh.row[cur][e]) - 1u)) == 0u ? all : 0u; // 0: an earlier coordinate has the id
+            }
+#pragma unroll
+            for (int i = 0; i < EPT; ++i) {
+                tl[i] = 0xffffffffu;
+                ls[i] = 0u;
+                if (m[i] & (m[i] - 1u)) {
+                    const uint32_t pc = (uint32_t)__popc(m[i]);
+                    tl[i] = atomicAdd(&sh.cntTL[id[i] & (C - 1)], (1u << 16) + pc);
+                    ls[i] = atomicAdd(&sh.cntAll, pc);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < EPT; ++i) {
+                if (m[i] == 0u) continue;
+                if (m[i] & (m[i] - 1u)) {
+                    sh.coff[p[i]] = (uint16_t)(tl[i] & 0xffffu);
+                    sh.soff[p[i]] = (uint16_t)(NZ + ls[i]);
+                } else sh.soff[p[i]] = (uint16_t)(tid + i * THREADS);
+            }
         }
         if (warp == NW - 3) { // where each coordinate's entries start in each CTA's record
             for (int j = lane; j <= kLB; j += 32) {
@@ -757,48 +791,44 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         // ---- the records' places: the head has its own (one per block); the workers' records come from the pool, of which
         //      a CTA takes a piece for several blocks at a time. A block that the pool has no room for is walked in place
         //      like one that is too long.
-        if (tid == 0) {
-            unsigned long long need = 0;
-            int sl = B.over;
-            uint32_t len[kMaxC];
+        if (warp == 0) { // (a lane per CTA of the cluster)
+            const bool in = lane < C;
+            const uint32_t n_c = in ? sh.rc[kLB][lane] : 0u;
+            const uint32_t len = in ? sub_bytes((int)n_c, (int)(sh.cntTL[lane] >> 16), false) : 0u;
+            uint32_t incl = len;
 #pragma unroll
-            for (int c = 0; c < kMaxC; ++c) {
-                if (c >= C) continue;
-                len[c] = sub_bytes(sh.rc[kLB][c], (int)(sh.cntTL[c] >> 16), false);
-                need += len[c];
-                if (sh.rc[kLB][c] > P.nzcap) sl = 1; // more of them fall to one CTA than its record holds
+            for (int o = 1; o < kMaxC; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
             }
-            if (!sl && sh.pool_at + need > sh.pool_end) {
+            const uint32_t need = __shfl_sync(0xffffffffu, incl, kMaxC - 1);
+            // 1: longer than the arrays, or more of the entries fall to one CTA than its record holds
+            int sl = B.over || __any_sync(0xffffffffu, n_c > (uint32_t)P.nzcap) ? 1 : 0;
+            unsigned long long at = sh.pool_at, pool_end = sh.pool_end;
+            if (!sl && at + need > pool_end) {
                 const unsigned long long take = need > P.pool_piece ? need : P.pool_piece;
-                unsigned long long at = atomicAdd(P.cursor, take);
-                sh.pool_at = at;
-                sh.pool_end = at + take < P.pool_cap ? at + take : P.pool_cap;
-                if (at + need > P.pool_cap) { sl = 2; sh.pool_end = 0ull; }
+                if (lane == 0) at = atomicAdd(P.cursor, take);
+                at = __shfl_sync(0xffffffffu, at, 0);
+                pool_end = at + take < P.pool_cap ? at + take : P.pool_cap;
+                if (at + need > P.pool_cap) { sl = 2; pool_end = 0ull; }
             }
-            sh.walk = sl;
-            unsigned long long at = sh.pool_at;
-#pragma unroll
-            for (int c = 0; c < kMaxC; ++c) {
-                if (c >= C) continue;
-                BlkDir d;
-                if (sl) { // nothing to stage: the workers copy the first bytes of the head instead
-                    d.offset = (unsigned long long)bid * sizeof(ChainHead);
-                    d.bytes = 16u;
-                    d.flags = 1u;
-                } else {
-                    d.offset = P.pool_off + at;
-                    d.bytes = len[c];
-                    d.flags = 0u;
-                    sh.sub_off[c] = d.offset;
-                    at += len[c];
-                }
-                if (bid == P.drop_block) d.bytes = 0u;
-                P.dirS[bid * C + c] = d;
+            if (in) {
+                BlkDir d; // nothing to stage: the workers copy the first bytes of the head instead
+                d.offset = sl ? (unsigned long long)bid * sizeof(ChainHead) : P.pool_off + at + (incl - len);
+                d.bytes = bid == P.drop_block ? 0u : (sl ? 16u : len);
+                d.flags = sl ? 1u : 0u;
+                sh.sub_off[lane] = d.offset;
+                P.dirS[bid * C + lane] = d;
             }
-            if (!sl) sh.pool_at = at;
-            out.cnt = cnt;
-            out.flags = sl ? 1 : 0;
-            out.pad[0] = out.pad[1] = 0;
+            __syncwarp();
+            if (lane == 0) {
+                sh.walk = sl;
+                sh.pool_at = sl ? at : at + need;
+                sh.pool_end = pool_end;
+                out.cnt = cnt;
+                out.flags = sl ? 1 : 0;
+                out.pad[0] = out.pad[1] = 0;
+            }
         }
         __syncthreads();
         PRE_T(2);
@@ -888,7 +918,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
             for (int i = tid; i < kLB * kLB; i += THREADS) out.G[i] = sh.G[i >> 5][i & 31];
         if (warp == 0) out.hdr[lane] = B.hdr[lane];
         if (warp == NW - 1 && bid + 2 < end) pre_make_block<LOSS, NZ, HT>(P, sh, bid + 2);
-        if (have_next) pre_scan<NZ, HT, THREADS>(P, sh, N.total, nxt, C, carry);
+        if (have_next) pre_scan<NZ, HT, THREADS>(P, sh, N.total, nxt, carry);
         __syncthreads();
         PRE_T(5);
         // ---- cross Gram matrix: a warp per coordinate j of the next block; lane l collects x_j . x_l
