@@ -116,9 +116,11 @@ void destroy_impl(chicle_glm *h)
     for (int i = 0; i < lookahead_max_slices(); ++i) {
         if (h->la_ev_prep && h->la_ev_prep[i]) (void)cudaEventDestroy(h->la_ev_prep[i]);
         if (h->la_ev_done && h->la_ev_done[i]) (void)cudaEventDestroy(h->la_ev_done[i]);
+        if (h->la_ev_begun && h->la_ev_begun[i]) (void)cudaEventDestroy(h->la_ev_begun[i]);
     }
     delete[] h->la_ev_prep;
     delete[] h->la_ev_done;
+    delete[] h->la_ev_begun;
     while (!h->owned.empty()) dev_free(h, h->owned.back());
     if (h->h_status) (void)cudaFreeHost(h->h_status);
     if (h->h_gap) (void)cudaFreeHost(h->h_gap);
@@ -226,10 +228,12 @@ chicle_status_t chicle_glm_create(const chicle_matrix_t *X, const float *labels,
         const int ns = lookahead_max_slices();
         h->la_ev_prep = new (std::nothrow) cudaEvent_t[(size_t)ns]();
         h->la_ev_done = new (std::nothrow) cudaEvent_t[(size_t)ns]();
-        if (!h->la_ev_prep || !h->la_ev_done) return bail(CHICLE_ERR_OOM, "host allocation failed");
+        h->la_ev_begun = new (std::nothrow) cudaEvent_t[(size_t)ns]();
+        if (!h->la_ev_prep || !h->la_ev_done || !h->la_ev_begun) return bail(CHICLE_ERR_OOM, "host allocation failed");
         for (int i = 0; i < ns; ++i)
             if ((e = cudaEventCreateWithFlags(&h->la_ev_prep[i], cudaEventDisableTiming)) != cudaSuccess ||
-                (e = cudaEventCreateWithFlags(&h->la_ev_done[i], cudaEventDisableTiming)) != cudaSuccess)
+                (e = cudaEventCreateWithFlags(&h->la_ev_done[i], cudaEventDisableTiming)) != cudaSuccess ||
+                (e = cudaEventCreateWithFlags(&h->la_ev_begun[i], cudaEventDisableTiming)) != cudaSuccess)
                 return bail_cuda(e, "cudaEventCreate");
     }
 
@@ -421,22 +425,21 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
         h->ord.start = new_bk + 2 * nbk;
         (void)cudaMemsetAsync(new_bk, 0, nbk * sizeof(uint32_t), h->stream);
         // the look-ahead solver's per-round records (their number depends on K); without them the blocked solver runs
-        dev_free(h, h->la_rec); dev_free(h, h->la_dir); dev_free(h, h->la_cursor); dev_free(h, h->la_blk_base); dev_free(h, h->la_slice);
-        h->la_rec = nullptr; h->la_dir = nullptr; h->la_cursor = nullptr; h->la_blk_base = nullptr; h->la_slice = nullptr;
+        dev_free(h, h->la_rec); dev_free(h, h->la_dir); dev_free(h, h->la_slice);
+        h->la_rec = nullptr; h->la_dir = nullptr; h->la_slice = nullptr;
         const bool dense_fmt = h->fmt == CHICLE_FMT_DENSE_ROWMAJOR;
         if (dense_fmt ? h->dim <= lookahead_max_dense_dim() : h->dim <= lookahead_max_dim()) {
             lookahead_plan(*h, K);
             unsigned char *rec = nullptr, *dir = nullptr;
             if (alloc_into(h, rec, (size_t)h->la_regions * h->la_region_bytes) && alloc_into(h, dir, h->la_dir_bytes) &&
-                alloc_into(h, h->la_cursor, 64) &&
-                alloc_into(h, h->la_blk_base, (size_t)lookahead_max_slices() * ((size_t)K + 1)) &&
-                alloc_into(h, h->la_slice, (size_t)lookahead_max_slices() * 2 * (size_t)K)) {
+                alloc_into(h, h->la_slice, (size_t)lookahead_max_slices() * (3 * (size_t)K + 2) + 64)) {
                 h->la_rec = rec;
                 h->la_dir = dir;
-                (void)cudaMemsetAsync(h->la_cursor, 0, 64 * sizeof(unsigned long long), h->stream);
+                h->la_timing = reinterpret_cast<unsigned long long *>(h->la_slice) + (size_t)lookahead_max_slices() * (3 * (size_t)K + 2);
+                (void)cudaMemsetAsync(h->la_timing, 0, 64 * sizeof(unsigned long long), h->stream);
             } else {
-                dev_free(h, rec); dev_free(h, dir); dev_free(h, h->la_cursor); dev_free(h, h->la_blk_base); dev_free(h, h->la_slice);
-                h->la_cursor = nullptr; h->la_blk_base = nullptr; h->la_slice = nullptr;
+                dev_free(h, rec); dev_free(h, dir); dev_free(h, h->la_slice);
+                h->la_slice = nullptr;
             }
         }
     }

@@ -122,7 +122,7 @@ struct Glm {
     // not be allocated: the blocked solver runs instead). The buffer is a ring of regions, one slice of a round each.
     void *la_rec = nullptr;
     void *la_dir = nullptr;          // per region: cluster-size entries per block
-    unsigned long long *la_cursor = nullptr; // [r]: bytes of region r's pool handed out; [8..]: timing scratch
+    unsigned long long *la_timing = nullptr; // scratch of a -DCHICLE_LA_TIMING build (behind la_slice)
     size_t la_region_bytes = 0, la_pool_off = 0, la_pool_piece = 0, la_dir_bytes = 0;
     int64_t la_region_blocks = 0;    // blocks a region has records for
     int la_regions = 0;
@@ -135,10 +135,11 @@ struct Glm {
     size_t la_smem = 0;              // dynamic shared memory of the chain kernel
     int la_last_slices = 0;          // slices of the last round
     int solver_launches = 0;         // kernels the local solvers launched in the round being enqueued
-    int64_t *la_blk_base = nullptr;  // per slice K+1: first block of each partition in the slice's numbering of the blocks
-    int64_t *la_slice = nullptr;     // per slice 2K: every partition's step count and first step in that slice
+    int64_t *la_slice = nullptr;     // per slice 3K+2: every partition's step count, its first step, its first block in the
+                                     // slice's numbering of the blocks (K+1), bytes of the region's pool handed out
     cudaStream_t la_stream = nullptr; // side stream (lowest priority) for the later slices' prepare kernels
     cudaEvent_t *la_ev_prep = nullptr; // per slice: its records are written
+    cudaEvent_t *la_ev_begun = nullptr; // per slice: the CTAs of its chain launch have begun
     cudaEvent_t *la_ev_done = nullptr; // per slice: its chain launch is done (its region is free)
     bool time_prepare = false; // record ev[4] between the prepare and the chain kernel (round statistics asked for)
 

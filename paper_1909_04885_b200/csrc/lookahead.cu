@@ -2001,22 +2001,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     cluster_wait();
 }
 
-// blk_base of every slice in one launch: slice s of partition k takes slice[(2s) K + k] steps
-__global__ void k_block_bases_slices(const int64_t *__restrict__ slice, int32_t K, int64_t *__restrict__ blk_base)
-{
-    if (threadIdx.x != 0) return;
-    const int s = blockIdx.x;
-    const int64_t *steps = slice + (size_t)s * 2 * (size_t)K;
-    int64_t *out = blk_base + (size_t)s * ((size_t)K + 1);
-    int64_t run = 0;
-    for (int32_t k = 0; k < K; ++k) {
-        out[k] = run;
-        run += (steps[k] + kLB - 1) / kLB;
-    }
-    out[K] = run;
-}
-
-template <int LOSS, bool DENSE, bool FLAT, bool TAB> cudaError_t launch_chain(Glm &g, const LookParams &P)
+template <int LOSS, bool DENSE, bool FLAT, bool TAB> cudaError_t launch_chain(Glm &g, const LookParams &P, cudaEvent_t begun)
 {
     auto kern = k_lookahead_chain<LOSS, DENSE, FLAT, TAB>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.la_smem);
@@ -2026,13 +2011,19 @@ template <int LOSS, bool DENSE, bool FLAT, bool TAB> cudaError_t launch_chain(Gl
     cfg.blockDim = dim3(kChainThreads, 1, 1);
     cfg.dynamicSmemBytes = g.la_smem;
     cfg.stream = g.stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 1u << g.la_logC;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (begun) {
+        attr[1].id = cudaLaunchAttributeLaunchCompletionEvent;
+        attr[1].val.launchCompletionEvent.event = begun;
+        attr[1].val.launchCompletionEvent.flags = 0;
+        cfg.numAttrs = 2;
+    }
     e = cudaLaunchKernelEx(&cfg, kern, P);
 #ifdef CHICLE_LA_TIMING
     if (e == cudaSuccess) {
@@ -2106,31 +2097,33 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
     return e;
 }
 
-template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P)
+template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P, cudaEvent_t begun = nullptr)
 {
     constexpr bool tables = LOSS == CHICLE_LOSS_LOGISTIC_DUAL;
     const bool flat = g.la_hotc == 0;
     if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR)
-        return tables && P.tab_bins ? launch_chain<LOSS, true, false, tables>(g, P) : launch_chain<LOSS, true, false, false>(g, P);
-    if (tables && P.tab_bins) return flat ? launch_chain<LOSS, false, true, tables>(g, P) : launch_chain<LOSS, false, false, tables>(g, P);
-    return flat ? launch_chain<LOSS, false, true, false>(g, P) : launch_chain<LOSS, false, false, false>(g, P);
+        return tables && P.tab_bins ? launch_chain<LOSS, true, false, tables>(g, P, begun) : launch_chain<LOSS, true, false, false>(g, P, begun);
+    if (tables && P.tab_bins) return flat ? launch_chain<LOSS, false, true, tables>(g, P, begun) : launch_chain<LOSS, false, false, tables>(g, P, begun);
+    return flat ? launch_chain<LOSS, false, true, false>(g, P, begun) : launch_chain<LOSS, false, false, false>(g, P, begun);
 }
 
 // A round's launches, slice after slice (consecutive pieces of every partition's walk). The first slice's prepare
 // kernel runs on the handle's stream; the later ones on the side stream, where they fill the SMs the chain kernels
 // leave idle; every chain launch waits for its slice's prepare kernel. The records of slice s lie in region s mod R
 // of the record buffer, so the prepare kernel of slice s also waits for the chain launch of slice s - R.
+// A chain launch needs whole SMs (whole clusters of them), a prepare kernel spreads over whatever is free: one that gets
+// in between two chain launches holds the second up until it is through (1 M sparse rows, K = 16: 0.7 of 5.4 ms). So
+// slice s + 1's prepare kernel is let go once the CTAs of slice s's chain launch have begun. (Order of starts only:
+// what is read and overwritten is ordered by the other events.)
 template <int LOSS> cudaError_t launch_slices(Glm &g, std::vector<LookParams> &P)
 {
     const int S = (int)P.size(), R = g.la_regions;
-    cudaError_t e = cudaMemsetAsync(g.la_cursor, 0, 4 * sizeof(unsigned long long), g.stream);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     if (!g.la_overlap) {
         // the chains take most of the SMs: the prepare kernels get the whole GPU between the chain launches instead of
         // the few SMs beside them
         for (int s = 0; s < S && e == cudaSuccess; ++s) {
-            if (s > 0) e = cudaMemsetAsync(g.la_cursor + (s % R), 0, sizeof(unsigned long long), g.stream);
-            if (e == cudaSuccess) e = launch_prepare_on<LOSS>(g, P[s], g.stream);
+            e = launch_prepare_on<LOSS>(g, P[s], g.stream);
             if (s == 0 && g.time_prepare) (void)cudaEventRecord(g.ev[4], g.stream);
             if (e == cudaSuccess) e = launch_chain_on<LOSS>(g, P[s]);
         }
@@ -2141,28 +2134,18 @@ template <int LOSS> cudaError_t launch_slices(Glm &g, std::vector<LookParams> &P
     if (g.time_prepare) (void)cudaEventRecord(g.ev[4], g.stream);
     if (S > 1) {
         e = cudaEventRecord(g.la_ev_prep[0], g.stream);
-        if (e != cudaSuccess) return e;
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(g.la_stream, g.la_ev_prep[0], 0); // behind all of the caller's stream so far
     }
-    e = launch_chain_on<LOSS>(g, P[0]); // enqueued before the side stream's work: it takes its SMs first
-    if (e != cudaSuccess || S == 1) return e;
-    e = cudaEventRecord(g.la_ev_done[0], g.stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(g.la_stream, g.la_ev_prep[0], 0);
-    auto prepare_side = [&](int s) -> cudaError_t {
-        cudaError_t e2 = cudaMemsetAsync(g.la_cursor + (s % R), 0, sizeof(unsigned long long), g.la_stream);
-        if (e2 == cudaSuccess) e2 = launch_prepare_on<LOSS>(g, P[s], g.la_stream);
-        if (e2 == cudaSuccess) e2 = cudaEventRecord(g.la_ev_prep[s], g.la_stream);
-        return e2;
-    };
-    for (int s = 1; s < R && s < S && e == cudaSuccess; ++s) e = prepare_side(s);
-    for (int s = 1; s < S && e == cudaSuccess; ++s) {
-        if (s + R - 1 < S) { // its region is free once the chain launch of slice s - 1 is done
-            e = cudaStreamWaitEvent(g.la_stream, g.la_ev_done[s - 1], 0);
-            if (e == cudaSuccess) e = prepare_side(s + R - 1);
-            if (e != cudaSuccess) break;
-        }
-        e = cudaStreamWaitEvent(g.stream, g.la_ev_prep[s], 0);
-        if (e == cudaSuccess) e = launch_chain_on<LOSS>(g, P[s]);
-        if (e == cudaSuccess && s + 1 < S) e = cudaEventRecord(g.la_ev_done[s], g.stream);
+    for (int s = 0; s < S && e == cudaSuccess; ++s) {
+        if (s > 0) e = cudaStreamWaitEvent(g.stream, g.la_ev_prep[s], 0);
+        if (e == cudaSuccess) e = launch_chain_on<LOSS>(g, P[s], s + 1 < S ? g.la_ev_begun[s] : nullptr);
+        if (s + 1 == S || e != cudaSuccess) break;
+        e = cudaEventRecord(g.la_ev_done[s], g.stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(g.la_stream, g.la_ev_begun[s], 0);
+        // (its region is free once the chain launch of slice s + 1 - R is done)
+        if (e == cudaSuccess && s + 1 >= R) e = cudaStreamWaitEvent(g.la_stream, g.la_ev_done[s + 1 - R], 0);
+        if (e == cudaSuccess) e = launch_prepare_on<LOSS>(g, P[s + 1], g.la_stream);
+        if (e == cudaSuccess) e = cudaEventRecord(g.la_ev_prep[s + 1], g.la_stream);
     }
     return e;
 }
@@ -2243,7 +2226,7 @@ void lookahead_plan(Glm &g, int32_t K)
     }
     g.la_smem = chain_layout(g.la_nzcap, g.la_hotc, dense, g.la_tab_bins).total;
 
-    // slices: at most a sixteenth of the walk, but at least 256 blocks per partition; three regions
+    // slices: at most a sixteenth of the walk, but at least 256 blocks per partition; two regions
     const int64_t n = g.n_coord;
     const int64_t max_nk = (n + K - 1) / K + 1;
     const int64_t max_nb = (max_nk + kLB - 1) / kLB;
@@ -2256,10 +2239,10 @@ void lookahead_plan(Glm &g, int32_t K)
     int64_t region_blocks = whole ? n / kLB + K + 1 : per_part * K + K;
     if (region_blocks > n / kLB + K + 1) region_blocks = n / kLB + K + 1;
     g.la_region_blocks = region_blocks;
-    g.la_regions = whole ? 1 : 3;
+    g.la_regions = whole ? 1 : 2;
     {
         const char *env = getenv("CHICLE_LA_SLICES"); // forced slicing (tests): the ring as large problems have it
-        if (env && atoi(env) > 1) g.la_regions = 3;
+        if (env && atoi(env) > 1) g.la_regions = 2;
     }
     const double frac = whole ? 1.0 : (double)region_blocks / (double)(n / kLB + 1);
     const size_t C = (size_t)1 << logC;
@@ -2296,8 +2279,10 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
     }
     if (total <= 0 || total > 0x7fffffff) return cudaErrorInvalidConfiguration;
     // Slices: fractions 0 = F_0 < F_1 < ... < F_S = 1 of every partition's walk. The first slice is small (its
-    // prepare kernel is the one nothing hides), the next ones double, up to a sixteenth of the walk or 256 blocks of
-    // the longest partition, whichever is more; a slice must fit a region of the record buffer.
+    // prepare kernel is the one nothing hides), the next ones are 1.3 times as long as the one before (a slice is
+    // prepared on the SMs beside the chains while the one before is walked: when both take about as long per block,
+    // doubling makes every chain launch of the ramp wait), up to a sixteenth of the walk or 256 blocks of the longest
+    // partition, whichever is more; a slice must fit a region of the record buffer.
     // CHICLE_LA_SLICES=1 keeps every round in one piece (to time the prepare kernel alone), CHICLE_LA_SLICES=n cuts
     // into n equal slices whatever the length (to test the slicing on small problems).
     const int max_slices = lookahead_max_slices();
@@ -2310,7 +2295,7 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
         while (at < 1.0 && (int)F.size() < max_slices) {
             at += len;
             F.push_back(at < 1.0 ? at : 1.0);
-            len = len * 2.0 < cap ? len * 2.0 : cap;
+            len = len * 1.3 < cap ? len * 1.3 : cap;
         }
         F.back() = 1.0;
     };
@@ -2330,7 +2315,8 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
     std::vector<int64_t> blocks;
     for (int attempt = 0; attempt < 24; ++attempt) {
         const int Sn = (int)F.size() - 1;
-        h.assign((size_t)Sn * 2 * (size_t)K, 0);
+        h.assign((size_t)Sn * (3 * (size_t)K + 2), 0); // per slice: step counts, first steps, first blocks (K + 1), 0 for the cursor
+        const size_t per = 3 * (size_t)K + 2;
         blocks.assign((size_t)Sn, 0);
         int64_t worst = 0;
         for (int32_t k = 0; k < K; ++k) {
@@ -2341,9 +2327,11 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
                 cut = cut < prev ? prev : (cut > nbk ? nbk : cut);
                 const int64_t first = prev * kLB;
                 const int64_t last = s + 1 == Sn ? steps[(size_t)k] : cut * kLB;
-                h[((size_t)s * 2) * (size_t)K + (size_t)k] = last - first;
-                h[((size_t)s * 2 + 1) * (size_t)K + (size_t)k] = first;
+                int64_t *hs = h.data() + (size_t)s * per;
+                hs[k] = last - first;
+                hs[K + k] = first;
                 blocks[(size_t)s] += (last - first + kLB - 1) / kLB;
+                hs[2 * K + k + 1] = blocks[(size_t)s];
                 prev = cut;
             }
         }
@@ -2360,8 +2348,6 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
     // a pageable source: the runtime has taken its copy of these words when the call returns
     cudaError_t e = cudaMemcpyAsync(g.la_slice, h.data(), h.size() * sizeof(int64_t), cudaMemcpyHostToDevice, g.stream);
     if (e != cudaSuccess) return e;
-    k_block_bases_slices<<<Sn, 32, 0, g.stream>>>(g.la_slice, K, g.la_blk_base);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const char *drop = getenv("CHICLE_TEST_DROP_RECORD"); // test aid: leave one block's records unpublished
     const size_t C = (size_t)1 << g.la_logC;
     const bool tables = g.la_tab_bins > 0 && S.sigma * g.max_sqnorm <= tab_max_q(g.la_tab_bins) * S.lam_n;
@@ -2372,16 +2358,17 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
         p = LookParams{};
         p.S = S;
         p.S.H = 0;
-        p.S.steps_k = g.la_slice + ((size_t)s * 2) * (size_t)K;
-        p.S.first_k = g.la_slice + ((size_t)s * 2 + 1) * (size_t)K;
+        int64_t *hs = g.la_slice + (size_t)s * (3 * (size_t)K + 2);
+        p.S.steps_k = hs;
+        p.S.first_k = hs + K;
         p.rec = static_cast<unsigned char *>(g.la_rec) + (size_t)r * g.la_region_bytes;
         p.dirS = static_cast<BlkDir *>(g.la_dir) + (size_t)r * (size_t)g.la_region_blocks * C;
-        p.cursor = g.la_cursor + r;
-        p.timing = g.la_cursor + 8;
+        p.cursor = reinterpret_cast<unsigned long long *>(hs + 3 * K + 1);
+        p.timing = g.la_timing;
         p.pool_off = g.la_pool_off;
         p.pool_cap = g.la_region_bytes - g.la_pool_off;
         p.pool_piece = g.la_pool_piece;
-        p.blk_base = g.la_blk_base + (size_t)s * ((size_t)K + 1);
+        p.blk_base = hs + 2 * K;
         p.K = K;
         p.logC = g.la_logC;
         p.depth = g.la_depth;
@@ -2396,7 +2383,7 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
         p.model_out = s == Sn - 1 ? 1 : 0;
     }
     g.la_last_slices = Sn;
-    g.solver_launches += 1 + 2 * Sn; // block tables, then a prepare and a chain launch per slice
+    g.solver_launches += 2 * Sn; // a prepare and a chain launch per slice
     switch (g.loss) {
     case CHICLE_LOSS_HINGE_DUAL: return launch_slices<CHICLE_LOSS_HINGE_DUAL>(g, P);
     case CHICLE_LOSS_LOGISTIC_DUAL: return launch_slices<CHICLE_LOSS_LOGISTIC_DUAL>(g, P);
