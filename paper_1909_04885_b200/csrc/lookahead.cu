@@ -52,7 +52,9 @@ constexpr int kLB = 32;            // steps per block
 constexpr int kMaxC = 8;           // CTAs per cluster at most (the portable limit)
 constexpr int kDenseSlice = 384;   // columns of a dense row that one CTA of a cluster can take (a worker thread each)
 constexpr int kDenseEasy = 128;    // and what it takes where the cluster may be larger
-constexpr int kIdBits = 26;        // entry ids of a staged non-zero (problems with more ids take the blocked solver)
+// Where the model entry of an id is, in kIdBits bits: its place in its CTA's part of the model in shared memory (below hotc),
+// or the id itself (never below hotc, see k_lookahead_chain). Problems with more ids take the blocked solver.
+constexpr int kIdBits = 26;
 constexpr uint32_t kIdMask = (1u << kIdBits) - 1u;
 constexpr int kChainThreads = 512;
 constexpr int kSubSlots = 4;       // worker records in shared memory: blocks b .. b + 3
@@ -61,6 +63,7 @@ constexpr int kHeadSlots = 2;      // recurrence records (and tables of the logi
 constexpr int kWorkWarps = 12;
 constexpr int kWorkThreads = kWorkWarps * 32;
 constexpr int kBarWork = 1;        // named barrier of the worker warps
+constexpr int kRecordWarp = 8;     // fetches the workers' records
 constexpr int kFeedWarp = 4;       // in CTA 0: fetches the recurrence records and writes the new states (see the kernel)
 
 // Per-step constants for the recurrence warp (see coordinate_step for p0 .. p3).
@@ -84,24 +87,31 @@ struct alignas(16) ChainHead {
 };
 static_assert(sizeof(ChainHead) % 16 == 0, "bulk copy size");
 
-// What one CTA's workers read for one block. Behind it (sparse): val[n] f32, meta[n] u32 (entry id in the low bits,
-// the coordinate's place in the block above them, the top bit marks an id that several coordinates of the block
-// have), ids[T] u32 (those shared ids), cpos[n] u16 (for a non-zero with a shared id: its place in the id's list;
-// the lists lie one after the other, each in ascending coordinate order), off[T + 1] u16 (where each list starts).
-// Dense: val[cnt][slice of the row, padded to a multiple of four].
+// What one CTA's workers read for one block. Behind it (sparse): val[n] f32, meta[n] u32 (low bits: where the entry's
+// part of the model is, see kIdBits; the coordinate's place in the block above them; the top bit marks an id that several
+// coordinates of the block have), both row after row; then the entries of those shared ids once more, one list per id,
+// each in ascending coordinate order: ids[T] u32 (the same low bits, list length - 1 above them), lval[nl] f32,
+// lst[T] u16 (where each list starts), lrow[nl] u8 (coordinates).
+// Dense: val[cnt][slice of the row, dense_stride floats].
 struct alignas(16) SubHead {
     int32_t n;     // non-zeros of the block that fall to this CTA
     int32_t T;     // shared ids among them
+    int32_t nl;    // entries with a shared id
     int32_t cnt;
-    int32_t flags; // bit 0 as in ChainHead (the record is then this head alone)
     uint16_t roff[kLB + 8]; // where each coordinate's non-zeros start ([32] = n)
 };
 static_assert(sizeof(SubHead) == 96, "sub-record head");
 
-__host__ __device__ constexpr uint32_t sub_bytes(int n, int T, bool dense)
+__host__ __device__ constexpr uint32_t sub_bytes(uint32_t n, uint32_t T, uint32_t nl)
 {
-    return ((uint32_t)sizeof(SubHead) + (dense ? 4u * n : 8u * n + 4u * T + 2u * n + 2u * (T + 1)) + 15u) & ~15u;
+    return ((uint32_t)sizeof(SubHead) + 8u * n + 6u * T + 5u * nl + 15u) & ~15u;
 }
+// Dense rows in a record: 16-byte pieces of consecutive rows lie on different banks.
+__host__ __device__ constexpr int dense_stride(int cols) { return (((cols + 3) / 4) | 1) * 4; }
+__host__ __device__ constexpr uint32_t sub_bytes_dense(int cnt, int cols) { return ((uint32_t)sizeof(SubHead) + 4u * (uint32_t)(cnt * dense_stride(cols)) + 15u) & ~15u; }
+// A record's slot in shared memory: room for nzcap entries of which half are shared (a block that needs more is walked in
+// place).
+__host__ __device__ constexpr uint32_t sub_room(int nzcap) { return sub_bytes((uint32_t)nzcap, (uint32_t)nzcap / 4u, (uint32_t)nzcap / 2u); }
 
 struct alignas(16) BlkDir { // where a record is
     unsigned long long offset; // bytes from the start of the launch's region of the record buffer (a multiple of 16)
@@ -656,6 +666,8 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
     constexpr int NW = THREADS / 32, EPT = NZ / THREADS;
     static_assert(NZ % THREADS == 0 && NW >= 8, "entries per thread; a warp per CTA of the cluster");
     const int C = 1 << P.logC;
+    const int64_t hot_all = (int64_t)P.hotc << P.logC;
+    const uint32_t hot_total = (uint32_t)(hot_all < P.S.dim ? hot_all : P.S.dim);
     const int64_t lo = P.n_blocks * (int64_t)blockIdx.x / gridDim.x, hi = P.n_blocks * ((int64_t)blockIdx.x + 1) / gridDim.x;
     if (lo >= hi) return;
     if (P.K < kBaseStaged)
@@ -794,7 +806,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         if (warp == 0) { // (a lane per CTA of the cluster)
             const bool in = lane < C;
             const uint32_t n_c = in ? sh.rc[kLB][lane] : 0u;
-            const uint32_t len = in ? sub_bytes((int)n_c, (int)(sh.cntTL[lane] >> 16), false) : 0u;
+            const uint32_t len = in ? sub_bytes(n_c, sh.cntTL[lane] >> 16, sh.cntTL[lane] & 0xffffu) : 0u;
             uint32_t incl = len;
 #pragma unroll
             for (int o = 1; o < kMaxC; o <<= 1) {
@@ -802,8 +814,8 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 if (lane >= o) incl += y;
             }
             const uint32_t need = __shfl_sync(0xffffffffu, incl, kMaxC - 1);
-            // 1: longer than the arrays, or more of the entries fall to one CTA than its record holds
-            int sl = B.over || __any_sync(0xffffffffu, n_c > (uint32_t)P.nzcap) ? 1 : 0;
+            // 1: longer than the arrays, or more falls to one CTA than its record holds
+            int sl = B.over || __any_sync(0xffffffffu, len > sub_room(P.nzcap)) ? 1 : 0;
             unsigned long long at = sh.pool_at, pool_end = sh.pool_end;
             if (!sl && at + need > pool_end) {
                 const unsigned long long take = need > P.pool_piece ? need : P.pool_piece;
@@ -843,10 +855,8 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 const int n_c = sh.rc[kLB][tid], T_c = (int)(sh.cntTL[tid] >> 16);
                 h.n = n_c;
                 h.T = T_c;
+                h.nl = (int)(sh.cntTL[tid] & 0xffffu);
                 h.cnt = cnt;
-                h.flags = 0;
-                // the end of the last list
-                reinterpret_cast<uint16_t *>(P.rec + sh.sub_off[tid] + sizeof(SubHead) + 10u * n_c + 4u * T_c)[T_c] = (uint16_t)(sh.cntTL[tid] & 0xffffu);
             }
             for (int i = tid; i < C * (kLB + 8); i += THREADS) {
                 const int c = i / (kLB + 8), j = i - c * (kLB + 8);
@@ -864,15 +874,20 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 const int lower = __popc(m & ((1u << j) - 1u));
                 const float x = sh.val[cur][e];
                 unsigned char *rec = P.rec + sh.sub_off[cls] + sizeof(SubHead);
-                const uint32_t n_c = sh.rc[kLB][cls], T_c = sh.cntTL[cls] >> 16;
+                const uint32_t n_c = sh.rc[kLB][cls], T_c = sh.cntTL[cls] >> 16, nl_c = sh.cntTL[cls] & 0xffffu;
+                const uint32_t where = (uint32_t)id < hot_total ? (uint32_t)id >> P.logC : (uint32_t)id;
                 reinterpret_cast<float *>(rec)[place] = x;
-                reinterpret_cast<uint32_t *>(rec + 4u * n_c)[place] = (uint32_t)id | ((uint32_t)j << kIdBits) | (shared_id ? 0x80000000u : 0u);
-                uint16_t *cpos_g = reinterpret_cast<uint16_t *>(rec + 8u * n_c + 4u * T_c);
-                cpos_g[place] = shared_id ? (uint16_t)(sh.coff[p] + lower) : (uint16_t)0;
-                if (shared_id) sh.lval[sh.soff[p] - NZ + lower] = x;
-                if (tl[i] != 0xffffffffu) {
-                    reinterpret_cast<uint32_t *>(rec + 8u * n_c)[tl[i] >> 16] = (uint32_t)id;
-                    (cpos_g + n_c)[tl[i] >> 16] = (uint16_t)(tl[i] & 0xffffu);
+                reinterpret_cast<uint32_t *>(rec + 4u * n_c)[place] = where | ((uint32_t)j << kIdBits) | (shared_id ? 0x80000000u : 0u);
+                if (shared_id) {
+                    sh.lval[sh.soff[p] - NZ + lower] = x;
+                    const uint32_t at = sh.coff[p] + lower;
+                    unsigned char *lists = rec + 8u * n_c + 4u * T_c;
+                    reinterpret_cast<float *>(lists)[at] = x;
+                    (lists + 4u * nl_c + 2u * T_c)[at] = (unsigned char)j;
+                    if (tl[i] != 0xffffffffu) {
+                        reinterpret_cast<uint32_t *>(rec + 8u * n_c)[tl[i] >> 16] = where | ((uint32_t)(__popc(m) - 1) << kIdBits);
+                        reinterpret_cast<uint16_t *>(lists + 4u * nl_c)[tl[i] >> 16] = (uint16_t)(tl[i] & 0xffffu);
+                    }
                 }
             }
         }
@@ -954,10 +969,8 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
             }
         __syncthreads();
         PRE_T(6);
-        // (a next block that is walked in place because more of its entries fall to one CTA than a record holds takes
-        // nothing over either)
-        bool keep = carry;
-        for (int c = 0; c < C && keep; ++c) keep = sh.pre[nxt][(N.total + 31) >> 5][c] <= P.nzcap;
+        // (a next block that is walked in place takes nothing over: the recurrence warp drops it)
+        const bool keep = carry;
         for (int i = tid; i < kLB * kLB; i += THREADS) out.X[i] = keep ? sh.G[i >> 5][i & 31] : 0.0f;
         if (tid < kLB) out.q0n[tid] = keep ? sh.q0n[tid] : 0.0f;
         for (int p = tid; p < HT / 4; p += THREADS) {
@@ -1019,7 +1032,7 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
         sh.coord[tid] = c;
     } else if (tid == 2 * kLB) {
         unsigned long long need = 0;
-        for (int c = 0; c < C; ++c) need += sub_bytes(cnt * ((cols_of(c) + 3) & ~3), 0, true);
+        for (int c = 0; c < C; ++c) need += sub_bytes_dense(cnt, cols_of(c));
         unsigned long long at = atomicAdd(P.cursor, need);
         sh.walk = at + need > P.pool_cap ? 1 : 0; // no room: walked in place
         for (int c = 0; c < C; ++c) {
@@ -1030,7 +1043,7 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
                 d.flags = 1u;
             } else {
                 d.offset = P.pool_off + at;
-                d.bytes = sub_bytes(cnt * ((cols_of(c) + 3) & ~3), 0, true);
+                d.bytes = sub_bytes_dense(cnt, cols_of(c));
                 d.flags = 0u;
                 at += d.bytes;
             }
@@ -1046,7 +1059,7 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
     const bool walk = sh.walk != 0;
     if (!walk && tid < C) {
         SubHead &h = *reinterpret_cast<SubHead *>(P.rec + sh.sub_off[tid]);
-        h.n = cnt * cols_of(tid); h.T = 0; h.cnt = cnt; h.flags = 0;
+        h.n = cnt * cols_of(tid); h.T = 0; h.nl = 0; h.cnt = cnt;
     }
     // ---- headers: warp 0 this block's coordinates, warp 1 the next block's
     if (warp < 2) {
@@ -1091,7 +1104,7 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
                 }
                 const int e = e0 + 4 * sub, c = e / slice;
                 float *val_g = reinterpret_cast<float *>(P.rec + (walk || c >= C ? 0 : sh.sub_off[c]) + sizeof(SubHead));
-                const int st = (cols_of(c) + 3) & ~3;
+                const int st = dense_stride(cols_of(c));
 #pragma unroll
                 for (int u = 0; u < RPW; ++u) {
                     const int j = warp * RPW + u * per + lane / lpr;
@@ -1110,12 +1123,12 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
                         v[u] = f < cols && sh.coord[j] >= 0 ? P.S.values[(int64_t)sh.coord[j] * dim + e] : 0.0f;
                     }
                     float *val_g = reinterpret_cast<float *>(P.rec + (walk || c >= C ? 0 : sh.sub_off[c]) + sizeof(SubHead));
-                    const int st = c < C ? (cols_of(c) + 3) & ~3 : 0;
+                    const int st = c < C ? dense_stride(cols_of(c)) : 0, padded = c < C ? (cols_of(c) + 3) & ~3 : 0;
 #pragma unroll
                     for (int u = 0; u < RPW; ++u) {
                         const int j = warp * RPW + u;
                         sh.row[j * stride + f] = v[u];
-                        if (j < cnt && !walk && c < C && e - c * slice < st) val_g[j * st + (e - c * slice)] = v[u]; // (with the zero padding)
+                        if (j < cnt && !walk && c < C && e - c * slice < padded) val_g[j * st + (e - c * slice)] = v[u]; // (with the zero padding)
                     }
                 }
             }
@@ -1299,19 +1312,21 @@ struct alignas(16) ChainCtl {
     uint64_t headfull[kHeadSlots]; // the same for the recurrence warp's records (CTA 0)
     uint64_t pbar[2];              // CTA 0: the partial dot products of a block have arrived from all CTAs
     uint64_t dbar[2];              // a block's deltas have arrived from CTA 0
+    uint64_t subfree[kSubSlots];   // the worker warps are through with the slot's record
     uint64_t ackbar;               // CTA 0: every CTA has applied all updates (before a block is walked in place)
     alignas(16) float pbuf[2][kMaxC][kLB];
     alignas(16) float dbuf[2][kLB];
     alignas(16) float sbuf[2][kLB]; // CTA 0: the block's new states (arrive with its deltas)
     float sink[32]; // where a lane's stores go that have no target
+    int walk[kSubSlots]; // whether the slot's block is walked in place
     int abort_flag;
     int done; // the CTA's workers are through (the warps with no role sleep until then)
 };
 
 // Shared-memory layout of the chain kernel (sizes fixed at launch): control, recurrence records, logistic tables,
-// worker records, products, the CTA's part of the model.
+// worker records, the CTA's part of the model.
 struct ChainLayout {
-    uint32_t heads, tabs, subs, sub_stride, prod, w, total;
+    uint32_t heads, tabs, subs, sub_stride, w, total;
 };
 __host__ __device__ inline ChainLayout chain_layout(int nzcap, int hotc, bool dense, int tab_bins)
 {
@@ -1319,9 +1334,8 @@ __host__ __device__ inline ChainLayout chain_layout(int nzcap, int hotc, bool de
     L.heads = (uint32_t)((sizeof(ChainCtl) + 127) & ~(size_t)127);
     L.tabs = L.heads + kHeadSlots * (uint32_t)sizeof(ChainHead);
     L.subs = L.tabs + kHeadSlots * tab_bytes(tab_bins);
-    L.sub_stride = dense ? sub_bytes(kLB * hotc, 0, true) : sub_bytes(nzcap, nzcap / 2, false);
-    L.prod = L.subs + kSubSlots * L.sub_stride;
-    L.w = L.prod + 4u * (uint32_t)(dense ? kLB : nzcap);
+    L.sub_stride = dense ? sub_bytes_dense(kLB, hotc) : sub_room(nzcap);
+    L.w = L.subs + kSubSlots * L.sub_stride;
     L.total = L.w + 4u * (uint32_t)(hotc > 0 ? hotc : 4);
     return L;
 }
@@ -1338,7 +1352,6 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     const ChainLayout L = chain_layout(P.nzcap, P.hotc, DENSE, TAB ? P.tab_bins : 0);
     ChainCtl &ctl = *reinterpret_cast<ChainCtl *>(smem_chain);
     float *W = reinterpret_cast<float *>(smem_chain + L.w);
-    float *prod = reinterpret_cast<float *>(smem_chain + L.prod);
     volatile int *abort_flag = &ctl.abort_flag;
 
     const int64_t nk = S.part_off[k + 1] - S.part_off[k];
@@ -1359,7 +1372,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     if (tid == 0) {
         ctl.abort_flag = 0;
         ctl.done = 0;
-        for (int i = 0; i < kSubSlots; ++i) mbar_init(smem_u32(&ctl.subfull[i]), 1);
+        for (int i = 0; i < kSubSlots; ++i) {
+            mbar_init(smem_u32(&ctl.subfull[i]), 1);
+            mbar_init(smem_u32(&ctl.subfree[i]), kWorkWarps);
+        }
         for (int i = 0; i < kHeadSlots; ++i) mbar_init(smem_u32(&ctl.headfull[i]), 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&ctl.pbar[i]), 1);
@@ -1621,16 +1637,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             issue_head(b + kHeadSlots, slot);
         }
     }
-    if (is_worker && nb > 0) {
-        // ============================== the worker warps ========================================================
-        const int wt = (warp - 1 - (warp >> 2)) * 32 + lane; // 0 .. kWorkThreads - 1
-        const uint32_t p_bar0 = mapa_u32(smem_u32(&ctl.pbar[0]), 0u);
-        const uint32_t p_buf0 = mapa_u32(smem_u32(&ctl.pbuf[0][crank][0]), 0u);
-        const uint32_t ack_bar = mapa_u32(smem_u32(&ctl.ackbar), 0u);
-        const int dstride = (hot_mine + 3) & ~3; // dense: floats per row of a record
-        auto sub_at = [&](int blk) { return smem_chain + L.subs + (size_t)(blk & (kSubSlots - 1)) * L.sub_stride; };
-        // The directory entry of a block is loaded a block ahead of its use (an unconditional load from a clamped
-        // address, so that nothing has to wait for it at the point of issue).
+    if (warp == kRecordWarp && nb > 0) {
+        // ============================== the workers' records, four blocks ahead =======================================
+        // (directory entries are loaded a block ahead of their use; walk[slot] is written before the arrival that, with the
+        // record's bytes, completes the slot's barrier)
         auto load_dir = [&](int blk, uint32_t (&d)[4]) {
             const int at = blk < nb ? blk : nb - 1;
             asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
@@ -1638,333 +1648,232 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                          : "l"(P.dirS + (((bid0 + at) << logC) + crank))
                          : "memory");
         };
-        auto issue_sub = [&](int blk, const uint32_t (&d)[4]) {
-            const uint32_t bar = smem_u32(&ctl.subfull[blk & (kSubSlots - 1)]);
-            // (the slot is only ever written by the copy engine and read by loads that are done by now)
+        uint32_t d[4];
+        load_dir(0, d);
+#pragma unroll 1
+        for (int blk = 0; blk < nb; ++blk) {
+            const int slot = blk & (kSubSlots - 1);
+            if (blk >= kSubSlots && !mbar_wait_cluster(smem_u32(&ctl.subfree[slot]), (uint32_t)(blk / kSubSlots - 1) & 1u, abort_flag, S.status)) break;
             const unsigned long long offset = ((unsigned long long)d[1] << 32) | d[0];
             uint32_t bytes = d[2] <= L.sub_stride ? d[2] : 0u;
             if (!CHICLE_IN_BOUNDS(S.status, (offset & 15ull) == 0ull && offset + bytes <= P.pool_off + P.pool_cap))
                 bytes = 0u; // (an entry that points outside the region: as if no record had been written)
-            const bool mine = blk < nb && wt == 0;
-            if (mine && bytes == 0) {
-                // no record: nothing will arrive, say so now
-                atomicOr(S.status, ST_WAIT_TIMEOUT);
-                *abort_flag = 1;
+            if (bytes == 0u) { // no record: nothing will arrive, say so now
+                if (lane == 0) {
+                    atomicOr(S.status, ST_WAIT_TIMEOUT);
+                    *abort_flag = 1;
+                }
+                break;
             }
-            mbar_arrive_expect_tx_if(bar, bytes, mine && bytes != 0);
-            bulk_g2s_if(smem_u32(sub_at(blk)), P.rec + offset, bytes, bar, mine && bytes != 0);
-        };
-        // which of the blocks b .. b + 3 are walked in place
-        bool sl0, sl1, sl2, sl3;
-        {
-            uint32_t d[4];
-            load_dir(0, d); issue_sub(0, d); sl0 = (d[3] & 1u) != 0u;
-            load_dir(1, d); issue_sub(1, d); sl1 = nb > 1 && (d[3] & 1u) != 0u;
-            load_dir(2, d); issue_sub(2, d); sl2 = nb > 2 && (d[3] & 1u) != 0u;
-            load_dir(3, d); issue_sub(3, d); sl3 = nb > 3 && (d[3] & 1u) != 0u;
+            if (lane == 0) ctl.walk[slot] = (int)(d[3] & 1u);
+            __syncwarp();
+            const uint32_t bar = smem_u32(&ctl.subfull[slot]);
+            mbar_arrive_expect_tx_if(bar, bytes, lane == 0);
+            bulk_g2s_if(smem_u32(smem_chain + L.subs) + (uint32_t)slot * L.sub_stride, P.rec + offset, bytes, bar, lane == 0);
+            load_dir(blk + 1, d);
         }
+    }
+    if (is_worker && nb > 0) {
+        // ============================== the worker warps ========================================================
+        // Two barriers per block: behind its update (the model is as block b left it) and behind the dot products taken
+        // against that model. Every warp waits for deltas and records by itself; a warp whose wait runs out does nothing
+        // and says so at the next barrier's vote, so that all warps still meet there.
+        const int wt = (warp - 1 - (warp >> 2)) * 32 + lane; // 0 .. kWorkThreads - 1
+        const uint32_t p_bar0 = mapa_u32(smem_u32(&ctl.pbar[0]), 0u);
+        const uint32_t p_buf0 = mapa_u32(smem_u32(&ctl.pbuf[0][crank][0]), 0u);
+        const uint32_t ack_bar = mapa_u32(smem_u32(&ctl.ackbar), 0u);
+        const uint32_t a_w = smem_u32(W), a_sink = smem_u32(&ctl.sink[lane]);
+        const uint32_t hotc = (uint32_t)P.hotc;
+        const bool cold_ids = FLAT || (int64_t)hot_total < S.dim;  // some ids are not in shared memory
+        const int dstride = dense_stride(hot_mine);                // dense: floats per row of a record
+        const int depth = P.depth;
+        auto record = [&](int blk) { return smem_chain + L.subs + (size_t)(blk & (kSubSlots - 1)) * L.sub_stride; };
         int fg = 0; // staged blocks whose dot products have been sent
-        bool failed = false; // this warp gave up a wait (voted on at the next barrier)
+        bool ok = true;
 #ifdef CHICLE_LA_TIMING
         long long wd = 0, ws = 0, wg = 0, ws1 = 0, wg0 = 0, wg1 = 0, t0 = clock64(), t1 = 0;
 #endif
-
-        // Block x's dot products against the model as it is now (this CTA's part), sent to CTA 0.
-        auto take_dots = [&](int x) -> bool {
-            // Every warp waits for the record by itself (a barrier costs more than 200 cycles); a warp whose wait runs out
-            // skips the work and says so at the next barrier's vote, so that all warps still meet there.
-            bool ok = mbar_wait_cluster(smem_u32(&ctl.subfull[x & (kSubSlots - 1)]), (uint32_t)(x >> 2) & 1u, abort_flag, S.status);
-            if (DENSE) ok = work_bar_and(ok); // (dense rows: the products of the call before have been read)
-            if (!ok) {
-                failed = true;
-                ++fg;
-                return !DENSE;
+        // The loop starts `depth` blocks early: those turns only take the first blocks' dot products (one place in the
+        // code for every phase keeps the loop small: the warps run at the pace instructions can be fetched).
+        bool sl0 = false, sl1 = false; // whether blocks b and b + 1 are walked in place
+#pragma unroll 1
+        for (int b = -depth; b < nb; ++b) {
+            const uint32_t par = (uint32_t)(b & 1);
+            if (b >= 0) {
+                // (walked in place by CTA 0: every update before it has been applied here, the barriers behind the block
+                // before say so; wait for the walk to end)
+                if (sl0 && wt == 0) mbar_arrive_remote_release(ack_bar);
+                ok = ok && mbar_wait_cluster(smem_u32(&ctl.dbar[par]), (uint32_t)(b >> 1) & 1u, abort_flag, S.status);
+                if (sl0) fence_cluster(); // the walk's ordinary stores into this CTA's part of the model
+                mbar_arrive_expect_tx_if(smem_u32(&ctl.dbar[par]), d_bytes, wt == 0 && ok); // for block b + 2
+                LA_T(wd);
+                if (ok && !sl0) {
+                    // ---- block b's update of this CTA's part of the model
+                    const float *dl = ctl.dbuf[par];
+                    const unsigned char *rec = record(b);
+                    const SubHead &h = *reinterpret_cast<const SubHead *>(rec);
+                    const float *val = reinterpret_cast<const float *>(rec + sizeof(SubHead));
+                    if (DENSE) {
+                        if (wt < hot_mine) {
+                            float s0 = 0.0f, s1 = 0.0f;
+                            const int cnt = h.cnt;
+                            if (cnt == kLB) { // all loads first
+                                float x[kLB];
+#pragma unroll
+                                for (int j = 0; j < kLB; ++j) x[j] = val[j * dstride + wt];
+#pragma unroll
+                                for (int j = 0; j < kLB; j += 4) {
+                                    const float4 d = *reinterpret_cast<const float4 *>(dl + j);
+                                    s0 = fmaf(d.x, x[j], s0);
+                                    s1 = fmaf(d.y, x[j + 1], s1);
+                                    s0 = fmaf(d.z, x[j + 2], s0);
+                                    s1 = fmaf(d.w, x[j + 3], s1);
+                                }
+                            } else
+                                for (int j = 0; j < cnt; ++j) s0 = fmaf(dl[j], val[j * dstride + wt], s0);
+                            W[wt] = fmaf(sigma, s0 + s1, W[wt]);
+                        }
+                    } else {
+                        // A thread per entry: one whose id no other coordinate of the block has is applied (no two threads
+                        // touch the same word). One store per entry, its address chosen without a branch: the model word, or
+                        // a word that nobody reads; ids beyond the part in shared memory are added to at L2, nothing waits.
+                        constexpr int U = FLAT ? 4 : 2;
+                        const int n = h.n;
+                        const uint32_t *meta = reinterpret_cast<const uint32_t *>(val + n);
+                        for (int e0 = wt; e0 < n; e0 += U * kWorkThreads) {
+                            uint32_t m[U];
+                            float p[U], w[U];
+#pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                const int e = e0 + u * kWorkThreads;
+                                m[u] = e < n ? meta[e] : 0x80000000u;
+                                p[u] = e < n ? val[e] : 0.0f;
+                            }
+#pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                const uint32_t v = m[u] & kIdMask;
+                                p[u] = sigma * (p[u] * dl[(m[u] >> kIdBits) & 31u]);
+                                if (!FLAT) w[u] = lds_f32(a_w + 4u * (v < hotc ? v : 0u));
+                            }
+#pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                const uint32_t v = m[u] & kIdMask;
+                                const bool mine = (m[u] >> 31) == 0u;
+                                if (!FLAT) sts_f32(mine && v < hotc ? a_w + 4u * v : a_sink, p[u] + w[u]);
+                                if (cold_ids) {
+                                    const bool far = mine && v >= hotc && p[u] != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
+                                    red_add_if(Uk + (far ? v : 0u), p[u], far);
+                                }
+                            }
+                        }
+                        // Eight threads per shared id: each adds every eighth entry of the list, then the partial sums are added
+                        // in a fixed order.
+                        const int T = h.T, nl = h.nl, q = wt & 7;
+                        const uint32_t *ids = meta + n;
+                        const float *lval = reinterpret_cast<const float *>(ids + T);
+                        const uint16_t *lst = reinterpret_cast<const uint16_t *>(lval + nl);
+                        const unsigned char *lrow = reinterpret_cast<const unsigned char *>(lst + T);
+                        for (int t4 = wt >> 3; t4 < ((T + 3) & ~3); t4 += kWorkThreads / 8) { // (whole warps)
+                            const bool on = t4 < T;
+                            const uint32_t id = on ? ids[t4] : 0u, v = id & kIdMask;
+                            const int first = on ? lst[t4] : 0, len = on ? (int)((id >> kIdBits) & 31u) + 1 : 0;
+                            float sum = 0.0f;
+                            for (int o = q; o < len; o += 8)
+                                if (CHICLE_IN_BOUNDS(S.status, first + o < nl)) sum = fmaf(lval[first + o], dl[lrow[first + o] & 31], sum);
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 4);
+                            if (on && q == 0 && sum != 0.0f) {
+                                if (v < hotc) sts_f32(a_w + 4u * v, fmaf(sigma, sum, lds_f32(a_w + 4u * v)));
+                                else if (CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim)) atomicAdd(Uk + v, sigma * sum);
+                            }
+                        }
+                    }
+                }
+                LA_T(ws1);
+                ok = work_bar_and(ok);
+                LA_T(ws);
+                if (lane == 0) mbar_arrive(smem_u32(&ctl.subfree[b & (kSubSlots - 1)])); // block b's slot is free
+                if (!ok) { aborted = true; break; }
+            }
+            // ---- dot products: of block b + depth against the model as it is now. A block right behind a walked one starts
+            //      from the model as the walk left it: with depth 2 its products wait for that.
+            bool sl2 = false;
+            if (b + depth < nb) {
+                ok = mbar_wait_cluster(smem_u32(&ctl.subfull[(b + depth) & (kSubSlots - 1)]), (uint32_t)((b + depth) / kSubSlots) & 1u, abort_flag, S.status);
+                sl2 = ctl.walk[(b + depth) & (kSubSlots - 1)] != 0;
             }
             LA_T(wg0);
-            const unsigned char *rec = sub_at(x);
-            const SubHead &h = *reinterpret_cast<const SubHead *>(rec);
-            // (debug build) a record whose sizes do not fit its slot is not read: as if its wait had run out
-            if (!CHICLE_IN_BOUNDS(S.status, h.cnt >= 0 && h.cnt <= kLB &&
-                                                (DENSE || (h.n >= 0 && h.n <= P.nzcap && h.T >= 0 && h.T <= P.nzcap / 2 && h.roff[kLB] == h.n)))) {
-                failed = true;
+            const bool late = depth == 2 && sl0 && !sl1 && b + 1 < nb, due = b + depth < nb && !sl2 && (depth == 1 || !sl1);
+#pragma unroll 1
+            for (int x = late ? b + 1 : b + depth; ok && (late || due) && x <= (due ? b + depth : b + 1); x += depth - 1 > 0 ? depth - 1 : 1) {
+                const unsigned char *rec = record(x);
+                const SubHead &h = *reinterpret_cast<const SubHead *>(rec);
+                // (debug build) a record whose sizes do not fit its slot is not read: as if its wait had run out
+                if (!CHICLE_IN_BOUNDS(S.status, h.cnt >= 0 && h.cnt <= kLB && (DENSE || (h.n >= 0 && h.T >= 0 && h.nl >= 0 && h.roff[kLB] == h.n &&
+                                                    sub_bytes((uint32_t)h.n, (uint32_t)h.T, (uint32_t)h.nl) <= L.sub_stride)))) {
+                    ok = false;
+                    break;
+                }
+                const float *val = reinterpret_cast<const float *>(rec + sizeof(SubHead));
+                const uint32_t slot = (uint32_t)(fg & 1);
                 ++fg;
-                return !DENSE;
-            }
-            const float *val = reinterpret_cast<const float *>(rec + sizeof(SubHead));
-            const uint32_t slot = (uint32_t)(fg & 1);
-            if (DENSE) {
-                if (wt < kLB * 8) {
-                    const int j = wt >> 3, qq = wt & 7;
-                    float acc = 0.0f;
+                if (wt >= kLB * 8) continue;
+                // eight threads per coordinate
+                const int j = wt >> 3, q = wt & 7;
+                float acc = 0.0f;
+                if (DENSE) {
                     if (j < h.cnt) {
                         const float4 *v4 = reinterpret_cast<const float4 *>(val + j * dstride), *w4 = reinterpret_cast<const float4 *>(W);
 #pragma unroll 4
-                        for (int e = qq; e < dstride >> 2; e += 8) {
+                        for (int e = q; e < (hot_mine + 3) >> 2; e += 8) {
                             const float4 a = v4[e], w = w4[e];
                             acc = fmaf(a.x, w.x, acc); acc = fmaf(a.y, w.y, acc); acc = fmaf(a.z, w.z, acc); acc = fmaf(a.w, w.w, acc);
                         }
                     }
-                    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-                    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-                    acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-                    if (qq == 0) prod[j] = acc;
-                }
-                work_bar();
-                if (wt < kLB) {
-                    st_async_f32(p_buf0 + (slot * (uint32_t)(kMaxC * kLB) + (uint32_t)wt) * 4u, prod[wt], p_bar0 + slot * 8u);
-                }
-            } else {
-                const int n = h.n;
-                const uint32_t *meta = reinterpret_cast<const uint32_t *>(val + n);
-                // Eight threads per coordinate, each its every eighth non-zero: the first two with all loads issued
-                // before anything is used. Ids below hot_total from shared memory; the others from row k of the
-                // update workspace (read at L2: the updates are made there by reductions) and from v.
-                if (FLAT && wt < kLB * 8) {
-                    // (no id in shared memory: every gather goes to L2, eight per thread in flight)
-                    const int j = wt >> 3, qq = wt & 7;
-                    const int lo = h.roff[j] + qq, hi = h.roff[j + 1];
-                    float acc = 0.0f;
-                    for (int e0 = lo; e0 < hi; e0 += 64) {
-                        float x8[8], u8[8];
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const int e = e0 + 8 * u;
-                            const bool on = e < hi;
-                            x8[u] = on ? val[e] : 0.0f;
-                            const uint32_t g = on ? (meta[e] & kIdMask) : 0u;
-                            u8[u] = ldcg_if(Uk + g, on && CHICLE_IN_BOUNDS(S.status, (int64_t)g < S.dim));
-                        }
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) acc = fmaf(x8[u], u8[u], acc);
-                    }
-                    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-                    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-                    acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-                    if (qq == 0) st_async_f32(p_buf0 + (slot * (uint32_t)(kMaxC * kLB) + (uint32_t)j) * 4u, acc, p_bar0 + slot * 8u);
-                } else if (!FLAT && wt < kLB * 8) {
-                    const int j = wt >> 3, qq = wt & 7;
-                    const int lo = h.roff[j] + qq, hi = h.roff[j + 1];
-                    float x[2], hv[2], uu[2];
-                    bool cold[2];
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const int e = lo + 8 * u;
-                        const bool on = e < hi;
-                        x[u] = on ? val[e] : 0.0f;
-                        const uint32_t g = on ? (meta[e] & kIdMask) : 0u;
-                        cold[u] = on && g >= hot_total && CHICLE_IN_BOUNDS(S.status, (int64_t)g < S.dim);
-                        hv[u] = W[g < hot_total ? (g >> logC) : 0u];
-                        uu[u] = ldcg_if(Uk + (cold[u] ? g : 0u), cold[u]);
-                    }
-                    float acc = x[0] * (cold[0] ? uu[0] : hv[0]);
-                    acc = fmaf(x[1], cold[1] ? uu[1] : hv[1], acc);
-                    // (longer coordinates: four at a time, again with all loads first: an id beyond the part of the
-                    // model in shared memory costs a round trip to L2, which the four share)
-                    for (int e0 = lo + 16; e0 < hi; e0 += 32) {
-                        float x4[4], h4[4], u4[4];
-                        bool c4[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int e = e0 + 8 * u;
-                            const bool on = e < hi;
-                            x4[u] = on ? val[e] : 0.0f;
-                            const uint32_t g = on ? (meta[e] & kIdMask) : 0u;
-                            c4[u] = on && g >= hot_total && CHICLE_IN_BOUNDS(S.status, (int64_t)g < S.dim);
-                            h4[u] = W[g < hot_total ? (g >> logC) : 0u];
-                            u4[u] = ldcg_if(Uk + (c4[u] ? g : 0u), c4[u]);
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) acc = fmaf(x4[u], c4[u] ? u4[u] : h4[u], acc);
-                    }
-                    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-                    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-                    acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-                    if (qq == 0) st_async_f32(p_buf0 + (slot * (uint32_t)(kMaxC * kLB) + (uint32_t)j) * 4u, acc, p_bar0 + slot * 8u);
-                }
-                LA_T(wg1);
-            }
-            ++fg;
-            return true;
-        };
-
-        // The loop starts `depth` blocks early: those turns only take the first blocks' dot products (one place in the
-        // code for every phase keeps the loop small: the warps run at the pace instructions can be fetched).
-        const int depth = P.depth;
-        if (depth == 2) { sl2 = sl0; sl3 = sl1; sl0 = false; sl1 = false; } // flags of blocks b .. b + 3 for b = -2
-        else { sl3 = sl2; sl2 = sl1; sl1 = sl0; sl0 = false; }              // ... for b = -1
-#pragma unroll 1
-        for (int b = -depth; b < nb && !aborted; ++b) {
-            uint32_t dn[4];
-            load_dir(b + kSubSlots, dn);
-            const uint32_t par = (uint32_t)(b & 1);
-            if (b < 0) {
-            } else if (sl0) {
-                // walked in place by CTA 0: every update before it has been applied here (the barrier that ended
-                // the block before); say so, and wait for the walk to end
-                if (wt == 0) mbar_arrive_remote_release(ack_bar);
-                bool ok = !failed && (wt >= 32 || mbar_wait_cluster(smem_u32(&ctl.dbar[par]), (uint32_t)(b >> 1) & 1u, abort_flag, S.status));
-                if (wt < 32) fence_cluster(); // the walk's ordinary stores into this CTA's part of the model
-                ok = work_bar_and(ok);
-                if (!ok) { aborted = true; break; }
-            } else {
-                bool ok = !failed && (wt >= 32 || mbar_wait_cluster(smem_u32(&ctl.dbar[par]), (uint32_t)(b >> 1) & 1u, abort_flag, S.status));
-                ok = work_bar_and(ok);
-                if (!ok) { aborted = true; break; }
-                LA_T(wd);
-                // ---- block b's update of this CTA's part of the model
-                const float *dl = ctl.dbuf[par];
-                const unsigned char *rec = sub_at(b);
-                const SubHead &h = *reinterpret_cast<const SubHead *>(rec);
-                const float *val = reinterpret_cast<const float *>(rec + sizeof(SubHead));
-                if (DENSE) {
-                    if (wt < hot_mine) {
-                        float sum = 0.0f;
-                        const int cnt = h.cnt;
-#pragma unroll 8
-                        for (int j = 0; j < cnt; ++j) sum = fmaf(dl[j], val[j * dstride + wt], sum);
-                        W[wt] = fmaf(sigma, sum, W[wt]);
-                    }
                 } else {
-                    const int n = h.n, T = h.T;
-                    const uint32_t *meta = reinterpret_cast<const uint32_t *>(val + n);
-                    const uint32_t *ids = meta + n;
-                    const uint16_t *cpos = reinterpret_cast<const uint16_t *>(ids + T);
-                    const uint16_t *offs = cpos + n;
-                    // (A) eight threads per coordinate. A non-zero whose id no other coordinate of the block has is
-                    //     applied at once (no two of a block's non-zeros touch the same word then); the others leave
-                    //     their product delta_j * x at their place in the id's list. One store per non-zero, its
-                    //     address chosen without a branch: the list place, the model word, or a word that nobody reads;
-                    //     ids beyond the part in shared memory add to the workspace row instead.
-                    if (FLAT && wt < kLB * 8) {
-                        // (no id in shared memory: a list place or a reduction at L2, eight non-zeros per turn)
-                        const int j = wt >> 3, qq = wt & 7;
-                        const int lo = h.roff[j] + qq, hi = h.roff[j + 1];
-                        const float d = dl[j];
-                        const uint32_t a_prod = smem_u32(prod), a_sink = smem_u32(&ctl.sink[lane]);
-                        for (int e0 = lo; e0 < hi; e0 += 64) {
-                            uint32_t m8[8];
-                            float p8[8];
-                            int c8[8];
+                    // all loads of a turn are issued before anything is used: an id beyond the part of the model in shared
+                    // memory costs a round trip to L2 (the updates are made there by reductions)
+                    constexpr int U = FLAT ? 8 : 4;
+                    const int lo = h.roff[j] + q, hi = h.roff[j + 1];
+                    const uint32_t *meta = reinterpret_cast<const uint32_t *>(val + h.n);
+                    for (int e0 = lo; e0 < hi; e0 += 8 * U) {
+                        float x[U], w[U];
+                        uint32_t m[U];
 #pragma unroll
-                            for (int u = 0; u < 8; ++u) {
-                                const int e = e0 + 8 * u;
-                                const bool on = e < hi;
-                                m8[u] = on ? meta[e] : 0u;
-                                p8[u] = on ? d * val[e] : 0.0f;
-                                c8[u] = on ? cpos[e] : 0;
-                            }
+                        for (int u = 0; u < U; ++u) {
+                            const int e = e0 + 8 * u;
+                            x[u] = e < hi ? val[e] : 0.0f;
+                            m[u] = e < hi ? meta[e] & kIdMask : 0u;
+                        }
 #pragma unroll
-                            for (int u = 0; u < 8; ++u) {
-                                const bool shared_id = (m8[u] >> 31) != 0u && CHICLE_IN_BOUNDS(S.status, c8[u] < P.nzcap);
-                                sts_f32(shared_id ? a_prod + 4u * (uint32_t)c8[u] : a_sink, p8[u]);
-                                const bool far = (m8[u] >> 31) == 0u && p8[u] != 0.0f && // (beyond the coordinate's end p8 is 0)
-                                                 CHICLE_IN_BOUNDS(S.status, (int64_t)(m8[u] & kIdMask) < S.dim);
-                                red_add_if(Uk + (far ? (m8[u] & kIdMask) : 0u), sigma * p8[u], far);
+                        for (int u = 0; u < U; ++u) {
+                            if (FLAT) {
+                                const bool on = e0 + 8 * u < hi && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim);
+                                w[u] = ldcg_if(Uk + (on ? m[u] : 0u), on);
+                            } else if (!cold_ids) {
+                                w[u] = lds_f32(a_w + 4u * (CHICLE_IN_BOUNDS(S.status, m[u] < hotc) ? m[u] : 0u));
+                            } else {
+                                const bool cold = m[u] >= hotc && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim);
+                                const float far = ldcg_if(Uk + (cold ? m[u] : 0u), cold);
+                                const float near = lds_f32(a_w + 4u * (m[u] < hotc ? m[u] : 0u));
+                                w[u] = cold ? far : near;
                             }
                         }
-                    } else if (!FLAT && wt < kLB * 8) {
-                        const int j = wt >> 3, qq = wt & 7;
-                        const int lo = h.roff[j] + qq, hi = h.roff[j + 1];
-                        const float d = dl[j];
-                        const uint32_t a_prod = smem_u32(prod), a_w = smem_u32(W), a_sink = smem_u32(&ctl.sink[lane]);
-                        uint32_t m[2];
-                        float p[2], w2[2];
-                        int cp[2];
-                        bool on[2];
 #pragma unroll
-                        for (int u = 0; u < 2; ++u) {
-                            const int e = lo + 8 * u;
-                            on[u] = e < hi;
-                            m[u] = on[u] ? meta[e] : 0u;
-                            p[u] = on[u] ? d * val[e] : 0.0f;
-                            cp[u] = on[u] ? cpos[e] : 0;
-                        }
-#pragma unroll
-                        for (int u = 0; u < 2; ++u) {
-                            const uint32_t g = m[u] & kIdMask;
-                            w2[u] = W[(on[u] && g < hot_total) ? (g >> logC) : 0u];
-                        }
-#pragma unroll
-                        for (int u = 0; u < 2; ++u) {
-                            const uint32_t g = m[u] & kIdMask;
-                            const bool shared_id = (m[u] >> 31) != 0u, hot = g < hot_total;
-                            const bool list_ok = CHICLE_IN_BOUNDS(S.status, !shared_id || cp[u] < P.nzcap);
-                            const uint32_t addr = (!on[u] || !list_ok) ? a_sink : (shared_id ? a_prod + 4u * (uint32_t)cp[u] : (hot ? a_w + 4u * (g >> logC) : a_sink));
-                            sts_f32(addr, shared_id ? p[u] : fmaf(sigma, p[u], w2[u]));
-                            const bool far = on[u] && !shared_id && !hot && p[u] != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)g < S.dim);
-                            red_add_if(Uk + (far ? g : 0u), sigma * p[u], far); // a reduction at L2, nothing waits for it
-                        }
-                        for (int e = lo + 16; e < hi; e += 8) {
-                            const uint32_t mm = meta[e];
-                            const uint32_t g = mm & kIdMask;
-                            const float pp = d * val[e];
-                            if (mm & 0x80000000u) {
-                                if (CHICLE_IN_BOUNDS(S.status, cpos[e] < P.nzcap)) prod[cpos[e]] = pp;
-                            } else if (g < hot_total) W[g >> logC] = fmaf(sigma, pp, W[g >> logC]);
-                            else if (pp != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)g < S.dim)) atomicAdd(Uk + g, sigma * pp);
-                        }
-                    }
-                    work_bar();
-                    LA_T(ws1);
-                    // (B) four threads per shared id: each adds every fourth entry of the list (at most 8: a list has
-                    //     at most 32), then the four partial sums are added in a fixed order; two ids per thread and
-                    //     pass, all loads first
-                    const int quarter = wt & 3;
-                    constexpr int kIdsPerPass = kWorkThreads / 4;
-                    for (int tb = 0; tb < T; tb += 2 * kIdsPerPass) {
-                        float sum[2];
-                        uint32_t g3[2];
-                        bool on[2];
-                        int o0[2], o1[2];
-#pragma unroll
-                        for (int u = 0; u < 2; ++u) {
-                            const int t = tb + u * kIdsPerPass + (wt >> 2);
-                            on[u] = t < T;
-                            o0[u] = on[u] ? offs[t] + quarter : 0;
-                            o1[u] = on[u] ? offs[t + 1] : 0;
-                            g3[u] = on[u] ? ids[t] : 0u;
-                            if (!CHICLE_IN_BOUNDS(S.status, o1[u] <= P.nzcap && (int64_t)g3[u] < S.dim)) { o1[u] = 0; on[u] = false; }
-                        }
-                        float vv[2][8];
-#pragma unroll
-                        for (int u = 0; u < 2; ++u)
-#pragma unroll
-                            for (int qq = 0; qq < 8; ++qq) {
-                                const int o = o0[u] + 4 * qq;
-                                vv[u][qq] = o < o1[u] ? prod[o] : 0.0f;
-                            }
-#pragma unroll
-                        for (int u = 0; u < 2; ++u) {
-                            sum[u] = ((vv[u][0] + vv[u][1]) + (vv[u][2] + vv[u][3])) + ((vv[u][4] + vv[u][5]) + (vv[u][6] + vv[u][7]));
-                            sum[u] += __shfl_xor_sync(0xffffffffu, sum[u], 1);
-                            sum[u] += __shfl_xor_sync(0xffffffffu, sum[u], 2);
-                        }
-#pragma unroll
-                        for (int u = 0; u < 2; ++u)
-                            if (quarter == 0 && on[u] && sum[u] != 0.0f) {
-                                if (g3[u] < hot_total) W[g3[u] >> logC] = fmaf(sigma, sum[u], W[g3[u] >> logC]);
-                                else atomicAdd(Uk + g3[u], sigma * sum[u]);
-                            }
+                        for (int u = 0; u < U; ++u) acc = fmaf(x[u], w[u], acc);
                     }
                 }
-                work_bar();
+                acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+                acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+                acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+                if (q == 0) st_async_f32(p_buf0 + (slot * (uint32_t)(kMaxC * kLB) + (uint32_t)j) * 4u, acc, p_bar0 + slot * 8u);
             }
-            if (b >= 0) {
-                mbar_arrive_expect_tx_if(smem_u32(&ctl.dbar[par]), d_bytes, wt == 0); // for block b + 2
-                issue_sub(b + kSubSlots, dn); // block b's slot is free
-            }
-            LA_T(ws);
-            // dot products: of block b + 2 against the model as it is now; of block b + 1 first if block b was walked in
-            // place (a block right behind a walked one starts from the model as the walk left it)
-#pragma unroll 1
-            for (int ahead = depth == 1 || sl0 ? 1 : 2; ahead <= depth; ++ahead) {
-                // (one block ahead: block b + 1 after block b's update, whatever block b was)
-                const bool due = b + ahead < nb && !sl1 && (ahead == 1 || !sl2);
-                if (due && !take_dots(b + ahead)) { aborted = true; break; }
-            }
-            if (aborted) break;
-            sl0 = sl1; sl1 = sl2; sl2 = sl3;
-            sl3 = b + kSubSlots < nb && (dn[3] & 1u) != 0u;
+            LA_T(wg1);
+            ok = work_bar_and(ok);
+            if (!ok) { aborted = true; break; }
+            sl0 = depth == 1 ? sl2 : sl1;
+            sl1 = sl2;
             LA_T(wg);
         }
 #ifdef CHICLE_LA_TIMING
@@ -2032,8 +1941,7 @@ template <int LOSS, bool DENSE, bool FLAT, bool TAB> cudaError_t launch_chain(Gl
         (void)cudaMemcpy(t, P.timing, sizeof(t), cudaMemcpyDeviceToHost);
         const double nb = t[3] ? (double)t[3] : 1.0;
         fprintf(stderr, "lookahead chain, cycles per block (partition 0): waiting for dot products %.0f, recurrence %.0f, deltas %.0f; "
-                "workers of CTA 0: waiting for deltas %.0f, update: row-wise %.0f, lists and copy issue %.0f, dot products: record wait %.0f, "
-                "products %.0f, sums and sending %.0f (%llu blocks)\n",
+                "workers of CTA 0: waiting for deltas %.0f, update %.0f, barrier %.0f, record wait %.0f, products %.0f, barrier %.0f (%llu blocks)\n",
                 t[0] / nb, t[1] / nb, t[2] / nb, t[4] / nb, t[7] / nb, t[5] / nb, t[8] / nb, t[9] / nb, t[6] / nb, t[3]);
     }
 #endif
@@ -2247,13 +2155,13 @@ void lookahead_plan(Glm &g, int32_t K)
     const double frac = whole ? 1.0 : (double)region_blocks / (double)(n / kLB + 1);
     const size_t C = (size_t)1 << logC;
     size_t pool;
-    if (dense) pool = (size_t)region_blocks * C * sub_bytes(kLB * slice, 0, true);
+    if (dense) pool = (size_t)region_blocks * C * sub_bytes_dense(kLB, slice);
     else {
-        const double all = 14.0 * (double)g.nnz;
+        const double all = 16.0 * (double)g.nnz;
         double part = whole ? all : 1.2 * frac * all + (double)(1 << 20);
         if (part > all) part = all;
         // (what the prepare kernel's CTAs hold in advance: a piece of about four blocks each)
-        g.la_pool_piece = ((size_t)(4.0 * 14.0 * 32.0 * (double)g.nnz / (double)g.n_coord) + 4096) & ~(size_t)255; // (records start on 16-byte boundaries)
+        g.la_pool_piece = ((size_t)(4.0 * 12.0 * 32.0 * (double)g.nnz / (double)g.n_coord) + 4096) & ~(size_t)255; // (records start on 16-byte boundaries)
         part += (double)g.la_pool_piece * (double)(region_blocks < 2 * (int64_t)g.sm_count ? region_blocks : 2 * (int64_t)g.sm_count);
         pool = (size_t)part + (size_t)region_blocks * C * 128 + 4096;
     }
