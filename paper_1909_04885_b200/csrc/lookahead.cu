@@ -62,7 +62,6 @@ constexpr int kHeadSlots = 2;      // recurrence records (and tables of the logi
 // Worker warps: all but the warps that share warp 0's scheduler (warp ids 0, 4, 8, 12), which stay out of its way.
 constexpr int kWorkWarps = 12;
 constexpr int kWorkThreads = kWorkWarps * 32;
-constexpr int kBarWork = 1;        // named barrier of the worker warps
 constexpr int kRecordWarp = 8;     // fetches the workers' records
 constexpr int kFeedWarp = 4;       // in CTA 0: fetches the recurrence records and writes the new states (see the kernel)
 
@@ -1266,15 +1265,20 @@ __device__ __forceinline__ uint32_t mbar_try_wait_cluster(uint32_t a, uint32_t p
         : "memory");
     return ok;
 }
-// Bounded wait of one warp on an mbarrier that another CTA of the cluster completes (every lane must call it). No
-// pauses of its own (try_wait suspends the thread for a while by itself; the waits of the pipeline are short and on
-// its critical path); gives up after about a second, or when the CTA is aborting. The result is the same on all
-// lanes. One warp per CTA waits this way at a time.
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int *abort_flag, uint32_t *status)
+// One look without suspension: 16 cycles with the vote, against 47 for try_wait with a time hint.
+__device__ __forceinline__ uint32_t mbar_test(uint32_t a, uint32_t parity)
 {
-    // every lane looks at the barrier (one instruction for the warp either way) and the lanes agree by a vote, so
-    // that the warp stays together
-    if (__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity) != 0u)) return true;
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(a), "r"(parity)
+        : "memory");
+    return ok;
+}
+// (not inlined: one copy keeps the loops of the kernel small)
+__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int *abort_flag, uint32_t *status)
+{
     const long long t_start = clock64();
     for (;;) {
         bool ok = false;
@@ -1292,19 +1296,14 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
         }
     }
 }
-// The worker warps' barrier, with a vote: all of them take the same decision after a wait.
-__device__ __forceinline__ bool work_bar_and(bool ok)
+// Bounded wait of one warp on an mbarrier (every lane must call it). No pauses of its own (try_wait suspends the thread
+// for a while by itself; the waits of the pipeline are short and on its critical path); gives up after about a second, or
+// when the CTA is aborting. The result is the same on all lanes: every lane looks at the barrier (one instruction for the
+// warp either way) and the lanes agree by a vote, so that the warp stays together.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int *abort_flag, uint32_t *status)
 {
-    uint32_t r;
-    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.and.pred p, %2, %3, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(r)
-                 : "r"((uint32_t)ok), "n"(kBarWork), "n"(kWorkThreads)
-                 : "memory");
-    return r != 0;
-}
-__device__ __forceinline__ void work_bar()
-{
-    asm volatile("bar.sync %0, %1;" ::"n"(kBarWork), "n"(kWorkThreads) : "memory");
+    if (__all_sync(0xffffffffu, mbar_test(bar, parity) != 0u)) return true;
+    return mbar_wait_slow(bar, parity, abort_flag, status);
 }
 
 struct alignas(16) ChainCtl {
@@ -1313,6 +1312,7 @@ struct alignas(16) ChainCtl {
     uint64_t pbar[2];              // CTA 0: the partial dot products of a block have arrived from all CTAs
     uint64_t dbar[2];              // a block's deltas have arrived from CTA 0
     uint64_t subfree[kSubSlots];   // the worker warps are through with the slot's record
+    uint64_t updone, dotsdone;     // the worker warps have applied a block's update / taken a turn's dot products
     uint64_t ackbar;               // CTA 0: every CTA has applied all updates (before a block is walked in place)
     alignas(16) float pbuf[2][kMaxC][kLB];
     alignas(16) float dbuf[2][kLB];
@@ -1381,6 +1381,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             mbar_init(smem_u32(&ctl.pbar[i]), 1);
             mbar_init(smem_u32(&ctl.dbar[i]), 1);
         }
+        mbar_init(smem_u32(&ctl.updone), kWorkWarps);
+        mbar_init(smem_u32(&ctl.dotsdone), kWorkWarps);
         mbar_init(smem_u32(&ctl.ackbar), (uint32_t)C);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // armed for the first two blocks before anybody can send
@@ -1673,16 +1675,18 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             load_dir(blk + 1, d);
         }
     }
-    if (is_worker && nb > 0) {
+    if (is_worker) {
         // ============================== the worker warps ========================================================
-        // Two barriers per block: behind its update (the model is as block b left it) and behind the dot products taken
-        // against that model. Every warp waits for deltas and records by itself; a warp whose wait runs out does nothing
-        // and says so at the next barrier's vote, so that all warps still meet there.
+        // Every warp waits by itself, for deltas, for records and for the other warps: `updone` completes when all have
+        // applied a block's update (the dot products that follow read the model), `dotsdone` when all have taken a turn's
+        // dot products (the update that follows writes it). Arriving and waiting are apart, so that what does not touch the
+        // model is done in between. A warp whose wait runs out leaves, and the abort flag ends the others' waits.
         const int wt = (warp - 1 - (warp >> 2)) * 32 + lane; // 0 .. kWorkThreads - 1
         const uint32_t p_bar0 = mapa_u32(smem_u32(&ctl.pbar[0]), 0u);
         const uint32_t p_buf0 = mapa_u32(smem_u32(&ctl.pbuf[0][crank][0]), 0u);
         const uint32_t ack_bar = mapa_u32(smem_u32(&ctl.ackbar), 0u);
-        const uint32_t a_w = smem_u32(W), a_sink = smem_u32(&ctl.sink[lane]);
+        const uint32_t updone = smem_u32(&ctl.updone), dotsdone = smem_u32(&ctl.dotsdone);
+        float *const sink = &ctl.sink[lane];
         const uint32_t hotc = (uint32_t)P.hotc;
         const bool cold_ids = FLAT || (int64_t)hot_total < S.dim;  // some ids are not in shared memory
         const int dstride = dense_stride(hot_mine);                // dense: floats per row of a record
@@ -1697,17 +1701,19 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         // code for every phase keeps the loop small: the warps run at the pace instructions can be fetched).
         bool sl0 = false, sl1 = false; // whether blocks b and b + 1 are walked in place
 #pragma unroll 1
-        for (int b = -depth; b < nb; ++b) {
+        for (int b = nb > 0 ? -depth : 0; b < nb; ++b) {
             const uint32_t par = (uint32_t)(b & 1);
             if (b >= 0) {
-                // (walked in place by CTA 0: every update before it has been applied here, the barriers behind the block
-                // before say so; wait for the walk to end)
-                if (sl0 && wt == 0) mbar_arrive_remote_release(ack_bar);
+                ok = mbar_wait_cluster(dotsdone, (uint32_t)(b + depth - 1) & 1u, abort_flag, S.status);
+                // (a block walked in place by CTA 0: every update before it has been applied here, and no dot product reads
+                // the model any more; wait for the walk to end)
+                if (sl0 && ok && wt == 0) mbar_arrive_remote_release(ack_bar);
                 ok = ok && mbar_wait_cluster(smem_u32(&ctl.dbar[par]), (uint32_t)(b >> 1) & 1u, abort_flag, S.status);
+                if (!ok) break;
                 if (sl0) fence_cluster(); // the walk's ordinary stores into this CTA's part of the model
-                mbar_arrive_expect_tx_if(smem_u32(&ctl.dbar[par]), d_bytes, wt == 0 && ok); // for block b + 2
+                mbar_arrive_expect_tx_if(smem_u32(&ctl.dbar[par]), d_bytes, wt == 0); // for block b + 2
                 LA_T(wd);
-                if (ok && !sl0) {
+                if (!sl0) {
                     // ---- block b's update of this CTA's part of the model
                     const float *dl = ctl.dbuf[par];
                     const unsigned char *rec = record(b);
@@ -1734,12 +1740,50 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                             W[wt] = fmaf(sigma, s0 + s1, W[wt]);
                         }
                     } else {
+                        // Eight threads per shared id: each adds every eighth entry of the list (at most four: all loads of a
+                        // thread first), then the partial sums are added in a fixed order.
+                        const int n = h.n, T = h.T, nl = h.nl, q = wt & 7;
+                        const uint32_t *meta = reinterpret_cast<const uint32_t *>(val + n);
+                        const uint32_t *ids = meta + n;
+                        const float *lval = reinterpret_cast<const float *>(ids + T);
+                        const uint16_t *lst = reinterpret_cast<const uint16_t *>(lval + nl);
+                        const unsigned char *lrow = reinterpret_cast<const unsigned char *>(lst + T);
+                        for (int t4 = wt >> 3; t4 < ((T + 3) & ~3); t4 += kWorkThreads / 8) { // (whole warps)
+                            const bool on = t4 < T;
+                            const uint32_t id = on ? ids[t4] : 0u, v = id & kIdMask;
+                            const int len = on ? (int)((id >> kIdBits) & 31u) + 1 : 0, first = (on ? lst[t4] : 0) + q;
+                            const bool more = __any_sync(0xffffffffu, len > 8);
+                            float x[4] = {0.f, 0.f, 0.f, 0.f};
+                            int r[4] = {0, 0, 0, 0};
+                            auto take = [&](int u) {
+                                if (q + 8 * u < len && CHICLE_IN_BOUNDS(S.status, first + 8 * u < nl)) {
+                                    x[u] = lval[first + 8 * u];
+                                    r[u] = lrow[first + 8 * u] & 31;
+                                }
+                            };
+                            take(0);
+                            const float w = W[!FLAT && v < hotc ? v : 0u];
+                            if (more) { take(1); take(2); take(3); }
+                            float sum = x[0] * dl[r[0]];
+                            if (more) {
+                                sum = fmaf(x[1], dl[r[1]], sum);
+                                sum = fmaf(x[2], dl[r[2]], sum);
+                                sum = fmaf(x[3], dl[r[3]], sum);
+                            }
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+                            sum += __shfl_xor_sync(0xffffffffu, sum, 4);
+                            const bool mine = on && q == 0, near = !FLAT && v < hotc;
+                            if (!FLAT) *(mine && near ? W + v : sink) = fmaf(sigma, sum, w);
+                            if (cold_ids) {
+                                const bool far = mine && !near && sum != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
+                                red_add_if(Uk + (far ? v : 0u), sigma * sum, far);
+                            }
+                        }
                         // A thread per entry: one whose id no other coordinate of the block has is applied (no two threads
                         // touch the same word). One store per entry, its address chosen without a branch: the model word, or
                         // a word that nobody reads; ids beyond the part in shared memory are added to at L2, nothing waits.
                         constexpr int U = FLAT ? 4 : 2;
-                        const int n = h.n;
-                        const uint32_t *meta = reinterpret_cast<const uint32_t *>(val + n);
                         for (int e0 = wt; e0 < n; e0 += U * kWorkThreads) {
                             uint32_t m[U];
                             float p[U], w[U];
@@ -1753,60 +1797,41 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                             for (int u = 0; u < U; ++u) {
                                 const uint32_t v = m[u] & kIdMask;
                                 p[u] = sigma * (p[u] * dl[(m[u] >> kIdBits) & 31u]);
-                                if (!FLAT) w[u] = lds_f32(a_w + 4u * (v < hotc ? v : 0u));
+                                if (!FLAT) w[u] = W[v < hotc ? v : 0u];
                             }
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
                                 const uint32_t v = m[u] & kIdMask;
-                                const bool mine = (m[u] >> 31) == 0u;
-                                if (!FLAT) sts_f32(mine && v < hotc ? a_w + 4u * v : a_sink, p[u] + w[u]);
+                                const bool mine = (m[u] >> 31) == 0u, near = !FLAT && v < hotc;
+                                if (!FLAT) *(mine && near ? W + v : sink) = p[u] + w[u];
                                 if (cold_ids) {
-                                    const bool far = mine && v >= hotc && p[u] != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
+                                    const bool far = mine && !near && p[u] != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
                                     red_add_if(Uk + (far ? v : 0u), p[u], far);
                                 }
                             }
                         }
-                        // Eight threads per shared id: each adds every eighth entry of the list, then the partial sums are added
-                        // in a fixed order.
-                        const int T = h.T, nl = h.nl, q = wt & 7;
-                        const uint32_t *ids = meta + n;
-                        const float *lval = reinterpret_cast<const float *>(ids + T);
-                        const uint16_t *lst = reinterpret_cast<const uint16_t *>(lval + nl);
-                        const unsigned char *lrow = reinterpret_cast<const unsigned char *>(lst + T);
-                        for (int t4 = wt >> 3; t4 < ((T + 3) & ~3); t4 += kWorkThreads / 8) { // (whole warps)
-                            const bool on = t4 < T;
-                            const uint32_t id = on ? ids[t4] : 0u, v = id & kIdMask;
-                            const int first = on ? lst[t4] : 0, len = on ? (int)((id >> kIdBits) & 31u) + 1 : 0;
-                            float sum = 0.0f;
-                            for (int o = q; o < len; o += 8)
-                                if (CHICLE_IN_BOUNDS(S.status, first + o < nl)) sum = fmaf(lval[first + o], dl[lrow[first + o] & 31], sum);
-                            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-                            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-                            sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-                            if (on && q == 0 && sum != 0.0f) {
-                                if (v < hotc) sts_f32(a_w + 4u * v, fmaf(sigma, sum, lds_f32(a_w + 4u * v)));
-                                else if (CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim)) atomicAdd(Uk + v, sigma * sum);
-                            }
-                        }
                     }
                 }
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(updone);
+                    mbar_arrive(smem_u32(&ctl.subfree[b & (kSubSlots - 1)])); // block b's slot is free
+                }
                 LA_T(ws1);
-                ok = work_bar_and(ok);
-                LA_T(ws);
-                if (lane == 0) mbar_arrive(smem_u32(&ctl.subfree[b & (kSubSlots - 1)])); // block b's slot is free
-                if (!ok) { aborted = true; break; }
             }
             // ---- dot products: of block b + depth against the model as it is now. A block right behind a walked one starts
             //      from the model as the walk left it: with depth 2 its products wait for that.
             bool sl2 = false;
             if (b + depth < nb) {
                 ok = mbar_wait_cluster(smem_u32(&ctl.subfull[(b + depth) & (kSubSlots - 1)]), (uint32_t)((b + depth) / kSubSlots) & 1u, abort_flag, S.status);
+                if (!ok) break;
                 sl2 = ctl.walk[(b + depth) & (kSubSlots - 1)] != 0;
             }
             LA_T(wg0);
             const bool late = depth == 2 && sl0 && !sl1 && b + 1 < nb, due = b + depth < nb && !sl2 && (depth == 1 || !sl1);
+            bool waited = b < 0; // for the update
 #pragma unroll 1
-            for (int x = late ? b + 1 : b + depth; ok && (late || due) && x <= (due ? b + depth : b + 1); x += depth - 1 > 0 ? depth - 1 : 1) {
+            for (int x = late ? b + 1 : b + depth; (late || due) && x <= (due ? b + depth : b + 1); ++x) {
                 const unsigned char *rec = record(x);
                 const SubHead &h = *reinterpret_cast<const SubHead *>(rec);
                 // (debug build) a record whose sizes do not fit its slot is not read: as if its wait had run out
@@ -1818,12 +1843,13 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 const float *val = reinterpret_cast<const float *>(rec + sizeof(SubHead));
                 const uint32_t slot = (uint32_t)(fg & 1);
                 ++fg;
-                if (wt >= kLB * 8) continue;
-                // eight threads per coordinate
-                const int j = wt >> 3, q = wt & 7;
+                // eight threads per coordinate (the first eight warps)
+                const int j = (wt >> 3) & (kLB - 1), q = wt & 7;
                 float acc = 0.0f;
                 if (DENSE) {
-                    if (j < h.cnt) {
+                    if (!waited && !mbar_wait_cluster(updone, par, abort_flag, S.status)) { ok = false; break; }
+                    waited = true;
+                    if (j < h.cnt && wt < kLB * 8) {
                         const float4 *v4 = reinterpret_cast<const float4 *>(val + j * dstride), *w4 = reinterpret_cast<const float4 *>(W);
 #pragma unroll 4
                         for (int e = q; e < (hot_mine + 3) >> 2; e += 8) {
@@ -1832,69 +1858,96 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                         }
                     }
                 } else {
-                    // all loads of a turn are issued before anything is used: an id beyond the part of the model in shared
-                    // memory costs a round trip to L2 (the updates are made there by reductions)
-                    constexpr int U = FLAT ? 8 : 4;
-                    const int lo = h.roff[j] + q, hi = h.roff[j + 1];
+                    // eight entries per thread and turn, all loads of a turn issued before anything is used: an id beyond the
+                    // part of the model in shared memory costs a round trip to L2 (the updates are made there by reductions)
+                    const int hi = wt < kLB * 8 ? h.roff[j + 1] : 0;
                     const uint32_t *meta = reinterpret_cast<const uint32_t *>(val + h.n);
-                    for (int e0 = lo; e0 < hi; e0 += 8 * U) {
-                        float x[U], w[U];
-                        uint32_t m[U];
+                    int e0 = h.roff[j] + q;
+                    float xx[8], ww[8];
+                    uint32_t mm[8];
+                    bool more;
+                    auto entry = [&](int u) {
+                        const int e = e0 + 8 * u;
+                        xx[u] = e < hi ? val[e] : 0.0f;
+                        mm[u] = e < hi ? meta[e] & kIdMask : 0u;
+                    };
+                    auto model = [&](int u) {
+                        if (FLAT) {
+                            const bool in = e0 + 8 * u < hi && CHICLE_IN_BOUNDS(S.status, (int64_t)mm[u] < S.dim);
+                            ww[u] = ldcg_if(Uk + (in ? mm[u] : 0u), in);
+                        } else if (!cold_ids) {
+                            ww[u] = W[CHICLE_IN_BOUNDS(S.status, mm[u] < hotc) ? mm[u] : 0u];
+                        } else {
+                            const bool cold = mm[u] >= hotc && CHICLE_IN_BOUNDS(S.status, (int64_t)mm[u] < S.dim);
+                            const float far = ldcg_if(Uk + (cold ? mm[u] : 0u), cold);
+                            const float near = W[mm[u] < hotc ? mm[u] : 0u];
+                            ww[u] = cold ? far : near;
+                        }
+                    };
+                    auto entries = [&]() {
+                        more = __any_sync(0xffffffffu, e0 + 32 < hi);
 #pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            const int e = e0 + 8 * u;
-                            x[u] = e < hi ? val[e] : 0.0f;
-                            m[u] = e < hi ? meta[e] & kIdMask : 0u;
+                        for (int u = 0; u < 4; ++u) entry(u);
+#pragma unroll
+                        for (int u = 4; u < 8; ++u) { xx[u] = 0.0f; ww[u] = 0.0f; mm[u] = 0u; }
+                        if (more) {
+#pragma unroll
+                            for (int u = 4; u < 8; ++u) entry(u);
+                        }
+                    };
+                    entries();
+                    if (!waited && !mbar_wait_cluster(updone, par, abort_flag, S.status)) { ok = false; break; }
+                    waited = true;
+                    for (;;) { // (whole warps)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) model(u);
+                        if (more) {
+#pragma unroll
+                            for (int u = 4; u < 8; ++u) model(u);
                         }
 #pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            if (FLAT) {
-                                const bool on = e0 + 8 * u < hi && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim);
-                                w[u] = ldcg_if(Uk + (on ? m[u] : 0u), on);
-                            } else if (!cold_ids) {
-                                w[u] = lds_f32(a_w + 4u * (CHICLE_IN_BOUNDS(S.status, m[u] < hotc) ? m[u] : 0u));
-                            } else {
-                                const bool cold = m[u] >= hotc && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim);
-                                const float far = ldcg_if(Uk + (cold ? m[u] : 0u), cold);
-                                const float near = lds_f32(a_w + 4u * (m[u] < hotc ? m[u] : 0u));
-                                w[u] = cold ? far : near;
-                            }
-                        }
+                        for (int u = 0; u < 4; ++u) acc = fmaf(xx[u], ww[u], acc);
+                        if (!more) break;
 #pragma unroll
-                        for (int u = 0; u < U; ++u) acc = fmaf(x[u], w[u], acc);
+                        for (int u = 4; u < 8; ++u) acc = fmaf(xx[u], ww[u], acc);
+                        e0 += 64;
+                        if (!__any_sync(0xffffffffu, e0 < hi)) break;
+                        entries();
                     }
                 }
                 acc += __shfl_xor_sync(0xffffffffu, acc, 1);
                 acc += __shfl_xor_sync(0xffffffffu, acc, 2);
                 acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-                if (q == 0) st_async_f32(p_buf0 + (slot * (uint32_t)(kMaxC * kLB) + (uint32_t)j) * 4u, acc, p_bar0 + slot * 8u);
+                if (q == 0 && wt < kLB * 8) st_async_f32(p_buf0 + (slot * (uint32_t)(kMaxC * kLB) + (uint32_t)j) * 4u, acc, p_bar0 + slot * 8u);
             }
+            if (ok && !waited) ok = mbar_wait_cluster(updone, par, abort_flag, S.status);
+            if (!ok) break;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(dotsdone);
             LA_T(wg1);
-            ok = work_bar_and(ok);
-            if (!ok) { aborted = true; break; }
             sl0 = depth == 1 ? sl2 : sl1;
             sl1 = sl2;
-            LA_T(wg);
         }
+        if (!ok && lane == 0) *abort_flag = 1;
+        aborted = !ok; // (otherwise: every update has been applied and every dot product taken by this warp; the last turn
+                       // waited for the other warps' updates)
 #ifdef CHICLE_LA_TIMING
         if (blockIdx.x == 0 && wt == 0) {
             unsigned long long *d = P.timing + 4;
             d[0] = wd; d[1] = ws; d[2] = wg; d[3] = ws1; d[4] = wg0; d[5] = wg1;
         }
 #endif
-    }
-    if (is_worker && !aborted) {
-        // the model goes back to row k: as it is, or after the round's last launch as the update U_k = (w - v) / sigma'
-        const int wt = (warp - 1 - (warp >> 2)) * 32 + lane;
-        work_bar();
-        const float inv_sigma = 1.0f / sigma;
-        for (int l = wt; l < hot_mine; l += kWorkThreads) {
-            const size_t g = DENSE ? (size_t)(slice0 + l) : ((size_t)l << logC) + crank;
-            Uk[g] = P.model_out ? (W[l] - S.vbase[g]) * inv_sigma : W[l];
+        if (!aborted) {
+            // the model goes back to row k: as it is, or after the round's last launch as the update U_k = (w - v) / sigma'
+            const float inv_sigma = 1.0f / sigma;
+            for (int l = wt; l < hot_mine; l += kWorkThreads) {
+                const size_t g = DENSE ? (size_t)(slice0 + l) : ((size_t)l << logC) + crank;
+                Uk[g] = P.model_out ? (W[l] - S.vbase[g]) * inv_sigma : W[l];
+            }
+            if (P.model_out)
+                for (size_t g = cold0 + ((size_t)wt << logC); g < (size_t)S.dim; g += (size_t)kWorkThreads << logC)
+                    Uk[g] = (__ldcg(Uk + g) - S.vbase[g]) * inv_sigma;
         }
-        if (P.model_out)
-            for (size_t g = cold0 + ((size_t)wt << logC); g < (size_t)S.dim; g += (size_t)kWorkThreads << logC)
-                Uk[g] = (__ldcg(Uk + g) - S.vbase[g]) * inv_sigma;
     }
     if (is_worker || nb == 0) {
         if ((tid & 31) == 0) *reinterpret_cast<volatile int *>(&ctl.done) = 1;
@@ -1941,8 +1994,8 @@ template <int LOSS, bool DENSE, bool FLAT, bool TAB> cudaError_t launch_chain(Gl
         (void)cudaMemcpy(t, P.timing, sizeof(t), cudaMemcpyDeviceToHost);
         const double nb = t[3] ? (double)t[3] : 1.0;
         fprintf(stderr, "lookahead chain, cycles per block (partition 0): waiting for dot products %.0f, recurrence %.0f, deltas %.0f; "
-                "workers of CTA 0: waiting for deltas %.0f, update %.0f, barrier %.0f, record wait %.0f, products %.0f, barrier %.0f (%llu blocks)\n",
-                t[0] / nb, t[1] / nb, t[2] / nb, t[4] / nb, t[7] / nb, t[5] / nb, t[8] / nb, t[9] / nb, t[6] / nb, t[3]);
+                "workers of CTA 0: waiting for deltas %.0f, update %.0f, record wait %.0f, products %.0f (%llu blocks)\n",
+                t[0] / nb, t[1] / nb, t[2] / nb, t[4] / nb, t[7] / nb, t[8] / nb, t[9] / nb, t[3]);
     }
 #endif
     return e;
