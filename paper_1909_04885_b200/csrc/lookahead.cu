@@ -58,10 +58,15 @@ constexpr int kIdBits = 26;
 constexpr uint32_t kIdMask = (1u << kIdBits) - 1u;
 constexpr int kChainThreads = 512;
 constexpr int kSubSlots = 4;       // worker records in shared memory: blocks b .. b + 3
-constexpr int kHeadSlots = 2;      // recurrence records (and tables of the logistic step, see tab_map) in shared memory
+// Recurrence records in shared memory: a record is fetched when the block that many before it is done, and takes 1 500 cycles
+// or more from memory, so two would set the pace (1 M sparse rows: 3 019 cycles a block, with three 2 600). With tables of the logistic step
+// (see tab_map: 32 KB or more each, fetched with the record) a block takes longer and two do.
+constexpr int kMaxHeadSlots = 3;
+__host__ __device__ constexpr int head_slots(bool tables) { return tables ? 2 : 3; }
 // Worker warps: all but the warps that share warp 0's scheduler (warp ids 0, 4, 8, 12), which stay out of its way.
 constexpr int kWorkWarps = 12;
 constexpr int kWorkThreads = kWorkWarps * 32;
+constexpr int kBarWork = 1;        // named barrier of the worker warps
 constexpr int kRecordWarp = 8;     // fetches the workers' records
 constexpr int kFeedWarp = 4;       // in CTA 0: fetches the recurrence records and writes the new states (see the kernel)
 
@@ -1306,13 +1311,15 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     return mbar_wait_slow(bar, parity, abort_flag, status);
 }
 
+// The worker warps' barrier: 35 cycles when all are there (with a vote 78, by arrivals on an mbarrier 181).
+__device__ __forceinline__ void work_bar() { asm volatile("bar.sync %0, %1;" ::"n"(kBarWork), "n"(kWorkThreads) : "memory"); }
+
 struct alignas(16) ChainCtl {
     uint64_t subfull[kSubSlots];   // count the bytes of the bulk copies into the workers' record slots
-    uint64_t headfull[kHeadSlots]; // the same for the recurrence warp's records (CTA 0)
+    uint64_t headfull[kMaxHeadSlots]; // the same for the recurrence warp's records (CTA 0)
     uint64_t pbar[2];              // CTA 0: the partial dot products of a block have arrived from all CTAs
     uint64_t dbar[2];              // a block's deltas have arrived from CTA 0
     uint64_t subfree[kSubSlots];   // the worker warps are through with the slot's record
-    uint64_t updone, dotsdone;     // the worker warps have applied a block's update / taken a turn's dot products
     uint64_t ackbar;               // CTA 0: every CTA has applied all updates (before a block is walked in place)
     alignas(16) float pbuf[2][kMaxC][kLB];
     alignas(16) float dbuf[2][kLB];
@@ -1332,8 +1339,9 @@ __host__ __device__ inline ChainLayout chain_layout(int nzcap, int hotc, bool de
 {
     ChainLayout L;
     L.heads = (uint32_t)((sizeof(ChainCtl) + 127) & ~(size_t)127);
-    L.tabs = L.heads + kHeadSlots * (uint32_t)sizeof(ChainHead);
-    L.subs = L.tabs + kHeadSlots * tab_bytes(tab_bins);
+    const uint32_t hs = (uint32_t)head_slots(tab_bins > 0);
+    L.tabs = L.heads + hs * (uint32_t)sizeof(ChainHead);
+    L.subs = L.tabs + hs * tab_bytes(tab_bins);
     L.sub_stride = dense ? sub_bytes_dense(kLB, hotc) : sub_room(nzcap);
     L.w = L.subs + kSubSlots * L.sub_stride;
     L.total = L.w + 4u * (uint32_t)(hotc > 0 ? hotc : 4);
@@ -1374,15 +1382,13 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         ctl.done = 0;
         for (int i = 0; i < kSubSlots; ++i) {
             mbar_init(smem_u32(&ctl.subfull[i]), 1);
-            mbar_init(smem_u32(&ctl.subfree[i]), kWorkWarps);
+            mbar_init(smem_u32(&ctl.subfree[i]), 1);
         }
-        for (int i = 0; i < kHeadSlots; ++i) mbar_init(smem_u32(&ctl.headfull[i]), 1);
+        for (int i = 0; i < kMaxHeadSlots; ++i) mbar_init(smem_u32(&ctl.headfull[i]), 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&ctl.pbar[i]), 1);
             mbar_init(smem_u32(&ctl.dbar[i]), 1);
         }
-        mbar_init(smem_u32(&ctl.updone), kWorkWarps);
-        mbar_init(smem_u32(&ctl.dotsdone), kWorkWarps);
         mbar_init(smem_u32(&ctl.ackbar), (uint32_t)C);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // armed for the first two blocks before anybody can send
@@ -1405,6 +1411,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     cluster_arrive();
     cluster_wait();
 
+    constexpr int HS = head_slots(TAB);
     const bool is_chain = crank == 0 && warp == 0;
     const bool is_worker = (warp & 3) != 0;
     bool aborted = false;
@@ -1424,13 +1431,14 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         const uint32_t s_dst = smem_u32(&ctl.sbuf[0][4 * q]), s_bar = smem_u32(&ctl.dbar[0]); // (this CTA's own)
         float xs[4] = {0.f, 0.f, 0.f, 0.f}; // what the block before contributes to this block's states
         int fp = 0, sc = 0;                // staged blocks and walked blocks so far
+        int slot = 0;                      // b mod the head slots
+        uint32_t turn = 0;                 // parity of b / the head slots
 #ifdef CHICLE_LA_TIMING
         long long tw = 0, tr = 0, te = 0, t0 = clock64(), t1 = 0;
 #endif
 #pragma unroll 1
         for (int b = 0; b < nb; ++b) {
-            const int slot = b & (kHeadSlots - 1);
-            if (!mbar_wait_cluster(smem_u32(&ctl.headfull[slot]), (uint32_t)(b / kHeadSlots) & 1u, abort_flag, S.status)) { aborted = true; break; }
+            if (!mbar_wait_cluster(smem_u32(&ctl.headfull[slot]), turn, abort_flag, S.status)) { aborted = true; break; }
             const ChainHead &H = *reinterpret_cast<const ChainHead *>(smem_chain + L.heads + (size_t)slot * sizeof(ChainHead));
             const int cnt = H.cnt;
             const uint32_t par = (uint32_t)(b & 1);
@@ -1604,6 +1612,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 LA_T(te);
             }
             __syncwarp();
+            if (++slot == HS) {
+                slot = 0;
+                turn ^= 1u;
+            }
         }
 #ifdef CHICLE_LA_TIMING
         if (blockIdx.x == 0 && lane == 0) {
@@ -1615,7 +1627,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     if (crank == 0 && warp == kFeedWarp && nb > 0) {
         // ============================== the feeder: what the recurrence warp need not do itself =====================
         // When a block's deltas have arrived here, the recurrence warp is done with the block's head: its new states go
-        // to global memory and the head (and table) two blocks on into its slot. (The recurrence warp waits for that
+        // to global memory and the head (and table) HS blocks on into its slot. (The recurrence warp waits for that
         // head before it sends deltas on this barrier again, so the feeder never misses a phase.)
         const uint32_t tab_len = TAB ? tab_bytes(P.tab_bins) : 0u;
         const uint32_t heads0 = smem_u32(smem_chain + L.heads), tabs0 = smem_u32(smem_chain + L.tabs);
@@ -1627,16 +1639,17 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             bulk_g2s_if(heads0 + (uint32_t)slot * (uint32_t)sizeof(ChainHead), P.rec + at * sizeof(ChainHead), (uint32_t)sizeof(ChainHead), bar, on);
             if (TAB) bulk_g2s_if(tabs0 + (uint32_t)slot * tab_len, P.rec + P.tab_off + at * tab_len, tab_len, bar, on);
         };
-        for (int i = 0; i < kHeadSlots; ++i) issue_head(i, i);
+        for (int i = 0; i < HS; ++i) issue_head(i, i);
+        int slot = 0;
 #pragma unroll 1
         for (int b = 0; b < nb; ++b) {
-            const int slot = b & (kHeadSlots - 1);
             if (!mbar_wait_cluster(smem_u32(&ctl.dbar[b & 1]), (uint32_t)(b >> 1) & 1u, abort_flag, S.status)) break;
             const ChainHead &H = *reinterpret_cast<const ChainHead *>(smem_chain + L.heads + (size_t)slot * sizeof(ChainHead));
             const int32_t c = H.hdr[lane].coord;
             if (lane < H.cnt && !(H.flags & 1) && CHICLE_IN_BOUNDS(S.status, c >= 0 && (int64_t)c < S.n_coord)) S.alpha[c] = ctl.sbuf[b & 1][lane];
             __syncwarp();
-            issue_head(b + kHeadSlots, slot);
+            issue_head(b + HS, slot);
+            slot = slot + 1 == HS ? 0 : slot + 1;
         }
     }
     if (warp == kRecordWarp && nb > 0) {
@@ -1677,15 +1690,13 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     }
     if (is_worker) {
         // ============================== the worker warps ========================================================
-        // Every warp waits by itself, for deltas, for records and for the other warps: `updone` completes when all have
-        // applied a block's update (the dot products that follow read the model), `dotsdone` when all have taken a turn's
-        // dot products (the update that follows writes it). Arriving and waiting are apart, so that what does not touch the
-        // model is done in between. A warp whose wait runs out leaves, and the abort flag ends the others' waits.
+        // Two barriers per block: in front of its update (no dot product reads the model any more) and behind it. Every
+        // warp waits for deltas and records by itself; one whose wait runs out does no more work but goes on meeting the
+        // others at the barriers (its abort flag ends their waits too).
         const int wt = (warp - 1 - (warp >> 2)) * 32 + lane; // 0 .. kWorkThreads - 1
         const uint32_t p_bar0 = mapa_u32(smem_u32(&ctl.pbar[0]), 0u);
         const uint32_t p_buf0 = mapa_u32(smem_u32(&ctl.pbuf[0][crank][0]), 0u);
         const uint32_t ack_bar = mapa_u32(smem_u32(&ctl.ackbar), 0u);
-        const uint32_t updone = smem_u32(&ctl.updone), dotsdone = smem_u32(&ctl.dotsdone);
         float *const sink = &ctl.sink[lane];
         const uint32_t hotc = (uint32_t)P.hotc;
         const bool cold_ids = FLAT || (int64_t)hot_total < S.dim;  // some ids are not in shared memory
@@ -1704,16 +1715,18 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         for (int b = nb > 0 ? -depth : 0; b < nb; ++b) {
             const uint32_t par = (uint32_t)(b & 1);
             if (b >= 0) {
-                ok = mbar_wait_cluster(dotsdone, (uint32_t)(b + depth - 1) & 1u, abort_flag, S.status);
-                // (a block walked in place by CTA 0: every update before it has been applied here, and no dot product reads
-                // the model any more; wait for the walk to end)
-                if (sl0 && ok && wt == 0) mbar_arrive_remote_release(ack_bar);
+                // (a block walked in place by CTA 0: every update before it has been applied here; once no dot product reads
+                // the model any more, say so, and wait for the walk to end)
+                if (sl0) {
+                    work_bar();
+                    if (wt == 0) mbar_arrive_remote_release(ack_bar);
+                }
                 ok = ok && mbar_wait_cluster(smem_u32(&ctl.dbar[par]), (uint32_t)(b >> 1) & 1u, abort_flag, S.status);
-                if (!ok) break;
                 if (sl0) fence_cluster(); // the walk's ordinary stores into this CTA's part of the model
-                mbar_arrive_expect_tx_if(smem_u32(&ctl.dbar[par]), d_bytes, wt == 0); // for block b + 2
+                mbar_arrive_expect_tx_if(smem_u32(&ctl.dbar[par]), d_bytes, wt == 0 && ok); // for block b + 2
+                work_bar();
                 LA_T(wd);
-                if (!sl0) {
+                if (!sl0 && ok) {
                     // ---- block b's update of this CTA's part of the model
                     const float *dl = ctl.dbuf[par];
                     const unsigned char *rec = record(b);
@@ -1812,26 +1825,25 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                         }
                     }
                 }
-                __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(updone);
-                    mbar_arrive(smem_u32(&ctl.subfree[b & (kSubSlots - 1)])); // block b's slot is free
-                }
                 LA_T(ws1);
             }
             // ---- dot products: of block b + depth against the model as it is now. A block right behind a walked one starts
             //      from the model as the walk left it: with depth 2 its products wait for that.
             bool sl2 = false;
             if (b + depth < nb) {
-                ok = mbar_wait_cluster(smem_u32(&ctl.subfull[(b + depth) & (kSubSlots - 1)]), (uint32_t)((b + depth) / kSubSlots) & 1u, abort_flag, S.status);
-                if (!ok) break;
+                ok = ok && mbar_wait_cluster(smem_u32(&ctl.subfull[(b + depth) & (kSubSlots - 1)]), (uint32_t)((b + depth) / kSubSlots) & 1u, abort_flag, S.status);
                 sl2 = ctl.walk[(b + depth) & (kSubSlots - 1)] != 0;
             }
             LA_T(wg0);
             const bool late = depth == 2 && sl0 && !sl1 && b + 1 < nb, due = b + depth < nb && !sl2 && (depth == 1 || !sl1);
-            bool waited = b < 0; // for the update
+            bool met = b < 0; // the barrier behind the update
+            auto meet = [&]() {
+                if (!met) work_bar();
+                if (!met && wt == 0) mbar_arrive(smem_u32(&ctl.subfree[b & (kSubSlots - 1)])); // block b's slot is free
+                met = true;
+            };
 #pragma unroll 1
-            for (int x = late ? b + 1 : b + depth; (late || due) && x <= (due ? b + depth : b + 1); ++x) {
+            for (int x = late ? b + 1 : b + depth; ok && (late || due) && x <= (due ? b + depth : b + 1); ++x) {
                 const unsigned char *rec = record(x);
                 const SubHead &h = *reinterpret_cast<const SubHead *>(rec);
                 // (debug build) a record whose sizes do not fit its slot is not read: as if its wait had run out
@@ -1847,8 +1859,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 const int j = (wt >> 3) & (kLB - 1), q = wt & 7;
                 float acc = 0.0f;
                 if (DENSE) {
-                    if (!waited && !mbar_wait_cluster(updone, par, abort_flag, S.status)) { ok = false; break; }
-                    waited = true;
+                    meet();
                     if (j < h.cnt && wt < kLB * 8) {
                         const float4 *v4 = reinterpret_cast<const float4 *>(val + j * dstride), *w4 = reinterpret_cast<const float4 *>(W);
 #pragma unroll 4
@@ -1896,8 +1907,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                         }
                     };
                     entries();
-                    if (!waited && !mbar_wait_cluster(updone, par, abort_flag, S.status)) { ok = false; break; }
-                    waited = true;
+                    meet();
                     for (;;) { // (whole warps)
 #pragma unroll
                         for (int u = 0; u < 4; ++u) model(u);
@@ -1920,17 +1930,13 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 acc += __shfl_xor_sync(0xffffffffu, acc, 4);
                 if (q == 0 && wt < kLB * 8) st_async_f32(p_buf0 + (slot * (uint32_t)(kMaxC * kLB) + (uint32_t)j) * 4u, acc, p_bar0 + slot * 8u);
             }
-            if (ok && !waited) ok = mbar_wait_cluster(updone, par, abort_flag, S.status);
-            if (!ok) break;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(dotsdone);
+            meet();
             LA_T(wg1);
             sl0 = depth == 1 ? sl2 : sl1;
             sl1 = sl2;
         }
         if (!ok && lane == 0) *abort_flag = 1;
-        aborted = !ok; // (otherwise: every update has been applied and every dot product taken by this warp; the last turn
-                       // waited for the other warps' updates)
+        aborted = !ok; // (otherwise: every update has been applied, the last barrier says so)
 #ifdef CHICLE_LA_TIMING
         if (blockIdx.x == 0 && wt == 0) {
             unsigned long long *d = P.timing + 4;
