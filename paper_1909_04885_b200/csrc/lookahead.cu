@@ -37,6 +37,7 @@
 // A block with more non-zeros than the shared-memory buffers hold is flagged by the prepare kernel: the pipeline
 // drains, warp 0 of CTA 0 walks the block coordinate by coordinate against the whole model, and the pipeline starts
 // again behind it. Rounds that span several local epochs run the pair of kernels once per epoch.
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -56,15 +57,15 @@ constexpr int kDenseEasy = 128;    // and what it takes where the cluster may be
 // or the id itself (never below hotc, see k_lookahead_chain). Problems with more ids take the blocked solver.
 constexpr int kIdBits = 26;
 constexpr uint32_t kIdMask = (1u << kIdBits) - 1u;
-constexpr int kChainThreads = 512;
+constexpr int kChainThreads = 352;
 constexpr int kSubSlots = 4;       // worker records in shared memory: blocks b .. b + 3
 // Recurrence records in shared memory: a record is fetched when the block that many before it is done, and takes 1 500 cycles
 // or more from memory, so two would set the pace (1 M sparse rows: 3 019 cycles a block, with three 2 600). With tables of the logistic step
 // (see tab_map: 32 KB or more each, fetched with the record) a block takes longer and two do.
 constexpr int kMaxHeadSlots = 3;
 __host__ __device__ constexpr int head_slots(bool tables) { return tables ? 2 : 3; }
-// Worker warps: all but the warps that share warp 0's scheduler (warp ids 0, 4, 8, 12), which stay out of its way.
-constexpr int kWorkWarps = 12;
+// Worker warps: warps 1 .. 10 but for those that share warp 0's scheduler (warp ids 0, 4, 8), which stay out of its way.
+constexpr int kWorkWarps = 8;
 constexpr int kWorkThreads = kWorkWarps * 32;
 constexpr int kBarWork = 1;        // named barrier of the worker warps
 constexpr int kRecordWarp = 8;     // fetches the workers' records
@@ -122,6 +123,10 @@ struct alignas(16) BlkDir { // where a record is
     uint32_t bytes;            // a multiple of 16; 0: no record was written
     uint32_t flags;            // bit 0: the block is walked coordinate by coordinate
 };
+
+// Kinds of data the chain kernel is instantiated for: sparse with the whole model in shared memory, with its most frequent
+// ids there, with none; dense rows.
+constexpr int kHot = 0, kCold = 1, kFlat = 2, kDense = 3;
 
 struct LookParams {
     SolverParams S;
@@ -237,6 +242,36 @@ __device__ __forceinline__ float ldcg_if(const float *p, bool on)
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.f32 %0, 0f00000000;\n\t@q ld.global.cg.f32 %0, [%1];\n\t}"
                  : "=f"(v) : "l"(p), "r"((uint32_t)on) : "memory");
     return v;
+}
+// The same from shared memory; ldcg_or gives `other` where it does not load.
+__device__ __forceinline__ float lds_f32_if(uint32_t a, bool on)
+{
+    float v;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.f32 %0, 0f00000000;\n\t@q ld.shared.f32 %0, [%1];\n\t}" : "=f"(v) : "r"(a), "r"((uint32_t)on) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t lds_u32_if(uint32_t a, bool on)
+{
+    uint32_t v;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t@q ld.shared.u32 %0, [%1];\n\t}" : "=r"(v) : "r"(a), "r"((uint32_t)on) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t lds_u16_if(uint32_t a, bool on)
+{
+    uint32_t v;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t@q ld.shared.u16 %0, [%1];\n\t}" : "=r"(v) : "r"(a), "r"((uint32_t)on) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t lds_u8_if(uint32_t a, bool on)
+{
+    uint32_t v;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t@q ld.shared.u8 %0, [%1];\n\t}" : "=r"(v) : "r"(a), "r"((uint32_t)on) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ldcg_or(const float *p, bool on, float other)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q ld.global.cg.f32 %0, [%1];\n\t}" : "+f"(other) : "l"(p), "r"((uint32_t)on) : "memory");
+    return other;
 }
 __device__ __forceinline__ void red_add_if(float *p, float v, bool on)
 {
@@ -437,6 +472,7 @@ template <int NZ, int HT, int THREADS> struct PreShared {
     float sq[kLB], al[kLB], lb[kLB];
     uint16_t rc[kLB + 1][kMaxC];        // where coordinate j's entries start in CTA c's record
     uint32_t cntTL[kMaxC], cntAll;      // per CTA: shared ids (high half) and their list entries (low half); all list entries
+    uint32_t cntLong[kMaxC];            // per CTA: ids with up to four list entries (high half) and with more (low half)
     unsigned long long sub_off[kMaxC];
     int32_t walk;
     unsigned long long pool_at, pool_end; // what this CTA holds of the pool
@@ -684,7 +720,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         }
     for (int p = tid; p < HT; p += THREADS) { sh.key[p] = -1; sh.mask[p] = 0u; }
     for (int p = tid; p < 2 * kLB * kHDS; p += THREADS) (&sh.D[0][0][0])[p] = 0.0f;
-    if (tid < kMaxC) sh.cntTL[tid] = 0u;
+    if (tid < kMaxC) sh.cntTL[tid] = sh.cntLong[tid] = 0u;
     if (tid == 0) { sh.cntAll = 0u; sh.pool_at = sh.pool_end = 0ull; }
     __syncthreads();
     // blocks that are fetched: the run, and the one behind it where the last block has a cross Gram matrix with it
@@ -766,7 +802,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         //      shape that depends on the list's length alone.)
         uint32_t tl[EPT];
         {
-            uint32_t p[EPT], m[EPT], ls[EPT];
+            uint32_t p[EPT], m[EPT], ls[EPT], rk[EPT];
             int32_t id[EPT];
 #pragma unroll
             for (int i = 0; i < EPT; ++i) {
@@ -782,7 +818,9 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 ls[i] = 0u;
                 if (m[i] & (m[i] - 1u)) {
                     const uint32_t pc = (uint32_t)__popc(m[i]);
-                    tl[i] = atomicAdd(&sh.cntTL[id[i] & (C - 1)], (1u << 16) + pc);
+                    tl[i] = atomicAdd(&sh.cntTL[id[i] & (C - 1)], (1u << 16) + pc) & 0xffffu; // where its list starts
+                    rk[i] = atomicAdd(&sh.cntLong[id[i] & (C - 1)], pc > 4u ? 1u : 0x10000u); // its number among the long or the short ones
+                    tl[i] |= (pc > 4u ? rk[i] & 0xffffu : 0x8000u | (rk[i] >> 16)) << 16;
                     ls[i] = atomicAdd(&sh.cntAll, pc);
                 }
             }
@@ -889,8 +927,9 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                     reinterpret_cast<float *>(lists)[at] = x;
                     (lists + 4u * nl_c + 2u * T_c)[at] = (unsigned char)j;
                     if (tl[i] != 0xffffffffu) {
-                        reinterpret_cast<uint32_t *>(rec + 8u * n_c)[tl[i] >> 16] = where | ((uint32_t)(__popc(m) - 1) << kIdBits);
-                        reinterpret_cast<uint16_t *>(lists + 4u * nl_c)[tl[i] >> 16] = (uint16_t)(tl[i] & 0xffffu);
+                        const uint32_t t = tl[i] >> 31 ? (sh.cntLong[cls] & 0xffffu) + ((tl[i] >> 16) & 0x7fffu) : tl[i] >> 16; // long lists first
+                        reinterpret_cast<uint32_t *>(rec + 8u * n_c)[t] = where | ((uint32_t)(__popc(m) - 1) << kIdBits);
+                        reinterpret_cast<uint16_t *>(lists + 4u * nl_c)[t] = (uint16_t)(tl[i] & 0xffffu);
                     }
                 }
             }
@@ -981,7 +1020,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
             reinterpret_cast<int4 *>(sh.key)[p] = make_int4(-1, -1, -1, -1);
             reinterpret_cast<uint4 *>(sh.mask)[p] = make_uint4(0u, 0u, 0u, 0u);
         }
-        if (tid < kMaxC) sh.cntTL[tid] = 0u;
+        if (tid < kMaxC) sh.cntTL[tid] = sh.cntLong[tid] = 0u;
         if (tid == 0) sh.cntAll = 0u;
         __syncthreads();
         PRE_T(7);
@@ -1213,9 +1252,10 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Data and the signal that it has landed travel together: an asynchronous store completes bytes on the receiver's
 // mbarrier, straight from registers.
-__device__ __forceinline__ void st_async_f32(uint32_t remote, float v, uint32_t remote_bar)
+__device__ __forceinline__ void st_async_f32_if(uint32_t remote, float v, uint32_t remote_bar, bool on)
 {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(remote), "f"(v), "r"(remote_bar)
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];\n\t}" ::"r"(remote), "f"(v),
+                 "r"(remote_bar), "r"((uint32_t)on)
                  : "memory");
 }
 __device__ __forceinline__ void st_async_f32x4_if(uint32_t remote, float a, float b, float c, float d, uint32_t remote_bar, bool on)
@@ -1348,9 +1388,10 @@ __host__ __device__ inline ChainLayout chain_layout(int nzcap, int hotc, bool de
     return L;
 }
 
-template <int LOSS, bool DENSE, bool FLAT, bool TAB>
+template <int LOSS, int KIND, bool TAB>
 __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const LookParams P)
 {
+    constexpr bool DENSE = KIND == kDense;
     extern __shared__ __align__(128) unsigned char smem_chain[];
     const SolverParams &S = P.S;
     const int logC = P.logC, C = 1 << logC;
@@ -1413,7 +1454,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
 
     constexpr int HS = head_slots(TAB);
     const bool is_chain = crank == 0 && warp == 0;
-    const bool is_worker = (warp & 3) != 0;
+    const bool is_worker = (warp & 3) != 0; // warps 1 2 3 5 6 7 9 10
     bool aborted = false;
 
     if (is_chain && nb > 0) {
@@ -1693,102 +1734,103 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         // Two barriers per block: in front of its update (no dot product reads the model any more) and behind it. Every
         // warp waits for deltas and records by itself; one whose wait runs out does no more work but goes on meeting the
         // others at the barriers (its abort flag ends their waits too).
+        // What these warps are bound by is the number of instructions they issue, most of them the same in every warp
+        // (addresses, waits, loop ends): hence eight warps and not twelve, 32-bit shared-memory addresses and one instance
+        // of the kernel per kind of data.
         const int wt = (warp - 1 - (warp >> 2)) * 32 + lane; // 0 .. kWorkThreads - 1
         const uint32_t p_bar0 = mapa_u32(smem_u32(&ctl.pbar[0]), 0u);
         const uint32_t p_buf0 = mapa_u32(smem_u32(&ctl.pbuf[0][crank][0]), 0u);
         const uint32_t ack_bar = mapa_u32(smem_u32(&ctl.ackbar), 0u);
-        float *const sink = &ctl.sink[lane];
+        const uint32_t a_w = smem_u32(W), a_sink = smem_u32(&ctl.sink[lane]), stride = L.sub_stride;
+        const uint32_t subs0 = smem_u32(smem_chain + L.subs), subs_end = subs0 + kSubSlots * stride;
         const uint32_t hotc = (uint32_t)P.hotc;
-        const bool cold_ids = FLAT || (int64_t)hot_total < S.dim;  // some ids are not in shared memory
         const int dstride = dense_stride(hot_mine);                // dense: floats per row of a record
         const int depth = P.depth;
-        auto record = [&](int blk) { return smem_chain + L.subs + (size_t)(blk & (kSubSlots - 1)) * L.sub_stride; };
+        const int jd = wt >> 3, qd = wt & 7;                       // dot products: eight threads per coordinate
+        uint32_t r_upd = subs0, r_dot = subs0;                     // records of blocks b and b + depth
         int fg = 0; // staged blocks whose dot products have been sent
         bool ok = true;
 #ifdef CHICLE_LA_TIMING
         long long wd = 0, ws = 0, wg = 0, ws1 = 0, wg0 = 0, wg1 = 0, t0 = clock64(), t1 = 0;
 #endif
-        // The loop starts `depth` blocks early: those turns only take the first blocks' dot products (one place in the
-        // code for every phase keeps the loop small: the warps run at the pace instructions can be fetched).
+        // The loop starts `depth` blocks early: those turns only take the first blocks' dot products.
         bool sl0 = false, sl1 = false; // whether blocks b and b + 1 are walked in place
 #pragma unroll 1
         for (int b = nb > 0 ? -depth : 0; b < nb; ++b) {
-            const uint32_t par = (uint32_t)(b & 1);
             if (b >= 0) {
-                // (a block walked in place by CTA 0: every update before it has been applied here; once no dot product reads
-                // the model any more, say so, and wait for the walk to end)
+                const uint32_t par = (uint32_t)(b & 1), dbar = smem_u32(&ctl.dbar[0]) + 8u * par;
                 if (sl0) {
+                    // (walked in place by CTA 0: every update before it has been applied here; once no dot product reads the
+                    // model any more, say so, and wait for the walk to end)
                     work_bar();
                     if (wt == 0) mbar_arrive_remote_release(ack_bar);
                 }
-                ok = ok && mbar_wait_cluster(smem_u32(&ctl.dbar[par]), (uint32_t)(b >> 1) & 1u, abort_flag, S.status);
+                ok = ok && mbar_wait_cluster(dbar, (uint32_t)(b >> 1) & 1u, abort_flag, S.status);
                 if (sl0) fence_cluster(); // the walk's ordinary stores into this CTA's part of the model
-                mbar_arrive_expect_tx_if(smem_u32(&ctl.dbar[par]), d_bytes, wt == 0 && ok); // for block b + 2
+                mbar_arrive_expect_tx_if(dbar, d_bytes, wt == 0 && ok); // for block b + 2
                 work_bar();
                 LA_T(wd);
                 if (!sl0 && ok) {
                     // ---- block b's update of this CTA's part of the model
-                    const float *dl = ctl.dbuf[par];
-                    const unsigned char *rec = record(b);
-                    const SubHead &h = *reinterpret_cast<const SubHead *>(rec);
-                    const float *val = reinterpret_cast<const float *>(rec + sizeof(SubHead));
+                    const uint32_t dl = smem_u32(&ctl.dbuf[0][0]) + par * (uint32_t)(kLB * 4);
+                    const int4 head = lds_s32x4(r_upd); // n, T, nl, cnt
+                    const uint32_t val = r_upd + (uint32_t)sizeof(SubHead);
                     if (DENSE) {
-                        if (wt < hot_mine) {
+                        for (int col = wt; col < hot_mine; col += kWorkThreads) {
                             float s0 = 0.0f, s1 = 0.0f;
-                            const int cnt = h.cnt;
-                            if (cnt == kLB) { // all loads first
+                            const uint32_t at = val + 4u * (uint32_t)col, row = 4u * (uint32_t)dstride;
+                            if (head.w == kLB) { // all loads first
                                 float x[kLB];
 #pragma unroll
-                                for (int j = 0; j < kLB; ++j) x[j] = val[j * dstride + wt];
+                                for (int j = 0; j < kLB; ++j) x[j] = lds_f32(at + (uint32_t)j * row);
 #pragma unroll
                                 for (int j = 0; j < kLB; j += 4) {
-                                    const float4 d = *reinterpret_cast<const float4 *>(dl + j);
+                                    const float4 d = lds_f32x4(dl + 4u * j);
                                     s0 = fmaf(d.x, x[j], s0);
                                     s1 = fmaf(d.y, x[j + 1], s1);
                                     s0 = fmaf(d.z, x[j + 2], s0);
                                     s1 = fmaf(d.w, x[j + 3], s1);
                                 }
                             } else
-                                for (int j = 0; j < cnt; ++j) s0 = fmaf(dl[j], val[j * dstride + wt], s0);
-                            W[wt] = fmaf(sigma, s0 + s1, W[wt]);
+                                for (int j = 0; j < head.w; ++j) s0 = fmaf(lds_f32(dl + 4u * j), lds_f32(at + (uint32_t)j * row), s0);
+                            W[col] = fmaf(sigma, s0 + s1, W[col]);
                         }
                     } else {
-                        // Eight threads per shared id: each adds every eighth entry of the list (at most four: all loads of a
-                        // thread first), then the partial sums are added in a fixed order.
-                        const int n = h.n, T = h.T, nl = h.nl, q = wt & 7;
-                        const uint32_t *meta = reinterpret_cast<const uint32_t *>(val + n);
-                        const uint32_t *ids = meta + n;
-                        const float *lval = reinterpret_cast<const float *>(ids + T);
-                        const uint16_t *lst = reinterpret_cast<const uint16_t *>(lval + nl);
-                        const unsigned char *lrow = reinterpret_cast<const unsigned char *>(lst + T);
-                        for (int t4 = wt >> 3; t4 < ((T + 3) & ~3); t4 += kWorkThreads / 8) { // (whole warps)
-                            const bool on = t4 < T;
-                            const uint32_t id = on ? ids[t4] : 0u, v = id & kIdMask;
-                            const int len = on ? (int)((id >> kIdBits) & 31u) + 1 : 0, first = (on ? lst[t4] : 0) + q;
-                            const bool more = __any_sync(0xffffffffu, len > 8);
-                            float x[4] = {0.f, 0.f, 0.f, 0.f};
-                            int r[4] = {0, 0, 0, 0};
+                        const int n = head.x, T = head.y, nl = head.z;
+                        const uint32_t meta = val + 4u * (uint32_t)n, ids = meta + 4u * (uint32_t)n, lval = ids + 4u * (uint32_t)T,
+                                       lst = lval + 4u * (uint32_t)nl, lrow = lst + 2u * (uint32_t)T;
+                        // Four threads per shared id: each adds every fourth entry of the list (lists of up to four entries come
+                        // last, so that few warps meet a longer one), then the partial sums are added in a fixed order.
+                        const int q = wt & 3;
+                        for (int t = wt >> 2; (t & ~7) < T; t += kWorkThreads / 4) { // (whole warps)
+                            const bool on = t < T;
+                            const uint32_t id = lds_u32_if(ids + 4u * (uint32_t)t, on), v = id & kIdMask;
+                            const int len = on ? (int)((id >> kIdBits) & 31u) + 1 : 0;
+                            const int first = (int)lds_u16_if(lst + 2u * (uint32_t)t, on) + q;
+                            const uint32_t a_val = lval + 4u * (uint32_t)first, a_row = lrow + (uint32_t)first;
+                            const bool near = KIND == kHot || (KIND == kCold && v < hotc);
+                            const float w = KIND == kFlat ? 0.0f : lds_f32(a_w + (near ? 4u * v : 0u));
+                            float x[8];
+                            uint32_t r[8];
                             auto take = [&](int u) {
-                                if (q + 8 * u < len && CHICLE_IN_BOUNDS(S.status, first + 8 * u < nl)) {
-                                    x[u] = lval[first + 8 * u];
-                                    r[u] = lrow[first + 8 * u] & 31;
-                                }
+                                const bool in = q + 4 * u < len && CHICLE_IN_BOUNDS(S.status, first + 4 * u < nl);
+                                x[u] = lds_f32_if(a_val + 16u * u, in);
+                                r[u] = lds_u8_if(a_row + 4u * u, in);
                             };
                             take(0);
-                            const float w = W[!FLAT && v < hotc ? v : 0u];
-                            if (more) { take(1); take(2); take(3); }
-                            float sum = x[0] * dl[r[0]];
-                            if (more) {
-                                sum = fmaf(x[1], dl[r[1]], sum);
-                                sum = fmaf(x[2], dl[r[2]], sum);
-                                sum = fmaf(x[3], dl[r[3]], sum);
-                            }
+                            float sum;
+                            if (__any_sync(0xffffffffu, len > 4)) {
+#pragma unroll
+                                for (int u = 1; u < 8; ++u) take(u);
+                                sum = x[0] * lds_f32(dl + 4u * (r[0] & 31u));
+#pragma unroll
+                                for (int u = 1; u < 8; ++u) sum = fmaf(x[u], lds_f32(dl + 4u * (r[u] & 31u)), sum);
+                            } else sum = x[0] * lds_f32(dl + 4u * (r[0] & 31u));
                             sum += __shfl_xor_sync(0xffffffffu, sum, 1);
                             sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-                            sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-                            const bool mine = on && q == 0, near = !FLAT && v < hotc;
-                            if (!FLAT) *(mine && near ? W + v : sink) = fmaf(sigma, sum, w);
-                            if (cold_ids) {
+                            const bool mine = on && q == 0;
+                            if (KIND != kFlat) sts_f32(mine && near ? a_w + 4u * v : a_sink, fmaf(sigma, sum, w));
+                            if (KIND != kHot) {
                                 const bool far = mine && !near && sum != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
                                 red_add_if(Uk + (far ? v : 0u), sigma * sum, far);
                             }
@@ -1796,28 +1838,31 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                         // A thread per entry: one whose id no other coordinate of the block has is applied (no two threads
                         // touch the same word). One store per entry, its address chosen without a branch: the model word, or
                         // a word that nobody reads; ids beyond the part in shared memory are added to at L2, nothing waits.
-                        constexpr int U = FLAT ? 4 : 2;
-                        for (int e0 = wt; e0 < n; e0 += U * kWorkThreads) {
+                        constexpr int U = KIND == kFlat ? 4 : 2;
+                        for (int e0 = wt; (e0 & ~31) < n; e0 += U * kWorkThreads) {
                             uint32_t m[U];
                             float p[U], w[U];
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
-                                const int e = e0 + u * kWorkThreads;
-                                m[u] = e < n ? meta[e] : 0x80000000u;
-                                p[u] = e < n ? val[e] : 0.0f;
+                                const bool in = e0 + u * kWorkThreads < n;
+                                const uint32_t at = 4u * (uint32_t)(e0 + u * kWorkThreads);
+                                m[u] = lds_u32_if(meta + at, in);
+                                p[u] = lds_f32_if(val + at, in);
+                                if (!in) m[u] = 0x80000000u;
                             }
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
                                 const uint32_t v = m[u] & kIdMask;
-                                p[u] = sigma * (p[u] * dl[(m[u] >> kIdBits) & 31u]);
-                                if (!FLAT) w[u] = W[v < hotc ? v : 0u];
+                                p[u] = sigma * (p[u] * lds_f32(dl + ((m[u] >> (kIdBits - 2)) & 124u)));
+                                if (KIND == kHot) w[u] = lds_f32(a_w + 4u * (CHICLE_IN_BOUNDS(S.status, v < hotc) ? v : 0u));
+                                if (KIND == kCold) w[u] = lds_f32(a_w + (v < hotc ? 4u * v : 0u));
                             }
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
                                 const uint32_t v = m[u] & kIdMask;
-                                const bool mine = (m[u] >> 31) == 0u, near = !FLAT && v < hotc;
-                                if (!FLAT) *(mine && near ? W + v : sink) = p[u] + w[u];
-                                if (cold_ids) {
+                                const bool mine = (m[u] >> 31) == 0u, near = KIND == kHot ? CHICLE_IN_BOUNDS(S.status, v < hotc) : (KIND == kCold && v < hotc);
+                                if (KIND != kFlat) sts_f32(mine && near ? a_w + 4u * v : a_sink, p[u] + w[u]);
+                                if (KIND != kHot) {
                                     const bool far = mine && !near && p[u] != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
                                     red_add_if(Uk + (far ? v : 0u), p[u], far);
                                 }
@@ -1825,82 +1870,86 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                         }
                     }
                 }
+                r_upd = r_upd + stride == subs_end ? subs0 : r_upd + stride;
                 LA_T(ws1);
             }
             // ---- dot products: of block b + depth against the model as it is now. A block right behind a walked one starts
             //      from the model as the walk left it: with depth 2 its products wait for that.
-            bool sl2 = false;
-            if (b + depth < nb) {
-                ok = ok && mbar_wait_cluster(smem_u32(&ctl.subfull[(b + depth) & (kSubSlots - 1)]), (uint32_t)((b + depth) / kSubSlots) & 1u, abort_flag, S.status);
-                sl2 = ctl.walk[(b + depth) & (kSubSlots - 1)] != 0;
+            bool sl2 = false, due = b + depth < nb, late = false;
+            if (due) {
+                const int slot = (b + depth) & (kSubSlots - 1);
+                ok = ok && mbar_wait_cluster(smem_u32(&ctl.subfull[0]) + 8u * slot, (uint32_t)((b + depth) / kSubSlots) & 1u, abort_flag, S.status);
+                sl2 = lds_s32(smem_u32(&ctl.walk[0]) + 4u * slot) != 0;
+                due = !sl2;
+            }
+            if (sl0 || sl1) {
+                late = depth == 2 && sl0 && !sl1 && b + 1 < nb;
+                due = due && (depth == 1 || !sl1);
             }
             LA_T(wg0);
-            const bool late = depth == 2 && sl0 && !sl1 && b + 1 < nb, due = b + depth < nb && !sl2 && (depth == 1 || !sl1);
             bool met = b < 0; // the barrier behind the update
             auto meet = [&]() {
                 if (!met) work_bar();
-                if (!met && wt == 0) mbar_arrive(smem_u32(&ctl.subfree[b & (kSubSlots - 1)])); // block b's slot is free
+                if (!met && wt == 0) mbar_arrive(smem_u32(&ctl.subfree[0]) + 8u * (b & (kSubSlots - 1))); // block b's slot is free
                 met = true;
             };
 #pragma unroll 1
-            for (int x = late ? b + 1 : b + depth; ok && (late || due) && x <= (due ? b + depth : b + 1); ++x) {
-                const unsigned char *rec = record(x);
-                const SubHead &h = *reinterpret_cast<const SubHead *>(rec);
+            while (ok && (late || due)) {
+                // (block b + 1's record lies in the slot before block b + 2's)
+                const uint32_t rec = !late ? r_dot : (r_dot == subs0 ? subs_end : r_dot) - stride, val = rec + (uint32_t)sizeof(SubHead);
+                if (late) late = false;
+                else due = false;
+                const int4 head = lds_s32x4(rec); // n, T, nl, cnt
                 // (debug build) a record whose sizes do not fit its slot is not read: as if its wait had run out
-                if (!CHICLE_IN_BOUNDS(S.status, h.cnt >= 0 && h.cnt <= kLB && (DENSE || (h.n >= 0 && h.T >= 0 && h.nl >= 0 && h.roff[kLB] == h.n &&
-                                                    sub_bytes((uint32_t)h.n, (uint32_t)h.T, (uint32_t)h.nl) <= L.sub_stride)))) {
+                if (!CHICLE_IN_BOUNDS(S.status, head.w >= 0 && head.w <= kLB && (DENSE || (head.x >= 0 && head.y >= 0 && head.z >= 0 &&
+                                                    sub_bytes((uint32_t)head.x, (uint32_t)head.y, (uint32_t)head.z) <= stride)))) {
                     ok = false;
                     break;
                 }
-                const float *val = reinterpret_cast<const float *>(rec + sizeof(SubHead));
                 const uint32_t slot = (uint32_t)(fg & 1);
                 ++fg;
-                // eight threads per coordinate (the first eight warps)
-                const int j = (wt >> 3) & (kLB - 1), q = wt & 7;
                 float acc = 0.0f;
                 if (DENSE) {
                     meet();
-                    if (j < h.cnt && wt < kLB * 8) {
-                        const float4 *v4 = reinterpret_cast<const float4 *>(val + j * dstride), *w4 = reinterpret_cast<const float4 *>(W);
+                    if (jd < head.w) {
+                        const uint32_t row = val + 4u * (uint32_t)(jd * dstride);
+                        float acc1 = 0.0f;
 #pragma unroll 4
-                        for (int e = q; e < (hot_mine + 3) >> 2; e += 8) {
-                            const float4 a = v4[e], w = w4[e];
-                            acc = fmaf(a.x, w.x, acc); acc = fmaf(a.y, w.y, acc); acc = fmaf(a.z, w.z, acc); acc = fmaf(a.w, w.w, acc);
+                        for (int e = qd; e < (hot_mine + 3) >> 2; e += 8) {
+                            const float4 a = lds_f32x4(row + 16u * e), w = lds_f32x4(a_w + 16u * e);
+                            acc = fmaf(a.x, w.x, acc); acc1 = fmaf(a.y, w.y, acc1); acc = fmaf(a.z, w.z, acc); acc1 = fmaf(a.w, w.w, acc1);
                         }
+                        acc += acc1;
                     }
                 } else {
                     // eight entries per thread and turn, all loads of a turn issued before anything is used: an id beyond the
                     // part of the model in shared memory costs a round trip to L2 (the updates are made there by reductions)
-                    const int hi = wt < kLB * 8 ? h.roff[j + 1] : 0;
-                    const uint32_t *meta = reinterpret_cast<const uint32_t *>(val + h.n);
-                    int e0 = h.roff[j] + q;
-                    float xx[8], ww[8];
-                    uint32_t mm[8];
+                    const uint32_t roff = rec + (uint32_t)offsetof(SubHead, roff) + 2u * (uint32_t)jd;
+                    const int first = (int)lds_u16(roff) + qd;
+                    int left = (int)lds_u16(roff + 2u) - first; // entries of this coordinate from this thread's next one on
+                    uint32_t a_val = val + 4u * (uint32_t)first, a_meta = a_val + 4u * (uint32_t)head.x;
+                    float x[8], w[8];
+                    uint32_t m[8];
                     bool more;
                     auto entry = [&](int u) {
-                        const int e = e0 + 8 * u;
-                        xx[u] = e < hi ? val[e] : 0.0f;
-                        mm[u] = e < hi ? meta[e] & kIdMask : 0u;
+                        x[u] = lds_f32_if(a_val + 32u * u, left > 8 * u);
+                        m[u] = lds_u32_if(a_meta + 32u * u, left > 8 * u) & kIdMask;
                     };
                     auto model = [&](int u) {
-                        if (FLAT) {
-                            const bool in = e0 + 8 * u < hi && CHICLE_IN_BOUNDS(S.status, (int64_t)mm[u] < S.dim);
-                            ww[u] = ldcg_if(Uk + (in ? mm[u] : 0u), in);
-                        } else if (!cold_ids) {
-                            ww[u] = W[CHICLE_IN_BOUNDS(S.status, mm[u] < hotc) ? mm[u] : 0u];
+                        if (KIND == kFlat) {
+                            const bool in = left > 8 * u && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim);
+                            w[u] = ldcg_if(Uk + (in ? m[u] : 0u), in);
+                        } else if (KIND == kHot) {
+                            w[u] = lds_f32(a_w + 4u * (CHICLE_IN_BOUNDS(S.status, m[u] < hotc) ? m[u] : 0u));
                         } else {
-                            const bool cold = mm[u] >= hotc && CHICLE_IN_BOUNDS(S.status, (int64_t)mm[u] < S.dim);
-                            const float far = ldcg_if(Uk + (cold ? mm[u] : 0u), cold);
-                            const float near = W[mm[u] < hotc ? mm[u] : 0u];
-                            ww[u] = cold ? far : near;
+                            const bool cold = m[u] >= hotc && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim);
+                            w[u] = ldcg_or(Uk + (cold ? m[u] : 0u), cold, lds_f32(a_w + (m[u] < hotc ? 4u * m[u] : 0u)));
                         }
                     };
                     auto entries = [&]() {
-                        more = __any_sync(0xffffffffu, e0 + 32 < hi);
+                        more = __any_sync(0xffffffffu, left > 32);
 #pragma unroll
                         for (int u = 0; u < 4; ++u) entry(u);
-#pragma unroll
-                        for (int u = 4; u < 8; ++u) { xx[u] = 0.0f; ww[u] = 0.0f; mm[u] = 0u; }
                         if (more) {
 #pragma unroll
                             for (int u = 4; u < 8; ++u) entry(u);
@@ -1908,6 +1957,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                     };
                     entries();
                     meet();
+#pragma unroll 1
                     for (;;) { // (whole warps)
 #pragma unroll
                         for (int u = 0; u < 4; ++u) model(u);
@@ -1916,21 +1966,24 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                             for (int u = 4; u < 8; ++u) model(u);
                         }
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) acc = fmaf(xx[u], ww[u], acc);
+                        for (int u = 0; u < 4; ++u) acc = fmaf(x[u], w[u], acc);
                         if (!more) break;
 #pragma unroll
-                        for (int u = 4; u < 8; ++u) acc = fmaf(xx[u], ww[u], acc);
-                        e0 += 64;
-                        if (!__any_sync(0xffffffffu, e0 < hi)) break;
+                        for (int u = 4; u < 8; ++u) acc = fmaf(x[u], w[u], acc);
+                        left -= 64;
+                        if (!__any_sync(0xffffffffu, left > 0)) break;
+                        a_val += 256u;
+                        a_meta += 256u;
                         entries();
                     }
                 }
                 acc += __shfl_xor_sync(0xffffffffu, acc, 1);
                 acc += __shfl_xor_sync(0xffffffffu, acc, 2);
                 acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-                if (q == 0 && wt < kLB * 8) st_async_f32(p_buf0 + (slot * (uint32_t)(kMaxC * kLB) + (uint32_t)j) * 4u, acc, p_bar0 + slot * 8u);
+                st_async_f32_if(p_buf0 + (slot * (uint32_t)(kMaxC * kLB) + (uint32_t)jd) * 4u, acc, p_bar0 + slot * 8u, qd == 0);
             }
             meet();
+            r_dot = r_dot + stride == subs_end ? subs0 : r_dot + stride;
             LA_T(wg1);
             sl0 = depth == 1 ? sl2 : sl1;
             sl1 = sl2;
@@ -1969,9 +2022,9 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     cluster_wait();
 }
 
-template <int LOSS, bool DENSE, bool FLAT, bool TAB> cudaError_t launch_chain(Glm &g, const LookParams &P, cudaEvent_t begun)
+template <int LOSS, int KIND, bool TAB> cudaError_t launch_chain_kind(Glm &g, const LookParams &P, cudaEvent_t begun)
 {
-    auto kern = k_lookahead_chain<LOSS, DENSE, FLAT, TAB>;
+    auto kern = k_lookahead_chain<LOSS, KIND, TAB>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.la_smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -2064,14 +2117,18 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
     return e;
 }
 
+template <int LOSS, int KIND, bool TABLES> cudaError_t launch_chain(Glm &g, const LookParams &P, cudaEvent_t begun)
+{
+    return TABLES && P.tab_bins ? launch_chain_kind<LOSS, KIND, TABLES>(g, P, begun) : launch_chain_kind<LOSS, KIND, false>(g, P, begun);
+}
+
 template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P, cudaEvent_t begun = nullptr)
 {
     constexpr bool tables = LOSS == CHICLE_LOSS_LOGISTIC_DUAL;
-    const bool flat = g.la_hotc == 0;
-    if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR)
-        return tables && P.tab_bins ? launch_chain<LOSS, true, false, tables>(g, P, begun) : launch_chain<LOSS, true, false, false>(g, P, begun);
-    if (tables && P.tab_bins) return flat ? launch_chain<LOSS, false, true, tables>(g, P, begun) : launch_chain<LOSS, false, false, tables>(g, P, begun);
-    return flat ? launch_chain<LOSS, false, true, false>(g, P, begun) : launch_chain<LOSS, false, false, false>(g, P, begun);
+    if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) return launch_chain<LOSS, kDense, tables>(g, P, begun);
+    if (g.la_hotc == 0) return launch_chain<LOSS, kFlat, tables>(g, P, begun);
+    if (((int64_t)g.la_hotc << g.la_logC) >= g.dim) return launch_chain<LOSS, kHot, tables>(g, P, begun);
+    return launch_chain<LOSS, kCold, tables>(g, P, begun);
 }
 
 // A round's launches, slice after slice (consecutive pieces of every partition's walk). The first slice's prepare
