@@ -171,7 +171,7 @@ __device__ __forceinline__ int32_t checked_id(const LookParams &P, int32_t id)
 }
 // The same search over a copy of blk_base in shared memory (a launch with at most kBaseStaged - 1 partitions; block
 // counts fit 32 bits): the dependent loads of the search cost 30 cycles each instead of an L2 round trip.
-constexpr int kBaseStaged = 260;
+constexpr int kBaseStaged = 132;
 __device__ __forceinline__ void block_to_part_staged(const int32_t *base, int32_t K, int64_t bid, int &k, int64_t &b)
 {
     int32_t lo = 0, hi = K;
@@ -447,6 +447,7 @@ struct PreBlock {
     int32_t nnz[kLB];
     int32_t roff[kLB + 1];            // where each coordinate's entries start in the flat array ([32] = all of them)
     float gsc[kLB], ys[kLB], as[kLB]; // per coordinate: its Gram scale, and what multiplies / enters from the earlier ones
+    float scl[kLB], inv[kLB];         // a power of two that brings the values below 2^15 (see pre_pairs), and its inverse
     int32_t k, cnt, total, over;      // partition; over: more non-zeros than the arrays hold (total is 0 then): walked in place
 };
 
@@ -458,13 +459,13 @@ template <int NZ, int HT, int THREADS> struct PreShared {
     uint16_t coff[HT];                  // a shared id: start of its list among the lists of its CTA's record
     int32_t idx[2][NZ];                 // the block's entries, and the next block's
     float val[2][NZ];
-    float lval[NZ];                     // the values of shared ids, one list per id, each in ascending coordinate order
+    float lval[NZ];                     // the scaled values of shared ids, one list per id, each in ascending coordinate order
     uint16_t slot[NZ];                  // table slot of each entry's id
-    uint16_t found[NZ];                 // the next block's entries: table slot of the id, 0xffff: this block does not have it
     uint8_t row[2][NZ];                 // coordinate of each entry
     uint32_t bal[2][CH + 1][kMaxC];     // per chunk and CTA: which of the entries fall to it
     uint16_t pre[2][CH + 1][kMaxC];     // and how many before the chunk
-    float G[kLB][kLB + 1];              // scaled Gram entries: the triangle, then the cross Gram matrix
+    int32_t G[2][kLB][kLB];             // Gram triangle and cross Gram matrix, fixed point (the low words lie in idx, see pre_pairs)
+    uint32_t work[THREADS / 32][2 * 32]; // per warp: entries whose pairs are still to be added; then its sums for A and q0n
     alignas(16) float D[2][kLB][kHDS];  // the entries with the kHD most frequent ids, dense
     PreBlock blk[kDirNew];
     int32_t coord[kDirNew][kLB];        // visiting-order entries
@@ -476,7 +477,6 @@ template <int NZ, int HT, int THREADS> struct PreShared {
     unsigned long long sub_off[kMaxC];
     int32_t walk;
     unsigned long long pool_at, pool_end; // what this CTA holds of the pool
-    float q0n[kLB];
     int32_t base[kBaseStaged];          // blk_base, and first step and step count of each partition (see pre_locate)
     int64_t off[kBaseStaged];
     int32_t steps[kBaseStaged];
@@ -562,6 +562,14 @@ template <int LOSS, int NZ, int HT, class Shared> __device__ __forceinline__ voi
     B.gsc[lane] = c >= 0 ? gram_scale<LOSS>(hd, P.S.sigma, P.S.inv_n) : 0.0f;
     B.ys[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 1.0f : hd.p3;
     B.as[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : hd.p1;
+    {
+        // |x| < 2^e for e = (exponent of |x|^2 + 2) / 2, rounded down
+        const uint32_t bits = c >= 0 ? __float_as_uint(sh.sq[lane]) : 0u;
+        const int ex = (int)(bits >> 23) - 127, e = (ex + 2) >> 1;
+        const bool usable = ex > -127 && ex < 128;
+        B.scl[lane] = usable ? __uint_as_float((uint32_t)(127 + 15 - e) << 23) : 0.0f;
+        B.inv[lane] = usable ? __uint_as_float((uint32_t)(127 - 15 + e) << 23) : 0.0f;
+    }
     constexpr int room = NZ < HT - kHD ? NZ : HT - kHD; // entries, and slots for their ids if none is shared
     const int m = n < room + 1 ? n : room + 1; // (more than the arrays hold is all that matters of a longer one)
     int incl = m;
@@ -596,50 +604,17 @@ template <int NZ, int THREADS, class Shared> __device__ __forceinline__ void pre
         }
     }
 }
-// (all warps: which entries of a fetched block fall to which CTA, its dense tile, and, with PROBE, where the table of the
-// current block has their ids)
-template <int NZ, int HT, int THREADS, class Shared>
-__device__ __forceinline__ void pre_scan(const LookParams &P, Shared &sh, int total, int buf, bool probe)
+// (a warp: which of 32 consecutive entries fall to which CTA, and their part of the dense tile; id < 0: no entry)
+template <class Shared> __device__ __forceinline__ void pre_classify(const LookParams &P, Shared &sh, int32_t id, int e, int buf)
 {
-    constexpr int EPT = NZ / THREADS;
     const int lane = threadIdx.x & 31;
-    int32_t id[EPT], seen[EPT];
-    uint32_t p[EPT];
-#pragma unroll
-    for (int i = 0; i < EPT; ++i) {
-        const int e = (int)threadIdx.x + i * THREADS;
-        id[i] = e < total ? checked_id(P, sh.idx[buf][e]) : -1;
-        p[i] = id[i] >= kHD ? home_slot<HT>(id[i]) : 0u;
+    uint32_t mine = __ballot_sync(0xffffffffu, id >= 0);
+    for (int bit = 0; bit < P.logC; ++bit) {
+        const uint32_t b = __ballot_sync(0xffffffffu, (id >> bit) & 1);
+        mine &= (lane >> bit) & 1 ? b : ~b;
     }
-    if (probe) {
-#pragma unroll
-        for (int i = 0; i < EPT; ++i) seen[i] = sh.key[p[i]];
-    }
-#pragma unroll
-    for (int i = 0; i < EPT; ++i) {
-        const int e = (int)threadIdx.x + i * THREADS;
-        if ((e & ~31) >= total) break; // (whole warps)
-        uint32_t mine = __ballot_sync(0xffffffffu, id[i] >= 0);
-        for (int bit = 0; bit < P.logC; ++bit) {
-            const uint32_t b = __ballot_sync(0xffffffffu, (id[i] >> bit) & 1);
-            mine &= (lane >> bit) & 1 ? b : ~b;
-        }
-        if (lane >> P.logC == 0) sh.bal[buf][e >> 5][lane] = mine; // lane c: the entries of CTA c
-        if (id[i] >= 0 && id[i] < kHD) sh.D[buf][sh.row[buf][e]][id[i]] = sh.val[buf][e];
-    }
-    if (probe) {
-#pragma unroll
-        for (int i = 0; i < EPT; ++i) {
-            const int e = (int)threadIdx.x + i * THREADS;
-            if (e >= total) break;
-            if (id[i] >= kHD)
-                for (int t = 0; t < HT && seen[i] != id[i] && seen[i] != -1; ++t) {
-                    p[i] = next_slot<HT>(p[i]);
-                    seen[i] = sh.key[p[i]];
-                }
-            sh.found[e] = id[i] >= kHD && seen[i] == id[i] ? (uint16_t)p[i] : (uint16_t)0xffffu;
-        }
-    }
+    if (lane >> P.logC == 0) sh.bal[buf][e >> 5][lane] = mine; // lane c: the entries of CTA c
+    if (id >= 0 && id < kHD) sh.D[buf][sh.row[buf][e]][id] = sh.val[buf][e];
 }
 // (warp c: how many of the entries before each chunk fall to CTA c)
 template <class Shared> __device__ __forceinline__ void pre_prefix(Shared &sh, int total, int buf, int c)
@@ -661,39 +636,58 @@ template <class Shared> __device__ __forceinline__ void pre_prefix(Shared &sh, i
     }
 }
 
-// Dot product of a coordinate's dense part (row j of `a`) with lane's row of `m`.
-__device__ __forceinline__ float pre_dense_dot(const float *a, const float *m)
+// The Gram matrices' entries come from two sources. The kHD most frequent ids: dense 32 x kHD tiles (pre_rows). All others:
+// an id that c coordinates have contributes c (c - 1) / 2 products, about 550 per block inside a block of 1 600 entries and
+// 1 300 to the cross Gram matrix: they are added one by one with shared-memory atomics, in fixed point, so that the sum
+// does not depend on the order. Values are scaled by a power of two below 2^15 / |x| (exact), a product is below 2^30 and
+// so is every partial sum of an entry (|sum| <= |x_l| |x_j|); what rounding a product to a whole number leaves goes to a second
+// word, 2^20 times finer: together finer than an fp32 sum is.
+// (Walking lists with shuffles in a fixed order took 14 000 of 31 000 cycles a block.)
+template <int NZ, class Shared>
+__device__ __forceinline__ void pre_pairs(Shared &sh, uint32_t item, bool on, int cur, const PreBlock &N)
 {
-    float acc = 0.0f;
-    const float4 *dj = reinterpret_cast<const float4 *>(a), *dm = reinterpret_cast<const float4 *>(m);
-#pragma unroll
-    for (int h = 0; h < kHD / 4; ++h) {
-        const float4 x = dj[h], y = dm[h];
-        acc = fmaf(x.x, y.x, acc); acc = fmaf(x.y, y.y, acc); acc = fmaf(x.z, y.z, acc); acc = fmaf(x.w, y.w, acc);
+    const int e = (int)(item & 4095u), p = (int)((item >> 12) & 4095u), next = (int)(item >> 24);
+    uint32_t m = 0u;
+    uint32_t at = 0u;
+    float x = 0.0f;
+    int col = 0;
+    if (on) {
+        const int buf = cur ^ next, j = sh.row[buf][e], so = sh.soff[p];
+        m = sh.mask[p];
+        x = sh.val[buf][e];
+        if (next) x *= N.scl[j];
+        else m &= (1u << j) - 1u;
+        at = so < NZ ? smem_u32(&sh.val[cur][so]) : smem_u32(&sh.lval[so - NZ]);
+        col = next * kLB * kLB + j;
     }
-    return acc;
+    int32_t *hi = &sh.G[0][0][0] + col, *lo = &sh.idx[cur][0] + col;
+    while (m) {
+        const int l = (__ffs((int)m) - 1) * kLB;
+        m &= m - 1u;
+        const float v = lds_f32(at) * x;
+        at += 4u;
+        const int h = __float2int_rn(v), r = __float2int_rn((v - (float)h) * 1048576.0f);
+        atomicAdd(hi + l, h);
+        if (r) atomicAdd(lo + l, r);
+    }
 }
-// Adds what the entries marked in `todo` (lanes of this chunk) contribute: mask, list address and value handed round by
-// shuffles, four entries per turn, so that their loads are under way together (the additions stay in ascending order).
-__device__ __forceinline__ void pre_add_listed(uint32_t todo, uint32_t m_l, uint32_t at_l, float x_l, float &acc)
+
+// What the states at round start contribute: the warps' sums (sh.work) together, off A and into q0n; the block's constants
+// go out. (A warp; one block behind the loop, so that it needs no barrier of its own.)
+template <int NW, class Shared> __device__ __forceinline__ void pre_finish_head(const LookParams &P, Shared &sh, int64_t bid)
 {
-    const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
-    while (todo) {
-        float v[4], x[4];
+    const int lane = threadIdx.x & 31;
+    ChainHead &out = *reinterpret_cast<ChainHead *>(P.rec + (size_t)bid * sizeof(ChainHead));
+    float qg = 0.0f, qx = 0.0f;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const bool any = todo != 0u;
-            const int src = any ? __ffs(todo) - 1 : 0;
-            todo &= todo - 1u; // (0 stays 0)
-            const uint32_t m = __shfl_sync(0xffffffffu, m_l, src), at = __shfl_sync(0xffffffffu, at_l, src);
-            x[u] = __shfl_sync(0xffffffffu, x_l, src);
-            const bool on = any && ((m >> lane) & 1u);
-            v[u] = 0.0f;
-            if (on) v[u] = lds_f32(at + 4u * (uint32_t)__popc(m & lt));
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc = fmaf(x[u], v[u], acc);
+    for (int w = 0; w < NW; ++w) {
+        qg += __uint_as_float(sh.work[w][lane]);
+        qx += __uint_as_float(sh.work[w][32 + lane]);
     }
+    CHdr hd = sh.blk[bid & (kDirNew - 1)].hdr[lane];
+    hd.A -= qg;
+    out.hdr[lane] = hd;
+    out.q0n[lane] = qx;
 }
 
 template <int LOSS, int NZ, int HT, int THREADS, int PER_SM>
@@ -741,7 +735,8 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
     pre_fetch_rows<NZ, THREADS>(P, sh, lo, (int)(lo & 1));
     cp_async_wait_all();
     __syncthreads();
-    pre_scan<NZ, HT, THREADS>(P, sh, sh.blk[lo & (kDirNew - 1)].total, (int)(lo & 1), false);
+    for (int e = tid; (e & ~31) < sh.blk[lo & (kDirNew - 1)].total; e += THREADS)
+        pre_classify(P, sh, e < sh.blk[lo & (kDirNew - 1)].total ? checked_id(P, sh.idx[lo & 1][e]) : -1, e, (int)(lo & 1));
     __syncthreads();
     if (warp < C) pre_prefix(sh, sh.blk[lo & (kDirNew - 1)].total, (int)(lo & 1), warp);
     __syncthreads();
@@ -765,6 +760,8 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         if (warp == NW - 1 && bid + 2 < end) pre_fetch_extents<LOSS>(P, sh, bid + 2);
         if (warp == NW - 2 && bid + 3 < end) pre_fetch_order(P, sh, bid + 3);
         for (int p = tid; p < kLB * kHDS; p += THREADS) (&sh.D[nxt][0][0])[p] = 0.0f;
+        for (int p = tid; p < 2 * kLB * kLB; p += THREADS) (&sh.G[0][0][0])[p] = 0;
+        if (warp == NW - 4 && bid > lo) pre_finish_head<NW>(P, sh, bid - 1);
         // ---- every id into the table
         {
             int32_t id[EPT], seen[EPT];
@@ -907,21 +904,23 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
 #pragma unroll
             for (int i = 0; i < EPT; ++i) {
                 const int e = tid + i * THREADS;
-                if (e >= total) break;
-                const int32_t id = checked_id(P, sh.idx[cur][e]);
+                const int32_t id = e < total ? checked_id(P, sh.idx[cur][e]) : 0;
+                sh.idx[cur][e] = 0; // (from here on: the low words of the Gram matrices)
+                if (e >= total) continue;
                 const int cls = id & (C - 1), j = sh.row[cur][e], p = sh.slot[e];
                 const int place = sh.pre[cur][e >> 5][cls] + __popc(sh.bal[cur][e >> 5][cls] & ((1u << lane) - 1u));
                 const uint32_t m = sh.mask[p];
                 const bool shared_id = (m & (m - 1u)) != 0u;
                 const int lower = __popc(m & ((1u << j) - 1u));
-                const float x = sh.val[cur][e];
+                const float x = sh.val[cur][e], scaled = x * B.scl[j];
+                sh.val[cur][e] = scaled; // (the records have the value itself)
                 unsigned char *rec = P.rec + sh.sub_off[cls] + sizeof(SubHead);
                 const uint32_t n_c = sh.rc[kLB][cls], T_c = sh.cntTL[cls] >> 16, nl_c = sh.cntTL[cls] & 0xffffu;
                 const uint32_t where = (uint32_t)id < hot_total ? (uint32_t)id >> P.logC : (uint32_t)id;
                 reinterpret_cast<float *>(rec)[place] = x;
                 reinterpret_cast<uint32_t *>(rec + 4u * n_c)[place] = where | ((uint32_t)j << kIdBits) | (shared_id ? 0x80000000u : 0u);
                 if (shared_id) {
-                    sh.lval[sh.soff[p] - NZ + lower] = x;
+                    sh.lval[sh.soff[p] - NZ + lower] = scaled;
                     const uint32_t at = sh.coff[p] + lower;
                     unsigned char *lists = rec + 8u * n_c + 4u * T_c;
                     reinterpret_cast<float *>(lists)[at] = x;
@@ -934,88 +933,101 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 }
             }
         }
-        __syncthreads();
-        PRE_T(3);
-        // ---- Gram triangle: a warp per coordinate j, lane l collects x_j . x_l over j's entries in ascending order. The
-        //      lanes first look at 32 entries at once and keep those whose id an earlier coordinate has too; only these
-        //      are then walked.
-        if (!walk)
-            for (int j = warp; j < kLB; j += NW) {
-                float acc = 0.0f;
-                const int n = B.nnz[j], r0 = B.roff[j];
-                if (n) {
-                    const uint32_t below = (1u << j) - 1u;
-                    acc = pre_dense_dot(&sh.D[cur][j][0], &sh.D[cur][lane][0]);
-                    for (int e0 = 0; e0 < n; e0 += 32) {
-                        uint32_t m_l = 0u, at_l = 0u;
-                        float x_l = 0.0f;
-                        if (e0 + lane < n) {
-                            const int p = sh.slot[r0 + e0 + lane];
-                            if (p >= kHD) { // (the dense tile has the others)
-                                m_l = sh.mask[p];
-                                at_l = smem_u32(&sh.lval[0]) + 4u * (uint32_t)(sh.soff[p] - NZ);
-                                x_l = sh.val[cur][r0 + e0 + lane];
-                            }
-                        }
-                        pre_add_listed(__ballot_sync(0xffffffffu, (m_l & below) != 0u), m_l, at_l, x_l, acc);
-                    }
-                    if (lane >= j) acc = 0.0f;
-                }
-                acc *= B.gsc[j] * B.ys[lane];
-                sh.G[lane][j] = acc; // row l, column j
-                float q0 = acc * B.as[lane];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) q0 += __shfl_xor_sync(0xffffffffu, q0, o);
-                if (lane == 0) B.hdr[j].A -= q0;
-            }
         cp_async_wait_all(); // the next block's rows, the extents after it, the order after that
         __syncthreads();
-        PRE_T(4);
-        // ---- the head's Gram triangle and constants; the next block's entries looked up in this block's table
-        if (!walk)
-            for (int i = tid; i < kLB * kLB; i += THREADS) out.G[i] = sh.G[i >> 5][i & 31];
-        if (warp == 0) out.hdr[lane] = B.hdr[lane];
+        PRE_T(3);
+        // ---- the next block's entries: which CTA's they are, their dense tile, and (table of this block) which of this
+        //      block's coordinates have their ids; the pairs of both Gram matrices, 32 entries with some at a time
         if (warp == NW - 1 && bid + 2 < end) pre_make_block<LOSS, NZ, HT>(P, sh, bid + 2);
-        if (have_next) pre_scan<NZ, HT, THREADS>(P, sh, N.total, nxt, carry);
-        __syncthreads();
-        PRE_T(5);
-        // ---- cross Gram matrix: a warp per coordinate j of the next block; lane l collects x_j . x_l
-        if (have_next && warp < C) pre_prefix(sh, N.total, nxt, warp);
-        if (carry)
-            for (int j = warp; j < kLB; j += NW) {
-                float acc = 0.0f;
-                const int n = N.nnz[j], r0 = N.roff[j];
-                if (n) {
-                    acc = pre_dense_dot(&sh.D[nxt][j][0], &sh.D[cur][lane][0]);
-                    for (int e0 = 0; e0 < n; e0 += 32) {
-                        uint32_t m_l = 0u, at_l = 0u;
-                        float x_l = 0.0f;
-                        if (e0 + lane < n) {
-                            const int p = sh.found[r0 + e0 + lane];
-                            if (p != 0xffff) {
-                                m_l = sh.mask[p];
-                                const int so = sh.soff[p];
-                                at_l = so < NZ ? smem_u32(&sh.val[cur][so]) : smem_u32(&sh.lval[so - NZ]);
-                                x_l = sh.val[nxt][r0 + e0 + lane];
-                            }
-                        }
-                        pre_add_listed(__ballot_sync(0xffffffffu, m_l != 0u), m_l, at_l, x_l, acc);
-                    }
-                    if (lane >= cnt) acc = 0.0f;
+        {
+            uint32_t *todo = sh.work[warp];
+            int have = 0;
+            auto push = [&](bool on, uint32_t item) {
+                const uint32_t b = __ballot_sync(0xffffffffu, on);
+                if (on) todo[have + __popc(b & ((1u << lane) - 1u))] = item;
+                have += __popc(b);
+                __syncwarp();
+                if (have >= 32) {
+                    have -= 32;
+                    const uint32_t mine = todo[have + lane];
+                    __syncwarp();
+                    pre_pairs<NZ>(sh, mine, true, cur, N);
                 }
-                acc *= N.gsc[j] * B.ys[lane];
-                sh.G[lane][j] = acc; // row l (this block), column j (next block)
-                float q0 = acc * B.as[lane];
+            };
+            const int ntotal = have_next ? N.total : 0;
+            int32_t id[EPT], seen[EPT];
+            uint32_t p[EPT];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) q0 += __shfl_xor_sync(0xffffffffu, q0, o);
-                if (lane == 0) sh.q0n[j] = q0;
+            for (int i = 0; i < EPT; ++i) {
+                const int e = tid + i * THREADS;
+                id[i] = e < ntotal ? checked_id(P, sh.idx[nxt][e]) : -1;
+                p[i] = id[i] >= kHD ? home_slot<HT>(id[i]) : 0u;
             }
+#pragma unroll
+            for (int i = 0; i < EPT; ++i) seen[i] = carry ? sh.key[p[i]] : -1;
+            if (!walk) {
+#pragma unroll 1
+                for (int e = tid; (e & ~31) < total; e += THREADS) {
+                    const uint32_t s = e < total ? sh.slot[e] : 0u;
+                    push(s >= (uint32_t)kHD && (sh.mask[s] & ((1u << sh.row[cur][e]) - 1u)) != 0u, (uint32_t)e | s << 12);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < EPT; ++i) {
+                const int e = tid + i * THREADS;
+                if ((e & ~31) >= ntotal) break; // (whole warps)
+                pre_classify(P, sh, id[i], e, nxt);
+                if (!carry) continue;
+                if (id[i] >= kHD)
+                    for (int t = 0; t < HT && seen[i] != id[i] && seen[i] != -1; ++t) {
+                        p[i] = next_slot<HT>(p[i]);
+                        seen[i] = sh.key[p[i]];
+                    }
+                push(id[i] >= kHD && seen[i] == id[i], (uint32_t)e | p[i] << 12 | 1u << 24);
+            }
+            const uint32_t mine = lane < have ? todo[lane] : 0u;
+            __syncwarp();
+            if (have) pre_pairs<NZ>(sh, mine, lane < have, cur, N);
+        }
         __syncthreads();
-        PRE_T(6);
-        // (a next block that is walked in place takes nothing over: the recurrence warp drops it)
-        const bool keep = carry;
-        for (int i = tid; i < kLB * kLB; i += THREADS) out.X[i] = keep ? sh.G[i >> 5][i & 31] : 0.0f;
-        if (tid < kLB) out.q0n[tid] = keep ? sh.q0n[tid] : 0.0f;
+        PRE_T(4);
+        // ---- rows l = warp, warp + NW of both matrices, lane = column: the dense part, both together, scaled
+        if (have_next && warp < C) pre_prefix(sh, N.total, nxt, warp);
+        {
+            constexpr int R = kLB / NW;
+            float g[R], x[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) g[r] = x[r] = 0.0f;
+            const float4 *dj = reinterpret_cast<const float4 *>(&sh.D[cur][lane][0]), *nj = reinterpret_cast<const float4 *>(&sh.D[nxt][lane][0]);
+#pragma unroll
+            for (int h = 0; h < kHD / 4; ++h) {
+                const float4 a = dj[h], b = nj[h];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float4 c = *reinterpret_cast<const float4 *>(&sh.D[cur][warp + r * NW][4 * h]);
+                    g[r] = fmaf(a.x, c.x, g[r]); g[r] = fmaf(a.y, c.y, g[r]); g[r] = fmaf(a.z, c.z, g[r]); g[r] = fmaf(a.w, c.w, g[r]);
+                    x[r] = fmaf(b.x, c.x, x[r]); x[r] = fmaf(b.y, c.y, x[r]); x[r] = fmaf(b.z, c.z, x[r]); x[r] = fmaf(b.w, c.w, x[r]);
+                }
+            }
+            float qg = 0.0f, qx = 0.0f;
+            const float gsc = B.gsc[lane], inv = B.inv[lane], ngsc = carry ? N.gsc[lane] : 0.0f, ninv = carry ? N.inv[lane] : 0.0f;
+            const int32_t *low = &sh.idx[cur][0];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int l = warp + r * NW;
+                const float il = B.inv[l], yl = B.ys[l], al = B.as[l];
+                float v = fmaf(fmaf((float)low[l * kLB + lane], 1.0f / 1048576.0f, (float)sh.G[0][l][lane]), il * inv, g[r]) * (gsc * yl);
+                v = lane > l && !walk ? v : 0.0f;
+                out.G[l * kLB + lane] = v;
+                qg = fmaf(v, al, qg);
+                v = fmaf(fmaf((float)low[kLB * kLB + l * kLB + lane], 1.0f / 1048576.0f, (float)sh.G[1][l][lane]), il * ninv, x[r]) * (ngsc * yl);
+                v = l < cnt && carry ? v : 0.0f;
+                out.X[l * kLB + lane] = v;
+                qx = fmaf(v, al, qx);
+            }
+            sh.work[warp][lane] = __float_as_uint(qg);
+            sh.work[warp][32 + lane] = __float_as_uint(qx);
+        }
         for (int p = tid; p < HT / 4; p += THREADS) {
             reinterpret_cast<int4 *>(sh.key)[p] = make_int4(-1, -1, -1, -1);
             reinterpret_cast<uint4 *>(sh.mask)[p] = make_uint4(0u, 0u, 0u, 0u);
@@ -1023,8 +1035,9 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         if (tid < kMaxC) sh.cntTL[tid] = sh.cntLong[tid] = 0u;
         if (tid == 0) sh.cntAll = 0u;
         __syncthreads();
-        PRE_T(7);
+        PRE_T(5);
     }
+    if (warp == 0) pre_finish_head<NW>(P, sh, hi - 1);
 }
 
 // Short dense rows: every row has every id, so the lists are implicit: constants, Gram triangle, cross Gram matrix
@@ -2111,7 +2124,7 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
         (void)cudaMemcpy(t, P.timing + 16, sizeof(t), cudaMemcpyDeviceToHost);
         (void)cudaMemset(P.timing + 16, 0, sizeof(t));
         const double n = (double)nb;
-        fprintf(stderr, "lookahead prepare, cycles per block: insert %.0f, number %.0f, place %.0f, entries %.0f, gram %.0f, scan %.0f, cross %.0f, write %.0f\n", t[0] / n, t[1] / n, t[2] / n, t[3] / n, t[4] / n, t[5] / n, t[6] / n, t[7] / n);
+        fprintf(stderr, "lookahead prepare, cycles per block: insert %.0f, number %.0f, place %.0f, entries %.0f, scan and pairs %.0f, dense and write %.0f\n", t[0] / n, t[1] / n, t[2] / n, t[3] / n, t[4] / n, t[5] / n, t[6] / n, t[7] / n);
     }
 #endif
     return e;
