@@ -1,5 +1,6 @@
 // Host side of the C ABI declared in chicle.h: argument checks, the state machine, memory, and the order in
 // which the kernels of a round are enqueued. No arithmetic of the method happens here.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -287,15 +288,15 @@ chicle_status_t chicle_glm_create(const chicle_matrix_t *X, const float *labels,
                    alloc_into(h, keys[0], (size_t)dim) && alloc_into(h, keys[1], (size_t)dim) &&
                    alloc_into(h, vals[0], (size_t)dim) && alloc_into(h, vals[1], (size_t)dim) &&
                    alloc_into(h, hist, sort_hist_entries(dim)) && alloc_into(h, sums, sort_scan_tiles(dim) + 1) &&
-                   alloc_into(h, mass, 4);
+                   alloc_into(h, mass, (size_t)kMassWords);
         if (ok2 && ridge) ok2 = alloc_into(h, labels_new, (size_t)dim);
         if (!ok2) return bail(CHICLE_ERR_OOM, "device allocation failed (id ranking)");
         e = cudaMemsetAsync(counts, 0, (size_t)dim * 4, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(mass, 0, 32, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(mass, 0, kMassWords * 8, s);
         if (e == cudaSuccess) e = launch_frequency_remap(*h, counts, keys, vals, hist, sums, blocked_solver_hot_ids(), blocked_solver_short_cap(), mass);
         if (e == cudaSuccess && ridge) e = launch_gather_f32(*h, h->labels, h->old_of_new, dim, labels_new);
-        unsigned long long host_mass2[2] = {0, 0};
-        if (e == cudaSuccess) e = cudaMemcpyAsync(host_mass2, mass, 16, cudaMemcpyDeviceToHost, s);
+        unsigned long long host_mass2[kMassWords] = {};
+        if (e == cudaSuccess) e = cudaMemcpyAsync(host_mass2, mass, sizeof(host_mass2), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return bail_cuda(e, "id ranking kernels");
         if (ridge) {
@@ -307,7 +308,15 @@ chicle_status_t chicle_glm_create(const chicle_matrix_t *X, const float *labels,
         h->hot_variant = h->nnz > 0 && (double)host_mass2[0] >= 0.5 * (double)h->nnz ? 1 : 0;
         // more than 1 % of the coordinates would not fit the short staging rows: take the variant with longer rows
         if (h->hot_variant && (double)host_mass2[1] > 0.01 * (double)h->n_coord) h->hot_variant = 2;
+        const double n = (double)h->n_coord, mean = (double)h->nnz / n;
+        h->row_variance = std::max(0.0, (double)host_mass2[2] / n - mean * mean);
+        for (int i = 0; i < kRankClasses; ++i) {
+            h->blk_entries[i] = 32.0 * (double)host_mass2[4 + i] / n;
+            h->blk_shared_ids[i] = (double)host_mass2[4 + kRankClasses + i] / 1048576.0;
+            h->blk_shared[i] = (double)host_mass2[4 + 2 * kRankClasses + i] / 1048576.0;
+        }
         const char *force = getenv("CHICLE_FORCE_VARIANT"); // debugging aid
+        h->flat_ids = force && strcmp(force, "flat") == 0;
         if (force && strcmp(force, "flat") == 0) h->hot_variant = 0;
         if (force && strcmp(force, "hot") == 0) h->hot_variant = 1;
         if (force && strcmp(force, "hot128") == 0) h->hot_variant = 2;

@@ -71,6 +71,10 @@ cudaError_t radix_pass(const uint64_t *keys_in, const int32_t *vals_in, uint64_t
 
 struct SolverParams;
 
+// What the ranking of the ids finds out about the data (see launch_frequency_remap).
+constexpr int kRankClasses = 8; // ids mod 8: a CTA of the largest cluster takes one class
+constexpr int kMassWords = 4 + 3 * kRankClasses;
+
 // ---- handle -------------------------------------------------------------------------------------------------
 struct Glm {
     int device = 0;
@@ -100,6 +104,11 @@ struct Glm {
     float *perm_tmp = nullptr;     // dim, staging for translating v at the boundary
     int hot_variant = 0;           // 1 / 2: most non-zeros fall on the first ids, the solver keeps those in a direct
                                    // array (2: with room for coordinates of up to 128 entries); 0: flat ids
+    bool flat_ids = false;         // (tests) no part of the model in shared memory
+    // what a block of 32 random coordinates is expected to have on the ids of each class (id mod kRankClasses): entries, ids
+    // that several of the 32 have, entries with such an id; and the variance of a coordinate's number of entries
+    double blk_entries[kRankClasses] = {}, blk_shared_ids[kRankClasses] = {}, blk_shared[kRankClasses] = {};
+    double row_variance = 0.0;
 
     // partition
     int32_t K = 0;
@@ -129,7 +138,9 @@ struct Glm {
     int la_logC = 0;                 // log2 of the CTAs per partition (thread-block cluster)
     int la_depth = 2;                // blocks the dot products are taken ahead of the recurrence (2: with cross Gram matrices)
     bool la_overlap = true;          // prepare kernels beside the chain kernels (side stream) or alternating with them
-    int32_t la_nzcap = 0, la_hotc = 0; // non-zeros per worker record; entry ids per CTA kept in shared memory
+    uint32_t la_sub_room = 0;        // bytes of a worker record's slot in shared memory
+    int la_slots = 4;                // and how many slots
+    int32_t la_hotc = 0;             // entry ids per CTA kept in shared memory
     int32_t la_tab_bins = 0;         // logistic: bins per coordinate of the step's tables (0: none)
     size_t la_tab_off = 0;           // where they lie in a region
     size_t la_smem = 0;              // dynamic shared memory of the chain kernel

@@ -37,6 +37,7 @@
 // A block with more non-zeros than the shared-memory buffers hold is flagged by the prepare kernel: the pipeline
 // drains, warp 0 of CTA 0 walks the block coordinate by coordinate against the whole model, and the pipeline starts
 // again behind it. Rounds that span several local epochs run the pair of kernels once per epoch.
+#include <cmath>
 #include <cstddef>
 #include <cstdio>
 #include <cstdlib>
@@ -58,7 +59,7 @@ constexpr int kDenseEasy = 128;    // and what it takes where the cluster may be
 constexpr int kIdBits = 26;
 constexpr uint32_t kIdMask = (1u << kIdBits) - 1u;
 constexpr int kChainThreads = 352;
-constexpr int kSubSlots = 4;       // worker records in shared memory: blocks b .. b + 3
+constexpr int kSubSlots = 4;       // worker records in shared memory: blocks b .. b + 3 (three of them where long records leave no room, see lookahead_plan)
 // Recurrence records in shared memory: a record is fetched when the block that many before it is done, and takes 1 500 cycles
 // or more from memory, so two would set the pace (1 M sparse rows: 3 019 cycles a block, with three 2 600). With tables of the logistic step
 // (see tab_map: 32 KB or more each, fetched with the record) a block takes longer and two do.
@@ -114,9 +115,6 @@ __host__ __device__ constexpr uint32_t sub_bytes(uint32_t n, uint32_t T, uint32_
 // Dense rows in a record: 16-byte pieces of consecutive rows lie on different banks.
 __host__ __device__ constexpr int dense_stride(int cols) { return (((cols + 3) / 4) | 1) * 4; }
 __host__ __device__ constexpr uint32_t sub_bytes_dense(int cnt, int cols) { return ((uint32_t)sizeof(SubHead) + 4u * (uint32_t)(cnt * dense_stride(cols)) + 15u) & ~15u; }
-// A record's slot in shared memory: room for nzcap entries of which half are shared (a block that needs more is walked in
-// place).
-__host__ __device__ constexpr uint32_t sub_room(int nzcap) { return sub_bytes((uint32_t)nzcap, (uint32_t)nzcap / 4u, (uint32_t)nzcap / 2u); }
 
 struct alignas(16) BlkDir { // where a record is
     unsigned long long offset; // bytes from the start of the launch's region of the record buffer (a multiple of 16)
@@ -142,7 +140,8 @@ struct LookParams {
     int32_t K, logC;
     int32_t depth;               // 2: a block's dot products are taken two blocks ahead and corrected with the cross
                                  // Gram matrix; 1: one block ahead, no cross Gram matrix (the recurrence waits for them)
-    int32_t nzcap;               // non-zeros a worker record holds at most
+    uint32_t sub_room;           // bytes of a worker record's slot in shared memory (sparse; a block that needs more is walked in place)
+    int32_t slots;               // and how many slots there are (at least depth + 2)
     int32_t hotc;                // entry ids per CTA kept in shared memory
     int64_t n_blocks;
     int64_t drop_block;          // test aid: this block's records are left unpublished (-1: none)
@@ -243,7 +242,7 @@ __device__ __forceinline__ float ldcg_if(const float *p, bool on)
                  : "=f"(v) : "l"(p), "r"((uint32_t)on) : "memory");
     return v;
 }
-// The same from shared memory; ldcg_or gives `other` where it does not load.
+// The same from shared memory.
 __device__ __forceinline__ float lds_f32_if(uint32_t a, bool on)
 {
     float v;
@@ -267,11 +266,6 @@ __device__ __forceinline__ uint32_t lds_u8_if(uint32_t a, bool on)
     uint32_t v;
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t@q ld.shared.u8 %0, [%1];\n\t}" : "=r"(v) : "r"(a), "r"((uint32_t)on) : "memory");
     return v;
-}
-__device__ __forceinline__ float ldcg_or(const float *p, bool on, float other)
-{
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q ld.global.cg.f32 %0, [%1];\n\t}" : "+f"(other) : "l"(p), "r"((uint32_t)on) : "memory");
-    return other;
 }
 __device__ __forceinline__ void red_add_if(float *p, float v, bool on)
 {
@@ -854,7 +848,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
             }
             const uint32_t need = __shfl_sync(0xffffffffu, incl, kMaxC - 1);
             // 1: longer than the arrays, or more falls to one CTA than its record holds
-            int sl = B.over || __any_sync(0xffffffffu, len > sub_room(P.nzcap)) ? 1 : 0;
+            int sl = B.over || __any_sync(0xffffffffu, len > P.sub_room) ? 1 : 0;
             unsigned long long at = sh.pool_at, pool_end = sh.pool_end;
             if (!sl && at + need > pool_end) {
                 const unsigned long long take = need > P.pool_piece ? need : P.pool_piece;
@@ -1388,15 +1382,15 @@ struct alignas(16) ChainCtl {
 struct ChainLayout {
     uint32_t heads, tabs, subs, sub_stride, w, total;
 };
-__host__ __device__ inline ChainLayout chain_layout(int nzcap, int hotc, bool dense, int tab_bins)
+__host__ __device__ inline ChainLayout chain_layout(uint32_t sub_room, int slots, int hotc, bool dense, int tab_bins)
 {
     ChainLayout L;
     L.heads = (uint32_t)((sizeof(ChainCtl) + 127) & ~(size_t)127);
     const uint32_t hs = (uint32_t)head_slots(tab_bins > 0);
     L.tabs = L.heads + hs * (uint32_t)sizeof(ChainHead);
     L.subs = L.tabs + hs * tab_bytes(tab_bins);
-    L.sub_stride = dense ? sub_bytes_dense(kLB, hotc) : sub_room(nzcap);
-    L.w = L.subs + kSubSlots * L.sub_stride;
+    L.sub_stride = dense ? sub_bytes_dense(kLB, hotc) : sub_room;
+    L.w = L.subs + (uint32_t)slots * L.sub_stride;
     L.total = L.w + 4u * (uint32_t)(hotc > 0 ? hotc : 4);
     return L;
 }
@@ -1411,7 +1405,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     const uint32_t crank = cluster_ctarank();
     const int k = (int)(blockIdx.x >> logC);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const ChainLayout L = chain_layout(P.nzcap, P.hotc, DENSE, TAB ? P.tab_bins : 0);
+    const ChainLayout L = chain_layout(P.sub_room, P.slots, P.hotc, DENSE, TAB ? P.tab_bins : 0);
     ChainCtl &ctl = *reinterpret_cast<ChainCtl *>(smem_chain);
     float *W = reinterpret_cast<float *>(smem_chain + L.w);
     volatile int *abort_flag = &ctl.abort_flag;
@@ -1717,12 +1711,14 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                          : "l"(P.dirS + (((bid0 + at) << logC) + crank))
                          : "memory");
         };
+        const int slots = P.slots;
         uint32_t d[4];
         load_dir(0, d);
+        int slot = 0, before = 0;     // of this block and of the one before
+        uint32_t turn = 0, tbefore = 0; // parity of how often the slots have been filled
 #pragma unroll 1
         for (int blk = 0; blk < nb; ++blk) {
-            const int slot = blk & (kSubSlots - 1);
-            if (blk >= kSubSlots && !mbar_wait_cluster(smem_u32(&ctl.subfree[slot]), (uint32_t)(blk / kSubSlots - 1) & 1u, abort_flag, S.status)) break;
+            if (blk >= slots && !mbar_wait_cluster(smem_u32(&ctl.subfree[slot]), turn ^ 1u, abort_flag, S.status)) break;
             const unsigned long long offset = ((unsigned long long)d[1] << 32) | d[0];
             uint32_t bytes = d[2] <= L.sub_stride ? d[2] : 0u;
             if (!CHICLE_IN_BOUNDS(S.status, (offset & 15ull) == 0ull && offset + bytes <= P.pool_off + P.pool_cap))
@@ -1740,6 +1736,26 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             mbar_arrive_expect_tx_if(bar, bytes, lane == 0);
             bulk_g2s_if(smem_u32(smem_chain + L.subs) + (uint32_t)slot * L.sub_stride, P.rec + offset, bytes, bar, lane == 0);
             load_dir(blk + 1, d);
+            // The block before this one has arrived by now, and its dot products are a block's time away: the model entries
+            // beyond the part in shared memory that they will gather are brought into L2 (the records that stream through it
+            // push them out: with an entry or two per thread, what a block's gathers cost is one round trip to memory).
+            if ((KIND == kCold || KIND == kFlat) && blk > 0) {
+                if (!mbar_wait_cluster(smem_u32(&ctl.subfull[before]), tbefore, abort_flag, S.status)) break;
+                const uint32_t rec = smem_u32(smem_chain + L.subs) + (uint32_t)before * L.sub_stride;
+                const int n = ctl.walk[before] ? 0 : lds_s32(rec);
+                const uint32_t meta = rec + (uint32_t)sizeof(SubHead) + 4u * (uint32_t)n;
+                for (int e = lane; e < n; e += 32) {
+                    const uint32_t v = lds_u32_if(meta + 4u * (uint32_t)e, true) & kIdMask;
+                    if (v >= (uint32_t)P.hotc && (int64_t)v < S.dim) asm volatile("prefetch.global.L2 [%0];" ::"l"(Uk + v));
+                }
+                __syncwarp();
+            }
+            before = slot;
+            tbefore = turn;
+            if (++slot == slots) {
+                slot = 0;
+                turn ^= 1u;
+            }
         }
     }
     if (is_worker) {
@@ -1755,13 +1771,16 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         const uint32_t p_buf0 = mapa_u32(smem_u32(&ctl.pbuf[0][crank][0]), 0u);
         const uint32_t ack_bar = mapa_u32(smem_u32(&ctl.ackbar), 0u);
         const uint32_t a_w = smem_u32(W), a_sink = smem_u32(&ctl.sink[lane]), stride = L.sub_stride;
-        const uint32_t subs0 = smem_u32(smem_chain + L.subs), subs_end = subs0 + kSubSlots * stride;
+        const uint32_t subs0 = smem_u32(smem_chain + L.subs), subs_end = subs0 + (uint32_t)P.slots * stride;
         const uint32_t hotc = (uint32_t)P.hotc;
         const int dstride = dense_stride(hot_mine);                // dense: floats per row of a record
         const int depth = P.depth;
         const int jd = wt >> 3, qd = wt & 7;                       // dot products: eight threads per coordinate
         uint32_t r_upd = subs0, r_dot = subs0;                     // records of blocks b and b + depth
         int fg = 0; // staged blocks whose dot products have been sent
+        const int slots = P.slots;
+        int s_upd = 0, s_dot = 0;  // and these records' slots (the first turns take the dot products of blocks 0, ..)
+        uint32_t dot_turn = 0;     // parity of how often slot s_dot has been filled
         bool ok = true;
 #ifdef CHICLE_LA_TIMING
         long long wd = 0, ws = 0, wg = 0, ws1 = 0, wg0 = 0, wg1 = 0, t0 = clock64(), t1 = 0;
@@ -1890,9 +1909,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             //      from the model as the walk left it: with depth 2 its products wait for that.
             bool sl2 = false, due = b + depth < nb, late = false;
             if (due) {
-                const int slot = (b + depth) & (kSubSlots - 1);
-                ok = ok && mbar_wait_cluster(smem_u32(&ctl.subfull[0]) + 8u * slot, (uint32_t)((b + depth) / kSubSlots) & 1u, abort_flag, S.status);
-                sl2 = lds_s32(smem_u32(&ctl.walk[0]) + 4u * slot) != 0;
+                ok = ok && mbar_wait_cluster(smem_u32(&ctl.subfull[0]) + 8u * s_dot, dot_turn, abort_flag, S.status);
+                sl2 = lds_s32(smem_u32(&ctl.walk[0]) + 4u * s_dot) != 0;
                 due = !sl2;
             }
             if (sl0 || sl1) {
@@ -1903,7 +1921,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             bool met = b < 0; // the barrier behind the update
             auto meet = [&]() {
                 if (!met) work_bar();
-                if (!met && wt == 0) mbar_arrive(smem_u32(&ctl.subfree[0]) + 8u * (b & (kSubSlots - 1))); // block b's slot is free
+                if (!met && wt == 0) mbar_arrive(smem_u32(&ctl.subfree[0]) + 8u * s_upd); // block b's slot is free
                 met = true;
             };
 #pragma unroll 1
@@ -1956,7 +1974,13 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                             w[u] = lds_f32(a_w + 4u * (CHICLE_IN_BOUNDS(S.status, m[u] < hotc) ? m[u] : 0u));
                         } else {
                             const bool cold = m[u] >= hotc && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim);
-                            w[u] = ldcg_or(Uk + (cold ? m[u] : 0u), cold, lds_f32(a_w + (m[u] < hotc ? 4u * m[u] : 0u)));
+                            w[u] = ldcg_if(Uk + (cold ? m[u] : 0u), cold);
+                        }
+                    };
+                    auto near = [&](int u) { // (once all gathers are on their way)
+                        if (KIND == kCold) {
+                            const float h = lds_f32(a_w + (m[u] < hotc ? 4u * m[u] : 0u));
+                            w[u] = m[u] < hotc ? h : w[u];
                         }
                     };
                     auto entries = [&]() {
@@ -1979,6 +2003,12 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                             for (int u = 4; u < 8; ++u) model(u);
                         }
 #pragma unroll
+                        for (int u = 0; u < 4; ++u) near(u);
+                        if (more) {
+#pragma unroll
+                            for (int u = 4; u < 8; ++u) near(u);
+                        }
+#pragma unroll
                         for (int u = 0; u < 4; ++u) acc = fmaf(x[u], w[u], acc);
                         if (!more) break;
 #pragma unroll
@@ -1997,6 +2027,11 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             }
             meet();
             r_dot = r_dot + stride == subs_end ? subs0 : r_dot + stride;
+            if (++s_dot == slots) {
+                s_dot = 0;
+                dot_turn ^= 1u;
+            }
+            if (b >= 0) s_upd = s_upd + 1 == slots ? 0 : s_upd + 1;
             LA_T(wg1);
             sl0 = depth == 1 ? sl2 : sl1;
             sl1 = sl2;
@@ -2090,9 +2125,8 @@ constexpr int kPreMidNz = 3072;
 
 // true: the prepare kernel with arrays for 2 048 non-zeros per block serves (32 coordinates of 50 on average, with room)
 bool small_prepare(const Glm &g) { return 32.0 * (double)g.nnz / (double)g.n_coord * 1.25 <= (double)kPreSmallNz; }
-// true: arrays for 3 072 non-zeros per block serve (two CTAs of 512 threads share an SM; with 4 096 it is one). Blocks
-// with more are walked in place either way unless a cluster shares them out.
-bool mid_prepare(const Glm &g) { return g.la_logC == 0 || 32.0 * (double)g.nnz / (double)g.n_coord * 1.1 <= (double)kPreMidNz; }
+// true: arrays for 3 072 non-zeros per block serve
+bool mid_prepare(const Glm &g) { return 32.0 * (double)g.nnz / (double)g.n_coord * 1.1 <= (double)kPreMidNz; }
 
 // The prepare kernel of one launch's blocks on `stream`.
 template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, cudaStream_t stream)
@@ -2200,14 +2234,13 @@ void lookahead_plan(Glm &g, int32_t K)
 {
     const bool dense = g.fmt == CHICLE_FMT_DENSE_ROWMAJOR;
     int logC = 0;
-    if (!dense && g.hot_variant) {
+    if (!dense) {
         // a cluster per partition, on at most half of the SMs: the prepare kernels need the rest
         while (logC < 3 && ((int64_t)K << (logC + 1)) * 2 <= g.sm_count) ++logC;
         const char *env = getenv("CHICLE_LA_CLUSTER");
         if (env && env[0] >= '1' && env[0] <= '8' && env[1] == 0) {
             const int want = env[0] - '0';
             logC = want >= 8 ? 3 : (want >= 4 ? 2 : (want >= 2 ? 1 : 0));
-            while (logC > 0 && ((int64_t)K << logC) > g.sm_count) --logC;
         }
     }
     int slice = (int)((g.dim + 3) & ~(int64_t)3); // dense: columns per CTA
@@ -2243,25 +2276,50 @@ void lookahead_plan(Glm &g, int32_t K)
         const float q_max = (float)K * g.max_sqnorm / (g.lambda * (float)g.n_examples);
         for (int bins = 64; bins >= 32; bins >>= 1)
             if (q_max <= tab_max_q(bins)) g.la_tab_bins = bins;
-        if (dense && chain_layout(0, slice, true, g.la_tab_bins).total > budget) g.la_tab_bins = 0;
+        if (dense && chain_layout(0, kSubSlots, slice, true, g.la_tab_bins).total > budget) g.la_tab_bins = 0;
         const char *env = getenv("CHICLE_LA_TABLES"); // 0: none (tests)
         if (env && env[0] == '0') g.la_tab_bins = 0;
     }
-    if (dense) {
-        g.la_nzcap = 0;
-        g.la_hotc = slice;
-    } else if (!g.hot_variant) {
-        g.la_nzcap = 3072;
-        g.la_hotc = 0;
-    } else {
-        g.la_nzcap = logC == 0 ? 2048 : (logC == 1 ? 1536 : 1024);
-        const ChainLayout L0 = chain_layout(g.la_nzcap, 0, false, g.la_tab_bins);
+    g.la_slots = kSubSlots;
+    g.la_sub_room = 0;
+    g.la_hotc = slice;
+    if (!dense) {
+        // A slot holds the record that a block of 32 random coordinates is expected to make for a CTA (how many entries, and how
+        // many of them with ids that several of the 32 have: from the ids' frequencies, see launch_frequency_remap) and five
+        // standard deviations more; what is left keeps the model's most frequent ids. Where that leaves the model little, three
+        // slots do if dot products are taken one block ahead, and the root search on the chain instead of tables: a block
+        // without room is walked in place, 20 times slower.
+        const int C = 1 << logC;
+        uint32_t room = 256;
+        for (int c = 0; c < C; ++c) {
+            double n = 0.0, T = 0.0, nl = 0.0;
+            for (int i = c; i < kRankClasses; i += C) { n += g.blk_entries[i]; T += g.blk_shared_ids[i]; nl += g.blk_shared[i]; }
+            const double all = (double)kLB * (double)g.nnz / (double)g.n_coord, part = all > 0.0 ? n / all : 0.0;
+            const double n_hi = n + 5.0 * sqrt(n + part * part * kLB * g.row_variance), f = n > 0.0 ? n_hi / n : 1.0;
+            const double nl_hi = fmin(n_hi, f * nl + 5.0 * sqrt(nl)), T_hi = fmin(0.5 * nl_hi, f * T + 5.0 * sqrt(T));
+            if (n_hi > 65535.0) room = 0xffffffu; // (cut to what there is)
+            else {
+                const uint32_t r = sub_bytes((uint32_t)n_hi + 1u, (uint32_t)T_hi + 1u, (uint32_t)nl_hi + 1u) + 64u;
+                room = r > room ? r : room;
+            }
+        }
+        for (;;) {
+            const double left = (double)budget - (double)chain_layout(0, 0, 0, false, g.la_tab_bins).total - 64.0;
+            g.la_slots = g.la_depth == 1 && 4.0 * room > 0.6 * left ? 3 : kSubSlots;
+            if (g.la_tab_bins == 0 || (double)g.la_slots * room <= 0.8 * left) {
+                const uint32_t most = (uint32_t)(0.8 * left / g.la_slots) & ~15u;
+                g.la_sub_room = room < most ? room : most;
+                break;
+            }
+            g.la_tab_bins = 0;
+        }
+        const ChainLayout L0 = chain_layout(g.la_sub_room, g.la_slots, 0, false, g.la_tab_bins);
         int64_t hotc = ((int64_t)budget - (int64_t)L0.total - 64) / 4;
-        hotc = hotc < 0 ? 0 : (hotc / 32) * 32;
+        hotc = hotc < 0 || g.flat_ids ? 0 : (hotc / 32) * 32;
         const int64_t need = (g.dim + ((int64_t)1 << logC) - 1) >> logC; // per CTA for the whole model
         g.la_hotc = (int32_t)(hotc < need ? hotc : (need + 31) / 32 * 32);
     }
-    g.la_smem = chain_layout(g.la_nzcap, g.la_hotc, dense, g.la_tab_bins).total;
+    g.la_smem = chain_layout(g.la_sub_room, g.la_slots, g.la_hotc, dense, g.la_tab_bins).total;
 
     // slices: at most a sixteenth of the walk, but at least 256 blocks per partition; two regions
     const int64_t n = g.n_coord;
@@ -2409,7 +2467,8 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
         p.K = K;
         p.logC = g.la_logC;
         p.depth = g.la_depth;
-        p.nzcap = g.la_nzcap;
+        p.sub_room = g.la_sub_room;
+        p.slots = g.la_slots;
         p.hotc = g.la_hotc;
         p.n_blocks = blocks[(size_t)s];
         p.drop_block = (drop && s == 0) ? atoll(drop) : -1;

@@ -55,16 +55,57 @@ __global__ void k_mass_of_first(const uint32_t *__restrict__ counts, const int32
     if ((threadIdx.x & 31) == 0 && s) atomicAdd(out, s);
 }
 
-// out[1] += number of coordinates with more than `long_len` entries
+// What a block of 32 random coordinates is expected to have on the ids of class i = (new id) mod kRankClasses: out[i]
+// entries (the whole problem's, exactly), out[kRankClasses + i] ids that at least two of the 32 have and
+// out[2 kRankClasses + i] entries with such ids (both in units of 2^-20, so that the sums do not depend on their order).
+__global__ void k_expect_blocks(const uint32_t *__restrict__ counts, const int32_t *__restrict__ old_of_new, int64_t dim, double inv_n,
+                                unsigned long long *__restrict__ out)
+{
+    static_assert(kT % kRankClasses == 0, "a thread's ids are of one class");
+    unsigned long long all = 0, ids = 0, ent = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < dim; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t c = counts[old_of_new[i]];
+        const float p = fminf((float)((double)c * inv_n), 0.9999999f), l = log1pf(-p);
+        const float others = -expm1f(31.0f * l);                               // one of the other 31 has it
+        const float one = 32.0f * p * (1.0f - others), some = -expm1f(32.0f * l); // exactly one has it, some have it
+        all += c;
+        ids += (unsigned long long)(fmaxf(some - one, 0.0f) * 1048576.0f);
+        ent += (unsigned long long)(32.0f * p * others * 1048576.0f);
+    }
+#pragma unroll
+    for (int o = 16; o >= kRankClasses; o >>= 1) {
+        all += __shfl_xor_sync(0xffffffffu, all, o);
+        ids += __shfl_xor_sync(0xffffffffu, ids, o);
+        ent += __shfl_xor_sync(0xffffffffu, ent, o);
+    }
+    if ((threadIdx.x & 31) < kRankClasses) {
+        unsigned long long *o = out + (threadIdx.x & (kRankClasses - 1));
+        if (all) atomicAdd(o, all);
+        if (ids) atomicAdd(o + kRankClasses, ids);
+        if (ent) atomicAdd(o + 2 * kRankClasses, ent);
+    }
+}
+
+// out[1] += number of coordinates with more than `long_len` entries; out[2] += the sum of their squared lengths (each
+// counted as 65 536 at most)
 __global__ void k_count_long(const int64_t *__restrict__ indptr, int64_t n_coord, int32_t long_len,
                              unsigned long long *__restrict__ out)
 {
-    unsigned long long s = 0;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_coord; c += (int64_t)gridDim.x * blockDim.x)
-        s += (indptr[c + 1] - indptr[c]) > long_len ? 1u : 0u;
+    unsigned long long s = 0, q = 0;
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_coord; c += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t len = indptr[c + 1] - indptr[c], m = len < 65536 ? len : 65536;
+        s += len > long_len ? 1u : 0u;
+        q += (unsigned long long)(m * m);
+    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0 && s) atomicAdd(out + 1, s);
+    for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        q += __shfl_xor_sync(0xffffffffu, q, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (s) atomicAdd(out + 1, s);
+        if (q) atomicAdd(out + 2, q);
+    }
 }
 
 // dst[i] = src[map[i]]
@@ -76,8 +117,8 @@ __global__ void k_gather_f32(const float *__restrict__ src, const int32_t *__res
 
 } // namespace
 
-// counts: dim zeroed uint32; keys/vals: two arrays of dim each; mass: two zeroed 64-bit words (non-zeros on the first
-// hot_ids ids; coordinates longer than long_len).
+// counts: dim zeroed uint32; keys/vals: two arrays of dim each; mass: kMassWords zeroed 64-bit words (non-zeros on the first
+// hot_ids ids; coordinates longer than long_len; the sum of squared lengths; from word 4 on what k_expect_blocks sums).
 cudaError_t launch_frequency_remap(Glm &g, uint32_t *counts, uint64_t *keys[2], int32_t *vals[2], uint32_t *hist,
                                    uint32_t *scan_sums, int64_t hot_ids, int32_t long_len, unsigned long long *mass)
 {
@@ -97,6 +138,7 @@ cudaError_t launch_frequency_remap(Glm &g, uint32_t *counts, uint64_t *keys[2], 
     const int64_t first = hot_ids < dim ? hot_ids : dim;
     k_mass_of_first<<<blocks_for(first), kT, 0, g.stream>>>(counts, g.old_of_new, first, mass);
     k_count_long<<<wide, kT, 0, g.stream>>>(g.indptr, g.n_coord, long_len, mass);
+    k_expect_blocks<<<blocks_for(dim) < wide ? blocks_for(dim) : wide, kT, 0, g.stream>>>(counts, g.old_of_new, dim, 1.0 / (double)g.n_coord, mass + 4);
     return cudaGetLastError();
 }
 
