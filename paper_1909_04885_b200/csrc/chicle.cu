@@ -89,12 +89,22 @@ cudaError_t copy_in(void *dst, const void *src, size_t bytes, chicle_memspace_t 
 }
 
 // Reads and clears the device status word. Stream must be idle or the caller accepts a sync here.
+chicle_status_t status_of(chicle_glm *h, uint32_t bits);
+
 chicle_status_t check_status(chicle_glm *h)
 {
-    cudaError_t e = cudaMemcpyAsync(h->h_status, h->d_status, sizeof(uint32_t), cudaMemcpyDeviceToHost, h->stream);
+    // (a word that has been read since the last kernels that may set it need not be copied again)
+    cudaError_t e = h->status_read ? cudaSuccess : cudaMemcpyAsync(h->h_status, h->d_status, sizeof(uint32_t), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return fail_cuda(h, e, "status read");
-    const uint32_t bits = *h->h_status;
+    if (h->status_read) return CHICLE_OK;
+    return status_of(h, *h->h_status);
+}
+
+// (a word that says something is cleared: what it says is reported once)
+chicle_status_t status_of(chicle_glm *h, uint32_t bits)
+{
+    h->status_read = true;
     if (bits == 0) return CHICLE_OK;
     (void)cudaMemsetAsync(h->d_status, 0, sizeof(uint32_t), h->stream);
     if (bits & ST_BOUNDS) return fail(h, CHICLE_ERR_INTERNAL, "a bounds check of a CHICLE_DEBUG_BOUNDS build failed");
@@ -179,11 +189,12 @@ chicle_status_t chicle_glm_create(const chicle_matrix_t *X, const float *labels,
     h->dim = ridge ? X->n_rows : X->n_cols;
     h->n_examples = X->n_rows;
     h->lambda = lambda;
-    // (three attributes: cudaGetDeviceProperties takes 2.5 ms)
+    // (four attributes: cudaGetDeviceProperties takes 2.5 ms)
     int major = 0;
     e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->l2_bytes, cudaDevAttrL2CacheSize, device);
     if (e != cudaSuccess) { destroy_impl(h); return fail_cuda(nullptr, e, "cudaDeviceGetAttribute"); }
     if (major < 10) {
         destroy_impl(h);
@@ -208,8 +219,7 @@ chicle_status_t chicle_glm_create(const chicle_matrix_t *X, const float *labels,
     // 12 bytes past its last entry
     bool ok = alloc_into(h, h->values, nvals + 4) && alloc_into(h, h->labels, (size_t)h->n_examples) &&
               alloc_into(h, h->sqnorm, (size_t)h->n_coord) && alloc_into(h, h->alpha, (size_t)h->n_coord) &&
-              alloc_into(h, h->v, (size_t)h->dim) && alloc_into(h, h->d_status, 64) &&
-              alloc_into(h, h->gap_out, 8);
+              alloc_into(h, h->v, (size_t)h->dim) && alloc_into(h, h->d_status, 64);
     if (ok && !dense) ok = alloc_into(h, h->indptr, (size_t)h->n_coord + 1) && alloc_into(h, h->indices, nvals + 4);
     if (ok && ridge) ok = alloc_into(h, h->resid, (size_t)h->dim);
     h->gap_blocks = h->sm_count * 8;
@@ -322,6 +332,7 @@ chicle_status_t chicle_glm_create(const chicle_matrix_t *X, const float *labels,
         if (force && strcmp(force, "hot128") == 0) h->hot_variant = 2;
     }
     if (!dense) {
+        h->status_read = false;
         e = cudaStreamWaitEvent(s, h->la_ev_done[0], 0);
         if (e == cudaSuccess) e = launch_validate(*h, true, false);
         if (e != cudaSuccess) return bail_cuda(e, "validation kernels");
@@ -557,14 +568,14 @@ static chicle_status_t round_impl(chicle_glm_t *h, int64_t H, const int64_t *hos
     cudaStream_t s = h->stream;
     if (stats) (void)cudaEventRecord(h->ev[0], s);
     if (host_steps) {
-        // a pageable source: the runtime has taken its copy of the K words when the call returns
-        e = cudaMemcpyAsync(h->d_steps, host_steps, (size_t)h->K * sizeof(int64_t), cudaMemcpyHostToDevice, s);
+        e = launch_words(*h, h->d_steps, host_steps, (size_t)h->K);
         if (e != cudaSuccess) return fail_cuda(h, e, "step budgets to the device");
     }
     e = launch_permutation(*h, h->round, epochs, H, host_steps ? h->d_steps : nullptr);
     if (e != cudaSuccess) return fail_cuda(h, e, "visiting-order kernels");
     if (stats) (void)cudaEventRecord(h->ev[1], s);
     int variant = 0;
+    h->status_read = false;
     h->time_prepare = stats != nullptr;
     h->solver_launches = 0;
     h->round_steps = host_steps;
@@ -671,10 +682,10 @@ chicle_status_t chicle_duality_gap(chicle_glm_t *h, double *host_gap, double *ho
 {
     if (!h) return CHICLE_ERR_INVALID_ARG;
     cudaError_t e = cudaSetDevice(h->device);
-    if (e == cudaSuccess) e = launch_gap(*h);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_gap, h->gap_out, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = launch_gap(*h); // (its last kernel leaves the result and the status word in host memory)
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return fail_cuda(h, e, "duality-gap kernels");
-    const chicle_status_t st = check_status(h); // synchronises
+    const chicle_status_t st = status_of(h, *h->h_status);
     if (st != CHICLE_OK) return st;
     if (host_gap) *host_gap = h->h_gap[0];
     if (host_primal) *host_primal = h->h_gap[1];
@@ -705,9 +716,11 @@ chicle_status_t chicle_get_v(chicle_glm_t *h, float *out, int64_t len, chicle_me
 {
     if (h && h->new_of_old) {
         // translate from the library's ranked ids to the caller's: tmp[old] = v[new_of_old[old]]
+        const bool direct = out && len == h->dim && space == CHICLE_MEM_DEVICE; // (the caller's array takes it as it is)
         if (cudaSetDevice(h->device) == cudaSuccess) {
-            const cudaError_t e = launch_gather_f32(*h, h->v, h->new_of_old, h->dim, h->perm_tmp);
+            const cudaError_t e = launch_gather_f32(*h, h->v, h->new_of_old, h->dim, direct ? out : h->perm_tmp);
             if (e != cudaSuccess) return fail_cuda(h, e, "chicle_get_v");
+            if (direct) return check_status(h);
         }
         return copy_out(h, h->perm_tmp, h->dim, out, len, space, "chicle_get_v");
     }

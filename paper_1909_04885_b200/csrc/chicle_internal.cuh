@@ -158,14 +158,15 @@ struct Glm {
     int order_launches = 0;        // kernels launched for the last visiting orders
     double *gap_partials = nullptr; // gap kernel partial sums
     int gap_blocks = 0;
-    double *gap_out = nullptr;      // 8 doubles on the device
     uint32_t *d_status = nullptr;
+    bool status_read = false;       // no kernel that may set the status word has been launched since it was last read
     uint32_t *h_status = nullptr;   // pinned
     double *h_gap = nullptr;        // pinned, 8 doubles
 
     int64_t round = 0;
     int sm_count = 148;
     int max_smem_optin = 0;
+    int l2_bytes = 0;
     cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     std::string err;
 };
@@ -189,6 +190,7 @@ cudaError_t launch_frequency_remap(Glm &g, uint32_t *counts, uint64_t *keys[2], 
                                    uint32_t *scan_sums, int64_t hot_ids, int32_t long_len, unsigned long long *mass);
 cudaError_t launch_gather_f32(Glm &g, const float *src, const int32_t *map, int64_t n, float *dst); // dst[i] = src[map[i]]
 cudaError_t launch_lookahead_solver(Glm &g, const struct SolverParams &P);
+cudaError_t launch_words(Glm &g, int64_t *dst, const int64_t *src, size_t n); // small host arrays to the device
 void lookahead_plan(Glm &g, int32_t K); // fills the la_* sizes for a partition into K
 int lookahead_max_dense_dim();
 int lookahead_max_slices();

@@ -1040,7 +1040,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
 // issued before the first is used: three round trips to memory per block. (A warp per row, headers by its first lane, was
 // a chain of 24 of them: 72 000 cycles per block at 28 entries per row, with the tables.)
 constexpr int kPreThreads = 256;
-constexpr int kPreDensePerSm = 4;
+constexpr int kPreDensePerSm = 4, kPreDenseLongPerSm = 3;
 struct PreDenseShared {
     CHdr hdr[kLB];
     float gsc[2 * kLB], ys[kLB], as[kLB];
@@ -1050,16 +1050,16 @@ struct PreDenseShared {
     unsigned long long sub_off[kMaxC];
     alignas(16) float row[1];        // 64 rows of row_stride(columns at a time) floats: this block's, then the next block's
 };
-// Rows go through shared memory this many columns at a time (four CTAs per SM either way).
-constexpr int kDenseCols = 128;
+// Rows longer than this go through shared memory that many columns at a time.
+constexpr int kDenseCols = 64;
 // 16-byte pieces of consecutive rows lie on different banks
 __host__ __device__ constexpr int row_stride(int cols) { return (((cols + 3) / 4) | 1) * 4; }
 inline size_t pre_dense_bytes(int dim)
 {
-    return sizeof(PreDenseShared) + 2 * kLB * (size_t)row_stride(dim < kDenseCols ? dim : kDenseCols) * sizeof(float);
+    return sizeof(PreDenseShared) + (dim > kDenseCols ? 2 : 1) * 2 * kLB * (size_t)row_stride(dim < kDenseCols ? dim : kDenseCols) * sizeof(float);
 }
 
-template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const LookParams &P, const int64_t bid, PreDenseShared &sh)
+template <int LOSS, bool LONG> __device__ __forceinline__ void prepare_block_dense(const LookParams &P, const int64_t bid, PreDenseShared &sh)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr int NW = kPreThreads / 32;
@@ -1126,21 +1126,65 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
             sh.as[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : hd.p1;
         }
     }
-    // ---- x_l . x_j for this block's l and the 64 columns j: a thread has l = lp, lp + 16 and j = jq, jq + 16, .. (every
-    //      sum over the entries in ascending order). The rows pass through shared memory kDenseCols columns at a time, and
-    //      this block's go into the workers' records on the way.
+    // ---- x_l . x_j for this block's l and the 64 columns j. This block's rows go into the workers' records on the
+    //      way. LONG rows pass through shared memory kDenseCols columns at a time, fetched two pieces ahead by asynchronous copies
+    //      (with registers on the way, 64 of them per thread, a load's round trip was exposed for every piece: 100 000 rows of
+    //      500 took 295 us); four groups of 64 threads take every fourth four columns, a thread l = lp, lp + 8, .. and j = jq,
+    //      jq + 8, .. (4 x 8 sums: 12 loads of 16 bytes per 128 multiply-adds, against 48; pairs of tiles that lie below the
+    //      triangle are left out), and the groups' sums are added in order. Short rows leave such groups nothing to share: 2 x 4 sums, l = lp, lp + 16, j = jq, jq + 16, ..
+    constexpr int TL = LONG ? 4 : 2, TJ = LONG ? 8 : 4, GL = kLB / TL, GJ = 2 * kLB / TJ, GROUPS = kPreThreads / (GL * GJ);
     constexpr int RPW = 2 * kLB / NW; // rows a warp loads
     {
-        const int jq = tid & 15, lp = tid >> 4;
-        float acc[2][4];
+        const int jq = tid % GJ, lp = tid / GJ % GL, group = tid / (GL * GJ);
+        float acc[TL][TJ];
 #pragma unroll
-        for (int a = 0; a < 2; ++a)
+        for (int a = 0; a < TL; ++a)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][c] = 0.0f;
+            for (int c = 0; c < TJ; ++c) acc[a][c] = 0.0f;
+        auto fetch = [&](int e0, float *to) { // (LONG) the 64 rows' columns e0 ..
+            const int cols = dim - e0 < kDenseCols ? dim - e0 : kDenseCols, cols4 = (cols + 3) & ~3;
+            constexpr int V = kDenseCols / 4;
+            if ((dim & 3) == 0) {
+#pragma unroll
+                for (int i = tid; i < 2 * kLB * V; i += kPreThreads) {
+                    const int j = i / V, s = i % V, c = sh.coord[j];
+                    if (4 * s >= cols) continue;
+                    float *at = to + j * stride + 4 * s;
+                    if (c >= 0) cp_async16(smem_u32(at), P.S.values + (int64_t)c * dim + e0 + 4 * s);
+                    else *reinterpret_cast<float4 *>(at) = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            } else {
+#pragma unroll 4
+                for (int i = tid; i < 2 * kLB * kDenseCols; i += kPreThreads) {
+                    const int j = i / kDenseCols, s = i % kDenseCols, c = sh.coord[j];
+                    if (s >= cols4) continue;
+                    float *at = to + j * stride + s;
+                    if (c >= 0 && s < cols) cp_async4(smem_u32(at), P.S.values + (int64_t)c * dim + e0 + s);
+                    else *at = 0.0f;
+                }
+            }
+        };
+        if (LONG) {
+            fetch(0, sh.row);
+            cp_async_commit();
+            fetch(kDenseCols, sh.row + 2 * kLB * stride);
+            cp_async_commit();
+        }
         for (int e0 = 0; e0 < dim; e0 += kDenseCols) {
             const int cols = dim - e0 < kDenseCols ? dim - e0 : kDenseCols, cols4 = (cols + 3) & ~3;
-            if (e0 > 0) __syncthreads(); // the chunk before has been read
-            if ((dim & 3) == 0) { // rows start on 16-byte boundaries (and so do slices)
+            float *rows = sh.row + (LONG && ((e0 / kDenseCols) & 1) ? 2 * kLB * stride : 0);
+            if (LONG) {
+                cp_async_wait_but_one();
+                __syncthreads();
+                if (!walk)
+#pragma unroll
+                    for (int i = tid; i < kLB * (kDenseCols / 4); i += kPreThreads) {
+                        const int j = i / (kDenseCols / 4), s = 4 * (i % (kDenseCols / 4)), e = e0 + s, c = e / slice;
+                        if (j < cnt && s < cols && c < C) // (with the zero padding)
+                            *reinterpret_cast<float4 *>(reinterpret_cast<float *>(P.rec + sh.sub_off[c] + sizeof(SubHead)) + j * dense_stride(cols_of(c)) + (e - c * slice)) =
+                                *reinterpret_cast<const float4 *>(rows + j * stride + s);
+                    }
+            } else if ((dim & 3) == 0) { // rows start on 16-byte boundaries (and so do slices)
                 const int nv = cols >> 2;
                 const int lpr = nv <= 8 ? 8 : (nv <= 16 ? 16 : 32); // lanes per row
                 const int sub = lane & (lpr - 1), per = 32 / lpr;   // rows per turn
@@ -1182,20 +1226,21 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
                     }
                 }
             }
-            __syncthreads();
+            if (!LONG) __syncthreads();
             if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins && !walk && e0 == 0) write_table(P, bid, sh.hdr, kPreThreads);
             if (!walk) {
-                const float *rl = sh.row + lp * stride, *rj = sh.row + jq * stride;
-                for (int e = 0; e < cols; e += 4) {
-                    float4 xl[2], xj[4];
+                const float *rl = rows + lp * stride, *rj = rows + jq * stride;
+                for (int e = 4 * group; e < cols; e += 4 * GROUPS) {
+                    float4 xl[TL], xj[TJ];
 #pragma unroll
-                    for (int a = 0; a < 2; ++a) xl[a] = *reinterpret_cast<const float4 *>(rl + 16 * a * stride + e);
+                    for (int a = 0; a < TL; ++a) xl[a] = *reinterpret_cast<const float4 *>(rl + GL * a * stride + e);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) xj[c] = *reinterpret_cast<const float4 *>(rj + 16 * c * stride + e);
+                    for (int c = 0; c < TJ; ++c) xj[c] = *reinterpret_cast<const float4 *>(rj + GJ * c * stride + e);
 #pragma unroll
-                    for (int a = 0; a < 2; ++a)
+                    for (int a = 0; a < TL; ++a)
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
+                        for (int c = 0; c < TJ; ++c) {
+                            if (GJ * c < kLB && GL * a >= GJ * (c + 1)) continue; // (every l of the tile is at or beyond every j)
                             acc[a][c] = fmaf(xj[c].x, xl[a].x, acc[a][c]);
                             acc[a][c] = fmaf(xj[c].y, xl[a].y, acc[a][c]);
                             acc[a][c] = fmaf(xj[c].z, xl[a].z, acc[a][c]);
@@ -1203,19 +1248,43 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
                         }
                 }
             }
-        }
-#pragma unroll
-        for (int a = 0; a < 2; ++a)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int l = lp + 16 * a, j = jq + 16 * c;
-                const bool on = c < 2 ? l < j : l < cnt; // inside the block: earlier coordinates only
-                const float v = on ? acc[a][c] * (sh.gsc[j] * sh.ys[l]) : 0.0f;
-                sh.T[l][j] = v;
-                (c < 2 ? out.G : out.X)[l * kLB + (j & (kLB - 1))] = v;
+            if (LONG) {
+                __syncthreads(); // the piece has been read
+                if (e0 + 2 * kDenseCols < dim) fetch(e0 + 2 * kDenseCols, rows);
+                cp_async_commit();
             }
+        }
+        if (LONG) { // the groups' sums together, in order (sh.T[l][j]: bank l + j, no two of a warp's threads on one)
+#pragma unroll 1
+            for (int r = GROUPS - 1; r >= 0; --r) {
+                if (r < GROUPS - 1) __syncthreads();
+                if (group != r) continue;
+#pragma unroll
+                for (int a = 0; a < TL; ++a)
+#pragma unroll
+                    for (int c = 0; c < TJ; ++c) {
+                        float &t = sh.T[lp + GL * a][jq + GJ * c];
+                        if (r < GROUPS - 1) acc[a][c] += t;
+                        if (r > 0) t = acc[a][c];
+                    }
+            }
+        }
+        if (group == 0) {
+#pragma unroll
+            for (int a = 0; a < TL; ++a)
+#pragma unroll
+                for (int c = 0; c < TJ; ++c) {
+                    const int l = lp + GL * a, j = jq + GJ * c;
+                    const bool on = GJ * c < kLB ? l < j : l < cnt; // inside the block: earlier coordinates only
+                    sh.T[l][j] = on ? acc[a][c] * (sh.gsc[j] * sh.ys[l]) : 0.0f;
+                }
+        }
     }
     __syncthreads();
+    for (int i = tid; i < kLB * kLB; i += kPreThreads) {
+        out.G[i] = sh.T[i / kLB][i % kLB];
+        out.X[i] = sh.T[i / kLB][kLB + i % kLB];
+    }
     for (int j = warp; j < 2 * kLB; j += NW) { // what the states at round start contribute
         float q0 = sh.T[lane][j] * sh.as[lane];
 #pragma unroll
@@ -1230,12 +1299,12 @@ template <int LOSS> __device__ __forceinline__ void prepare_block_dense(const Lo
 }
 
 // (blocks blockIdx.x, blockIdx.x + gridDim.x, ...: see k_lookahead_prepare)
-template <int LOSS> __global__ void __launch_bounds__(kPreThreads, kPreDensePerSm) k_lookahead_prepare_dense(const LookParams P)
+template <int LOSS, bool LONG> __global__ void __launch_bounds__(kPreThreads, LONG ? kPreDenseLongPerSm : kPreDensePerSm) k_lookahead_prepare_dense(const LookParams P)
 {
     extern __shared__ __align__(16) unsigned char smem_pre[];
     PreDenseShared &sh = *reinterpret_cast<PreDenseShared *>(smem_pre);
     for (int64_t bid = blockIdx.x; bid < P.n_blocks; bid += gridDim.x) {
-        prepare_block_dense<LOSS>(P, bid, sh);
+        prepare_block_dense<LOSS, LONG>(P, bid, sh);
         __syncthreads();
     }
 }
@@ -1445,16 +1514,40 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             mbar_arrive_expect_tx(smem_u32(&ctl.dbar[i]), d_bytes);
         }
     }
-    for (int l = tid; l < hot_mine; l += kChainThreads) {
-        const size_t g = DENSE ? (size_t)(slice0 + l) : ((size_t)l << logC) + crank;
-        W[l] = P.model_in ? fmaf(sigma, Uk[g], S.vbase[g]) : Uk[g];
+    // (eight words per thread and turn, all loads first: a launch must not spend a memory round trip on every 352 words)
+    for (int l0 = tid; l0 < hot_mine; l0 += 8 * kChainThreads) {
+        float u[8], v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int l = l0 + i * kChainThreads;
+            const bool in = l < hot_mine;
+            const size_t g = !in ? 0 : (DENSE ? (size_t)(slice0 + l) : ((size_t)l << logC) + crank);
+            u[i] = ldcg_if(Uk + g, in);
+            v[i] = ldcg_if(S.vbase + g, in && P.model_in);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (l0 + i * kChainThreads < hot_mine) W[l0 + i * kChainThreads] = P.model_in ? fmaf(sigma, u[i], v[i]) : u[i];
     }
     if (DENSE && tid < 4 && hot_mine + tid < P.hotc) W[hot_mine + tid] = 0.0f; // (the padding of the last slice)
     // the ids beyond the part in shared memory that fall to this CTA (id mod C): the model in place
     const size_t cold0 = (size_t)hot_total + (((size_t)crank - (size_t)hot_total) & (size_t)(C - 1));
     if (P.model_in)
-        for (size_t g = cold0 + ((size_t)tid << logC); g < (size_t)S.dim; g += (size_t)kChainThreads << logC)
-            Uk[g] = fmaf(sigma, Uk[g], S.vbase[g]);
+        for (size_t g0 = cold0 + ((size_t)tid << logC); g0 < (size_t)S.dim; g0 += (size_t)(8 * kChainThreads) << logC) {
+            float u[8], v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const size_t g = g0 + ((size_t)(i * kChainThreads) << logC);
+                const bool in = g < (size_t)S.dim;
+                u[i] = ldcg_if(Uk + (in ? g : 0), in);
+                v[i] = ldcg_if(S.vbase + (in ? g : 0), in);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const size_t g = g0 + ((size_t)(i * kChainThreads) << logC);
+                if (g < (size_t)S.dim) Uk[g] = fmaf(sigma, u[i], v[i]);
+            }
+        }
     __syncthreads();
     cluster_arrive();
     cluster_wait();
@@ -2047,13 +2140,36 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         if (!aborted) {
             // the model goes back to row k: as it is, or after the round's last launch as the update U_k = (w - v) / sigma'
             const float inv_sigma = 1.0f / sigma;
-            for (int l = wt; l < hot_mine; l += kWorkThreads) {
-                const size_t g = DENSE ? (size_t)(slice0 + l) : ((size_t)l << logC) + crank;
-                Uk[g] = P.model_out ? (W[l] - S.vbase[g]) * inv_sigma : W[l];
+            for (int l0 = wt; l0 < hot_mine; l0 += 8 * kWorkThreads) {
+                float v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int l = l0 + i * kWorkThreads;
+                    const bool in = l < hot_mine && P.model_out;
+                    v[i] = ldcg_if(S.vbase + (!in ? 0 : (DENSE ? (size_t)(slice0 + l) : ((size_t)l << logC) + crank)), in);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int l = l0 + i * kWorkThreads;
+                    if (l < hot_mine) Uk[DENSE ? (size_t)(slice0 + l) : ((size_t)l << logC) + crank] = P.model_out ? (W[l] - v[i]) * inv_sigma : W[l];
+                }
             }
             if (P.model_out)
-                for (size_t g = cold0 + ((size_t)wt << logC); g < (size_t)S.dim; g += (size_t)kWorkThreads << logC)
-                    Uk[g] = (__ldcg(Uk + g) - S.vbase[g]) * inv_sigma;
+                for (size_t g0 = cold0 + ((size_t)wt << logC); g0 < (size_t)S.dim; g0 += (size_t)(8 * kWorkThreads) << logC) {
+                    float u[8], v[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const size_t g = g0 + ((size_t)(i * kWorkThreads) << logC);
+                        const bool in = g < (size_t)S.dim;
+                        u[i] = ldcg_if(Uk + (in ? g : 0), in);
+                        v[i] = ldcg_if(S.vbase + (in ? g : 0), in);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const size_t g = g0 + ((size_t)(i * kWorkThreads) << logC);
+                        if (g < (size_t)S.dim) Uk[g] = (u[i] - v[i]) * inv_sigma;
+                    }
+                }
         }
     }
     if (is_worker || nb == 0) {
@@ -2116,7 +2232,8 @@ template <int LOSS, int NZ, int HT, int THREADS, int PER_SM> cudaError_t launch_
     cudaError_t e = cudaFuncSetAttribute(pre, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared));
     if (e != cudaSuccess) return e;
     const unsigned nb = (unsigned)P.n_blocks;
-    pre<<<nb < sms * PER_SM ? nb : sms * PER_SM, THREADS, sizeof(Shared), stream>>>(P);
+    const unsigned grid = nb < sms * PER_SM ? nb : sms * PER_SM;
+    pre<<<grid, THREADS, sizeof(Shared), stream>>>(P);
     return cudaGetLastError();
 }
 
@@ -2137,10 +2254,10 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
     const int chain_sms = g.K << g.la_logC;
     const unsigned free_sms = (unsigned)(g.sm_count > chain_sms ? g.sm_count - chain_sms : 1);
     if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) {
-        const unsigned per_sm = kPreDensePerSm;
+        const unsigned per_sm = g.dim > kDenseCols ? kPreDenseLongPerSm : kPreDensePerSm;
         const size_t smem = pre_dense_bytes((int)g.dim);
         const unsigned grid = stream == g.stream || nb < free_sms * per_sm ? nb : free_sms * per_sm;
-        auto pre = k_lookahead_prepare_dense<LOSS>;
+        auto pre = g.dim > kDenseCols ? k_lookahead_prepare_dense<LOSS, true> : k_lookahead_prepare_dense<LOSS, false>;
         cudaError_t e = cudaFuncSetAttribute(pre, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         pre<<<grid, kPreThreads, smem, stream>>>(P);
@@ -2176,6 +2293,13 @@ template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P, cud
     if (g.la_hotc == 0) return launch_chain<LOSS, kFlat, tables>(g, P, begun);
     if (((int64_t)g.la_hotc << g.la_logC) >= g.dim) return launch_chain<LOSS, kHot, tables>(g, P, begun);
     return launch_chain<LOSS, kCold, tables>(g, P, begun);
+}
+
+constexpr size_t kWordsPerLaunch = 480;
+struct WordArgs { int64_t w[kWordsPerLaunch]; };
+__global__ void k_words(const __grid_constant__ WordArgs a, int n, int64_t *dst)
+{
+    for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = a.w[i];
 }
 
 // A round's launches, slice after slice (consecutive pieces of every partition's walk). The first slice's prepare
@@ -2223,6 +2347,20 @@ template <int LOSS> cudaError_t launch_slices(Glm &g, std::vector<LookParams> &P
 
 } // namespace
 
+// A few words of host memory to the device: as arguments of a kernel (a copy from pageable memory costs the host 15 us, and
+// the stream waits for it); many of them as a copy, of which the runtime has taken its own when the call returns.
+cudaError_t launch_words(Glm &g, int64_t *dst, const int64_t *src, size_t n)
+{
+    if (n > 8 * kWordsPerLaunch) return cudaMemcpyAsync(dst, src, n * sizeof(int64_t), cudaMemcpyHostToDevice, g.stream);
+    for (size_t at = 0; at < n; at += kWordsPerLaunch) {
+        WordArgs a;
+        const size_t m = n - at < kWordsPerLaunch ? n - at : kWordsPerLaunch;
+        std::memcpy(a.w, src + at, m * sizeof(int64_t));
+        k_words<<<1, 256, 0, g.stream>>>(a, (int)m, dst + at);
+    }
+    return cudaGetLastError();
+}
+
 int lookahead_max_dense_dim() { return kMaxC * kDenseSlice; }
 int lookahead_max_slices() { return 64; }
 int64_t lookahead_max_dim() { return (int64_t)1 << kIdBits; }
@@ -2237,6 +2375,11 @@ void lookahead_plan(Glm &g, int32_t K)
     if (!dense) {
         // a cluster per partition, on at most half of the SMs: the prepare kernels need the rest
         while (logC < 3 && ((int64_t)K << (logC + 1)) * 2 <= g.sm_count) ++logC;
+        // Many partitions on a long vector with flat ids: all their models together (less what 32 000 words of shared memory each keep) are
+        // more than L2 holds, and gathers go to memory. With two CTAs per partition half of the partitions run at a time, each
+        // with twice the shared memory (ridge, 2 M columns over 350 000 rows, K = 128: 10 400 cycles a block instead of 26 400;
+        // step 14.3 -> 12.6 ms. Four: 6 170, but a quarter of the partitions at a time: 14.8 ms).
+        if (logC == 0 && !g.hot_variant && g.l2_bytes > 0 && g.dim > 32000 && (double)K * (double)(g.dim - 32000) * 4.0 > (double)g.l2_bytes) logC = 1;
         const char *env = getenv("CHICLE_LA_CLUSTER");
         if (env && env[0] >= '1' && env[0] <= '8' && env[1] == 0) {
             const int want = env[0] - '0';
@@ -2440,8 +2583,7 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
         for (int s = 1; s <= n; ++s) F.push_back((double)s / n);
     }
     const int Sn = (int)F.size() - 1;
-    // a pageable source: the runtime has taken its copy of these words when the call returns
-    cudaError_t e = cudaMemcpyAsync(g.la_slice, h.data(), h.size() * sizeof(int64_t), cudaMemcpyHostToDevice, g.stream);
+    cudaError_t e = launch_words(g, g.la_slice, h.data(), h.size());
     if (e != cudaSuccess) return e;
     const char *drop = getenv("CHICLE_TEST_DROP_RECORD"); // test aid: leave one block's records unpublished
     const size_t C = (size_t)1 << g.la_logC;

@@ -82,6 +82,9 @@ k_sqnorm(const int64_t *__restrict__ indptr, const float *__restrict__ values, i
 // ---------------------------------------------------------------------------------------- aggregation (a5)
 // v[j] += sum_k U[k][j] with k ascending and an fp64 accumulator; U is cleared for the next round; for ridge
 // the residual v - y that the next round's solvers gather from is refreshed in the same pass.
+// Eight rows' loads are issued before the first of them is cleared (the compiler cannot move a load over the store to
+// another row): 128 rows of 350 000 took 614 us, one memory round trip per row.
+constexpr int kReduceRows = 8;
 template <int VEC>
 __global__ void __launch_bounds__(kThreads)
 k_reduce_updates(float *__restrict__ v, float *__restrict__ U, int K, int64_t dim, const float *__restrict__ y,
@@ -96,17 +99,24 @@ k_reduce_updates(float *__restrict__ v, float *__restrict__ U, int K, int64_t di
         } else {
             acc[0] = v[i];
         }
-#pragma unroll 16
-        for (int k = 0; k < K; ++k) {
-            if (VEC == 4) {
-                float4 *p = reinterpret_cast<float4 *>(U + (size_t)k * dim) + i;
-                const float4 t = *p;
-                acc[0] += t.x; acc[1 % VEC] += t.y; acc[2 % VEC] += t.z; acc[3 % VEC] += t.w;
-                *p = make_float4(0.f, 0.f, 0.f, 0.f);
-            } else {
-                float *p = U + (size_t)k * dim + i;
-                acc[0] += *p;
-                *p = 0.f;
+        for (int k0 = 0; k0 < K; k0 += kReduceRows) {
+            float t[kReduceRows][VEC];
+#pragma unroll
+            for (int u = 0; u < kReduceRows; ++u) {
+                const float *p = U + (size_t)(k0 + u < K ? k0 + u : k0) * dim + (size_t)VEC * i;
+                if (VEC == 4) {
+                    const float4 f = __ldcs(reinterpret_cast<const float4 *>(p));
+                    t[u][0] = f.x; t[u][1 % VEC] = f.y; t[u][2 % VEC] = f.z; t[u][3 % VEC] = f.w;
+                } else t[u][0] = __ldcs(p);
+            }
+#pragma unroll
+            for (int u = 0; u < kReduceRows; ++u) {
+                if (k0 + u >= K) break;
+                float *p = U + (size_t)(k0 + u) * dim + (size_t)VEC * i;
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) acc[j] += t[u][j];
+                if (VEC == 4) *reinterpret_cast<float4 *>(p) = make_float4(0.f, 0.f, 0.f, 0.f);
+                else *p = 0.f;
             }
         }
         if (VEC == 4) {
@@ -132,11 +142,16 @@ k_sum_updates(float *__restrict__ U, int K, int64_t dim, float *__restrict__ del
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < dim; i += (int64_t)gridDim.x * blockDim.x) {
         double acc = 0.0;
-#pragma unroll 16
-        for (int k = 0; k < K; ++k) {
-            float *p = U + (size_t)k * dim + i;
-            acc += *p;
-            *p = 0.f;
+        for (int k0 = 0; k0 < K; k0 += kReduceRows) {
+            float t[kReduceRows];
+#pragma unroll
+            for (int u = 0; u < kReduceRows; ++u) t[u] = __ldcs(U + (size_t)(k0 + u < K ? k0 + u : k0) * dim + i);
+#pragma unroll
+            for (int u = 0; u < kReduceRows; ++u) {
+                if (k0 + u >= K) break;
+                acc += t[u];
+                U[(size_t)(k0 + u) * dim + i] = 0.f;
+            }
         }
         delta[i] = (float)acc;
     }
@@ -216,6 +231,7 @@ __device__ __forceinline__ void gap_term(double dot, float label, float state, d
 constexpr int kGapRows = CHICLE_GAP_ROWS;   // coordinates a warp has in flight
 constexpr int kGapChunks = 2; // 32-entry chunks per coordinate held in registers (longer ones loop)
 
+constexpr int kGapDenseStaged = 3072; // longest dense row whose shared vector is staged (24 KB)
 template <int LOSS>
 __global__ void __launch_bounds__(kThreads)
 k_gap_partials(const int64_t *__restrict__ indptr, const int32_t *__restrict__ indices,
@@ -225,6 +241,7 @@ k_gap_partials(const int64_t *__restrict__ indptr, const int32_t *__restrict__ i
 {
     __shared__ double sh[kThreads][2];
     __shared__ double sh2[kWarpsPerBlock][2];
+    __shared__ alignas(16) double sv[kGapDenseStaged];
     const double inv_lam_n = 1.0 / lam_n;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t nw = (int64_t)gridDim.x * kWarpsPerBlock;
@@ -319,6 +336,29 @@ k_gap_partials(const int64_t *__restrict__ indptr, const int32_t *__restrict__ i
                 dot = fma((double)x.w, (double)vec[4 * j4 + 3], dot);
             }
             gap_term<LOSS>(dot, labels[c], state[c], inv_lam_n, s0, s1);
+        }
+    } else if (dim <= kGapDenseStaged && (dim & 3) == 0) {
+        // longer dense rows: a warp per two rows, 128-bit loads, the shared vector in shared memory as doubles (converting it
+        // for every row again took as long as the rows: 100 000 rows of 500, 85 us)
+        for (int j = threadIdx.x; j < (int)dim; j += kThreads) sv[j] = (double)vec[j];
+        __syncthreads();
+        const int nv = (int)(dim >> 2);
+        for (int64_t c = 2 * gw; c < n_coord; c += 2 * nw) {
+            const bool two = c + 1 < n_coord;
+            const float4 *r0 = reinterpret_cast<const float4 *>(values + c * dim), *r1 = two ? r0 + nv : r0;
+            double d0 = 0.0, d1 = 0.0;
+#pragma unroll 4
+            for (int j = lane; j < nv; j += 32) {
+                const float4 x = __ldcs(r0 + j), y = __ldcs(r1 + j);
+                const double2 a = *reinterpret_cast<const double2 *>(sv + 4 * j), b = *reinterpret_cast<const double2 *>(sv + 4 * j + 2);
+                d0 = fma((double)x.x, a.x, d0); d1 = fma((double)y.x, a.x, d1);
+                d0 = fma((double)x.y, a.y, d0); d1 = fma((double)y.y, a.y, d1);
+                d0 = fma((double)x.z, b.x, d0); d1 = fma((double)y.z, b.x, d1);
+                d0 = fma((double)x.w, b.y, d0); d1 = fma((double)y.w, b.y, d1);
+            }
+            d0 = warp_sum_d(d0);
+            d1 = warp_sum_d(d1);
+            if (lane < (two ? 2 : 1)) gap_term<LOSS>(lane ? d1 : d0, labels[c + lane], state[c + lane], inv_lam_n, s0, s1);
         }
     } else {
         for (int64_t c = gw; c < n_coord; c += nw) {
@@ -631,7 +671,7 @@ k_gap_stream(const int64_t *__restrict__ indptr, const int32_t *__restrict__ ind
 
 template <int LOSS>
 __global__ void k_gap_final(const double *__restrict__ partials, int nblocks, double n, double lambda,
-                            double *__restrict__ out)
+                            double *__restrict__ out, const uint32_t *status, uint32_t *status_out)
 {
     // 4 warps, one per partial sum: lane l adds blocks l, l+32, ... in order, then the 32 lanes are added in order
     __shared__ double lanes[4][32];
@@ -661,6 +701,8 @@ __global__ void k_gap_final(const double *__restrict__ partials, int nblocks, do
         out[0] = primal - dual;
         out[1] = primal;
         out[2] = dual;
+        *status_out = *status;
+        __threadfence_system();
     }
 }
 
@@ -805,7 +847,7 @@ template <int LOSS> cudaError_t launch_gap_loss(Glm &g)
         k_gap_partials<LOSS><<<nb, kThreads, 0, g.stream>>>(g.indptr, g.indices, g.values, g.labels, g.alpha, g.v, g.v, g.n_coord,
                                                             g.dim, lam_n, g.gap_partials, g.d_status);
     }
-    k_gap_final<LOSS><<<1, 128, 0, g.stream>>>(g.gap_partials, nb, n, (double)g.lambda, g.gap_out);
+    k_gap_final<LOSS><<<1, 128, 0, g.stream>>>(g.gap_partials, nb, n, (double)g.lambda, g.h_gap, g.d_status, g.h_status);
     return cudaGetLastError();
 }
 
