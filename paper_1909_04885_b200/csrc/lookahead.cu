@@ -1040,7 +1040,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
 // issued before the first is used: three round trips to memory per block. (A warp per row, headers by its first lane, was
 // a chain of 24 of them: 72 000 cycles per block at 28 entries per row, with the tables.)
 constexpr int kPreThreads = 256;
-constexpr int kPreDensePerSm = 4, kPreDenseLongPerSm = 3;
+constexpr int kPreDensePerSm = 4, kPreDenseLongPerSm = 2;
 struct PreDenseShared {
     CHdr hdr[kLB];
     float gsc[2 * kLB], ys[kLB], as[kLB];
@@ -1050,13 +1050,125 @@ struct PreDenseShared {
     unsigned long long sub_off[kMaxC];
     alignas(16) float row[1];        // 64 rows of row_stride(columns at a time) floats: this block's, then the next block's
 };
-// Rows longer than this go through shared memory that many columns at a time.
-constexpr int kDenseCols = 64;
+// Longer rows go through shared memory this many columns at a time.
+constexpr int kDenseCols = 128;
+constexpr int kDenseLong = 64; // what counts as long
 // 16-byte pieces of consecutive rows lie on different banks
 __host__ __device__ constexpr int row_stride(int cols) { return (((cols + 3) / 4) | 1) * 4; }
 inline size_t pre_dense_bytes(int dim)
 {
-    return sizeof(PreDenseShared) + (dim > kDenseCols ? 2 : 1) * 2 * kLB * (size_t)row_stride(dim < kDenseCols ? dim : kDenseCols) * sizeof(float);
+    return sizeof(PreDenseShared) + (dim > kDenseLong ? 2 : 1) * 2 * kLB * (size_t)row_stride(dim < kDenseCols ? dim : kDenseCols) * sizeof(float);
+}
+
+// Rows of more than kDenseLong columns: they pass through shared memory that many columns at a time, fetched two pieces ahead
+// by asynchronous copies. Every warp takes every eighth four columns of a piece, a thread l = lp, lp + 4, .. and j = jq,
+// jq + 8, .. (8 x 8 sums; pairs of tiles below the triangle are left out), and the warps' sums are added in a fixed order.
+// Shared-memory loads bound it (a 16-byte load of a warp takes four turns whatever it broadcasts): 16 of them per 208
+// multiply-adds, against 48 with 2 x 4 sums per thread over all columns; that and loads through registers, a round trip exposed
+// for every piece, took 295 us for 100 000 rows of 500.
+__device__ __forceinline__ void dense_gram_long(const LookParams &P, PreDenseShared &sh, int cnt, bool walk, int stride)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int dim = (int)P.S.dim, slice = P.hotc;
+    constexpr int TPR = kDenseCols / 4, RPT = kPreThreads / TPR; // threads per row of a piece, rows per turn
+    const int sub = 4 * (tid % TPR), row0 = tid / TPR; // of a piece: this thread's four columns of rows row0, row0 + RPT, ..
+    float *const buf0 = sh.row, *const buf1 = sh.row + 2 * kLB * stride;
+    auto fetch = [&](int e0, float *to) {
+#pragma unroll
+        for (int i = 0; i < 2 * kLB / RPT; ++i) {
+            float *at = to + (row0 + RPT * i) * stride + sub;
+            if (e0 + sub >= dim) continue;
+            const int c = sh.coord[row0 + RPT * i];
+            const float *src = P.S.values + (int64_t)c * dim + (e0 + sub);
+            if (c < 0) *reinterpret_cast<float4 *>(at) = make_float4(0.f, 0.f, 0.f, 0.f);
+            else if ((dim & 3) == 0) cp_async16(smem_u32(at), src);
+            else
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (e0 + sub + u < dim) cp_async4(smem_u32(at + u), src + u);
+                    else at[u] = 0.0f;
+                }
+        }
+        cp_async_commit();
+    };
+    fetch(0, buf0);
+    if (kDenseCols < dim) fetch(kDenseCols, buf1);
+    else cp_async_commit();
+    // where this thread's columns go in the records: CTA c's, `left` columns from its slice's end
+    int c = 0, first = 0;
+    const int jq = lane & 7, lp = lane >> 3;
+    float acc[8][8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 8; ++b) acc[a][b] = 0.0f;
+#pragma unroll 1
+    for (int e0 = 0; e0 < dim; e0 += kDenseCols) {
+        const int cols = dim - e0 < kDenseCols ? dim - e0 : kDenseCols;
+        float *rows = (e0 / kDenseCols) & 1 ? buf1 : buf0;
+        cp_async_wait_but_one();
+        __syncthreads();
+        if (!walk && sub < cols) {
+            while (e0 + sub - first >= slice) { first += slice; ++c; }
+            const int st = dense_stride(dim - first < slice ? dim - first : slice);
+            float *to = reinterpret_cast<float *>(P.rec + sh.sub_off[c] + sizeof(SubHead)) + (e0 + sub - first); // (padding included)
+#pragma unroll
+            for (int i = 0; i < kLB / RPT; ++i)
+                if (row0 + RPT * i < cnt)
+                    *reinterpret_cast<float4 *>(to + (row0 + RPT * i) * st) = *reinterpret_cast<const float4 *>(rows + (row0 + RPT * i) * stride + sub);
+        }
+        const float *rl = rows + lp * stride, *rj = rows + jq * stride;
+#pragma unroll 1
+        for (int e = 4 * warp; e < cols; e += 4 * (kPreThreads / 32)) {
+            float4 xl[8];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) xl[a] = *reinterpret_cast<const float4 *>(rl + 4 * a * stride + e);
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                const float4 xj = *reinterpret_cast<const float4 *>(rj + 8 * b * stride + e);
+#pragma unroll
+                for (int a = 0; a < 8; ++a) {
+                    if (b < 4 && 4 * a >= 8 * (b + 1)) continue; // (every l of the tile lies beyond every j)
+                    acc[a][b] = fmaf(xj.x, xl[a].x, acc[a][b]);
+                    acc[a][b] = fmaf(xj.y, xl[a].y, acc[a][b]);
+                    acc[a][b] = fmaf(xj.z, xl[a].z, acc[a][b]);
+                    acc[a][b] = fmaf(xj.w, xl[a].w, acc[a][b]);
+                }
+            }
+        }
+        __syncthreads(); // the piece has been read
+        if (e0 + 2 * kDenseCols < dim) fetch(e0 + 2 * kDenseCols, rows);
+        else cp_async_commit();
+    }
+    // the warps' sums: 4 .. 7 to 0 .. 3, 2 and 3 to 0 and 1, 1 to 0 (every lane has the same places in every warp)
+    float4 *part = reinterpret_cast<float4 *>(sh.row);
+    static_assert(4 * 64 * 32 <= 2 * 2 * kLB * row_stride(kDenseLong), "four warps' sums fit the rows' buffers");
+#pragma unroll
+    for (int half = 4; half > 0; half >>= 1) {
+        if (warp >= half && warp < 2 * half) {
+#pragma unroll
+            for (int a = 0; a < 8; ++a)
+#pragma unroll
+                for (int b = 0; b < 2; ++b)
+                    part[((warp - half) * 16 + 2 * a + b) * 32 + lane] = make_float4(acc[a][4 * b], acc[a][4 * b + 1], acc[a][4 * b + 2], acc[a][4 * b + 3]);
+        }
+        __syncthreads();
+        if (warp < half) {
+#pragma unroll
+            for (int a = 0; a < 8; ++a)
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const float4 t = part[(warp * 16 + 2 * a + b) * 32 + lane];
+                    acc[a][4 * b] += t.x; acc[a][4 * b + 1] += t.y; acc[a][4 * b + 2] += t.z; acc[a][4 * b + 3] += t.w;
+                }
+        }
+        if (half > 1) __syncthreads();
+    }
+    if (warp == 0)
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+            for (int b = 0; b < 8; ++b) sh.T[lp + 4 * a][jq + 8 * b] = acc[a][b];
 }
 
 template <int LOSS, bool LONG> __device__ __forceinline__ void prepare_block_dense(const LookParams &P, const int64_t bid, PreDenseShared &sh)
@@ -1126,165 +1238,90 @@ template <int LOSS, bool LONG> __device__ __forceinline__ void prepare_block_den
             sh.as[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : hd.p1;
         }
     }
-    // ---- x_l . x_j for this block's l and the 64 columns j. This block's rows go into the workers' records on the
-    //      way. LONG rows pass through shared memory kDenseCols columns at a time, fetched two pieces ahead by asynchronous copies
-    //      (with registers on the way, 64 of them per thread, a load's round trip was exposed for every piece: 100 000 rows of
-    //      500 took 295 us); four groups of 64 threads take every fourth four columns, a thread l = lp, lp + 8, .. and j = jq,
-    //      jq + 8, .. (4 x 8 sums: 12 loads of 16 bytes per 128 multiply-adds, against 48; pairs of tiles that lie below the
-    //      triangle are left out), and the groups' sums are added in order. Short rows leave such groups nothing to share: 2 x 4 sums, l = lp, lp + 16, j = jq, jq + 16, ..
-    constexpr int TL = LONG ? 4 : 2, TJ = LONG ? 8 : 4, GL = kLB / TL, GJ = 2 * kLB / TJ, GROUPS = kPreThreads / (GL * GJ);
-    constexpr int RPW = 2 * kLB / NW; // rows a warp loads
-    {
-        const int jq = tid % GJ, lp = tid / GJ % GL, group = tid / (GL * GJ);
-        float acc[TL][TJ];
+    // ---- x_l . x_j for this block's l and the 64 columns j. This block's rows go into the workers' records on the way.
+    if (LONG) dense_gram_long(P, sh, cnt, walk, stride);
+    else {
+        // a thread has l = lp, lp + 16 and j = jq, jq + 16, .. (every sum over the entries in ascending order)
+        constexpr int RPW = 2 * kLB / NW; // rows a warp loads
+        const int jq = tid & 15, lp = tid >> 4, cols4 = (dim + 3) & ~3;
+        float acc[2][4];
 #pragma unroll
-        for (int a = 0; a < TL; ++a)
+        for (int a = 0; a < 2; ++a)
 #pragma unroll
-            for (int c = 0; c < TJ; ++c) acc[a][c] = 0.0f;
-        auto fetch = [&](int e0, float *to) { // (LONG) the 64 rows' columns e0 ..
-            const int cols = dim - e0 < kDenseCols ? dim - e0 : kDenseCols, cols4 = (cols + 3) & ~3;
-            constexpr int V = kDenseCols / 4;
-            if ((dim & 3) == 0) {
+            for (int c = 0; c < 4; ++c) acc[a][c] = 0.0f;
+        float *val_g = reinterpret_cast<float *>(P.rec + (walk ? 0 : sh.sub_off[0]) + sizeof(SubHead)); // (one CTA per partition)
+        const int st = dense_stride(dim);
+        if ((dim & 3) == 0) { // rows start on 16-byte boundaries
+            const int nv = dim >> 2;
+            const int lpr = nv <= 8 ? 8 : 16;                 // lanes per row
+            const int sub = lane & (lpr - 1), per = 32 / lpr; // rows per turn
+            float4 v[RPW];
 #pragma unroll
-                for (int i = tid; i < 2 * kLB * V; i += kPreThreads) {
-                    const int j = i / V, s = i % V, c = sh.coord[j];
-                    if (4 * s >= cols) continue;
-                    float *at = to + j * stride + 4 * s;
-                    if (c >= 0) cp_async16(smem_u32(at), P.S.values + (int64_t)c * dim + e0 + 4 * s);
-                    else *reinterpret_cast<float4 *>(at) = make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-            } else {
-#pragma unroll 4
-                for (int i = tid; i < 2 * kLB * kDenseCols; i += kPreThreads) {
-                    const int j = i / kDenseCols, s = i % kDenseCols, c = sh.coord[j];
-                    if (s >= cols4) continue;
-                    float *at = to + j * stride + s;
-                    if (c >= 0 && s < cols) cp_async4(smem_u32(at), P.S.values + (int64_t)c * dim + e0 + s);
-                    else *at = 0.0f;
+            for (int u = 0; u < RPW; ++u) {
+                const int j = warp * RPW + u * per + lane / lpr;
+                v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (u * per < RPW && sub < nv && sh.coord[j] >= 0)
+                    v[u] = reinterpret_cast<const float4 *>(P.S.values + (int64_t)sh.coord[j] * dim)[sub];
+            }
+#pragma unroll
+            for (int u = 0; u < RPW; ++u) {
+                const int j = warp * RPW + u * per + lane / lpr;
+                if (u * per < RPW && sub < nv) {
+                    reinterpret_cast<float4 *>(sh.row + j * stride)[sub] = v[u];
+                    if (j < cnt && !walk) reinterpret_cast<float4 *>(val_g + j * st)[sub] = v[u];
                 }
             }
-        };
-        if (LONG) {
-            fetch(0, sh.row);
-            cp_async_commit();
-            fetch(kDenseCols, sh.row + 2 * kLB * stride);
-            cp_async_commit();
-        }
-        for (int e0 = 0; e0 < dim; e0 += kDenseCols) {
-            const int cols = dim - e0 < kDenseCols ? dim - e0 : kDenseCols, cols4 = (cols + 3) & ~3;
-            float *rows = sh.row + (LONG && ((e0 / kDenseCols) & 1) ? 2 * kLB * stride : 0);
-            if (LONG) {
-                cp_async_wait_but_one();
-                __syncthreads();
-                if (!walk)
-#pragma unroll
-                    for (int i = tid; i < kLB * (kDenseCols / 4); i += kPreThreads) {
-                        const int j = i / (kDenseCols / 4), s = 4 * (i % (kDenseCols / 4)), e = e0 + s, c = e / slice;
-                        if (j < cnt && s < cols && c < C) // (with the zero padding)
-                            *reinterpret_cast<float4 *>(reinterpret_cast<float *>(P.rec + sh.sub_off[c] + sizeof(SubHead)) + j * dense_stride(cols_of(c)) + (e - c * slice)) =
-                                *reinterpret_cast<const float4 *>(rows + j * stride + s);
-                    }
-            } else if ((dim & 3) == 0) { // rows start on 16-byte boundaries (and so do slices)
-                const int nv = cols >> 2;
-                const int lpr = nv <= 8 ? 8 : (nv <= 16 ? 16 : 32); // lanes per row
-                const int sub = lane & (lpr - 1), per = 32 / lpr;   // rows per turn
-                float4 v[RPW];
+        } else {
+            for (int f = lane; f < cols4; f += 32) {
+                float v[RPW];
 #pragma unroll
                 for (int u = 0; u < RPW; ++u) {
-                    const int j = warp * RPW + u * per + lane / lpr;
-                    v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (u * per < RPW && sub < nv && sh.coord[j] >= 0)
-                        v[u] = reinterpret_cast<const float4 *>(P.S.values + (int64_t)sh.coord[j] * dim + e0)[sub];
+                    const int j = warp * RPW + u;
+                    v[u] = f < dim && sh.coord[j] >= 0 ? P.S.values[(int64_t)sh.coord[j] * dim + f] : 0.0f;
                 }
-                const int e = e0 + 4 * sub, c = e / slice;
-                float *val_g = reinterpret_cast<float *>(P.rec + (walk || c >= C ? 0 : sh.sub_off[c]) + sizeof(SubHead));
-                const int st = dense_stride(cols_of(c));
 #pragma unroll
                 for (int u = 0; u < RPW; ++u) {
-                    const int j = warp * RPW + u * per + lane / lpr;
-                    if (u * per < RPW && sub < nv) {
-                        reinterpret_cast<float4 *>(sh.row + j * stride)[sub] = v[u];
-                        if (j < cnt && !walk) *reinterpret_cast<float4 *>(val_g + j * st + (e - c * slice)) = v[u];
-                    }
+                    const int j = warp * RPW + u;
+                    sh.row[j * stride + f] = v[u];
+                    if (j < cnt && !walk) val_g[j * st + f] = v[u]; // (with the zero padding)
                 }
-            } else {
-                for (int f = lane; f < cols4; f += 32) {
-                    const int e = e0 + f, c = e / slice;
-                    float v[RPW];
-#pragma unroll
-                    for (int u = 0; u < RPW; ++u) {
-                        const int j = warp * RPW + u;
-                        v[u] = f < cols && sh.coord[j] >= 0 ? P.S.values[(int64_t)sh.coord[j] * dim + e] : 0.0f;
-                    }
-                    float *val_g = reinterpret_cast<float *>(P.rec + (walk || c >= C ? 0 : sh.sub_off[c]) + sizeof(SubHead));
-                    const int st = c < C ? dense_stride(cols_of(c)) : 0, padded = c < C ? (cols_of(c) + 3) & ~3 : 0;
-#pragma unroll
-                    for (int u = 0; u < RPW; ++u) {
-                        const int j = warp * RPW + u;
-                        sh.row[j * stride + f] = v[u];
-                        if (j < cnt && !walk && c < C && e - c * slice < padded) val_g[j * st + (e - c * slice)] = v[u]; // (with the zero padding)
-                    }
-                }
-            }
-            if (!LONG) __syncthreads();
-            if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins && !walk && e0 == 0) write_table(P, bid, sh.hdr, kPreThreads);
-            if (!walk) {
-                const float *rl = rows + lp * stride, *rj = rows + jq * stride;
-                for (int e = 4 * group; e < cols; e += 4 * GROUPS) {
-                    float4 xl[TL], xj[TJ];
-#pragma unroll
-                    for (int a = 0; a < TL; ++a) xl[a] = *reinterpret_cast<const float4 *>(rl + GL * a * stride + e);
-#pragma unroll
-                    for (int c = 0; c < TJ; ++c) xj[c] = *reinterpret_cast<const float4 *>(rj + GJ * c * stride + e);
-#pragma unroll
-                    for (int a = 0; a < TL; ++a)
-#pragma unroll
-                        for (int c = 0; c < TJ; ++c) {
-                            if (GJ * c < kLB && GL * a >= GJ * (c + 1)) continue; // (every l of the tile is at or beyond every j)
-                            acc[a][c] = fmaf(xj[c].x, xl[a].x, acc[a][c]);
-                            acc[a][c] = fmaf(xj[c].y, xl[a].y, acc[a][c]);
-                            acc[a][c] = fmaf(xj[c].z, xl[a].z, acc[a][c]);
-                            acc[a][c] = fmaf(xj[c].w, xl[a].w, acc[a][c]);
-                        }
-                }
-            }
-            if (LONG) {
-                __syncthreads(); // the piece has been read
-                if (e0 + 2 * kDenseCols < dim) fetch(e0 + 2 * kDenseCols, rows);
-                cp_async_commit();
             }
         }
-        if (LONG) { // the groups' sums together, in order (sh.T[l][j]: bank l + j, no two of a warp's threads on one)
-#pragma unroll 1
-            for (int r = GROUPS - 1; r >= 0; --r) {
-                if (r < GROUPS - 1) __syncthreads();
-                if (group != r) continue;
+        __syncthreads();
+        if (!walk) {
+            const float *rl = sh.row + lp * stride, *rj = sh.row + jq * stride;
+            for (int e = 0; e < dim; e += 4) {
+                float4 xl[2], xj[4];
 #pragma unroll
-                for (int a = 0; a < TL; ++a)
+                for (int a = 0; a < 2; ++a) xl[a] = *reinterpret_cast<const float4 *>(rl + 16 * a * stride + e);
 #pragma unroll
-                    for (int c = 0; c < TJ; ++c) {
-                        float &t = sh.T[lp + GL * a][jq + GJ * c];
-                        if (r < GROUPS - 1) acc[a][c] += t;
-                        if (r > 0) t = acc[a][c];
+                for (int c = 0; c < 4; ++c) xj[c] = *reinterpret_cast<const float4 *>(rj + 16 * c * stride + e);
+#pragma unroll
+                for (int a = 0; a < 2; ++a)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        acc[a][c] = fmaf(xj[c].x, xl[a].x, acc[a][c]);
+                        acc[a][c] = fmaf(xj[c].y, xl[a].y, acc[a][c]);
+                        acc[a][c] = fmaf(xj[c].z, xl[a].z, acc[a][c]);
+                        acc[a][c] = fmaf(xj[c].w, xl[a].w, acc[a][c]);
                     }
             }
         }
-        if (group == 0) {
 #pragma unroll
-            for (int a = 0; a < TL; ++a)
+        for (int a = 0; a < 2; ++a)
 #pragma unroll
-                for (int c = 0; c < TJ; ++c) {
-                    const int l = lp + GL * a, j = jq + GJ * c;
-                    const bool on = GJ * c < kLB ? l < j : l < cnt; // inside the block: earlier coordinates only
-                    sh.T[l][j] = on ? acc[a][c] * (sh.gsc[j] * sh.ys[l]) : 0.0f;
-                }
-        }
+            for (int c = 0; c < 4; ++c) sh.T[lp + 16 * a][jq + 16 * c] = acc[a][c];
+    }
+    if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins && !walk) write_table(P, bid, sh.hdr, kPreThreads);
+    __syncthreads();
+    for (int i = tid; i < 2 * kLB * kLB; i += kPreThreads) { // scaled; inside the block: earlier coordinates only
+        const int l = (i >> 5) & 31, j = (i & 31) + (i >= kLB * kLB ? kLB : 0);
+        const bool on = j < kLB ? l < j : l < cnt;
+        const float v = on && !walk ? sh.T[l][j] * (sh.gsc[j] * sh.ys[l]) : 0.0f;
+        sh.T[l][j] = v;
+        out.G[i] = v; // (X lies behind G)
     }
     __syncthreads();
-    for (int i = tid; i < kLB * kLB; i += kPreThreads) {
-        out.G[i] = sh.T[i / kLB][i % kLB];
-        out.X[i] = sh.T[i / kLB][kLB + i % kLB];
-    }
     for (int j = warp; j < 2 * kLB; j += NW) { // what the states at round start contribute
         float q0 = sh.T[lane][j] * sh.as[lane];
 #pragma unroll
@@ -2254,10 +2291,10 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
     const int chain_sms = g.K << g.la_logC;
     const unsigned free_sms = (unsigned)(g.sm_count > chain_sms ? g.sm_count - chain_sms : 1);
     if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) {
-        const unsigned per_sm = g.dim > kDenseCols ? kPreDenseLongPerSm : kPreDensePerSm;
+        const unsigned per_sm = g.dim > kDenseLong ? kPreDenseLongPerSm : kPreDensePerSm;
         const size_t smem = pre_dense_bytes((int)g.dim);
         const unsigned grid = stream == g.stream || nb < free_sms * per_sm ? nb : free_sms * per_sm;
-        auto pre = g.dim > kDenseCols ? k_lookahead_prepare_dense<LOSS, true> : k_lookahead_prepare_dense<LOSS, false>;
+        auto pre = g.dim > kDenseLong ? k_lookahead_prepare_dense<LOSS, true> : k_lookahead_prepare_dense<LOSS, false>;
         cudaError_t e = cudaFuncSetAttribute(pre, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         pre<<<grid, kPreThreads, smem, stream>>>(P);
