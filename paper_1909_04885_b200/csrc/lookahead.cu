@@ -58,7 +58,7 @@ constexpr int kDenseEasy = 128;    // and what it takes where the cluster may be
 // or the id itself (never below hotc, see k_lookahead_chain). Problems with more ids take the blocked solver.
 constexpr int kIdBits = 26;
 constexpr uint32_t kIdMask = (1u << kIdBits) - 1u;
-constexpr int kChainThreads = 352;
+constexpr int kChainThreads = 384;
 constexpr int kSubSlots = 4;       // worker records in shared memory: blocks b .. b + 3 (three of them where long records leave no room, see lookahead_plan)
 // Recurrence records in shared memory: a record is fetched when the block that many before it is done, and takes 1 500 cycles
 // or more from memory, so two would set the pace (1 M sparse rows: 3 019 cycles a block, with three 2 600). With tables of the logistic step
@@ -66,11 +66,13 @@ constexpr int kSubSlots = 4;       // worker records in shared memory: blocks b 
 constexpr int kMaxHeadSlots = 3;
 __host__ __device__ constexpr int head_slots(bool tables) { return tables ? 2 : 3; }
 // Worker warps: warps 1 .. 10 but for those that share warp 0's scheduler (warp ids 0, 4, 8), which stay out of its way.
+// Warps 4 and 11 of CTA 0 take from the recurrence warp all that is not the recurrence (see the kernel).
 constexpr int kWorkWarps = 8;
 constexpr int kWorkThreads = kWorkWarps * 32;
 constexpr int kBarWork = 1;        // named barrier of the worker warps
 constexpr int kRecordWarp = 8;     // fetches the workers' records
-constexpr int kFeedWarp = 4;       // in CTA 0: fetches the recurrence records and writes the new states (see the kernel)
+constexpr int kStartWarp = 4;      // in CTA 0: the states that a block's recurrence starts from
+constexpr int kFeedWarp = 11;      // in CTA 0: what follows from a block's recurrence; fetches the recurrence records
 
 // Per-step constants for the recurrence warp (see coordinate_step for p0 .. p3).
 struct alignas(16) CHdr {
@@ -392,26 +394,26 @@ __device__ __forceinline__ void write_table(const LookParams &P, int64_t bid, co
         out[2 * i + 1] = hi;
     }
 }
-// a(c) from the table. h = q / 2; `row`: where the coordinate's table would have a bin of exponent 0; `on`: whether this
-// lane's result is wanted (the other lanes keep off the shared-memory pipe).
-__device__ __forceinline__ float tab_map(float c, float h, float off, uint32_t row, uint32_t neg, bool on, float4 &lo, float4 &hi)
+// a(c) from the table, as sgn * v + bias: the caller multiplies sgn into what a(c) is multiplied with next while the look-up is
+// under way. d = c - q / 2; `row`: where the coordinate's table would have a bin of exponent 0; `on`: whether this lane's
+// result is wanted (the other lanes keep off the shared-memory pipe).
+__device__ __forceinline__ float tab_map(float d, float off, uint32_t row, uint32_t neg, bool on, float4 &lo, float4 &hi, float &sgn, float &bias)
 {
-    const float d = c - h;
     const float x = fmaxf(fmaf(-fabsf(d), kTabInv, off), kTabXmin);
     const float ax = fabsf(x), y = 1.0f + ax;
     const uint32_t bits = __float_as_uint(y);
-    const float dl = ax - (__uint_as_float((bits & 0xffe00000u) | 0x00100000u) - 1.0f);
     const uint32_t at = ((bits & 0xffe00000u) >> 16) + (x < 0.0f ? row + neg : row); // 32 bytes a bin
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %9, 0;\n\t"
                  "@q ld.shared.v4.f32 {%0, %1, %2, %3}, [%8];\n\t@q ld.shared.v4.f32 {%4, %5, %6, %7}, [%8 + 16];\n\t}"
                  : "+f"(lo.x), "+f"(lo.y), "+f"(lo.z), "+f"(lo.w), "+f"(hi.x), "+f"(hi.y), "+f"(hi.z), "+f"(hi.w)
                  : "r"(at), "r"((uint32_t)on));
+    sgn = d > 0.0f ? -1.0f : 1.0f;
+    // (a state that is not finite gives a result that is not, as the root search would)
+    bias = fmaf(0.0f, d, d > 0.0f ? 1.0f : 0.0f);
+    const float dl = ax - (__uint_as_float((bits & 0xffe00000u) | 0x00100000u) - 1.0f);
     const float d2 = dl * dl, d4 = d2 * d2;
     const float p01 = fmaf(lo.y, dl, lo.x), p23 = fmaf(lo.w, dl, lo.z), p45 = fmaf(hi.y, dl, hi.x), p67 = fmaf(hi.w, dl, hi.z);
-    const float v = fmaf(fmaf(p67, d2, p45), d4, fmaf(p23, d2, p01));
-    // (a state that is not finite gives a result that is not, as the root search would)
-    const float bias = fmaf(0.0f, c, d > 0.0f ? 1.0f : 0.0f);
-    return fmaf(v, d > 0.0f ? -1.0f : 1.0f, bias);
+    return fmaf(fmaf(p67, d2, p45), d4, fmaf(p23, d2, p01));
 }
 
 // The most frequent ids (ids are frequency-ranked) are in most of a block's coordinates. Their part of the Gram
@@ -1394,6 +1396,16 @@ __device__ __forceinline__ void mbar_arrive_expect_tx_if(uint32_t bar, uint32_t 
                  "r"(bytes), "r"((uint32_t)on)
                  : "memory");
 }
+__device__ __forceinline__ void mbar_arrive_if(uint32_t bar, bool on)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %1, 0;\n\t@q mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void sts_f32x4_if(uint32_t a, float x, float y, float z, float w, bool on)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %5, 0;\n\t@q st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n\t}" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w),
+                 "r"((uint32_t)on)
+                 : "memory");
+}
 __device__ __forceinline__ float ld_cluster_f32(uint32_t remote)
 {
     float v;
@@ -1476,7 +1488,10 @@ struct alignas(16) ChainCtl {
     uint64_t ackbar;               // CTA 0: every CTA has applied all updates (before a block is walked in place)
     alignas(16) float pbuf[2][kMaxC][kLB];
     alignas(16) float dbuf[2][kLB];
-    alignas(16) float sbuf[2][kLB]; // CTA 0: the block's new states (arrive with its deltas)
+    uint64_t ready[2];             // CTA 0: the states that a block's recurrence starts from are in `start`
+    uint64_t out[2];               // CTA 0: the recurrence's results are in `res`
+    alignas(16) float start[2][3][kLB]; // states; the scalar map's constants (p2 and lq; with tables lq alone)
+    alignas(16) float res[2][kLB];
     float sink[32]; // where a lane's stores go that have no target
     int walk[kSubSlots]; // whether the slot's block is walked in place
     int abort_flag;
@@ -1530,7 +1545,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     const int hot_mine = DENSE ? ((int)S.dim - slice0 < P.hotc ? ((int)S.dim > slice0 ? (int)S.dim - slice0 : 0) : P.hotc)
                                : (hot_total > crank ? (int)((hot_total - crank + C - 1) >> logC) : 0);
 
-    const uint32_t d_bytes = crank == 0 ? 2u * kLB * 4u : (uint32_t)kLB * 4u; // what a block's deltas (CTA 0: and states) bring
+    const uint32_t d_bytes = (uint32_t)kLB * 4u; // what a block's deltas bring
     if (tid == 0) {
         ctl.abort_flag = 0;
         ctl.done = 0;
@@ -1542,6 +1557,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&ctl.pbar[i]), 1);
             mbar_init(smem_u32(&ctl.dbar[i]), 1);
+            mbar_init(smem_u32(&ctl.ready[i]), 1);
+            mbar_init(smem_u32(&ctl.out[i]), 1);
         }
         mbar_init(smem_u32(&ctl.ackbar), (uint32_t)C);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1591,36 +1608,26 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
 
     constexpr int HS = head_slots(TAB);
     const bool is_chain = crank == 0 && warp == 0;
-    const bool is_worker = (warp & 3) != 0; // warps 1 2 3 5 6 7 9 10
+    const bool is_worker = (warp & 3) != 0 && warp != kFeedWarp; // warps 1 2 3 5 6 7 9 10
     bool aborted = false;
 
     if (is_chain && nb > 0) {
         // ============================== the recurrence warp =====================================================
-        const int q = lane & 7, rep = lane >> 3;
+        const int q = lane & 7;
         const uint32_t tab_neg = TAB ? (uint32_t)(P.tab_bins - kTabNeg) * 32u : 0u;
-        // where the deltas go: the copy `rep` of lane q sends the lane's four values to CTAs rep and rep + 4
-        uint32_t d_dst[2], d_bar[2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const uint32_t c = (uint32_t)(rep + 4 * i) & (uint32_t)(C - 1);
-            d_dst[i] = mapa_u32(smem_u32(&ctl.dbuf[0][4 * q]), c);
-            d_bar[i] = mapa_u32(smem_u32(&ctl.dbar[0]), c);
-        }
-        const uint32_t s_dst = smem_u32(&ctl.sbuf[0][4 * q]), s_bar = smem_u32(&ctl.dbar[0]); // (this CTA's own)
         float xs[4] = {0.f, 0.f, 0.f, 0.f}; // what the block before contributes to this block's states
-        int fp = 0, sc = 0;                // staged blocks and walked blocks so far
+        int sc = 0;                        // walked blocks so far
         int slot = 0;                      // b mod the head slots
-        uint32_t turn = 0;                 // parity of b / the head slots
 #ifdef CHICLE_LA_TIMING
         long long tw = 0, tr = 0, te = 0, t0 = clock64(), t1 = 0;
 #endif
 #pragma unroll 1
         for (int b = 0; b < nb; ++b) {
-            if (!mbar_wait_cluster(smem_u32(&ctl.headfull[slot]), turn, abort_flag, S.status)) { aborted = true; break; }
-            const ChainHead &H = *reinterpret_cast<const ChainHead *>(smem_chain + L.heads + (size_t)slot * sizeof(ChainHead));
-            const int cnt = H.cnt;
             const uint32_t par = (uint32_t)(b & 1);
+            if (!mbar_wait_cluster(smem_u32(&ctl.ready[0]) + 8u * par, (uint32_t)(b >> 1) & 1u, abort_flag, S.status)) { aborted = true; break; }
+            const ChainHead &H = *reinterpret_cast<const ChainHead *>(smem_chain + L.heads + (size_t)slot * sizeof(ChainHead));
             if (H.flags & 1) {
+                const int cnt = H.cnt;
                 // ---- walked in place: wait until every CTA has applied all earlier updates, then coordinate by
                 //      coordinate against the whole model (the other CTAs' parts through the cluster's shared memory)
                 if (!mbar_wait_cluster(smem_u32(&ctl.ackbar), (uint32_t)sc & 1u, abort_flag, S.status)) { aborted = true; break; }
@@ -1666,53 +1673,41 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                     if (lane == 0) S.alpha[h.coord] = new_state;
                     __syncwarp();
                 }
-                // the walk's writes before the signal; the signal is a block of zero deltas
+                // the walk's writes before the signal (the feeder sends a block of zero deltas)
                 __threadfence();
                 fence_cluster();
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-                    st_async_f32x4_if(d_dst[i] + par * (uint32_t)(kLB * 4), 0.f, 0.f, 0.f, 0.f, d_bar[i] + par * 8u, rep + 4 * i < C);
-                st_async_f32x4_if(s_dst + par * (uint32_t)(kLB * 4), 0.f, 0.f, 0.f, 0.f, s_bar + par * 8u, rep == 0);
                 xs[0] = xs[1] = xs[2] = xs[3] = 0.0f;
             } else {
                 // ---- four coordinates at a time. Lane q (and its copies q + 8, q + 16, q + 24, which compute the
                 //      same) keeps the states of coordinates 4q .. 4q + 3. Group g: its lane walks its four coordinates
                 //      by itself, the four results are handed round, and every lane adds what they mean for its own
                 //      four, in this block and in the next.
-                float hp1[4], hp2[4], hp3[4], hlq[4], s[4], mine[4];
-                float hA[4], hB[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const CHdr &h = H.hdr[4 * q + i];
-                    hp1[i] = h.p1; hp2[i] = h.p2; hp3[i] = h.p3; hlq[i] = h.lq; hA[i] = h.A; hB[i] = h.B;
-                    mine[i] = 0.0f;
-                }
-                // with tables: half of q, and where each coordinate's table would have exponent 0
+                const uint32_t st0 = smem_u32(&ctl.start[0][0][0]) + par * (uint32_t)sizeof(ctl.start[0]) + 16u * (uint32_t)q;
+                const uint32_t res = smem_u32(&ctl.res[0][0]) + par * (uint32_t)(kLB * 4);
+                const float4 s0 = lds_f32x4(st0);
+                float4 k2 = make_float4(0.f, 0.f, 0.f, 0.f), k3 = k2;
+                if (LOSS != CHICLE_LOSS_HINGE_DUAL && !TAB) k2 = lds_f32x4(st0 + 128u);
+                if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL) k3 = lds_f32x4(st0 + 256u);
+                const float4 q0n = *reinterpret_cast<const float4 *>(&H.q0n[4 * q]);
+                const float hp2[4] = {k2.x, k2.y, k2.z, k2.w}, hlq[4] = {k3.x, k3.y, k3.z, k3.w};
+                float s[4] = {s0.x + xs[0], s0.y + xs[1], s0.z + xs[2], s0.w + xs[3]};
+                xs[0] = -q0n.x; xs[1] = -q0n.y; xs[2] = -q0n.z; xs[3] = -q0n.w;
+                // with tables: where each coordinate's table would have exponent 0
                 uint32_t row[4];
                 if (TAB) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        hp2[i] *= 0.5f;
+                    for (int i = 0; i < 4; ++i)
                         row[i] = smem_u32(smem_chain + L.tabs) + (uint32_t)slot * tab_bytes(P.tab_bins) + (uint32_t)((4 * q + i) * P.tab_bins) * 32u - (127u << 2) * 32u;
-                    }
                 }
                 float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo; // (the lanes whose result nobody wants keep what is there)
-                auto step_map = [&](float st, int i, bool on) {
-                    return TAB ? tab_map(st, hp2[i], hlq[i], row[i], tab_neg, on, lo, hi) : recurrence_map<LOSS>(st, hp2[i], hlq[i]);
+                // a state's result is sgn * v + bias (sgn = 1, bias = 0 without tables)
+                auto step_map = [&](float st, int i, bool on, float &sgn, float &bias) {
+                    if (TAB) return tab_map(st, hlq[i], row[i], tab_neg, on, lo, hi, sgn, bias);
+                    sgn = 1.0f;
+                    bias = 0.0f;
+                    return recurrence_map<LOSS>(st, hp2[i], hlq[i]);
                 };
-                const float4 q0n = *reinterpret_cast<const float4 *>(&H.q0n[4 * q]);
-                if (!mbar_wait_cluster(smem_u32(&ctl.pbar[fp & 1]), (uint32_t)(fp >> 1) & 1u, abort_flag, S.status)) { aborted = true; break; }
                 LA_T(tw);
-                float m0[4] = {0.f, 0.f, 0.f, 0.f};
-                for (int c = 0; c < C; ++c) { // the CTAs' partial sums in a fixed order
-                    const float4 pv = *reinterpret_cast<const float4 *>(&ctl.pbuf[fp & 1][c][4 * q]);
-                    m0[0] += pv.x; m0[1] += pv.y; m0[2] += pv.z; m0[3] += pv.w;
-                }
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < 4; ++i) s[i] = fmaf(hB[i], m0[i], hA[i]) + xs[i];
-                xs[0] = -q0n.x; xs[1] = -q0n.y; xs[2] = -q0n.z; xs[3] = -q0n.w;
                 const float4 *G4 = reinterpret_cast<const float4 *>(H.G); // G4[l * 8 + q]: row l, columns 4q .. 4q + 3
                 const float4 *X4 = reinterpret_cast<const float4 *>(H.X);
                 // (how far this is unrolled was measured: the code of the block loop has to stay near the instruction cache's
@@ -1728,16 +1723,21 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                     }
                     // inside the group (the numbers matter on the lanes with q == g, where blk holds the group's own
                     // triangle; the others run the same instructions on copies)
-                    float o[4];
-                    o[0] = step_map(s[0], 0, q == g);
-                    const float t1 = fmaf(o[0], blk[0].y, s[1]);
-                    o[1] = step_map(t1, 1, q == g);
-                    const float t2 = fmaf(o[1], blk[1].z, fmaf(o[0], blk[0].z, s[2]));
-                    o[2] = step_map(t2, 2, q == g);
-                    const float t3 = fmaf(o[2], blk[2].w, fmaf(o[1], blk[1].w, fmaf(o[0], blk[0].w, s[3])));
-                    o[3] = step_map(t3, 3, q == g);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) mine[i] = q == g ? o[i] : mine[i];
+                    float o[4], v, sg, bi;
+                    v = step_map(s[0], 0, q == g, sg, bi);
+                    o[0] = TAB ? fmaf(v, sg, bi) : v;
+                    const float t1 = TAB ? fmaf(v, sg * blk[0].y, fmaf(bi, blk[0].y, s[1])) : fmaf(v, blk[0].y, s[1]);
+                    v = step_map(t1, 1, q == g, sg, bi);
+                    o[1] = TAB ? fmaf(v, sg, bi) : v;
+                    const float u2 = fmaf(o[0], blk[0].z, s[2]);
+                    const float t2 = TAB ? fmaf(v, sg * blk[1].z, fmaf(bi, blk[1].z, u2)) : fmaf(v, blk[1].z, u2);
+                    v = step_map(t2, 2, q == g, sg, bi);
+                    o[2] = TAB ? fmaf(v, sg, bi) : v;
+                    const float u3 = fmaf(o[1], blk[1].w, fmaf(o[0], blk[0].w, s[3]));
+                    const float t3 = TAB ? fmaf(v, sg * blk[2].w, fmaf(bi, blk[2].w, u3)) : fmaf(v, blk[2].w, u3);
+                    v = step_map(t3, 3, q == g, sg, bi);
+                    o[3] = TAB ? fmaf(v, sg, bi) : v;
+                    sts_f32x4_if(res + 16u * (uint32_t)g, o[0], o[1], o[2], o[3], lane == g);
                     float og[4];
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) og[kk] = __shfl_sync(0xffffffffu, o[kk], g);
@@ -1755,45 +1755,11 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                     }
                 }
                 LA_T(tr);
-                if (TAB) { // (not kept in registers over the steps)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const CHdr &h = H.hdr[4 * q + i];
-                        hp1[i] = h.p1; hp3[i] = h.p3;
-                    }
-                }
-                float dl[4], st[4];
-                bool odd = false; // a step that is not finite
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const bool in = 4 * q + i < cnt;
-                    if (LOSS == CHICLE_LOSS_RIDGE_PRIMAL) {
-                        dl[i] = mine[i];
-                        st[i] = hp1[i] + mine[i];
-                    } else {
-                        dl[i] = hp3[i] * (mine[i] - hp1[i]);
-                        st[i] = hp3[i] * mine[i];
-                    }
-                    const bool fine = fabsf(dl[i]) <= CUDART_MAX_NORMAL_F;
-                    odd |= in && !fine;
-                    if (!fine) st[i] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? hp1[i] : hp3[i] * hp1[i];
-                    if (!in || !fine) dl[i] = 0.0f;
-                }
-                // armed for block fp + 2 before the deltas go out (its dot products are sent only after they arrive)
-                mbar_arrive_expect_tx_if(smem_u32(&ctl.pbar[fp & 1]), (uint32_t)(C * kLB * 4), lane == 0);
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-                    st_async_f32x4_if(d_dst[i] + par * (uint32_t)(kLB * 4), dl[0], dl[1], dl[2], dl[3], d_bar[i] + par * 8u, rep + 4 * i < C);
-                st_async_f32x4_if(s_dst + par * (uint32_t)(kLB * 4), st[0], st[1], st[2], st[3], s_bar + par * 8u, rep == 0);
-                ++fp;
-                if (__any_sync(0xffffffffu, odd) && lane == 0) atomicOr(S.status, ST_NONFINITE_STEP);
-                LA_T(te);
             }
             __syncwarp();
-            if (++slot == HS) {
-                slot = 0;
-                turn ^= 1u;
-            }
+            mbar_arrive_if(smem_u32(&ctl.out[0]) + 8u * par, lane == 0);
+            LA_T(te);
+            slot = slot + 1 == HS ? 0 : slot + 1;
         }
 #ifdef CHICLE_LA_TIMING
         if (blockIdx.x == 0 && lane == 0) {
@@ -1802,11 +1768,51 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         }
 #endif
     }
+    if (crank == 0 && warp == kStartWarp && nb > 0) {
+        // ============================== what a block's recurrence starts from =======================================
+        // A lane per coordinate: once the block's dot products are here (with tables: less half of q, see tab_map). In the
+        // recurrence warp itself, which keeps four coordinates per lane, this and what the feeder does took 1 090 cycles a
+        // block, most of them instruction fetches of code that runs once.
+        int fp = 0, slot = 0; // staged blocks so far; blk mod the head slots
+        uint32_t turn = 0;    // parity of blk / the head slots
+#pragma unroll 1
+        for (int blk = 0; blk < nb; ++blk) {
+            const uint32_t par = (uint32_t)(blk & 1);
+            // (a block walked in place waits for no dot products: not before the recurrence is through with `start`)
+            if (blk >= 2 && !mbar_wait_cluster(smem_u32(&ctl.out[0]) + 8u * par, (uint32_t)((blk >> 1) - 1) & 1u, abort_flag, S.status)) break;
+            if (!mbar_wait_cluster(smem_u32(&ctl.headfull[slot]), turn, abort_flag, S.status)) break;
+            const ChainHead &H = *reinterpret_cast<const ChainHead *>(smem_chain + L.heads + (size_t)slot * sizeof(ChainHead));
+            if (!(H.flags & 1)) {
+                const CHdr h = H.hdr[lane];
+                if (!mbar_wait_cluster(smem_u32(&ctl.pbar[fp & 1]), (uint32_t)(fp >> 1) & 1u, abort_flag, S.status)) break;
+                float m0 = 0.0f;
+                for (int c = 0; c < C; ++c) m0 += ctl.pbuf[fp & 1][c][lane]; // the CTAs' partial sums in a fixed order
+                ++fp;
+                const float s0 = fmaf(h.B, m0, h.A);
+                ctl.start[par][0][lane] = TAB ? s0 - 0.5f * h.p2 : s0;
+                ctl.start[par][1][lane] = h.p2;
+                ctl.start[par][2][lane] = h.lq;
+            }
+            __syncwarp();
+            mbar_arrive_if(smem_u32(&ctl.ready[0]) + 8u * par, lane == 0);
+            if (++slot == HS) {
+                slot = 0;
+                turn ^= 1u;
+            }
+        }
+    }
     if (crank == 0 && warp == kFeedWarp && nb > 0) {
-        // ============================== the feeder: what the recurrence warp need not do itself =====================
-        // When a block's deltas have arrived here, the recurrence warp is done with the block's head: its new states go
-        // to global memory and the head (and table) HS blocks on into its slot. (The recurrence warp waits for that
-        // head before it sends deltas on this barrier again, so the feeder never misses a phase.)
+        // ============================== the feeder: what follows from a block's recurrence ===========================
+        // Deltas to all CTAs' workers, the new states to global memory, and the head (and table) HS blocks on into the slot.
+        const int q = lane & 7, rep = lane >> 3;
+        // the copy `rep` of lane q sends four values to CTAs rep and rep + 4
+        uint32_t d_dst[2], d_bar[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t c = (uint32_t)(rep + 4 * i) & (uint32_t)(C - 1);
+            d_dst[i] = mapa_u32(smem_u32(&ctl.dbuf[0][4 * q]), c);
+            d_bar[i] = mapa_u32(smem_u32(&ctl.dbar[0]), c);
+        }
         const uint32_t tab_len = TAB ? tab_bytes(P.tab_bins) : 0u;
         const uint32_t heads0 = smem_u32(smem_chain + L.heads), tabs0 = smem_u32(smem_chain + L.tabs);
         auto issue_head = [&](int blk, int slot) {
@@ -1818,13 +1824,44 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             if (TAB) bulk_g2s_if(tabs0 + (uint32_t)slot * tab_len, P.rec + P.tab_off + at * tab_len, tab_len, bar, on);
         };
         for (int i = 0; i < HS; ++i) issue_head(i, i);
-        int slot = 0;
+        int fp = 0, slot = 0;
 #pragma unroll 1
         for (int b = 0; b < nb; ++b) {
-            if (!mbar_wait_cluster(smem_u32(&ctl.dbar[b & 1]), (uint32_t)(b >> 1) & 1u, abort_flag, S.status)) break;
+            const uint32_t par = (uint32_t)(b & 1);
+            if (!mbar_wait_cluster(smem_u32(&ctl.out[0]) + 8u * par, (uint32_t)(b >> 1) & 1u, abort_flag, S.status)) break;
             const ChainHead &H = *reinterpret_cast<const ChainHead *>(smem_chain + L.heads + (size_t)slot * sizeof(ChainHead));
-            const int32_t c = H.hdr[lane].coord;
-            if (lane < H.cnt && !(H.flags & 1) && CHICLE_IN_BOUNDS(S.status, c >= 0 && (int64_t)c < S.n_coord)) S.alpha[c] = ctl.sbuf[b & 1][lane];
+            const bool walked = (H.flags & 1) != 0;
+            float dl = 0.0f, st = 0.0f;
+            bool odd = false; // a step that is not finite
+            int32_t coord = -1;
+            if (!walked) {
+                const CHdr h = H.hdr[lane];
+                const float o = ctl.res[par][lane];
+                const bool in = lane < H.cnt;
+                if (LOSS == CHICLE_LOSS_RIDGE_PRIMAL) {
+                    dl = o;
+                    st = h.p1 + o;
+                } else {
+                    dl = h.p3 * (o - h.p1);
+                    st = h.p3 * o;
+                }
+                const bool fine = fabsf(dl) <= CUDART_MAX_NORMAL_F;
+                odd = in && !fine;
+                if (!fine) st = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? h.p1 : h.p3 * h.p1;
+                if (!in || !fine) dl = 0.0f;
+                coord = in ? h.coord : -1;
+                // armed for block fp + 2 before the deltas go out (its dot products are sent only after they arrive)
+                mbar_arrive_expect_tx_if(smem_u32(&ctl.pbar[fp & 1]), (uint32_t)(C * kLB * 4), lane == 0);
+                ++fp;
+            } else fence_cluster(); // (the walk's ordinary stores go before the signal)
+            float d4[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) d4[i] = __shfl_sync(0xffffffffu, dl, 4 * q + i);
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                st_async_f32x4_if(d_dst[i] + par * (uint32_t)(kLB * 4), d4[0], d4[1], d4[2], d4[3], d_bar[i] + par * 8u, rep + 4 * i < C);
+            if (coord >= 0 && CHICLE_IN_BOUNDS(S.status, (int64_t)coord < S.n_coord)) S.alpha[coord] = st;
+            if (__any_sync(0xffffffffu, odd) && lane == 0) atomicOr(S.status, ST_NONFINITE_STEP);
             __syncwarp();
             issue_head(b + HS, slot);
             slot = slot + 1 == HS ? 0 : slot + 1;
