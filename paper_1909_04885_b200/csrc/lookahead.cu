@@ -1956,6 +1956,30 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         bool sl0 = false, sl1 = false; // whether blocks b and b + 1 are walked in place
 #pragma unroll 1
         for (int b = nb > 0 ? -depth : 0; b < nb; ++b) {
+            bool sl2 = false, due = b + depth < nb, late = false;
+            // the record of the block whose dot products are next: whether it is walked in place
+            auto dot_record = [&]() {
+                if (!due) return;
+                ok = ok && mbar_wait_cluster(smem_u32(&ctl.subfull[0]) + 8u * s_dot, dot_turn, abort_flag, S.status);
+                sl2 = lds_s32(smem_u32(&ctl.walk[0]) + 4u * s_dot) != 0;
+                due = !sl2;
+            };
+            // Dense rows: a thread's part of both records is fetched before the deltas are waited for, so that these loads, the
+            // waits and the barrier are under way together (11 M logistic rows of 28: 25.5 -> 24.1 ms).
+            float xu[DENSE ? kLB : 1];
+            float4 xd[4];
+            if (DENSE) {
+                dot_record();
+                const uint32_t row = r_dot + (uint32_t)sizeof(SubHead) + 4u * (uint32_t)(jd * dstride), at = r_upd + (uint32_t)sizeof(SubHead) + 4u * (uint32_t)wt;
+                const bool up = b >= 0 && !sl0 && ok && wt < hot_mine && lds_s32(r_upd + 12u) == kLB, dot = ok && due && jd < lds_s32(r_dot + 12u);
+                if (up) // (few warps have columns)
+#pragma unroll
+                    for (int j = 0; j < kLB; ++j) xu[DENSE ? j : 0] = lds_f32(at + 4u * (uint32_t)(j * dstride));
+                if (dot)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) // (the row's first piece stands in for those it does not have)
+                        xd[i] = lds_f32x4(row + (qd + 8 * i < (hot_mine + 3) >> 2 ? 16u * (uint32_t)(qd + 8 * i) : 0u));
+            }
             if (b >= 0) {
                 const uint32_t par = (uint32_t)(b & 1), dbar = smem_u32(&ctl.dbar[0]) + 8u * par;
                 if (sl0) {
@@ -1981,7 +2005,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                             if (head.w == kLB) { // all loads first
                                 float x[kLB];
 #pragma unroll
-                                for (int j = 0; j < kLB; ++j) x[j] = lds_f32(at + (uint32_t)j * row);
+                                for (int j = 0; j < kLB; ++j) x[j] = xu[DENSE ? j : 0];
+                                if (col != wt)
+#pragma unroll
+                                    for (int j = 0; j < kLB; ++j) x[j] = lds_f32(at + (uint32_t)j * row);
 #pragma unroll
                                 for (int j = 0; j < kLB; j += 4) {
                                     const float4 d = lds_f32x4(dl + 4u * j);
@@ -2074,12 +2101,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             }
             // ---- dot products: of block b + depth against the model as it is now. A block right behind a walked one starts
             //      from the model as the walk left it: with depth 2 its products wait for that.
-            bool sl2 = false, due = b + depth < nb, late = false;
-            if (due) {
-                ok = ok && mbar_wait_cluster(smem_u32(&ctl.subfull[0]) + 8u * s_dot, dot_turn, abort_flag, S.status);
-                sl2 = lds_s32(smem_u32(&ctl.walk[0]) + 4u * s_dot) != 0;
-                due = !sl2;
-            }
+            if (!DENSE) dot_record();
             if (sl0 || sl1) {
                 late = depth == 2 && sl0 && !sl1 && b + 1 < nb;
                 due = due && (depth == 1 || !sl1);
@@ -2095,6 +2117,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             while (ok && (late || due)) {
                 // (block b + 1's record lies in the slot before block b + 2's)
                 const uint32_t rec = !late ? r_dot : (r_dot == subs0 ? subs_end : r_dot) - stride, val = rec + (uint32_t)sizeof(SubHead);
+                const bool fetched = !late;
                 if (late) late = false;
                 else due = false;
                 const int4 head = lds_s32x4(rec); // n, T, nl, cnt
@@ -2112,8 +2135,21 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                     if (jd < head.w) {
                         const uint32_t row = val + 4u * (uint32_t)(jd * dstride);
                         float acc1 = 0.0f;
+                        const int pieces = (hot_mine + 3) >> 2;
+                        int e = qd;
+                        if (fetched) {
+                            float4 w[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) w[i] = lds_f32x4(a_w + (qd + 8 * i < pieces ? 16u * (uint32_t)(qd + 8 * i) : 0u));
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                if (qd + 8 * i >= pieces) break;
+                                acc = fmaf(xd[i].x, w[i].x, acc); acc1 = fmaf(xd[i].y, w[i].y, acc1); acc = fmaf(xd[i].z, w[i].z, acc); acc1 = fmaf(xd[i].w, w[i].w, acc1);
+                            }
+                            e = qd + 32;
+                        }
 #pragma unroll 4
-                        for (int e = qd; e < (hot_mine + 3) >> 2; e += 8) {
+                        for (; e < pieces; e += 8) {
                             const float4 a = lds_f32x4(row + 16u * e), w = lds_f32x4(a_w + 16u * e);
                             acc = fmaf(a.x, w.x, acc); acc1 = fmaf(a.y, w.y, acc1); acc = fmaf(a.z, w.z, acc); acc1 = fmaf(a.w, w.w, acc1);
                         }
