@@ -1054,15 +1054,18 @@ struct PreDenseShared {
 };
 // Longer rows go through shared memory this many columns at a time.
 constexpr int kDenseCols = 128;
-constexpr int kDenseLong = 64; // what counts as long
+// What counts as long: more columns than this, or half as many where there are more blocks than the kernel for short rows
+// takes at once (10 000 rows of 100, 313 blocks: 14 us against 20; with many blocks the other one's fewer loads count).
+constexpr int kDenseLong = 128;
+inline bool dense_long(int64_t dim, int64_t blocks, int sms) { return dim > kDenseLong || (2 * dim > kDenseLong && blocks > (int64_t)sms * kPreDensePerSm); }
 // 16-byte pieces of consecutive rows lie on different banks
 __host__ __device__ constexpr int row_stride(int cols) { return (((cols + 3) / 4) | 1) * 4; }
-inline size_t pre_dense_bytes(int dim)
+inline size_t pre_dense_bytes(int dim, bool lng)
 {
-    return sizeof(PreDenseShared) + (dim > kDenseLong ? 2 : 1) * 2 * kLB * (size_t)row_stride(dim < kDenseCols ? dim : kDenseCols) * sizeof(float);
+    return sizeof(PreDenseShared) + (lng ? 2 : 1) * 2 * kLB * (size_t)row_stride(dim < kDenseCols ? dim : kDenseCols) * sizeof(float);
 }
 
-// Rows of more than kDenseLong columns: they pass through shared memory that many columns at a time, fetched two pieces ahead
+// Long rows (see dense_long): they pass through shared memory that many columns at a time, fetched two pieces ahead
 // by asynchronous copies. Every warp takes every eighth four columns of a piece, a thread l = lp, lp + 4, .. and j = jq,
 // jq + 8, .. (8 x 8 sums; pairs of tiles below the triangle are left out), and the warps' sums are added in a fixed order.
 // Shared-memory loads bound it (a 16-byte load of a warp takes four turns whatever it broadcasts): 16 of them per 208
@@ -1144,7 +1147,7 @@ __device__ __forceinline__ void dense_gram_long(const LookParams &P, PreDenseSha
     }
     // the warps' sums: 4 .. 7 to 0 .. 3, 2 and 3 to 0 and 1, 1 to 0 (every lane has the same places in every warp)
     float4 *part = reinterpret_cast<float4 *>(sh.row);
-    static_assert(4 * 64 * 32 <= 2 * 2 * kLB * row_stride(kDenseLong), "four warps' sums fit the rows' buffers");
+    static_assert(4 * 64 * 32 <= 2 * 2 * kLB * row_stride(kDenseLong / 2), "four warps' sums fit the rows' buffers");
 #pragma unroll
     for (int half = 4; half > 0; half >>= 1) {
         if (warp >= half && warp < 2 * half) {
@@ -1255,7 +1258,7 @@ template <int LOSS, bool LONG> __device__ __forceinline__ void prepare_block_den
         const int st = dense_stride(dim);
         if ((dim & 3) == 0) { // rows start on 16-byte boundaries
             const int nv = dim >> 2;
-            const int lpr = nv <= 8 ? 8 : 16;                 // lanes per row
+            const int lpr = nv <= 8 ? 8 : (nv <= 16 ? 16 : 32); // lanes per row
             const int sub = lane & (lpr - 1), per = 32 / lpr; // rows per turn
             float4 v[RPW];
 #pragma unroll
@@ -2364,10 +2367,11 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
     const int chain_sms = g.K << g.la_logC;
     const unsigned free_sms = (unsigned)(g.sm_count > chain_sms ? g.sm_count - chain_sms : 1);
     if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) {
-        const unsigned per_sm = g.dim > kDenseLong ? kPreDenseLongPerSm : kPreDensePerSm;
-        const size_t smem = pre_dense_bytes((int)g.dim);
+        const bool lng = dense_long(g.dim, nb, g.sm_count);
+        const unsigned per_sm = lng ? kPreDenseLongPerSm : kPreDensePerSm;
+        const size_t smem = pre_dense_bytes((int)g.dim, lng);
         const unsigned grid = stream == g.stream || nb < free_sms * per_sm ? nb : free_sms * per_sm;
-        auto pre = g.dim > kDenseLong ? k_lookahead_prepare_dense<LOSS, true> : k_lookahead_prepare_dense<LOSS, false>;
+        auto pre = lng ? k_lookahead_prepare_dense<LOSS, true> : k_lookahead_prepare_dense<LOSS, false>;
         cudaError_t e = cudaFuncSetAttribute(pre, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         pre<<<grid, kPreThreads, smem, stream>>>(P);
