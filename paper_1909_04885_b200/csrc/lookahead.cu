@@ -131,7 +131,6 @@ constexpr int kHot = 0, kCold = 1, kFlat = 2, kDense = 3;
 struct LookParams {
     SolverParams S;
     unsigned char *rec;          // this launch's region of the record buffer
-    BlkDir *dirH;                // one per block: the recurrence warp's record
     BlkDir *dirS;                // C per block: the workers' records
     unsigned long long *cursor;  // bytes of the pool handed out so far in this launch
     unsigned long long *timing;  // scratch words of a -DCHICLE_LA_TIMING build
