@@ -558,10 +558,10 @@ template <int LOSS, int NZ, int HT, class Shared> __device__ __forceinline__ voi
     B.ys[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 1.0f : hd.p3;
     B.as[lane] = LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : hd.p1;
     {
-        // |x| < 2^e for e = (exponent of |x|^2 + 2) / 2, rounded down
+        // |x| < 2^e for e = (exponent of |x|^2 + 2) / 2, rounded down (subnormal squares: the exponent of their first bit)
         const uint32_t bits = c >= 0 ? __float_as_uint(sh.sq[lane]) : 0u;
-        const int ex = (int)(bits >> 23) - 127, e = (ex + 2) >> 1;
-        const bool usable = ex > -127 && ex < 128;
+        const int ex = bits >> 23 ? (int)(bits >> 23) - 127 : -118 - __clz((int)bits), e = (ex + 2) >> 1;
+        const bool usable = bits != 0u && ex < 128;
         B.scl[lane] = usable ? __uint_as_float((uint32_t)(127 + 15 - e) << 23) : 0.0f;
         B.inv[lane] = usable ? __uint_as_float((uint32_t)(127 - 15 + e) << 23) : 0.0f;
     }
@@ -1005,17 +1005,18 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 }
             }
             float qg = 0.0f, qx = 0.0f;
+            // (the two inverse scales one after the other: their product is no fp32 number for two rows of norms below 1e-18)
             const float gsc = B.gsc[lane], inv = B.inv[lane], ngsc = carry ? N.gsc[lane] : 0.0f, ninv = carry ? N.inv[lane] : 0.0f;
             const int32_t *low = &sh.idx[cur][0];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const int l = warp + r * NW;
                 const float il = B.inv[l], yl = B.ys[l], al = B.as[l];
-                float v = fmaf(fmaf((float)low[l * kLB + lane], 1.0f / 1048576.0f, (float)sh.G[0][l][lane]), il * inv, g[r]) * (gsc * yl);
+                float v = fmaf(fmaf((float)low[l * kLB + lane], 1.0f / 1048576.0f, (float)sh.G[0][l][lane]) * il, inv, g[r]) * (gsc * yl);
                 v = lane > l && !walk ? v : 0.0f;
                 out.G[l * kLB + lane] = v;
                 qg = fmaf(v, al, qg);
-                v = fmaf(fmaf((float)low[kLB * kLB + l * kLB + lane], 1.0f / 1048576.0f, (float)sh.G[1][l][lane]), il * ninv, x[r]) * (ngsc * yl);
+                v = fmaf(fmaf((float)low[kLB * kLB + l * kLB + lane], 1.0f / 1048576.0f, (float)sh.G[1][l][lane]) * il, ninv, x[r]) * (ngsc * yl);
                 v = l < cnt && carry ? v : 0.0f;
                 out.X[l * kLB + lane] = v;
                 qx = fmaf(v, al, qx);
