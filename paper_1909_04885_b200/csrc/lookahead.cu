@@ -303,9 +303,13 @@ template <int LOSS> __device__ __forceinline__ float recurrence_map(float s, flo
 // a root search (two exponentials, two divisions and two reciprocals one behind the other: 510 cycles, now about 90).
 // a(c) is analytic but for branch points at c0 +- i pi (where 1 + q a (1 - a) = 0) and their mirror images at q - c0, and
 // a(q - c) = 1 - a(c), so u = min(c, q - c) is expanded about nodes whose distance grows like the distance to c0: with
-// x = (u - c0) / 3, four bins per octave of 1 + |x| on either side of c0. Beyond x = -7 (a below 1e-9) the last value
-// serves. In an fp32 emulation against the exact root the largest error of a is 1.6e-7 over q from 0 to 45 000, where
-// the two Halley steps of logistic_root leave 5.9e-7.
+// x = (u - c0) / 3, four bins per octave of 1 + |x| on either side of c0. Below c0 the table holds a e^-u instead, which goes
+// to 1, and the chain multiplies with e^u: a small a is as exact, relative to itself, as one near 1/2. Beyond x = -7 the last
+// value serves (it is within 1e-9 of 1). x comes from two lines, one for c and one for q - c, so that a state near 0 is not
+// rounded to the spacing of the numbers near q. Measured against the exact root, q from 0.001 to 40 000 and states from -40 on:
+// the largest error of a is 1.3e-7 (logistic_root: 4.6e-7); relative to a, root mean square, 7.1e-7 below c0 and 8e-8 above
+// (8.1e-7 and 2.8e-7). Polynomials of a itself below c0 and x from |c - q / 2| took 24.1 instead of 25.4 ms for a step on
+// 11 M rows of 28, and left a small a wrong by up to a thousandth at e^-12, by its own size at e^-20.
 constexpr int kTabNeg = 12;                // bins below c0: three octaves
 constexpr float kTabScale = 3.0f;
 constexpr float kTabInv = 1.0f / kTabScale;
@@ -320,13 +324,15 @@ __device__ __forceinline__ float tab_center(float q)
     const float E = 2.0f / (2.0f + q + rt);
     return logf(E) - (q > 1e-12f ? 2.0f * q / (q + rt) : 0.0f);
 }
-// What the chain adds to -|c - q / 2| / 3 to get x (kept inside the table whatever q is).
-__device__ __forceinline__ float tab_offset(float q, int bins)
+// The lines: x = min(c / 3 + off, q / 3 + off - c / 3).
+__device__ __forceinline__ float tab_offset(float q) { return -tab_center(q) * kTabInv; }
+// q as the chain takes it: no more than keeps x inside the table (the lines meet at c = q / 2).
+__device__ __forceinline__ float tab_q(float q, float off, int bins)
 {
     const float top = (float)(1 << ((bins - kTabNeg) >> 2));
-    return fminf((0.5f * q - tab_center(q)) * kTabInv, top * 0.999999f - 1.0f);
+    return fminf(q, 2.0f * kTabScale * (top * 0.999999f - 1.0f - off));
 }
-// Bin i of a coordinate's table: the coefficients of a(c0 + sgn * 3 * (|x|)) in |x| - (the bin's centre).
+// Bin i of a coordinate's table: the coefficients, in |x| - (the bin's centre), of a (x > 0) or a e^-u (x < 0).
 __device__ __forceinline__ void tab_bin(float q, float log_q, int bins, int i, float4 &lo, float4 &hi)
 {
     const int npos = bins - kTabNeg;
@@ -353,6 +359,8 @@ __device__ __forceinline__ void tab_bin(float q, float log_q, int bins, int i, f
     a[0] = e / (1.0f + e);
     p[0] = a[0] * (1.0f - a[0]);
     const float r = 1.0f / fmaf(q, p[0], 1.0f);
+    a[0] = fmaf(-p[0] * r, fmaf(q, a[0], z - c), a[0]); // (what rounding z to its spacing left)
+    p[0] = a[0] * (1.0f - a[0]);
 #pragma unroll
     for (int k = 0; k < 7; ++k) {
         float acc = 0.0f;
@@ -370,6 +378,19 @@ __device__ __forceinline__ void tab_bin(float q, float log_q, int bins, int i, f
         a[2] = -a[2];
         a[4] = -a[4];
         a[6] = -a[6];
+    }
+    if (neg) { // times e^-u: u = log a - log(1 - a) + q a, so a e^-u = (1 - a) e^(-q a); e^-u's own coefficients are (-1)^k / k!
+        const float g = (1.0f - a[0]) * expf(-q * a[0]) / a[0];
+#pragma unroll
+        for (int k = 7; k >= 0; --k) {
+            float acc = a[k], f = 1.0f;
+#pragma unroll
+            for (int m = 1; m <= k; ++m) {
+                f *= -1.0f / (float)m;
+                acc = fmaf(a[k - m], f, acc);
+            }
+            a[k] = acc * g;
+        }
     }
     float w = step;
 #pragma unroll
@@ -394,11 +415,13 @@ __device__ __forceinline__ void write_table(const LookParams &P, int64_t bid, co
     }
 }
 // a(c) from the table, as sgn * v + bias: the caller multiplies sgn into what a(c) is multiplied with next while the look-up is
-// under way. d = c - q / 2; `row`: where the coordinate's table would have a bin of exponent 0; `on`: whether this lane's
-// result is wanted (the other lanes keep off the shared-memory pipe).
-__device__ __forceinline__ float tab_map(float d, float off, uint32_t row, uint32_t neg, bool on, float4 &lo, float4 &hi, float &sgn, float &bias)
+// under way (e^u, too, is ready before the polynomial is). q, off, off2 (= q / 3 + off): see tab_q and tab_offset; `row`: where the
+// coordinate's table would have a bin of exponent 0; `on`: whether this lane's result is wanted (the other lanes keep off the shared-memory
+// pipe).
+__device__ __forceinline__ float tab_map(float c, float q, float off, float off2, uint32_t row, uint32_t neg, bool on, float4 &lo, float4 &hi, float &sgn, float &bias)
 {
-    const float x = fmaxf(fmaf(-fabsf(d), kTabInv, off), kTabXmin);
+    const float x = fmaxf(fminf(fmaf(c, kTabInv, off), fmaf(c, -kTabInv, off2)), kTabXmin);
+    const float t = q - c, u = fminf(c, t);
     const float ax = fabsf(x), y = 1.0f + ax;
     const uint32_t bits = __float_as_uint(y);
     const uint32_t at = ((bits & 0xffe00000u) >> 16) + (x < 0.0f ? row + neg : row); // 32 bytes a bin
@@ -406,9 +429,12 @@ __device__ __forceinline__ float tab_map(float d, float off, uint32_t row, uint3
                  "@q ld.shared.v4.f32 {%0, %1, %2, %3}, [%8];\n\t@q ld.shared.v4.f32 {%4, %5, %6, %7}, [%8 + 16];\n\t}"
                  : "+f"(lo.x), "+f"(lo.y), "+f"(lo.z), "+f"(lo.w), "+f"(hi.x), "+f"(hi.y), "+f"(hi.z), "+f"(hi.w)
                  : "r"(at), "r"((uint32_t)on));
-    sgn = d > 0.0f ? -1.0f : 1.0f;
+    float eu;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(eu) : "f"(u * 1.4426950409f));
+    eu = x < 0.0f ? eu : 1.0f;
+    sgn = t < c ? -eu : eu;
     // (a state that is not finite gives a result that is not, as the root search would)
-    bias = fmaf(0.0f, d, d > 0.0f ? 1.0f : 0.0f);
+    bias = fmaf(0.0f, c, t < c ? 1.0f : 0.0f);
     const float dl = ax - (__uint_as_float((bits & 0xffe00000u) | 0x00100000u) - 1.0f);
     const float d2 = dl * dl, d4 = d2 * d2;
     const float p01 = fmaf(lo.y, dl, lo.x), p23 = fmaf(lo.w, dl, lo.z), p45 = fmaf(hi.y, dl, hi.x), p67 = fmaf(hi.w, dl, hi.z);
@@ -549,7 +575,7 @@ template <int LOSS, int NZ, int HT, class Shared> __device__ __forceinline__ voi
         n = (int32_t)len;
         if (!CHICLE_IN_BOUNDS(P.S.status, rs >= 0 && len >= 0 && len <= 0x7fffffff && rs + len <= P.nnz)) { rs = 0; n = 0; }
         hd = make_hdr_of<LOSS>(P.S, c, sh.sq[lane], sh.al[lane], LOSS == CHICLE_LOSS_RIDGE_PRIMAL ? 0.0f : sh.lb[lane]);
-        if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) hd.lq = tab_offset(hd.p2, P.tab_bins);
+        if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) hd.lq = tab_offset(hd.p2);
     }
     B.hdr[lane] = hd;
     B.rs[lane] = rs;
@@ -1234,7 +1260,7 @@ template <int LOSS, bool LONG> __device__ __forceinline__ void prepare_block_den
         CHdr hd{0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (c >= 0) {
             hd = make_hdr<LOSS>(P.S, c);
-            if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) hd.lq = tab_offset(hd.p2, P.tab_bins);
+            if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) hd.lq = tab_offset(hd.p2);
         }
         sh.gsc[warp * kLB + lane] = c >= 0 ? gram_scale<LOSS>(hd, P.S.sigma, P.S.inv_n) : 0.0f;
         if (warp == 0) {
@@ -1493,7 +1519,7 @@ struct alignas(16) ChainCtl {
     alignas(16) float dbuf[2][kLB];
     uint64_t ready[2];             // CTA 0: the states that a block's recurrence starts from are in `start`
     uint64_t out[2];               // CTA 0: the recurrence's results are in `res`
-    alignas(16) float start[2][3][kLB]; // states; the scalar map's constants (p2 and lq; with tables lq alone)
+    alignas(16) float start[2][3][kLB]; // states; the scalar map's constants (p2 and lq; with tables tab_q and tab_offset)
     alignas(16) float res[2][kLB];
     float sink[32]; // where a lane's stores go that have no target
     int walk[kSubSlots]; // whether the slot's block is walked in place
@@ -1689,7 +1715,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 const uint32_t res = smem_u32(&ctl.res[0][0]) + par * (uint32_t)(kLB * 4);
                 const float4 s0 = lds_f32x4(st0);
                 float4 k2 = make_float4(0.f, 0.f, 0.f, 0.f), k3 = k2;
-                if (LOSS != CHICLE_LOSS_HINGE_DUAL && !TAB) k2 = lds_f32x4(st0 + 128u);
+                if (LOSS != CHICLE_LOSS_HINGE_DUAL) k2 = lds_f32x4(st0 + 128u);
                 if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL) k3 = lds_f32x4(st0 + 256u);
                 const float4 q0n = *reinterpret_cast<const float4 *>(&H.q0n[4 * q]);
                 const float hp2[4] = {k2.x, k2.y, k2.z, k2.w}, hlq[4] = {k3.x, k3.y, k3.z, k3.w};
@@ -1697,7 +1723,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 xs[0] = -q0n.x; xs[1] = -q0n.y; xs[2] = -q0n.z; xs[3] = -q0n.w;
                 // with tables: where each coordinate's table would have exponent 0
                 uint32_t row[4];
+                float off2[4];
                 if (TAB) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) off2[i] = fmaf(hp2[i], kTabInv, hlq[i]);
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
                         row[i] = smem_u32(smem_chain + L.tabs) + (uint32_t)slot * tab_bytes(P.tab_bins) + (uint32_t)((4 * q + i) * P.tab_bins) * 32u - (127u << 2) * 32u;
@@ -1705,7 +1734,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo; // (the lanes whose result nobody wants keep what is there)
                 // a state's result is sgn * v + bias (sgn = 1, bias = 0 without tables)
                 auto step_map = [&](float st, int i, bool on, float &sgn, float &bias) {
-                    if (TAB) return tab_map(st, hlq[i], row[i], tab_neg, on, lo, hi, sgn, bias);
+                    if (TAB) return tab_map(st, hp2[i], hlq[i], off2[i], row[i], tab_neg, on, lo, hi, sgn, bias);
                     sgn = 1.0f;
                     bias = 0.0f;
                     return recurrence_map<LOSS>(st, hp2[i], hlq[i]);
@@ -1773,7 +1802,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     }
     if (crank == 0 && warp == kStartWarp && nb > 0) {
         // ============================== what a block's recurrence starts from =======================================
-        // A lane per coordinate: once the block's dot products are here (with tables: less half of q, see tab_map). In the
+        // A lane per coordinate: once the block's dot products are here. In the
         // recurrence warp itself, which keeps four coordinates per lane, this and what the feeder does took 1 090 cycles a
         // block, most of them instruction fetches of code that runs once.
         int fp = 0, slot = 0; // staged blocks so far; blk mod the head slots
@@ -1792,8 +1821,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 for (int c = 0; c < C; ++c) m0 += ctl.pbuf[fp & 1][c][lane]; // the CTAs' partial sums in a fixed order
                 ++fp;
                 const float s0 = fmaf(h.B, m0, h.A);
-                ctl.start[par][0][lane] = TAB ? s0 - 0.5f * h.p2 : s0;
-                ctl.start[par][1][lane] = h.p2;
+                ctl.start[par][0][lane] = s0;
+                ctl.start[par][1][lane] = TAB ? tab_q(h.p2, h.lq, P.tab_bins) : h.p2;
                 ctl.start[par][2][lane] = h.lq;
             }
             __syncwarp();

@@ -20,3 +20,32 @@ def test_step_over_q(fmt, q):
                                             [w.values[w.indptr[i]:w.indptr[i + 1]] for i in range(515)]))
     w.lam = 4.0 * sq / q / 515
     run_parity(w, rounds=3)
+
+
+@pytest.mark.parametrize("q,margin", [(0.5, 4.0), (0.5, 12.0), (0.5, 24.0), (100.0, 0.0), (100.0, 14.0), (3e3, 0.0), (3.9e4, 0.0), (3.9e4, 16.0)])
+def test_small_states_relative_to_themselves(q, margin):
+    # every state ends between e^-margin and a few / q. A state is the sum of a few fp32 terms of 30 at most (2e-6 each way)
+    # and enters the result as e^state: 1e-5 leaves room for a handful of them, whatever the size of the result
+    import numpy as np
+    from parity_util import make_pair, rel_l2
+    n, d = 515, 7
+    w = tiny_dense(n, d, seed=3, loss="logistic", K=1, lam=1.0)
+    X = w.values.reshape(n, d)
+    w.labels = np.where(X[:, 0] >= 0, 1.0, -1.0).astype(np.float32)
+    X[:, 0] = w.labels * (1.0 + 0.1 * np.abs(X[:, 0]))
+    w.lam = float(np.float32((X.astype(np.float64) ** 2).sum(1).max() / q / n))
+    orc, glm = make_pair(w)
+    try:
+        orc.partition(1, 1)
+        glm.partition(1, 1)
+        v = np.zeros(d)
+        v[0] = np.float32(margin * w.lam * n)
+        orc.v[:] = v
+        glm.set_state(orc.state.astype(np.float32), v.astype(np.float32), 0)
+        orc.cocoa_round(40, 1.0)
+        glm.cocoa_round(40, 1.0)
+        at = orc.permutation(0, 0)[:40]
+        a, b = np.abs(glm.get_alpha()[at].astype(np.float64)), np.abs(orc.state[at])
+        assert (np.abs(a - b) / b).max() <= 1e-5, (np.abs(a - b) / b).max()
+    finally:
+        glm.close()
