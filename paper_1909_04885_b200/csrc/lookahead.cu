@@ -1514,7 +1514,7 @@ struct alignas(16) ChainCtl {
     uint64_t pbar[2];              // CTA 0: the partial dot products of a block have arrived from all CTAs
     uint64_t dbar[2];              // a block's deltas have arrived from CTA 0
     uint64_t subfree[kSubSlots];   // the worker warps are through with the slot's record
-    uint64_t ackbar;               // CTA 0: every CTA has applied all updates (before a block is walked in place)
+    uint64_t ackbar;               // CTA 0: every worker warp of every CTA is through with all blocks before the one that is walked in place
     alignas(16) float pbuf[2][kMaxC][kLB];
     alignas(16) float dbuf[2][kLB];
     uint64_t ready[2];             // CTA 0: the states that a block's recurrence starts from are in `start`
@@ -1589,7 +1589,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             mbar_init(smem_u32(&ctl.ready[i]), 1);
             mbar_init(smem_u32(&ctl.out[i]), 1);
         }
-        mbar_init(smem_u32(&ctl.ackbar), (uint32_t)C);
+        mbar_init(smem_u32(&ctl.ackbar), (uint32_t)(C * kWorkWarps));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // armed for the first two blocks before anybody can send
         for (int i = 0; i < 2; ++i) {
@@ -1917,6 +1917,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         uint32_t turn = 0, tbefore = 0; // parity of how often the slots have been filled
 #pragma unroll 1
         for (int blk = 0; blk < nb; ++blk) {
+            if (__any_sync(0xffffffffu, *abort_flag != 0)) break; // (no slot is refilled for workers that no longer wait for it)
             if (blk >= slots && !mbar_wait_cluster(smem_u32(&ctl.subfree[slot]), turn ^ 1u, abort_flag, S.status)) break;
             const unsigned long long offset = ((unsigned long long)d[1] << 32) | d[0];
             uint32_t bytes = d[2] <= L.sub_stride ? d[2] : 0u;
@@ -1959,9 +1960,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
     }
     if (is_worker) {
         // ============================== the worker warps ========================================================
-        // Two barriers per block: in front of its update (no dot product reads the model any more) and behind it. Every
-        // warp waits for deltas and records by itself; one whose wait runs out does no more work but goes on meeting the
-        // others at the barriers (its abort flag ends their waits too).
+        // Two barriers per block, whatever the block is: in front of its update (no dot product reads the model any more) and
+        // behind it. Every warp waits for deltas and records by itself; one whose wait runs out does no more work but goes on
+        // meeting the others at the barriers (its abort flag ends their waits too). Nothing that it reads from then on decides
+        // how often: a slot's walk flag may be rewritten under it, and a barrier that one warp leaves out never ends.
         // What these warps are bound by is the number of instructions they issue, most of them the same in every warp
         // (addresses, waits, loop ends): hence eight warps and not twelve, 32-bit shared-memory addresses and one instance
         // of the kernel per kind of data.
@@ -2015,10 +2017,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             if (b >= 0) {
                 const uint32_t par = (uint32_t)(b & 1), dbar = smem_u32(&ctl.dbar[0]) + 8u * par;
                 if (sl0) {
-                    // (walked in place by CTA 0: every update before it has been applied here; once no dot product reads the
-                    // model any more, say so, and wait for the walk to end)
-                    work_bar();
-                    if (wt == 0) mbar_arrive_remote_release(ack_bar);
+                    // (walked in place by CTA 0: this warp's part of every update before it has been applied, and its dot
+                    // products no longer read the model; say so, and wait for the walk to end)
+                    __syncwarp();
+                    if (lane == 0 && ok) mbar_arrive_remote_release(ack_bar);
                 }
                 ok = ok && mbar_wait_cluster(dbar, (uint32_t)(b >> 1) & 1u, abort_flag, S.status);
                 if (sl0) fence_cluster(); // the walk's ordinary stores into this CTA's part of the model
@@ -2142,7 +2144,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             bool met = b < 0; // the barrier behind the update
             auto meet = [&]() {
                 if (!met) work_bar();
-                if (!met && wt == 0) mbar_arrive(smem_u32(&ctl.subfree[0]) + 8u * s_upd); // block b's slot is free
+                if (!met && wt == 0 && ok) mbar_arrive(smem_u32(&ctl.subfree[0]) + 8u * s_upd); // block b's slot is free
                 met = true;
             };
 #pragma unroll 1
@@ -2157,6 +2159,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 if (!CHICLE_IN_BOUNDS(S.status, head.w >= 0 && head.w <= kLB && (DENSE || (head.x >= 0 && head.y >= 0 && head.z >= 0 &&
                                                     sub_bytes((uint32_t)head.x, (uint32_t)head.y, (uint32_t)head.z) <= stride)))) {
                     ok = false;
+                    *abort_flag = 1;
                     break;
                 }
                 const uint32_t slot = (uint32_t)(fg & 1);
