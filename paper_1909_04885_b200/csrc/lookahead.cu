@@ -1505,6 +1505,14 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     return mbar_wait_slow(bar, parity, abort_flag, status);
 }
 
+// The end of a bulk copy that is on its way, for a role that stops early: a CTA must not leave while one still writes to its
+// shared memory. Nothing but the copy itself is waited for (an abort does not end this), with a bound all the same. (Not
+// inlined: the block loops stay as small as they were.)
+__device__ __noinline__ void mbar_drain(uint32_t bar, uint32_t parity)
+{
+    for (int it = 0; it < (1 << 14) && !__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity) != 0u); ++it) { }
+}
+
 // The worker warps' barrier: 35 cycles when all are there (with a vote 78, by arrivals on an mbarrier 181).
 __device__ __forceinline__ void work_bar() { asm volatile("bar.sync %0, %1;" ::"n"(kBarWork), "n"(kWorkThreads) : "memory"); }
 
@@ -1856,7 +1864,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             if (TAB) bulk_g2s_if(tabs0 + (uint32_t)slot * tab_len, P.rec + P.tab_off + at * tab_len, tab_len, bar, on);
         };
         for (int i = 0; i < HS; ++i) issue_head(i, i);
-        int fp = 0, slot = 0;
+        int fp = 0, slot = 0, done = 0;
 #pragma unroll 1
         for (int b = 0; b < nb; ++b) {
             const uint32_t par = (uint32_t)(b & 1);
@@ -1897,7 +1905,9 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             __syncwarp();
             issue_head(b + HS, slot);
             slot = slot + 1 == HS ? 0 : slot + 1;
+            done = b + 1;
         }
+        for (int i = done; i < done + HS && i < nb; ++i) mbar_drain(smem_u32(&ctl.headfull[i % HS]), (uint32_t)(i / HS) & 1u);
     }
     if (warp == kRecordWarp && nb > 0) {
         // ============================== the workers' records, four blocks ahead =======================================
@@ -1914,6 +1924,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         uint32_t d[4];
         load_dir(0, d);
         int slot = 0, before = 0;     // of this block and of the one before
+        int fetched = 0;
         uint32_t turn = 0, tbefore = 0; // parity of how often the slots have been filled
 #pragma unroll 1
         for (int blk = 0; blk < nb; ++blk) {
@@ -1935,6 +1946,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             const uint32_t bar = smem_u32(&ctl.subfull[slot]);
             mbar_arrive_expect_tx_if(bar, bytes, lane == 0);
             bulk_g2s_if(smem_u32(smem_chain + L.subs) + (uint32_t)slot * L.sub_stride, P.rec + offset, bytes, bar, lane == 0);
+            fetched = blk + 1;
             load_dir(blk + 1, d);
             // The block before this one has arrived by now, and its dot products are a block's time away: the model entries
             // beyond the part in shared memory that they will gather are brought into L2 (the records that stream through it
@@ -1957,6 +1969,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 turn ^= 1u;
             }
         }
+        for (int i = fetched > slots ? fetched - slots : 0; i < fetched; ++i) mbar_drain(smem_u32(&ctl.subfull[i % slots]), (uint32_t)(i / slots) & 1u);
     }
     if (is_worker) {
         // ============================== the worker warps ========================================================
@@ -2325,7 +2338,11 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         const volatile int *done = &ctl.done;
         for (uint32_t it = 0; it < (1u << 24) && !*done; ++it) __nanosleep(2000);
     }
-    // nobody leaves while another CTA of the cluster may still write to, or read from, its shared memory
+    // nobody leaves while another CTA of the cluster may still write to, or read from, its shared memory (after an abort
+    // asynchronous stores may be on their way that no role waits for any more: a millisecond for them)
+    __syncwarp();
+    if (*abort_flag)
+        for (int i = 0; i < 16; ++i) __nanosleep(64000);
     __syncwarp();
     cluster_arrive();
     cluster_wait();
