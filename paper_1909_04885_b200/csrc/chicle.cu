@@ -715,8 +715,15 @@ chicle_status_t chicle_get_alpha(chicle_glm_t *h, float *out, int64_t len, chicl
 chicle_status_t chicle_get_v(chicle_glm_t *h, float *out, int64_t len, chicle_memspace_t space)
 {
     if (h && h->new_of_old) {
-        // translate from the library's ranked ids to the caller's: tmp[old] = v[new_of_old[old]]
-        const bool direct = out && len == h->dim && space == CHICLE_MEM_DEVICE; // (the caller's array takes it as it is)
+        // translate from the library's ranked ids to the caller's: tmp[old] = v[new_of_old[old]]. Only this device's own
+        // memory, at a whole float, is written in place (pinned host memory, another GPU's, an odd address: by a copy, which
+        // takes or refuses them).
+        bool direct = out && len == h->dim && space == CHICLE_MEM_DEVICE && (reinterpret_cast<uintptr_t>(out) & 3u) == 0;
+        if (direct) {
+            cudaPointerAttributes at{};
+            direct = cudaPointerGetAttributes(&at, out) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == h->device;
+            if (!direct) (void)cudaGetLastError();
+        }
         if (cudaSetDevice(h->device) == cudaSuccess) {
             const cudaError_t e = launch_gather_f32(*h, h->v, h->new_of_old, h->dim, direct ? out : h->perm_tmp);
             if (e != cudaSuccess) return fail_cuda(h, e, "chicle_get_v");
