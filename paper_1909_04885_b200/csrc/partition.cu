@@ -457,7 +457,7 @@ constexpr int kMapPer = CHICLE_NOALLOC_MAX_COORDS / (kMapC * kMapThreads); // id
 constexpr int kMapChunk = kMapThreads * kMapPer;
 constexpr int kMapCap = kMapChunk + 1024; // (the fullest eighth of 131 072 hashes: 16 384 + 8 standard deviations)
 constexpr int kMapSub = CHICLE_NOALLOC_MAX_COORDS / kMapC;
-constexpr int kMapMaxK = 512;  // more partitions: the member lists are made by comparison inside each partition
+constexpr int kMapMaxK = 512;  // more partitions: the member lists are made by comparison inside each partition (see launch_partition)
 constexpr int kMapWarps = kMapThreads / 32;
 
 struct MapShared {
@@ -726,7 +726,11 @@ cudaError_t launch_partition(Glm &g, int32_t K, uint64_t seed)
     const int64_t n = g.n_coord;
     // (the offsets are on the device already: equal blocks, or the sizes the caller gave)
     const Cuts cuts{g.part_off, K, 0, 0};
-    if (n <= CHICLE_NOALLOC_MAX_COORDS) return launch_map(n, seed, cuts, g.owner, g.members, g.ord.tmp, g.stream);
+    // More partitions than the one-launch kernel counts by: it compares every id with all of its partition, on eight SMs, which
+    // pays while there are few ids and no large partition. (20 000 ids, K = 513: 64 us a call against 128 on the path below;
+    // 131 072 ids, K = 2 000: 270 against 174; one partition of half of 131 072 ids: 17 ms against 0.15.)
+    const bool few = n <= 32768 && n * g.max_nk <= (int64_t)1 << 20;
+    if (n <= CHICLE_NOALLOC_MAX_COORDS && (K <= kMapMaxK || few)) return launch_map(n, seed, cuts, g.owner, g.members, g.ord.tmp, g.stream);
     // Which partition an id falls to needs its place in key order only where a cut lies inside its bucket: all other
     // ids get their bucket's partition, those (a K / n * 512 share) are put in order.
     const Segments S{nullptr, nullptr, 1, n, (uint32_t)order_buckets(n)};

@@ -63,3 +63,31 @@ def test_short_rounds(n, K, H):
         assert np.linalg.norm(a - orc.state) <= 1e-5 * np.linalg.norm(orc.state)
     finally:
         glm.close()
+
+
+# more than 512 partitions of given sizes: one that holds nearly all ids, a few large ones, small ones only; around the sizes
+# where the one-launch kernel stops
+@pytest.mark.parametrize("n,K,big", [(131072, 600, [130000]), (131072, 513, [40000, 40000, 40000]), (32768, 600, [10]), (32769, 1100, []), (2000, 600, [900]),
+                                     (32768, 1024, []), (20011, 4000, [3000])])
+def test_many_uneven_partitions(n, K, big):
+    import time
+    sizes = np.ones(K, np.int64)
+    sizes[7:7 + len(big)] = big
+    rest = [k for k in range(K) if not 7 <= k < 7 + len(big)]
+    left = n - int(sizes.sum())
+    sizes[rest] += left // len(rest)
+    sizes[rest[-1]] += n - int(sizes.sum())
+    orc, glm = make_pair(tiny_dense(n, 1, seed=1, K=K))
+    try:
+        orc.partition(K, 5, sizes)
+        glm.partition(K, 5, sizes)
+        check_partition(orc, glm, perm_rounds=(3,))
+        took = []
+        for _ in range(5):
+            t = time.perf_counter()
+            glm.partition(K, 6, sizes)
+            took.append(time.perf_counter() - t)
+        # a few launches over n ids (0.15 ms); comparing all pairs of the largest partition would be of the order of 20 ms
+        assert min(took) < 5e-3, took
+    finally:
+        glm.close()
