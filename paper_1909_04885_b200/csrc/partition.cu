@@ -64,6 +64,32 @@ constexpr int kCountThreads = 256;
 constexpr int kCountItems = 8;
 constexpr int kCountTile = kCountThreads * kCountItems;
 
+// The elements a CTA of the counting and scattering kernels takes: f(segment, first element, step, end). Tile t, t + tiles, .. of
+// one segment; or (tiles = 0) an equal share of all segments one after the other, counted in buckets. Segments of about the same
+// size take the first way. Where one is much longer than what its tiles' CTAs get through meanwhile, the second (see tiles_for).
+template <class F> __device__ __forceinline__ void for_my_elements(const Segments &S, int tiles, F f)
+{
+    if (tiles > 0) {
+        const int k = (int)(blockIdx.x / tiles), t = (int)(blockIdx.x % tiles);
+        f(k, S.first(k) + (int64_t)t * kCountTile, (int64_t)tiles * kCountTile, S.last(k));
+        return;
+    }
+    const int64_t all = S.bbase[S.K], end = all * ((int64_t)blockIdx.x + 1) / gridDim.x;
+    int64_t at = all * blockIdx.x / gridDim.x;
+    int lo = 0, hi = S.K; // bbase[lo] <= at < bbase[hi]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (S.bbase[mid] <= at) lo = mid;
+        else hi = mid;
+    }
+    for (int k = lo; at < end; ++k) {
+        const int64_t b0 = S.bbase[k], b1 = S.bbase[k + 1], stop = b1 < end ? b1 : end, first = S.first(k), last = S.last(k);
+        const int64_t until = first + (stop - b0) * kBucketMean;
+        f(k, first + (at - b0) * kBucketMean, (int64_t)kCountTile, until < last ? until : last);
+        at = stop;
+    }
+}
+
 // cursor[bucket] += its elements (zero on entry). LOCAL: a CTA counts in shared memory first and adds what it has of each
 // bucket; for segments of at most kLocalBuckets buckets whose CTAs have several elements of each (see launch_count): 1 M
 // coordinates in 16 segments took 31 us, a global atomic per coordinate.
@@ -73,32 +99,32 @@ __global__ void __launch_bounds__(kCountThreads)
 k_bucket_count(const Segments S, int tiles, const int32_t *__restrict__ ids, uint64_t ab, uint32_t *__restrict__ cursor)
 {
     __shared__ uint32_t mine[LOCAL ? kLocalBuckets : 1];
-    const int k = (int)(blockIdx.x / tiles), t = (int)(blockIdx.x % tiles);
-    const int64_t lo = S.first(k), hi = S.last(k);
-    const uint32_t nb = S.buckets(k);
-    uint32_t *cur = cursor + S.bucket0(k);
-    if (LOCAL) {
-        if (lo + (int64_t)t * kCountTile >= hi) return;
-        for (uint32_t b = threadIdx.x; b < nb; b += kCountThreads) mine[b] = 0u;
-        __syncthreads();
-    }
-    for (int64_t i0 = lo + (int64_t)t * kCountTile; i0 < hi; i0 += (int64_t)tiles * kCountTile) {
-        uint32_t b[kCountItems];
-#pragma unroll
-        for (int u = 0; u < kCountItems; ++u) {
-            const int64_t i = i0 + u * kCountThreads + threadIdx.x;
-            const uint32_t id = i < hi ? (ids ? (uint32_t)ids[i] : (uint32_t)i) : 0u;
-            b[u] = __umulhi((uint32_t)(mix64(ab ^ (uint64_t)id) >> 32), nb);
+    for_my_elements(S, tiles, [&](int k, int64_t from, int64_t step, int64_t hi) {
+        if (from >= hi) return;
+        const uint32_t nb = S.buckets(k);
+        uint32_t *cur = cursor + S.bucket0(k);
+        if (LOCAL) {
+            for (uint32_t b = threadIdx.x; b < nb; b += kCountThreads) mine[b] = 0u;
+            __syncthreads();
         }
+        for (int64_t i0 = from; i0 < hi; i0 += step) {
+            uint32_t b[kCountItems];
 #pragma unroll
-        for (int u = 0; u < kCountItems; ++u)
-            if (i0 + u * kCountThreads + threadIdx.x < hi) atomicAdd((LOCAL ? mine : cur) + b[u], 1u);
-    }
-    if (LOCAL) {
-        __syncthreads();
-        for (uint32_t b = threadIdx.x; b < nb; b += kCountThreads)
-            if (mine[b]) atomicAdd(cur + b, mine[b]);
-    }
+            for (int u = 0; u < kCountItems; ++u) {
+                const int64_t i = i0 + u * kCountThreads + threadIdx.x;
+                const uint32_t id = i < hi ? (ids ? (uint32_t)ids[i] : (uint32_t)i) : 0u;
+                b[u] = __umulhi((uint32_t)(mix64(ab ^ (uint64_t)id) >> 32), nb);
+            }
+#pragma unroll
+            for (int u = 0; u < kCountItems; ++u)
+                if (i0 + u * kCountThreads + threadIdx.x < hi) atomicAdd((LOCAL ? mine : cur) + b[u], 1u);
+        }
+        if (LOCAL) {
+            __syncthreads();
+            for (uint32_t b = threadIdx.x; b < nb; b += kCountThreads)
+                if (mine[b]) atomicAdd(cur + b, mine[b]);
+        }
+    });
 }
 
 // A CTA per segment. start[bucket] = first position of the bucket, cursor[bucket] the same (the scatter's running place);
@@ -179,32 +205,32 @@ k_bucket_scatter(const Segments S, int tiles, const int32_t *__restrict__ ids, u
                  const uint32_t *__restrict__ nbm, const int32_t *__restrict__ bowner, int32_t *__restrict__ owner,
                  int32_t *__restrict__ out)
 {
-    const int k = (int)(blockIdx.x / tiles), t = (int)(blockIdx.x % tiles);
-    const int64_t lo = S.first(k), hi = S.last(k);
-    const uint32_t nb = S.buckets(k), b0 = S.bucket0(k);
-    for (int64_t i0 = lo + (int64_t)t * kCountTile; i0 < hi; i0 += (int64_t)tiles * kCountTile) {
-        uint32_t id[kCountItems], b[kCountItems], m[kCountItems];
-#pragma unroll
-        for (int u = 0; u < kCountItems; ++u) {
-            const int64_t i = i0 + u * kCountThreads + threadIdx.x;
-            id[u] = i < hi ? (ids ? (uint32_t)ids[i] : (uint32_t)i) : 0u;
-            b[u] = b0 + __umulhi((uint32_t)(mix64(ab ^ (uint64_t)id[u]) >> 32), nb);
-            m[u] = i < hi ? nbm[b[u]] : 0u;
-        }
-        if (owner) {
+    for_my_elements(S, tiles, [&](int k, int64_t from, int64_t step, int64_t hi) {
+        const uint32_t nb = S.buckets(k), b0 = S.bucket0(k);
+        for (int64_t i0 = from; i0 < hi; i0 += step) {
+            uint32_t id[kCountItems], b[kCountItems], m[kCountItems];
 #pragma unroll
             for (int u = 0; u < kCountItems; ++u) {
                 const int64_t i = i0 + u * kCountThreads + threadIdx.x;
-                if (i < hi && m[u] == 0u) owner[i] = bowner[b[u]]; // (one segment of all ids: i is the id)
+                id[u] = i < hi ? (ids ? (uint32_t)ids[i] : (uint32_t)i) : 0u;
+                b[u] = b0 + __umulhi((uint32_t)(mix64(ab ^ (uint64_t)id[u]) >> 32), nb);
+                m[u] = i < hi ? nbm[b[u]] : 0u;
             }
+            if (owner) {
+#pragma unroll
+                for (int u = 0; u < kCountItems; ++u) {
+                    const int64_t i = i0 + u * kCountThreads + threadIdx.x;
+                    if (i < hi && m[u] == 0u) owner[i] = bowner[b[u]]; // (one segment of all ids: i is the id)
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kCountItems; ++u)
+                if (m[u]) m[u] = atomicAdd(cursor + b[u], 1u) + 1u;
+#pragma unroll
+            for (int u = 0; u < kCountItems; ++u)
+                if (m[u]) out[m[u] - 1u] = (int32_t)id[u];
         }
-#pragma unroll
-        for (int u = 0; u < kCountItems; ++u)
-            if (m[u]) m[u] = atomicAdd(cursor + b[u], 1u) + 1u;
-#pragma unroll
-        for (int u = 0; u < kCountItems; ++u)
-            if (m[u]) out[m[u] - 1u] = (int32_t)id[u];
-    }
+    });
 }
 
 template <int CAP> struct OrderShared {
@@ -689,12 +715,22 @@ cudaError_t launch_map(int64_t n, uint64_t seed, const Cuts &cuts, int32_t *owne
     return cudaGetLastError();
 }
 
-// tiles per segment for the counting and scattering kernels: enough CTAs to fill the GPU, no more than the longest needs
+// tiles per segment for the counting and scattering kernels: enough CTAs to fill the GPU, no more than the longest needs; 0
+// (see for_my_elements): the longest segment's CTAs would have more than four times what a CTA has on average, and more than
+// four tiles (10 M coordinates in 1 200 segments, half of them in one: 6.9 ms with a CTA for each, 0.21 this way)
 inline int tiles_for(const Glm &g, int64_t longest, int K)
 {
-    const int64_t want = ((int64_t)g.sm_count * 8 + K - 1) / K, have = (longest + kCountTile - 1) / kCountTile;
-    const int64_t t = want < have ? want : have;
-    return (int)(t < 1 ? 1 : t);
+    const int64_t ctas = (int64_t)g.sm_count * 8, want = (ctas + K - 1) / K, have = (longest + kCountTile - 1) / kCountTile;
+    const int64_t t = want < have ? want : have, even = g.n_coord / ctas;
+    if (K > 1 && longest / t > 4 * (even > kCountTile ? even : kCountTile)) return 0;
+    return (int)t;
+}
+// CTAs of such a launch
+inline unsigned ctas_for(const Glm &g, int tiles, int K)
+{
+    if (tiles > 0) return (unsigned)tiles * (unsigned)K;
+    const int64_t most = (int64_t)g.sm_count * 8;
+    return (unsigned)(g.n_buckets < most ? g.n_buckets : most);
 }
 
 template <int CAP, int THREADS>
@@ -713,12 +749,13 @@ cudaError_t launch_order(unsigned grid, const int32_t *src, const uint32_t *star
 int64_t order_buckets(int64_t nk) { return (nk + kBucketMean - 1) / kBucketMean; }
 
 // most, most_buckets: of the largest segment. A CTA counts by itself if it has four elements and more of a bucket.
-static void launch_count(const Segments &S, int segments, int64_t most, uint32_t most_buckets, int tiles, const int32_t *ids, uint64_t ab,
-                         uint32_t *cursor, cudaStream_t stream)
+static void launch_count(const Glm &g, const Segments &S, int segments, int64_t most, uint32_t most_buckets, int tiles, const int32_t *ids,
+                         uint64_t ab, uint32_t *cursor, cudaStream_t stream)
 {
-    const int64_t per_cta = most / tiles < kCountTile ? kCountTile : most / tiles;
-    if (most_buckets <= kLocalBuckets && per_cta >= 4 * (int64_t)most_buckets) k_bucket_count<true><<<tiles * segments, kCountThreads, 0, stream>>>(S, tiles, ids, ab, cursor);
-    else k_bucket_count<false><<<tiles * segments, kCountThreads, 0, stream>>>(S, tiles, ids, ab, cursor);
+    const int64_t per_cta = tiles == 0 ? 0 : (most / tiles < kCountTile ? kCountTile : most / tiles);
+    const unsigned ctas = ctas_for(g, tiles, segments);
+    if (most_buckets <= kLocalBuckets && per_cta >= 4 * (int64_t)most_buckets) k_bucket_count<true><<<ctas, kCountThreads, 0, stream>>>(S, tiles, ids, ab, cursor);
+    else k_bucket_count<false><<<ctas, kCountThreads, 0, stream>>>(S, tiles, ids, ab, cursor);
 }
 
 cudaError_t launch_partition(Glm &g, int32_t K, uint64_t seed)
@@ -737,7 +774,7 @@ cudaError_t launch_partition(Glm &g, int32_t K, uint64_t seed)
     const uint64_t s = mix64(seed);
     const int tiles = tiles_for(g, n, 1);
     OrderWorkspace &w = g.ord;
-    launch_count(S, 1, n, S.nb, tiles, nullptr, s, w.cursor, g.stream);
+    launch_count(g, S, 1, n, S.nb, tiles, nullptr, s, w.cursor, g.stream);
     k_bucket_scan<<<1, kScanThreads, 0, g.stream>>>(S, w.start, w.cursor, w.nbm, w.bowner, cuts, nullptr, 0, 0);
     k_bucket_scatter<<<tiles, kCountThreads, 0, g.stream>>>(S, tiles, nullptr, s, w.cursor, w.nbm, w.bowner, g.owner, w.tmp);
     cudaError_t e = launch_order<2 * kBucketMean, 256>(S.nb, w.tmp, w.start, w.nbm, nullptr, s, w.cursor, nullptr, cuts, g.owner, g.stream);
@@ -793,9 +830,9 @@ cudaError_t launch_permutation(Glm &g, int64_t round, int64_t epochs, int64_t H,
             err = launch_order<4096, 1024>((unsigned)g.K, g.members, nullptr, nullptr, g.part_off, ab, nullptr, out, none, nullptr, g.stream);
             g.order_launches += 1;
         } else {
-            launch_count(S, g.K, g.max_nk, (uint32_t)order_buckets(g.max_nk), tiles, g.members, ab, w.cursor, g.stream);
+            launch_count(g, S, g.K, g.max_nk, (uint32_t)order_buckets(g.max_nk), tiles, g.members, ab, w.cursor, g.stream);
             k_bucket_scan<<<g.K, kScanThreads, 0, g.stream>>>(S, w.start, w.cursor, w.nbm, nullptr, none, steps, H, e);
-            k_bucket_scatter<<<tiles * g.K, kCountThreads, 0, g.stream>>>(S, tiles, g.members, ab, w.cursor, w.nbm, nullptr, nullptr, w.tmp);
+            k_bucket_scatter<<<ctas_for(g, tiles, g.K), kCountThreads, 0, g.stream>>>(S, tiles, g.members, ab, w.cursor, w.nbm, nullptr, nullptr, w.tmp);
             err = launch_order<2 * kBucketMean, 256>((unsigned)g.n_buckets, w.tmp, w.start, w.nbm, nullptr, ab, w.cursor, out, none, nullptr, g.stream);
             g.order_launches += 4;
         }

@@ -91,3 +91,28 @@ def test_many_uneven_partitions(n, K, big):
         assert min(took) < 5e-3, took
     finally:
         glm.close()
+
+
+# visiting orders where one partition is much longer than the others (its elements are shared out over all CTAs): sizes around
+# the rule's line, short and whole orders
+@pytest.mark.parametrize("n,K,big", [(300007, 1300, 200000), (300007, 1300, 5000), (300007, 40, 260000), (150001, 20000, 120000), (9300, 1200, 8101)])
+def test_orders_of_uneven_partitions(n, K, big):
+    sizes = np.ones(K, np.int64)
+    sizes[K // 2] = big
+    rest = [k for k in range(K) if k != K // 2]
+    sizes[rest] += (n - int(sizes.sum())) // len(rest)
+    sizes[rest[-1]] += n - int(sizes.sum())
+    orc, glm = make_pair(tiny_dense(n, 1, seed=1, K=K))
+    try:
+        orc.partition(K, 5, sizes)
+        glm.partition(K, 5, sizes)
+        check_partition(orc, glm, perm_rounds=(0, 7))
+        H = 1 if int(sizes.min()) < 3 else 3
+        for r in range(2):
+            orc.cocoa_round(H, float(K))
+            glm.cocoa_round(H, float(K))
+        a = glm.get_alpha().astype(np.float64)
+        # 32-bit products of one term, three steps a partition
+        assert np.linalg.norm(a - orc.state) <= 1e-5 * np.linalg.norm(orc.state)
+    finally:
+        glm.close()
