@@ -483,7 +483,8 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
     h->n_buckets = h_off[2 * K + 1];
     h->K = K;
     h->seed = seed;
-    e = cudaMemcpyAsync(part_off, h_off, 2 * ((size_t)K + 1) * 8, cudaMemcpyHostToDevice, h->stream);
+    // (the bucket offsets too, where the visiting orders use them: a copy of pageable memory, 131 072 partitions: MB each)
+    e = cudaMemcpyAsync(part_off, h_off, (h->max_nk > kOrderOneCta ? 2 : 1) * ((size_t)K + 1) * 8, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(U, 0, (size_t)K * (size_t)h->dim * 4, h->stream);
     int64_t *d_coff = nullptr;
     int32_t *d_ctask = nullptr;

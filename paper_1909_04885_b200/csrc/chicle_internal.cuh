@@ -58,6 +58,7 @@ struct OrderWorkspace {
     uint32_t *table = nullptr;     // 256 counters per tile
     uint32_t *scan_sums = nullptr; // one per scan tile
 };
+constexpr int64_t kOrderOneCta = 4096; // partitions of up to this many coordinates are put in order without buckets
 int64_t order_buckets(int64_t nk); // buckets of a segment of nk elements
 
 size_t sort_hist_entries(int64_t n);

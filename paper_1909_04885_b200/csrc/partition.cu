@@ -826,8 +826,8 @@ cudaError_t launch_permutation(Glm &g, int64_t round, int64_t epochs, int64_t H,
         if (g.max_nk <= 2 * kBucketMean) {
             err = launch_order<2 * kBucketMean, 256>((unsigned)g.K, g.members, nullptr, nullptr, g.part_off, ab, nullptr, out, none, nullptr, g.stream);
             g.order_launches += 1;
-        } else if (g.max_nk <= 4096) {
-            err = launch_order<4096, 1024>((unsigned)g.K, g.members, nullptr, nullptr, g.part_off, ab, nullptr, out, none, nullptr, g.stream);
+        } else if (g.max_nk <= kOrderOneCta) {
+            err = launch_order<(int)kOrderOneCta, 1024>((unsigned)g.K, g.members, nullptr, nullptr, g.part_off, ab, nullptr, out, none, nullptr, g.stream);
             g.order_launches += 1;
         } else {
             launch_count(g, S, g.K, g.max_nk, (uint32_t)order_buckets(g.max_nk), tiles, g.members, ab, w.cursor, g.stream);
