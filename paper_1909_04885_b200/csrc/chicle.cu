@@ -83,6 +83,23 @@ template <typename T> bool alloc_into(chicle_glm *h, T *&dst, size_t count)
     return dst != nullptr;
 }
 
+// Device arrays of one call, released when it returns (its work has ended by then).
+struct Temporaries {
+    chicle_glm *h;
+    std::vector<void *> owned;
+    template <typename T> bool alloc(T *&p, size_t count)
+    {
+        owned.reserve(owned.size() + 1);
+        if (!alloc_into(h, p, count)) return false;
+        owned.push_back(p);
+        return true;
+    }
+    ~Temporaries()
+    {
+        for (void *p : owned) dev_free(h, p);
+    }
+};
+
 cudaError_t copy_in(void *dst, const void *src, size_t bytes, chicle_memspace_t space, cudaStream_t s)
 {
     return cudaMemcpyAsync(dst, src, bytes, space == CHICLE_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, s);
@@ -390,6 +407,31 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
     if (e != cudaSuccess) return fail_cuda(h, e, "cudaSetDevice");
     const int64_t n = h->n_coord;
 
+    // A placement of chunks travels as two temporary device arrays. Sparse: how long the rows of each partition are decides what
+    // the solver is planned for.
+    Temporaries temp{h, {}};
+    int64_t *d_coff = nullptr;
+    int32_t *d_ctask = nullptr;
+    const bool by_chunks = chunks && h->fmt != CHICLE_FMT_DENSE_ROWMAJOR;
+    double chunk_mean = h->chunk_mean;
+    if (chunks) {
+        std::vector<unsigned long long> entries((size_t)K);
+        unsigned long long *d_entries = nullptr;
+        if (!temp.alloc(d_coff, (size_t)chunks->C + 1) || !temp.alloc(d_ctask, (size_t)chunks->C) || !temp.alloc(d_entries, (size_t)K))
+            return fail(h, CHICLE_ERR_OOM, "device allocation failed (chunk placement)");
+        e = cudaMemcpyAsync(d_coff, chunks->off, ((size_t)chunks->C + 1) * 8, cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(d_ctask, chunks->task, (size_t)chunks->C * 4, cudaMemcpyHostToDevice, h->stream);
+        if (e == cudaSuccess && by_chunks) {
+            e = cudaMemsetAsync(d_entries, 0, (size_t)K * 8, h->stream);
+            if (e == cudaSuccess) e = launch_chunk_entries(*h, chunks->C, d_coff, d_ctask, d_entries);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(entries.data(), d_entries, (size_t)K * 8, cudaMemcpyDeviceToHost, h->stream);
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        if (e != cudaSuccess) return fail_cuda(h, e, "chunk placement");
+        if (by_chunks)
+            for (int32_t k = 0; k < K; ++k) chunk_mean = std::max(chunk_mean, (double)entries[(size_t)k] / (double)sizes[k]);
+    }
+
     // Allocate everything new first so that a failure leaves the handle as it was.
     int32_t *owner = h->owner, *members = h->members, *perm = h->perm;
     bool fresh = false;
@@ -411,7 +453,9 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
     float *U = h->U;
     int64_t *part_off = h->part_off;
     int64_t *h_off = h->h_part_off;
-    const bool regrow = K != h->K || !h->U;
+    // (partitions by chunks want longer record slots, and longer arrays where their rows are long: see lookahead_plan)
+    const bool regrow = K != h->K || !h->U || by_chunks != h->by_chunks ||
+                        (by_chunks && lookahead_arrays(*h, true, chunk_mean) != lookahead_arrays(*h, true, h->chunk_mean));
     if (regrow) {
         // synchronise before releasing buffers that queued kernels may still use (the side stream's kernels are
         // ordered before the end of the caller's stream in every round that completed; after a failed launch they
@@ -447,6 +491,8 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
         // the look-ahead solver's per-round records (their number depends on K); without them the blocked solver runs
         dev_free(h, h->la_rec); dev_free(h, h->la_dir); dev_free(h, h->la_slice);
         h->la_rec = nullptr; h->la_dir = nullptr; h->la_slice = nullptr;
+        h->by_chunks = by_chunks;
+        h->chunk_mean = chunk_mean;
         const bool dense_fmt = h->fmt == CHICLE_FMT_DENSE_ROWMAJOR;
         if (dense_fmt ? h->dim <= lookahead_max_dense_dim() : h->dim <= lookahead_max_dim()) {
             lookahead_plan(*h, K);
@@ -486,25 +532,13 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
     // (the bucket offsets too, where the visiting orders use them: a copy of pageable memory, 131 072 partitions: MB each)
     e = cudaMemcpyAsync(part_off, h_off, (h->max_nk > kOrderOneCta ? 2 : 1) * ((size_t)K + 1) * 8, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(U, 0, (size_t)K * (size_t)h->dim * 4, h->stream);
-    int64_t *d_coff = nullptr;
-    int32_t *d_ctask = nullptr;
     if (chunks && e == cudaSuccess) {
-        // the placement travels as two temporary device arrays, released once the kernels that read them are done
-        if (!alloc_into(h, d_coff, (size_t)chunks->C + 1) || !alloc_into(h, d_ctask, (size_t)chunks->C)) {
-            dev_free(h, d_coff);
-            h->K = 0;
-            return fail(h, CHICLE_ERR_OOM, "device allocation failed (chunk placement)");
-        }
-        e = cudaMemcpyAsync(d_coff, chunks->off, ((size_t)chunks->C + 1) * 8, cudaMemcpyHostToDevice, h->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(d_ctask, chunks->task, (size_t)chunks->C * 4, cudaMemcpyHostToDevice, h->stream);
-        if (e == cudaSuccess) e = launch_partition_chunks(*h, K, chunks->C, d_coff, d_ctask);
+        e = launch_partition_chunks(*h, K, chunks->C, d_coff, d_ctask);
     } else if (e == cudaSuccess) {
         e = launch_partition(*h, K, seed);
     }
     // the host copy of part_off is reused by later calls, so finish the upload before returning
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (d_coff) dev_free(h, d_coff);
-    if (d_ctask) dev_free(h, d_ctask);
     if (e != cudaSuccess) {
         h->K = 0; // the partition map is not valid: a new partition call is required
         return fail_cuda(h, e, "partition kernels");
@@ -611,11 +645,17 @@ static chicle_status_t round_impl(chicle_glm_t *h, int64_t H, const int64_t *hos
         r.solver_launches = steps > 0 ? (h->solver_launches > 0 ? h->solver_launches : 1) : 0;
         r.order_launches = h->order_launches;
         *stats = r;
-        if (logging)
+        if (logging) {
+            uint32_t *walked = h->h_status + 1;
+            *walked = 0;
+            (void)cudaMemcpyAsync(walked, h->d_status + kStatusWalked, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+            (void)cudaMemsetAsync(h->d_status + kStatusWalked, 0, sizeof(uint32_t), s);
+            (void)cudaStreamSynchronize(s);
             fprintf(stderr, "[chicle] round %lld: K=%d steps=%lld solver=%d slices=%d ctas/partition=%d launches=%d; ms: orders %.3f, "
-                    "local solvers %.3f (first prepare %.3f), aggregation %.3f\n", (long long)(h->round - 1), (int)h->K,
+                    "local solvers %.3f (first prepare %.3f), aggregation %.3f; blocks walked in place: %u\n", (long long)(h->round - 1), (int)h->K,
                     (long long)r.steps, (int)r.solver_variant, (int)r.solver_slices, (int)r.cluster_ctas,
-                    (int)(r.solver_launches + r.order_launches + 1), r.ms_permutation, r.ms_local, r.ms_prepare, r.ms_reduce);
+                    (int)(r.solver_launches + r.order_launches + 1), r.ms_permutation, r.ms_local, r.ms_prepare, r.ms_reduce, *walked);
+        }
     }
     return CHICLE_OK;
 }

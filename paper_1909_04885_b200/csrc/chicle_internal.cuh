@@ -21,6 +21,7 @@ enum : uint32_t {
 };
 
 constexpr int kStatusMaxNorm = 8; // the word of the status buffer where the largest squared norm is found
+constexpr int kStatusWalked = 9;  // and the one that counts the look-ahead solver's blocks that were walked in place
 
 // A -DCHICLE_DEBUG_BOUNDS build checks every index that the solvers and the gap kernels load from memory (visiting
 // order entries, row extents, entry ids, record directory entries, record sizes) before it is used as an address.
@@ -106,6 +107,8 @@ struct Glm {
     int hot_variant = 0;           // 1 / 2: most non-zeros fall on the first ids, the solver keeps those in a direct
                                    // array (2: with room for coordinates of up to 128 entries); 0: flat ids
     bool flat_ids = false;         // (tests) no part of the model in shared memory
+    bool by_chunks = false;        // sparse: the partitions follow the coordinates' numbers (chunks), not a random order
+    double chunk_mean = 0.0;       // largest average of a partition's numbers of entries that partitions by chunks have had
     // what a block of 32 random coordinates is expected to have on the ids of each class (id mod kRankClasses): entries, ids
     // that several of the 32 have, entries with such an id; and the variance of a coordinate's number of entries
     double blk_entries[kRankClasses] = {}, blk_shared_ids[kRankClasses] = {}, blk_shared[kRankClasses] = {};
@@ -177,6 +180,7 @@ cudaError_t launch_validate(Glm &g, bool values = true, bool rest = true); // th
 cudaError_t launch_sqnorm(Glm &g);
 cudaError_t launch_partition(Glm &g, int32_t K, uint64_t seed);           // fills owner, members
 cudaError_t launch_partition_chunks(Glm &g, int32_t K, int64_t C, const int64_t *chunk_off, const int32_t *chunk_task); // device arrays
+cudaError_t launch_chunk_entries(Glm &g, int64_t C, const int64_t *chunk_off, const int32_t *chunk_task, unsigned long long *entries); // += per task
 cudaError_t launch_permutation(Glm &g, int64_t round, int64_t epochs, int64_t H, const int64_t *steps); // fills perm[epochs * n_coord]
                                                                           // as far as a round of H steps (or the device's K budgets) walks
 cudaError_t launch_local_solver(Glm &g, int64_t H, float sigma_prime, int *variant);
@@ -193,6 +197,7 @@ cudaError_t launch_gather_f32(Glm &g, const float *src, const int32_t *map, int6
 cudaError_t launch_lookahead_solver(Glm &g, const struct SolverParams &P);
 cudaError_t launch_words(Glm &g, int64_t *dst, const int64_t *src, size_t n); // small host arrays to the device
 void lookahead_plan(Glm &g, int32_t K); // fills the la_* sizes for a partition into K
+int lookahead_arrays(const Glm &g, bool by_chunks, double chunk_mean); // which of the sparse prepare kernels would serve
 int lookahead_max_dense_dim();
 int lookahead_max_slices();
 int64_t lookahead_max_dim();

@@ -449,6 +449,8 @@ template <int HT> __device__ __forceinline__ uint32_t home_slot(int32_t id)
 {
     return id < kHD ? (uint32_t)id : kHD + __umulhi((uint32_t)id * 2654435761u, (uint32_t)(HT - kHD));
 }
+// entries that a block may have: the arrays', and slots for their ids if none is shared
+__host__ __device__ constexpr int pre_room(int nz, int ht) { return nz < ht - kHD ? nz : ht - kHD; }
 template <int HT> __device__ __forceinline__ uint32_t next_slot(uint32_t p) { return p + 1 < (uint32_t)HT ? p + 1 : kHD; }
 
 // ------------------------------------------------------------------------------------------------ prepare
@@ -591,7 +593,9 @@ template <int LOSS, int NZ, int HT, class Shared> __device__ __forceinline__ voi
         B.scl[lane] = usable ? __uint_as_float((uint32_t)(127 + 15 - e) << 23) : 0.0f;
         B.inv[lane] = usable ? __uint_as_float((uint32_t)(127 - 15 + e) << 23) : 0.0f;
     }
-    constexpr int room = NZ < HT - kHD ? NZ : HT - kHD; // entries, and slots for their ids if none is shared
+    constexpr int room = pre_room(NZ, HT);
+    // (a low word of the Gram matrices takes as many terms of 2^19 at most, see pre_pairs)
+    static_assert((int64_t)room << 19 < (int64_t)1 << 31, "the low words' range");
     const int m = n < room + 1 ? n : room + 1; // (more than the arrays hold is all that matters of a longer one)
     int incl = m;
 #pragma unroll
@@ -884,6 +888,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 pool_end = at + take < P.pool_cap ? at + take : P.pool_cap;
                 if (at + need > P.pool_cap) { sl = 2; pool_end = 0ull; }
             }
+            if (sl && lane == 0) atomicAdd(P.S.status + kStatusWalked, 1u);
             if (in) {
                 BlkDir d; // nothing to stage: the workers copy the first bytes of the head instead
                 d.offset = sl ? (unsigned long long)bid * sizeof(ChainHead) : P.pool_off + at + (incl - len);
@@ -1228,6 +1233,7 @@ template <int LOSS, bool LONG> __device__ __forceinline__ void prepare_block_den
         for (int c = 0; c < C; ++c) need += sub_bytes_dense(cnt, cols_of(c));
         unsigned long long at = atomicAdd(P.cursor, need);
         sh.walk = at + need > P.pool_cap ? 1 : 0; // no room: walked in place
+        if (sh.walk) atomicAdd(P.S.status + kStatusWalked, 1u);
         for (int c = 0; c < C; ++c) {
             BlkDir d;
             if (sh.walk) {
@@ -2399,13 +2405,31 @@ template <int LOSS, int NZ, int HT, int THREADS, int PER_SM> cudaError_t launch_
     return cudaGetLastError();
 }
 
-constexpr int kPreSmallNz = 2048;
-constexpr int kPreMidNz = 3072;
+constexpr int kPreSmallNz = 2048, kPreSmallHt = 2048;
+constexpr int kPreMidNz = 3072, kPreMidHt = 4096;
+constexpr int kPreLargeNz = 4096, kPreLargeHt = 4096;
 
-// true: the prepare kernel with arrays for 2 048 non-zeros per block serves (32 coordinates of 50 on average, with room)
-bool small_prepare(const Glm &g) { return 32.0 * (double)g.nnz / (double)g.n_coord * 1.25 <= (double)kPreSmallNz; }
-// true: arrays for 3 072 non-zeros per block serve
-bool mid_prepare(const Glm &g) { return 32.0 * (double)g.nnz / (double)g.n_coord * 1.1 <= (double)kPreMidNz; }
+// Whether the prepare kernel with arrays for `nz` non-zeros and `ht` ids per block serves: blocks of average rows `spare` times
+// over; partitions by chunks, whose rows may be the long ones, blocks of the longest partition's average rows and three standard
+// deviations more. (400 000 rows of 45 on average, sorted by length, K = 64: 3.3 ms a round with the arrays for 2 048, 1.9 with the
+// larger ones; the same rows over K = 8 and 16, whose partitions differ less, 2.5 -> 2.2 and 2.2 -> 1.9 with the smaller ones.)
+bool arrays_serve(const Glm &g, bool by_chunks, double chunk_mean, int nz, int ht, double spare)
+{
+    const double mean = (double)g.nnz / (double)g.n_coord;
+    return kLB * mean * spare <= (double)nz && (!by_chunks || kLB * chunk_mean + 3.0 * sqrt(kLB * g.row_variance) <= (double)pre_room(nz, ht));
+}
+// The prepare kernel that serves: 0 small (32 coordinates of 50 on average, with room), 1, 2 the longest blocks
+int arrays_of(const Glm &g, bool by_chunks, double chunk_mean)
+{
+    return arrays_serve(g, by_chunks, chunk_mean, kPreSmallNz, kPreSmallHt, 1.25) ? 0 : (arrays_serve(g, by_chunks, chunk_mean, kPreMidNz, kPreMidHt, 1.1) ? 1 : 2);
+}
+int arrays_of(const Glm &g) { return arrays_of(g, g.by_chunks, g.chunk_mean); }
+// entries of a block that it has room for
+int prepare_room(const Glm &g)
+{
+    const int a = arrays_of(g);
+    return a == 0 ? pre_room(kPreSmallNz, kPreSmallHt) : (a == 1 ? pre_room(kPreMidNz, kPreMidHt) : pre_room(kPreLargeNz, kPreLargeHt));
+}
 
 // The prepare kernel of one launch's blocks on `stream`.
 template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, cudaStream_t stream)
@@ -2428,9 +2452,10 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
     }
     cudaError_t e;
     const unsigned sms = stream == g.stream ? (unsigned)g.sm_count : free_sms;
-    if (small_prepare(g)) e = launch_prepare<LOSS, kPreSmallNz, 2048, 512, 2>(P, sms, stream);
-    else if (mid_prepare(g)) e = launch_prepare<LOSS, kPreMidNz, 4096, 1024, 1>(P, sms, stream);
-    else e = launch_prepare<LOSS, 4096, 4096, 1024, 1>(P, sms, stream);
+    const int arrays = arrays_of(g);
+    if (arrays == 0) e = launch_prepare<LOSS, kPreSmallNz, kPreSmallHt, 512, 2>(P, sms, stream);
+    else if (arrays == 1) e = launch_prepare<LOSS, kPreMidNz, kPreMidHt, 1024, 1>(P, sms, stream);
+    else e = launch_prepare<LOSS, kPreLargeNz, kPreLargeHt, 1024, 1>(P, sms, stream);
 #ifdef CHICLE_LA_TIMING
     if (e == cudaSuccess) {
         unsigned long long t[8] = {0};
@@ -2524,6 +2549,7 @@ cudaError_t launch_words(Glm &g, int64_t *dst, const int64_t *src, size_t n)
     return cudaGetLastError();
 }
 
+int lookahead_arrays(const Glm &g, bool by_chunks, double chunk_mean) { return arrays_of(g, by_chunks, chunk_mean); }
 int lookahead_max_dense_dim() { return kMaxC * kDenseSlice; }
 int lookahead_max_slices() { return 64; }
 int64_t lookahead_max_dim() { return (int64_t)1 << kIdBits; }
@@ -2592,29 +2618,36 @@ void lookahead_plan(Glm &g, int32_t K)
     if (!dense) {
         // A slot holds the record that a block of 32 random coordinates is expected to make for a CTA (how many entries, and how
         // many of them with ids that several of the 32 have: from the ids' frequencies, see launch_frequency_remap) and five
-        // standard deviations more; what is left keeps the model's most frequent ids. Where that leaves the model little, three
-        // slots do if dot products are taken one block ahead, and the root search on the chain instead of tables: a block
-        // without room is walked in place, 20 times slower.
+        // standard deviations more (`room`). Partitions by chunks may be sorted by class, time or length: the record of a block as
+        // long as the prepare kernel takes, whatever its rows share (`most`). (400 000 rows of 50, sorted by topic, K = 8: 82 ms a
+        // round with the first, 2.3 with the second.) What is left keeps the model's most frequent ids. Where that leaves the
+        // model little, three slots do if dot products are taken one block ahead, and the root search on the chain instead of
+        // tables: a block without room is walked in place, 20 times slower. (`most` for random partitions too: 2 M ridge columns
+        // over K = 128 12.5 -> 12.8 ms, logistic rows of 80 over K = 64, which lose their tables, 2.8 -> 3.8.)
         const int C = 1 << logC;
-        uint32_t room = 256;
+        uint32_t room = 256, most = 256;
+        const double cap = (double)prepare_room(g); // (a block with more entries is walked in place anyway)
         for (int c = 0; c < C; ++c) {
             double n = 0.0, T = 0.0, nl = 0.0;
             for (int i = c; i < kRankClasses; i += C) { n += g.blk_entries[i]; T += g.blk_shared_ids[i]; nl += g.blk_shared[i]; }
             const double all = (double)kLB * (double)g.nnz / (double)g.n_coord, part = all > 0.0 ? n / all : 0.0;
-            const double n_hi = n + 5.0 * sqrt(n + part * part * kLB * g.row_variance), f = n > 0.0 ? n_hi / n : 1.0;
+            double n_hi = n + 5.0 * sqrt(n + part * part * kLB * g.row_variance);
+            if (g.by_chunks) n_hi = fmax(n_hi, part * cap + 5.0 * sqrt(part * cap));
+            n_hi = fmin(n_hi, cap);
+            const double f = n > 0.0 ? fmax(1.0, n_hi / n) : 1.0;
             const double nl_hi = fmin(n_hi, f * nl + 5.0 * sqrt(nl)), T_hi = fmin(0.5 * nl_hi, f * T + 5.0 * sqrt(T));
-            if (n_hi > 65535.0) room = 0xffffffu; // (cut to what there is)
-            else {
-                const uint32_t r = sub_bytes((uint32_t)n_hi + 1u, (uint32_t)T_hi + 1u, (uint32_t)nl_hi + 1u) + 64u;
-                room = r > room ? r : room;
-            }
+            const uint32_t r = sub_bytes((uint32_t)n_hi + 1u, (uint32_t)T_hi + 1u, (uint32_t)nl_hi + 1u) + 64u;
+            const uint32_t m = sub_bytes((uint32_t)n_hi + 1u, (uint32_t)(0.5 * n_hi) + 1u, (uint32_t)n_hi + 1u) + 64u;
+            room = r > room ? r : room;
+            most = m > most ? m : most;
         }
+        if (g.by_chunks) room = most;
         for (;;) {
             const double left = (double)budget - (double)chain_layout(0, 0, 0, false, g.la_tab_bins).total - 64.0;
             g.la_slots = g.la_depth == 1 && 4.0 * room > 0.6 * left ? 3 : kSubSlots;
             if (g.la_tab_bins == 0 || (double)g.la_slots * room <= 0.8 * left) {
-                const uint32_t most = (uint32_t)(0.8 * left / g.la_slots) & ~15u;
-                g.la_sub_room = room < most ? room : most;
+                const uint32_t limit = (uint32_t)(0.8 * left / g.la_slots) & ~15u;
+                g.la_sub_room = room < limit ? room : limit;
                 break;
             }
             g.la_tab_bins = 0;
@@ -2623,6 +2656,9 @@ void lookahead_plan(Glm &g, int32_t K)
         int64_t hotc = ((int64_t)budget - (int64_t)L0.total - 64) / 4;
         hotc = hotc < 0 || g.flat_ids ? 0 : (hotc / 32) * 32;
         const int64_t need = (g.dim + ((int64_t)1 << logC) - 1) >> logC; // per CTA for the whole model
+        // (what the whole model leaves goes to the slots: rows may be more alike than their ids' frequencies say)
+        const int64_t spare = (4 * (hotc - (need + 31) / 32 * 32) / g.la_slots) & ~(int64_t)15;
+        if (spare > 0 && g.la_sub_room < most) g.la_sub_room += (uint32_t)((int64_t)(most - g.la_sub_room) < spare ? most - g.la_sub_room : spare);
         g.la_hotc = (int32_t)(hotc < need ? hotc : (need + 31) / 32 * 32);
     }
     g.la_smem = chain_layout(g.la_sub_room, g.la_slots, g.la_hotc, dense, g.la_tab_bins).total;

@@ -798,6 +798,20 @@ __global__ void k_owner_from_chunks(int64_t n, int64_t C, const int64_t *__restr
     }
 }
 
+// entries[t] += stored entries of task t's chunks
+__global__ void k_chunk_entries(int64_t C, const int64_t *__restrict__ chunk_off, const int32_t *__restrict__ chunk_task,
+                                const int64_t *__restrict__ indptr, unsigned long long *__restrict__ entries)
+{
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < C) atomicAdd(entries + chunk_task[c], (unsigned long long)(indptr[chunk_off[c + 1]] - indptr[chunk_off[c]]));
+}
+
+cudaError_t launch_chunk_entries(Glm &g, int64_t C, const int64_t *chunk_off, const int32_t *chunk_task, unsigned long long *entries)
+{
+    k_chunk_entries<<<blocks_for(C, 256), 256, 0, g.stream>>>(C, chunk_off, chunk_task, g.indptr, entries);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_partition_chunks(Glm &g, int32_t K, int64_t C, const int64_t *chunk_off, const int32_t *chunk_task)
 {
     const int64_t n = g.n_coord;
