@@ -2692,7 +2692,9 @@ void lookahead_plan(Glm &g, int32_t K)
         // (what the prepare kernel's CTAs hold in advance: a piece of about four blocks each)
         g.la_pool_piece = ((size_t)(4.0 * 12.0 * 32.0 * (double)g.nnz / (double)g.n_coord) + 4096) & ~(size_t)255; // (records start on 16-byte boundaries)
         part += (double)g.la_pool_piece * (double)(region_blocks < 2 * (int64_t)g.sm_count ? region_blocks : 2 * (int64_t)g.sm_count);
-        pool = (size_t)part + (size_t)region_blocks * C * 128 + 4096;
+        // (what is left of a piece when the next block's records are longer: up to a quarter where rows share most ids. Without this,
+        // rows of 50 over 100 ids, 1 M of them over K = 128, had no room for 610 of 32 000 blocks: 4.7 instead of 3.4 ms a round)
+        pool = (size_t)part + (size_t)region_blocks * (C * 128 + 1408) + 4096;
     }
     const size_t heads = ((size_t)region_blocks * sizeof(ChainHead) + 255) & ~(size_t)255;
     const size_t tabs = (size_t)region_blocks * tab_bytes(g.la_tab_bins);

@@ -56,7 +56,7 @@ def logged_walks(kind, n, K, chunks):
 
 
 @pytest.mark.parametrize("kind,n,K,chunks", [("topics", 40000, 8, True), ("topics", 40000, 64, True), ("lengths", 100000, 16, True),
-                                             ("lengths", 100000, 64, True), ("alike", 60000, 8, False)])
+                                             ("lengths", 100000, 64, True), ("alike", 60000, 8, False), ("alike", 1024000, 128, False)])
 def test_no_block_is_walked_in_place(kind, n, K, chunks):
     assert logged_walks(kind, n, K, chunks) == 0
 
