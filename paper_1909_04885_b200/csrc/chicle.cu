@@ -495,17 +495,21 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
         h->chunk_mean = chunk_mean;
         const bool dense_fmt = h->fmt == CHICLE_FMT_DENSE_ROWMAJOR;
         if (dense_fmt ? h->dim <= lookahead_max_dense_dim() : h->dim <= lookahead_max_dim()) {
-            lookahead_plan(*h, K);
-            unsigned char *rec = nullptr, *dir = nullptr;
-            if (alloc_into(h, rec, (size_t)h->la_regions * h->la_region_bytes) && alloc_into(h, dir, h->la_dir_bytes) &&
-                alloc_into(h, h->la_slice, (size_t)lookahead_max_slices() * (3 * (size_t)K + 2) + 64)) {
-                h->la_rec = rec;
-                h->la_dir = dir;
-                h->la_timing = reinterpret_cast<unsigned long long *>(h->la_slice) + (size_t)lookahead_max_slices() * (3 * (size_t)K + 2);
-                (void)cudaMemsetAsync(h->la_timing, 0, 64 * sizeof(unsigned long long), h->stream);
-            } else {
-                dev_free(h, rec); dev_free(h, dir); dev_free(h, h->la_slice);
-                h->la_slice = nullptr;
+            // (the logistic tables are the largest part of the records, 32 to 64 KB a block: without room for them, without them)
+            for (bool tables = true; !h->la_rec; tables = false) {
+                lookahead_plan(*h, K, tables);
+                unsigned char *rec = nullptr, *dir = nullptr;
+                if (alloc_into(h, rec, (size_t)h->la_regions * h->la_region_bytes) && alloc_into(h, dir, h->la_dir_bytes) &&
+                    alloc_into(h, h->la_slice, (size_t)lookahead_max_slices() * (3 * (size_t)K + 2) + 64)) {
+                    h->la_rec = rec;
+                    h->la_dir = dir;
+                    h->la_timing = reinterpret_cast<unsigned long long *>(h->la_slice) + (size_t)lookahead_max_slices() * (3 * (size_t)K + 2);
+                    (void)cudaMemsetAsync(h->la_timing, 0, 64 * sizeof(unsigned long long), h->stream);
+                } else {
+                    dev_free(h, rec); dev_free(h, dir); dev_free(h, h->la_slice);
+                    h->la_slice = nullptr;
+                    if (h->la_tab_bins == 0) break;
+                }
             }
         }
     }

@@ -196,7 +196,7 @@ cudaError_t launch_frequency_remap(Glm &g, uint32_t *counts, uint64_t *keys[2], 
 cudaError_t launch_gather_f32(Glm &g, const float *src, const int32_t *map, int64_t n, float *dst); // dst[i] = src[map[i]]
 cudaError_t launch_lookahead_solver(Glm &g, const struct SolverParams &P);
 cudaError_t launch_words(Glm &g, int64_t *dst, const int64_t *src, size_t n); // small host arrays to the device
-void lookahead_plan(Glm &g, int32_t K); // fills the la_* sizes for a partition into K
+void lookahead_plan(Glm &g, int32_t K, bool tables); // fills the la_* sizes for a partition into K (logistic: with or without tables)
 int lookahead_arrays(const Glm &g, bool by_chunks, double chunk_mean); // which of the sparse prepare kernels would serve
 int lookahead_max_dense_dim();
 int lookahead_max_slices();

@@ -2557,7 +2557,7 @@ int64_t lookahead_max_dim() { return (int64_t)1 << kIdBits; }
 // Sizes the look-ahead solver for a partition into K: CTAs per cluster, what stays in shared memory, and the record
 // buffer: `regions` regions that each hold one slice of a round (the recurrence records of its blocks, then a pool
 // for the workers' records).
-void lookahead_plan(Glm &g, int32_t K)
+void lookahead_plan(Glm &g, int32_t K, bool want_tables)
 {
     const bool dense = g.fmt == CHICLE_FMT_DENSE_ROWMAJOR;
     int logC = 0;
@@ -2604,7 +2604,7 @@ void lookahead_plan(Glm &g, int32_t K)
     // logistic tables: as many bins as the largest q = sigma' |x|^2 / (lambda n) at sigma' = K needs (a round with a larger
     // sigma' solves the roots on the chain), if two blocks' tables fit beside the rest
     g.la_tab_bins = 0;
-    if (g.loss == CHICLE_LOSS_LOGISTIC_DUAL) {
+    if (g.loss == CHICLE_LOSS_LOGISTIC_DUAL && want_tables) {
         const float q_max = (float)K * g.max_sqnorm / (g.lambda * (float)g.n_examples);
         for (int bins = 64; bins >= 32; bins >>= 1)
             if (q_max <= tab_max_q(bins)) g.la_tab_bins = bins;

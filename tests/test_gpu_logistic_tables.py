@@ -49,3 +49,27 @@ def test_small_states_relative_to_themselves(q, margin):
         assert (np.abs(a - b) / b).max() <= 1e-5, (np.abs(a - b) / b).max()
     finally:
         glm.close()
+
+
+@pytest.mark.parametrize("fmt", ["dense", "csr"])
+def test_no_memory_for_tables(fmt, monkeypatch):
+    # an allocator that refuses what the tables would take (32 KB a block): the look-ahead solver runs without them
+    from paper_1909_04885_b200 import binding
+    w = tiny_dense(4000, 28, seed=3, loss="logistic", K=4) if fmt == "dense" else tiny_csr(4000, 60, seed=3, loss="logistic", K=4)
+    serve = binding._TorchAllocator._alloc
+    refused = []
+
+    def limited(self, ctx, nbytes):
+        if nbytes > (3_000_000 if fmt == "dense" else 6_000_000):
+            refused.append(nbytes)
+            return None
+        return serve(self, ctx, nbytes)
+    monkeypatch.setattr(binding._TorchAllocator, "_alloc", limited)
+    run_parity(w, rounds=2)
+    assert len(refused) == 1
+    glm = binding.from_workload(w)
+    try:
+        glm.partition(4, 1)
+        assert glm.cocoa_round(0, 4.0, stats=True)["solver_variant"] in (4, 5)
+    finally:
+        glm.close()
