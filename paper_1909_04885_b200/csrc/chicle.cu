@@ -703,10 +703,12 @@ chicle_status_t chicle_export_state_of(chicle_glm_t *h, const uint8_t *host_keep
     if (h->K <= 0) return fail(h, CHICLE_ERR_BAD_STATE, "chicle_export_state_of needs a partition");
     if (!host_keep || !dev_out || len != h->n_coord)
         return fail(h, CHICLE_ERR_INVALID_ARG, "chicle_export_state_of: keep or out is NULL, or len is not the number of coordinates");
+    std::vector<uint8_t> own; // (pageable: read when the call returns, which a pinned array need not be)
+    try { own.assign(host_keep, host_keep + h->K); } catch (...) { return fail(h, CHICLE_ERR_OOM, "host allocation failed"); }
     cudaError_t e = cudaSetDevice(h->device);
     // (the K words of the step budgets are free between rounds: the K bytes travel through them)
     unsigned char *d_keep = reinterpret_cast<unsigned char *>(h->d_steps);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_keep, host_keep, (size_t)h->K, cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_keep, own.data(), (size_t)h->K, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = launch_mask_state(*h, d_keep, dev_out);
     if (e != cudaSuccess) return fail_cuda(h, e, "chicle_export_state_of");
     return CHICLE_OK;

@@ -2536,10 +2536,14 @@ template <int LOSS> cudaError_t launch_slices(Glm &g, std::vector<LookParams> &P
 } // namespace
 
 // A few words of host memory to the device: as arguments of a kernel (a copy from pageable memory costs the host 15 us, and
-// the stream waits for it); many of them as a copy, of which the runtime has taken its own when the call returns.
+// the stream waits for it); many of them as a copy from pageable memory, which the runtime has read when the call returns (the
+// caller's array may be pinned, and is then read when the stream gets there).
 cudaError_t launch_words(Glm &g, int64_t *dst, const int64_t *src, size_t n)
 {
-    if (n > 8 * kWordsPerLaunch) return cudaMemcpyAsync(dst, src, n * sizeof(int64_t), cudaMemcpyHostToDevice, g.stream);
+    if (n > 8 * kWordsPerLaunch) {
+        const std::vector<int64_t> own(src, src + n);
+        return cudaMemcpyAsync(dst, own.data(), n * sizeof(int64_t), cudaMemcpyHostToDevice, g.stream);
+    }
     for (size_t at = 0; at < n; at += kWordsPerLaunch) {
         WordArgs a;
         const size_t m = n - at < kWordsPerLaunch ? n - at : kWordsPerLaunch;
