@@ -1085,10 +1085,11 @@ struct PreDenseShared {
 };
 // Longer rows go through shared memory this many columns at a time.
 constexpr int kDenseCols = 128;
-// What counts as long: more columns than this, or half as many where there are more blocks than the kernel for short rows
-// takes at once (10 000 rows of 100, 313 blocks: 14 us against 20; with many blocks the other one's fewer loads count).
+// What counts as long: more columns than this (all of a shorter row is in shared memory at once). Up to here the kernel for short
+// rows is the faster one, with few blocks and with many: a round on rows of 100, 10 000 over K = 4: 133 us against 139 with
+// the other one, 100 000 over 64: 185 against 204, 1 M over 64: 1 571 against 1 933; rows of 128: 133 / 138, 197 / 212, 1 769 / 2 037.
 constexpr int kDenseLong = 128;
-inline bool dense_long(int64_t dim, int64_t blocks, int sms) { return dim > kDenseLong || (2 * dim > kDenseLong && blocks > (int64_t)sms * kPreDensePerSm); }
+inline bool dense_long(int64_t dim) { return dim > kDenseLong; }
 // 16-byte pieces of consecutive rows lie on different banks
 __host__ __device__ constexpr int row_stride(int cols) { return (((cols + 3) / 4) | 1) * 4; }
 inline size_t pre_dense_bytes(int dim, bool lng)
@@ -1178,7 +1179,7 @@ __device__ __forceinline__ void dense_gram_long(const LookParams &P, PreDenseSha
     }
     // the warps' sums: 4 .. 7 to 0 .. 3, 2 and 3 to 0 and 1, 1 to 0 (every lane has the same places in every warp)
     float4 *part = reinterpret_cast<float4 *>(sh.row);
-    static_assert(4 * 64 * 32 <= 2 * 2 * kLB * row_stride(kDenseLong / 2), "four warps' sums fit the rows' buffers");
+    static_assert(4 * 64 * 32 <= 2 * 2 * kLB * row_stride(kDenseCols), "four warps' sums fit the rows' buffers");
 #pragma unroll
     for (int half = 4; half > 0; half >>= 1) {
         if (warp >= half && warp < 2 * half) {
@@ -2440,7 +2441,7 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
     const int chain_sms = g.K << g.la_logC;
     const unsigned free_sms = (unsigned)(g.sm_count > chain_sms ? g.sm_count - chain_sms : 1);
     if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) {
-        const bool lng = dense_long(g.dim, nb, g.sm_count);
+        const bool lng = dense_long(g.dim);
         const unsigned per_sm = lng ? kPreDenseLongPerSm : kPreDensePerSm;
         const size_t smem = pre_dense_bytes((int)g.dim, lng);
         const unsigned grid = stream == g.stream || nb < free_sms * per_sm ? nb : free_sms * per_sm;
@@ -2591,12 +2592,12 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
     }
     g.la_logC = logC;
     // Beside chains on at most half of the SMs the prepare kernels run on the side stream; otherwise they alternate with
-    // the chain launches and have the whole GPU meanwhile (config 5, K = 128: 171 against 542 ms per round).
+    // the chain launches and have the whole GPU meanwhile (2 M ridge columns over K = 128: 12.5 against 584 ms a step).
     g.la_overlap = ((int64_t)K << logC) * 2 <= g.sm_count;
-    // Two blocks ahead pays where the chains bound the round: dense rows (the recurrence itself is the cost) and sparse
-    // data with a cluster per partition. One CTA per partition on sparse data means many partitions: there the prepare
-    // kernels bound the round and run 40 % faster without the cross Gram matrices (measured on the hashed workload: K = 64
-    // 157 against 219 ms per round; K = 16 with four CTAs per partition 253 against 308 ms the other way round).
+    // Two blocks ahead pays where the chains bound the round: dense rows (10 000 of 100, K = 4: 186 against 247 us a step) and
+    // sparse data with a cluster per partition (1 M rows of 50, K = 16: 4.0 against 5.2 ms; 45 M of 39: 156 against 278). One CTA
+    // per partition on sparse data means many partitions: there the prepare kernels bound the round, and are shorter without
+    // the cross Gram matrices (5.6 M hashed rows, a round with K = 64 and one with K = 16: 31.0 against 32.0 ms).
     g.la_depth = (dense || logC >= 1) && g.la_overlap ? 2 : 1;
     {
         const char *env = getenv("CHICLE_LA_DEPTH");
