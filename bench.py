@@ -149,17 +149,17 @@ def throughput(units, seconds_max):
 
 def read_profile_numbers():
     """Figures taken from committed ncu / timing-build summaries: DRAM bytes of the local solvers' kernels per
-    coordinate step for the headline shape (captured at reduced size; None once the solver source has changed since),
-    and the on-chip cost of one dependent step of the recurrence."""
+    coordinate step for the headline shape (captured at reduced size), and the on-chip cost of one dependent step of the
+    recurrence. None once the solver source has changed since."""
     import hashlib
     out = {"traffic_bytes_per_step": None, "t_step_ns": None}
     try:
         kv = dict(l.split(None, 1) for l in open(os.path.join(ROOT, "profiles", "local_scd_traffic.txt")) if l.strip() and l[0] != "#")
         kv = {k: v.strip() for k, v in kv.items()}
-        out["t_step_ns"] = float(kv["t_step_ns"])
         src = b"".join(open(os.path.join(ROOT, "paper_1909_04885_b200", "csrc", f), "rb").read()
                        for f in ("lookahead.cu", "solver_common.cuh"))
         if hashlib.sha256(src).hexdigest() == kv.get("solver_source_sha256"):
+            out["t_step_ns"] = float(kv["t_step_ns"])
             out["traffic_bytes_per_step"] = float(kv["dram_bytes_per_step_config4"])
             out["traffic_note"] = kv.get("note")
     except Exception:

@@ -266,7 +266,7 @@ chicle_status_t chicle_get_info(const chicle_glm_t *h, int64_t *round, int32_t *
  * counterpart: this entry point exists for deployment reasons only.) Who needs it: code that asks for a partition
  * map from a place where the device allocator is off limits, e.g. a serving or real-time loop whose memory pool was
  * sized and frozen at start-up, a thread that holds a lock the allocator also wants, or a process whose device
- * memory is handed out by another component. chicle_partition allocates its sort workspace and the K x dim update
+ * memory is handed out by another component. chicle_partition allocates its workspaces and the K x dim update
  * buffers; this call allocates nothing, on the host or on the device: no cudaMalloc, cudaFree, or framework
  * allocator. Its workspace (1 MB) is a static device array that every GPU loading this library holds until
  * the process ends.

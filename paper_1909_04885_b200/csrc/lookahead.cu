@@ -11,7 +11,8 @@
 // one warp runs it block after block without waiting for a model update, while the other warps, and the other CTAs
 // of the partition's thread-block cluster, apply block b's update to the model and take block b + 2's dot products.
 //
-//   k_lookahead_prepare   one CTA per block; nothing in it depends on the model. Writes the block's records: for
+//   k_lookahead_prepare   nothing in it depends on the model; a CTA takes a run of consecutive blocks (k_lookahead_prepare_dense:
+//                         a block at a time). Writes each block's records: for
 //                         the recurrence warp the per-step constants, the scaled Gram triangle and the scaled cross
 //                         Gram matrix with the next block; for each CTA of the cluster the block's non-zeros whose
 //                         entry id falls to that CTA (id mod cluster size), packed row after row, and for the ids
@@ -52,7 +53,8 @@ namespace {
 
 constexpr int kLB = 32;            // steps per block
 constexpr int kMaxC = 8;           // CTAs per cluster at most (the portable limit)
-constexpr int kDenseSlice = 384;   // columns of a dense row that one CTA of a cluster can take (a worker thread each)
+constexpr int kDenseSlice = 384;   // columns of a dense row that one CTA of a cluster can take: four blocks' slices fill its shared memory (an
+                                   // update takes the columns beyond kWorkThreads in a second turn)
 constexpr int kDenseEasy = 128;    // and what it takes where the cluster may be larger
 // Where the model entry of an id is, in kIdBits bits: its place in its CTA's part of the model in shared memory (below hotc),
 // or the id itself (never below hotc, see k_lookahead_chain). Problems with more ids take the blocked solver.
@@ -300,7 +302,7 @@ template <int LOSS> __device__ __forceinline__ float recurrence_map(float s, flo
 // ---- The logistic step from tables. a(c) = sigmoid(root of z + q sigmoid(z) = c) is a function of the state c alone once
 // the coordinate's q is known, and q does not depend on the model: the prepare kernel tabulates a(c) for each of a
 // block's coordinates as Taylor polynomials of degree 7, and a step of the chain is a look-up and a polynomial instead of
-// a root search (two exponentials, two divisions and two reciprocals one behind the other: 510 cycles, now about 90).
+// a root search (two exponentials, two divisions and two reciprocals one behind the other: 510 cycles, now 119).
 // a(c) is analytic but for branch points at c0 +- i pi (where 1 + q a (1 - a) = 0) and their mirror images at q - c0, and
 // a(q - c) = 1 - a(c), so u = min(c, q - c) is expanded about nodes whose distance grows like the distance to c0: with
 // x = (u - c0) / 3, four bins per octave of 1 + |x| on either side of c0. Below c0 the table holds a e^-u instead, which goes
@@ -1373,7 +1375,7 @@ template <int LOSS, bool LONG> __device__ __forceinline__ void prepare_block_den
     if (tid < kLB) out.hdr[tid] = sh.hdr[tid];
 }
 
-// (blocks blockIdx.x, blockIdx.x + gridDim.x, ...: see k_lookahead_prepare)
+// (blocks blockIdx.x, blockIdx.x + gridDim.x, ..)
 template <int LOSS, bool LONG> __global__ void __launch_bounds__(kPreThreads, LONG ? kPreDenseLongPerSm : kPreDensePerSm) k_lookahead_prepare_dense(const LookParams P)
 {
     extern __shared__ __align__(16) unsigned char smem_pre[];
@@ -1612,7 +1614,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             mbar_arrive_expect_tx(smem_u32(&ctl.dbar[i]), d_bytes);
         }
     }
-    // (eight words per thread and turn, all loads first: a launch must not spend a memory round trip on every 352 words)
+    // (eight words per thread and turn, all loads first: a launch must not spend a memory round trip on every 384 words)
     for (int l0 = tid; l0 < hot_mine; l0 += 8 * kChainThreads) {
         float u[8], v[8];
 #pragma unroll
@@ -2004,7 +2006,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         uint32_t dot_turn = 0;     // parity of how often slot s_dot has been filled
         bool ok = true;
 #ifdef CHICLE_LA_TIMING
-        long long wd = 0, ws = 0, wg = 0, ws1 = 0, wg0 = 0, wg1 = 0, t0 = clock64(), t1 = 0;
+        long long wd = 0, ws1 = 0, wg0 = 0, wg1 = 0, t0 = clock64(), t1 = 0;
 #endif
         // The loop starts `depth` blocks early: those turns only take the first blocks' dot products.
         bool sl0 = false, sl1 = false; // whether blocks b and b + 1 are walked in place
@@ -2299,7 +2301,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
 #ifdef CHICLE_LA_TIMING
         if (blockIdx.x == 0 && wt == 0) {
             unsigned long long *d = P.timing + 4;
-            d[0] = wd; d[1] = ws; d[2] = wg; d[3] = ws1; d[4] = wg0; d[5] = wg1;
+            d[0] = wd; d[3] = ws1; d[4] = wg0; d[5] = wg1;
         }
 #endif
         if (!aborted) {
@@ -2464,7 +2466,7 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
         (void)cudaMemcpy(t, P.timing + 16, sizeof(t), cudaMemcpyDeviceToHost);
         (void)cudaMemset(P.timing + 16, 0, sizeof(t));
         const double n = (double)nb;
-        fprintf(stderr, "lookahead prepare, cycles per block: insert %.0f, number %.0f, place %.0f, entries %.0f, scan and pairs %.0f, dense and write %.0f\n", t[0] / n, t[1] / n, t[2] / n, t[3] / n, t[4] / n, t[5] / n, t[6] / n, t[7] / n);
+        fprintf(stderr, "lookahead prepare, cycles per block: insert %.0f, number %.0f, place %.0f, entries %.0f, scan and pairs %.0f, dense and write %.0f\n", t[0] / n, t[1] / n, t[2] / n, t[3] / n, t[4] / n, t[5] / n);
     }
 #endif
     return e;
@@ -2583,8 +2585,8 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
     int slice = (int)((g.dim + 3) & ~(int64_t)3); // dense: columns per CTA
     if (dense) {
         // Long rows are shared out over a cluster: slices of about 128 columns where the SMs allow it for all partitions at
-        // once, else as few CTAs as slices of 384 columns need (a worker thread per column, four blocks' slices in shared
-        // memory); the clusters then take turns.
+        // once, else as few CTAs as slices of 384 columns need (the most that
+        // four blocks' slices leave room for); the clusters then take turns.
         auto cut = [&](int lg) { return (int)((((g.dim + (1 << lg) - 1) >> lg) + 3) & ~(int64_t)3); };
         while (logC < 3 && cut(logC) > kDenseSlice) ++logC;
         while (logC < 3 && cut(logC) > kDenseEasy && ((int64_t)K << (logC + 1)) <= g.sm_count) ++logC;
