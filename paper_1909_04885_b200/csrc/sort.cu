@@ -1,5 +1,5 @@
 // Stable least-significant-digit radix sort pass (8 bits) over (64-bit key, 32-bit value) pairs.
-// Used by the partition step (order ids by their mixed key) and the per-round visiting orders.
+// Used by the ranking of the ids at create, and to group the members of more than 256 partitions.
 //
 // One pass = digit histogram per tile -> exclusive scan of the digit-major table -> stable scatter.
 // The scatter ranks items inside a tile in index order: each warp owns a contiguous run of the tile and

@@ -2,7 +2,7 @@
 
 ``chicle_partition_noalloc`` is for callers that cannot allocate device memory at the moment they need a partition
 map (a memory pool frozen at start-up, a serving loop with a fixed budget, a thread holding a lock the allocator
-needs). It keeps its sort workspace in a fixed array inside the library, shared by all calls, so this test calls it
+needs). It keeps what workspace it needs in a fixed array inside the library, shared by all calls, so this test calls it
 twice in a row with different arguments to show that leftovers of one call do not leak into the next, and compares
 both results with ``chicle_partition`` bit for bit (integer work: no tolerance). This file is collected last on
 purpose: a failure here cannot hide the other GPU tests from a run that stops at the first failure.
