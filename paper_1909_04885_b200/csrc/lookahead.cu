@@ -270,6 +270,17 @@ __device__ __forceinline__ uint32_t lds_u8_if(uint32_t a, bool on)
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t@q ld.shared.u8 %0, [%1];\n\t}" : "=r"(v) : "r"(a), "r"((uint32_t)on) : "memory");
     return v;
 }
+// Atomics on shared memory, only where `on` holds (a thread's several are under way together).
+__device__ __forceinline__ void red_shared_add_if(uint32_t a, int32_t v, bool on)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q red.shared.add.s32 [%0], %1;\n\t}" ::"r"(a), "r"(v), "r"((uint32_t)on) : "memory");
+}
+// Two fused multiply-adds in one instruction, each rounded as usual.
+__device__ __forceinline__ void fma2(float2 &acc, float ax, float ay, float bx, float by)
+{
+    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%0, %1};\n\tfma.rn.f32x2 c, a, b, c;\n\tmov.b64 {%0, %1}, c;\n\t}"
+        : "+f"(acc.x), "+f"(acc.y) : "f"(ax), "f"(ay), "f"(bx), "f"(by));
+}
 __device__ __forceinline__ void red_add_if(float *p, float v, bool on)
 {
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q red.global.add.f32 [%0], %1;\n\t}" ::"l"(p), "f"(v), "r"((uint32_t)on) : "memory");
@@ -444,16 +455,17 @@ __device__ __forceinline__ float tab_map(float c, float q, float off, float off2
 }
 
 // The most frequent ids (ids are frequency-ranked) are in most of a block's coordinates. Their part of the Gram
-// matrices is taken from dense 32 x kHD tiles; only the other entries are walked through the table. Table slot: the id itself below kHD, a hashed slot above.
+// matrices is taken from dense 32 x kHD tiles; only the other entries are walked through the table.
 constexpr int kHD = 32;
 constexpr int kHDS = kHD + 4; // row stride of the tiles: 16-byte loads of consecutive rows fall on different banks
-template <int HT> __device__ __forceinline__ uint32_t home_slot(int32_t id)
-{
-    return id < kHD ? (uint32_t)id : kHD + __umulhi((uint32_t)id * 2654435761u, (uint32_t)(HT - kHD));
-}
+// Table slots: the ids below kDir have their own (no key, no tries); HT hashed ones behind them for the others.
+// (As many as shared memory leaves: at two CTAs per SM nothing is free.)
+constexpr int kDir = 768;
+// Hashed slots: HT of them, a power of two; the t-th try lies t places behind the one before, which reaches every one.
+template <int HT> __device__ __forceinline__ uint32_t home_place(int32_t id) { return __umulhi((uint32_t)id * 2654435761u, (uint32_t)HT); }
+template <int HT> __device__ __forceinline__ uint32_t next_place(uint32_t p, int t) { return (p + (uint32_t)t) & (uint32_t)(HT - 1); }
 // entries that a block may have: the arrays', and slots for their ids if none is shared
 __host__ __device__ constexpr int pre_room(int nz, int ht) { return nz < ht - kHD ? nz : ht - kHD; }
-template <int HT> __device__ __forceinline__ uint32_t next_slot(uint32_t p) { return p + 1 < (uint32_t)HT ? p + 1 : kHD; }
 
 // ------------------------------------------------------------------------------------------------ prepare
 // A CTA takes a run of consecutive blocks, so that a block's rows are fetched once: they serve as the next block of the
@@ -461,8 +473,13 @@ template <int HT> __device__ __forceinline__ uint32_t next_slot(uint32_t p) { re
 // run ahead of their use: while block b is worked on, the rows of b + 1, the row extents and constants of b + 2 and the
 // visiting-order entries of b + 3 are under way. Passes over the block's non-zeros take them as one flat array (32 at a
 // time whatever the rows' lengths).
-// What bounds it is instruction issue and shared-memory latency; before (a CTA per block, each fetching its own rows and
-// its successor's in three dependent round trips) a block of 1 600 non-zeros took 63 000 cycles at three CTAs per SM.
+// What bounds it is the number of instructions and shared-memory turns (each at 55 to 60 % of what the SM can do), and the barriers
+// between the phases; before (a CTA per block, each fetching its own rows and its successor's in three dependent round trips) a
+// block of 1 600 non-zeros took 63 000 cycles at three CTAs per SM. Rows of 50 on 1 M coordinates, a slice of 4 096 blocks on the whole
+// GPU: 255 us; with slots without tries for frequent ids, entries' findings kept in registers, one atomic per numbered id and the
+// pairs shared out evenly 225 us (instructions a block 40 700 -> 35 200); step 4.01 -> 3.59 ms, ridge 12.5 -> 11.1 (longer blocks
+// have more tries to save). A thread's several entries together, all loads first: 46 100 instructions, 272 us. 640 or 416
+// threads: 254 and 244 us; 256 us at 384.
 constexpr int kDirNew = 4; // (metadata slots: a power of two)
 
 // One block's coordinates as the kernel keeps them: constants of the steps and extents of the rows.
@@ -476,30 +493,46 @@ struct PreBlock {
     int32_t k, cnt, total, over;      // partition; over: more non-zeros than the arrays hold (total is 0 then): walked in place
 };
 
+// The shared ids of a CTA of the cluster, counted while they are numbered: list entries, ids with up to four of them, ids with
+// more. One word holds all three where the arrays are small (one atomic per id); else the short lists have their own.
+template <int NZ> struct PreCount {
+    static constexpr bool kOne = NZ <= 2048;
+    static constexpr int kLongBit = kOne ? 23 : 16;
+    static_assert(!kOne || (NZ < 1 << 12 && NZ / 2 < 1 << 11 && NZ / 5 < 1 << 9), "the fields of the one word");
+    static_assert(NZ <= 4096, "the fields of two words");
+    __device__ static uint32_t entries(uint32_t w) { return kOne ? w & 0xfffu : w & 0xffffu; }
+    __device__ static uint32_t longs(uint32_t w) { return w >> kLongBit; }
+    __device__ static uint32_t shorts(uint32_t w, uint32_t s) { return kOne ? (w >> 12) & 0x7ffu : s; }
+};
+// A CTA's record of the block: where its parts are (bytes behind the head), and where its lists start in lval.
+struct alignas(16) PreRec {
+    unsigned long long at; // from the start of the region
+    uint32_t meta, ids;
+    uint32_t lval, lst, lrow;
+    uint16_t base, longs;
+};
+
 template <int NZ, int HT, int THREADS> struct PreShared {
     static constexpr int CH = NZ / 32;  // chunks of 32 entries
-    alignas(16) int32_t key[HT];        // id in a table slot, -1 = empty
-    alignas(16) uint32_t mask[HT];      // bit j: coordinate j of the block has this id
-    uint16_t soff[HT];                  // where the id's values are: an entry of val (one coordinate has it), or NZ + a place in lval
-    uint16_t coff[HT];                  // a shared id: start of its list among the lists of its CTA's record
-    int32_t idx[2][NZ];                 // the block's entries, and the next block's
-    float val[2][NZ];
-    float lval[NZ];                     // the scaled values of shared ids, one list per id, each in ascending coordinate order
-    uint16_t slot[NZ];                  // table slot of each entry's id
-    uint8_t row[2][NZ];                 // coordinate of each entry
+    static constexpr int TS = kDir + HT; // table slots
+    alignas(16) int32_t key[HT];        // id in a hashed slot, -1 = empty
+    alignas(16) uint32_t mask[TS];      // bit j: coordinate j of the block has this id
+    uint16_t lists[TS];                   // one coordinate has the id: its entry; several: where the id's list starts among those of its CTA (12 bits), CTA
+    alignas(128) int32_t idx[2][NZ];    // the block's entries, and the next block's
+    float val[3][NZ];                   // [2]: the scaled values of shared ids, one list per id, each in ascending coordinate order
+    uint8_t row[3][NZ];                 // coordinate of each entry
     uint32_t bal[2][CH + 1][kMaxC];     // per chunk and CTA: which of the entries fall to it
     uint16_t pre[2][CH + 1][kMaxC];     // and how many before the chunk
-    int32_t G[2][kLB][kLB];             // Gram triangle and cross Gram matrix, fixed point (the low words lie in idx, see pre_pairs)
-    uint32_t work[THREADS / 32][2 * 32]; // per warp: entries whose pairs are still to be added; then its sums for A and q0n
+    alignas(128) int32_t G[2][kLB][kLB]; // Gram triangle and cross Gram matrix, fixed point (the low words lie in idx, see pre_pairs)
+    uint32_t work[THREADS / 32][3 * 32]; // per warp: entries whose pairs are still to be added; then its sums for A and q0n
     alignas(16) float D[2][kLB][kHDS];  // the entries with the kHD most frequent ids, dense
     PreBlock blk[kDirNew];
     int32_t coord[kDirNew][kLB];        // visiting-order entries
     int64_t ip[2][kLB];                 // fetched for a block: row extents, squared norms, states, labels
     float sq[kLB], al[kLB], lb[kLB];
     uint16_t rc[kLB + 1][kMaxC];        // where coordinate j's entries start in CTA c's record
-    uint32_t cntTL[kMaxC], cntAll;      // per CTA: shared ids (high half) and their list entries (low half); all list entries
-    uint32_t cntLong[kMaxC];            // per CTA: ids with up to four list entries (high half) and with more (low half)
-    unsigned long long sub_off[kMaxC];
+    uint32_t cnt[kMaxC], cntShort[kMaxC]; // per CTA: its shared ids, see PreCount
+    PreRec rec[kMaxC];
     int32_t walk;
     unsigned long long pool_at, pool_end; // what this CTA holds of the pool
     int32_t base[kBaseStaged];          // blk_base, and first step and step count of each partition (see pre_locate)
@@ -631,17 +664,17 @@ template <int NZ, int THREADS, class Shared> __device__ __forceinline__ void pre
         }
     }
 }
-// (a warp: which of 32 consecutive entries fall to which CTA, and their part of the dense tile; id < 0: no entry)
-template <class Shared> __device__ __forceinline__ void pre_classify(const LookParams &P, Shared &sh, int32_t id, int e, int buf)
+// (a warp: which of 32 consecutive entries fall to which CTA, and their part of the dense tile; id < 0: no entry. flip: per bit of a CTA's
+// number, all ones where this lane's number has a 0 there)
+template <class Shared> __device__ __forceinline__ void pre_classify(const LookParams &P, Shared &sh, int32_t id, int e, int buf, const uint32_t (&flip)[3])
 {
     const int lane = threadIdx.x & 31;
     uint32_t mine = __ballot_sync(0xffffffffu, id >= 0);
-    for (int bit = 0; bit < P.logC; ++bit) {
-        const uint32_t b = __ballot_sync(0xffffffffu, (id >> bit) & 1);
-        mine &= (lane >> bit) & 1 ? b : ~b;
-    }
+#pragma unroll
+    for (int bit = 0; bit < 3; ++bit)
+        if (bit < P.logC) mine &= __ballot_sync(0xffffffffu, (id & (1 << bit)) != 0) ^ flip[bit];
     if (lane >> P.logC == 0) sh.bal[buf][e >> 5][lane] = mine; // lane c: the entries of CTA c
-    if (id >= 0 && id < kHD) sh.D[buf][sh.row[buf][e]][id] = sh.val[buf][e];
+    if ((uint32_t)id < (uint32_t)kHD) sh.D[buf][sh.row[buf][e]][id] = sh.val[buf][e];
 }
 // (warp c: how many of the entries before each chunk fall to CTA c)
 template <class Shared> __device__ __forceinline__ void pre_prefix(Shared &sh, int total, int buf, int c)
@@ -669,35 +702,75 @@ template <class Shared> __device__ __forceinline__ void pre_prefix(Shared &sh, i
 // does not depend on the order. Values are scaled by a power of two below 2^15 / |x| (exact), a product is below 2^30 and
 // so is every partial sum of an entry (|sum| <= |x_l| |x_j|); what rounding a product to a whole number leaves goes to a second
 // word, 2^20 times finer: together finer than an fp32 sum is.
-// (Walking lists with shuffles in a fixed order took 14 000 of 31 000 cycles a block.)
+// (Walking lists with shuffles in a fixed order took 14 000 of 31 000 cycles a block; a lane per entry, whose loops last as long as the
+// longest of 32, 7 500 instructions a block of 1 600 entries, against 1 500 with the pairs shared out.)
+// Entry (l, j) of a matrix lies at place l ^ j of row j: the 32 entries whose pairs a warp adds together come from one or two
+// coordinates j and have any l, so its atomics fall on different banks.
+__device__ __forceinline__ int gram_place(int l, int j) { return j * kLB + (l ^ j); }
+// A warp takes 32 entries with pairs at a time and shares their pairs out evenly: pair t of the 32 entries' belongs to the last
+// entry whose pairs start at or before t.
 template <int NZ, class Shared>
 __device__ __forceinline__ void pre_pairs(Shared &sh, uint32_t item, bool on, int cur, const PreBlock &N)
 {
-    const int e = (int)(item & 4095u), p = (int)((item >> 12) & 4095u), next = (int)(item >> 24);
-    uint32_t m = 0u;
-    uint32_t at = 0u;
+    const int lane = threadIdx.x & 31;
+    int n = 0;          // pairs of this lane's entry
+    uint32_t with = 0u; // where the values and coordinates are that it is paired with (as an index of val[0], row[0])
+    uint32_t to = 0u;   // row of G (next, j), and j
     float x = 0.0f;
-    int col = 0;
     if (on) {
-        const int buf = cur ^ next, j = sh.row[buf][e], so = sh.soff[p];
-        m = sh.mask[p];
+        const int e = (int)(item & 4095u), p = (int)((item >> 12) & 8191u), next = (int)(item >> 25);
+        const int buf = cur ^ next, j = sh.row[buf][e], off = sh.lists[p];
+        uint32_t m = sh.mask[p];
+        with = (m & (m - 1u)) == 0u ? (uint32_t)(cur * NZ + off) : (uint32_t)(2 * NZ + sh.rec[off >> 12].base + (off & 4095));
         x = sh.val[buf][e];
         if (next) x *= N.scl[j];
         else m &= (1u << j) - 1u;
-        at = so < NZ ? smem_u32(&sh.val[cur][so]) : smem_u32(&sh.lval[so - NZ]);
-        col = next * kLB * kLB + j;
+        n = __popc(m);
+        to = (uint32_t)(next * kLB * kLB + j * kLB + j) * 4u; // (its place for l = 0; the others by the bits of 4 l)
     }
-    int32_t *hi = &sh.G[0][0][0] + col, *lo = &sh.idx[cur][0] + col;
-    while (m) {
-        const int l = (__ffs((int)m) - 1) * kLB;
-        m &= m - 1u;
-        const float v = lds_f32(at) * x;
-        at += 4u;
-        const int h = __float2int_rn(v), r = __float2int_rn((v - (float)h) * 1048576.0f);
-        atomicAdd(hi + l, h);
-        if (r) atomicAdd(lo + l, r);
+    int start = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, start, o);
+        if (lane >= o) start += t;
+    }
+    const int all = __shfl_sync(0xffffffffu, start, 31);
+    start -= n;
+    with -= (uint32_t)start; // (of the pair t: with + t)
+    const uint32_t hi = smem_u32(&sh.G[0][0][0]), lo = smem_u32(&sh.idx[cur][0]), val0 = smem_u32(&sh.val[0][0]), row0 = smem_u32(&sh.row[0][0]);
+    int before = -1;    // entries that start before the 32 pairs, less one
+#pragma unroll 1
+    for (int t0 = 0; t0 < all; t0 += 32) {
+        const uint32_t at = (uint32_t)(start - t0);
+        const uint32_t starts = __reduce_or_sync(0xffffffffu, n > 0 && at < 32u ? 1u << at : 0u);
+        const int from = before + __popc(starts & (0xffffffffu >> (31 - lane)));
+        before += __popc(starts);
+        const uint32_t u = __shfl_sync(0xffffffffu, with, from) + (uint32_t)(t0 + lane);
+        const uint32_t g = __shfl_sync(0xffffffffu, to, from);
+        const float y = __shfl_sync(0xffffffffu, x, from);
+        if (t0 + lane < all) {
+            const float v = lds_f32(val0 + 4u * u) * y;
+            const uint32_t word = g ^ (4u * lds_u8_if(row0 + u, true));
+            const int h = __float2int_rn(v), r = __float2int_rn((v - (float)h) * 1048576.0f);
+            red_shared_add_if(hi + word, h, true);
+            red_shared_add_if(lo + word, r, r != 0);
+        }
     }
 }
+
+// (a warp: the pairs of `have` listed entries)
+template <int NZ, class Shared>
+__device__ __forceinline__ void pre_listed(Shared &sh, int have, int cur, const PreBlock &N)
+{
+    const uint32_t *todo = sh.work[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int at = 0; at < have; at += 32) pre_pairs<NZ>(sh, at + lane < have ? todo[at + lane] : 0u, at + lane < have, cur, N);
+    __syncwarp();
+}
+// (not inlined: for lists longer than usual, between their parts)
+template <int NZ, class Shared>
+__device__ __noinline__ void pre_listed_early(Shared &sh, int have, int cur, const PreBlock &N) { pre_listed<NZ>(sh, have, cur, N); }
 
 // What the states at round start contribute: the warps' sums (sh.work) together, off A and into q0n; the block's constants
 // go out. (A warp; one block behind the loop, so that it needs no barrier of its own.)
@@ -720,7 +793,7 @@ template <int NW, class Shared> __device__ __forceinline__ void pre_finish_head(
 template <int LOSS, int NZ, int HT, int THREADS, int PER_SM>
 __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const LookParams P)
 {
-    extern __shared__ __align__(16) unsigned char smem_pre[];
+    extern __shared__ __align__(128) unsigned char smem_pre[];
     using Shared = PreShared<NZ, HT, THREADS>;
     Shared &sh = *reinterpret_cast<Shared *>(smem_pre);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -739,11 +812,13 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 sh.steps[i] = (int32_t)steps_of(P, i, P.S.part_off[i + 1] - P.S.part_off[i]);
             }
         }
-    for (int p = tid; p < HT; p += THREADS) { sh.key[p] = -1; sh.mask[p] = 0u; }
+    for (int p = tid; p < HT; p += THREADS) sh.key[p] = -1;
+    for (int p = tid; p < Shared::TS; p += THREADS) sh.mask[p] = 0u;
     for (int p = tid; p < 2 * kLB * kHDS; p += THREADS) (&sh.D[0][0][0])[p] = 0.0f;
-    if (tid < kMaxC) sh.cntTL[tid] = sh.cntLong[tid] = 0u;
-    if (tid == 0) { sh.cntAll = 0u; sh.pool_at = sh.pool_end = 0ull; }
+    if (tid < kMaxC) sh.cnt[tid] = sh.cntShort[tid] = 0u;
+    if (tid == 0) sh.pool_at = sh.pool_end = 0ull;
     __syncthreads();
+    const uint32_t flip[3] = {lane & 1 ? 0u : ~0u, lane & 2 ? 0u : ~0u, lane & 4 ? 0u : ~0u};
     // blocks that are fetched: the run, and the one behind it where the last block has a cross Gram matrix with it
     int64_t end = hi;
     if (P.depth >= 2 && hi < P.n_blocks && pre_locate(P, sh, hi).k == pre_locate(P, sh, hi - 1).k) end = hi + 1;
@@ -763,7 +838,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
     cp_async_wait_all();
     __syncthreads();
     for (int e = tid; (e & ~31) < sh.blk[lo & (kDirNew - 1)].total; e += THREADS)
-        pre_classify(P, sh, e < sh.blk[lo & (kDirNew - 1)].total ? checked_id(P, sh.idx[lo & 1][e]) : -1, e, (int)(lo & 1));
+        pre_classify(P, sh, e < sh.blk[lo & (kDirNew - 1)].total ? checked_id(P, sh.idx[lo & 1][e]) : -1, e, (int)(lo & 1), flip);
     __syncthreads();
     if (warp < C) pre_prefix(sh, sh.blk[lo & (kDirNew - 1)].total, (int)(lo & 1), warp);
     __syncthreads();
@@ -786,98 +861,85 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         if (have_next) pre_fetch_rows<NZ, THREADS>(P, sh, bid + 1, nxt);
         if (warp == NW - 1 && bid + 2 < end) pre_fetch_extents<LOSS>(P, sh, bid + 2);
         if (warp == NW - 2 && bid + 3 < end) pre_fetch_order(P, sh, bid + 3);
-        for (int p = tid; p < kLB * kHDS; p += THREADS) (&sh.D[nxt][0][0])[p] = 0.0f;
-        for (int p = tid; p < 2 * kLB * kLB; p += THREADS) (&sh.G[0][0][0])[p] = 0;
+        for (int p = tid; p < kLB * kHDS / 4; p += THREADS) reinterpret_cast<float4 *>(&sh.D[nxt][0][0])[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int p = tid; p < 2 * kLB * kLB / 4; p += THREADS) reinterpret_cast<int4 *>(&sh.G[0][0][0])[p] = make_int4(0, 0, 0, 0);
         if (warp == NW - 4 && bid > lo) pre_finish_head<NW>(P, sh, bid - 1);
-        // ---- every id into the table
-        {
-            int32_t id[EPT], seen[EPT];
-            uint32_t p[EPT];
+        // ---- every id into the table. What a thread has found out about its entries stays in registers for the whole block:
+        //      id, table slot, coordinate, mask of the coordinates that have the id. (32 entries of a warp after the other, and not a
+        //      thread's several together: what bounds this kernel is the number of instructions.)
+        int32_t id[EPT];
+        uint32_t slot[EPT], m[EPT]; // (slot: its coordinate in the high half)
 #pragma unroll
-            for (int i = 0; i < EPT; ++i) {
-                const int e = tid + i * THREADS;
-                id[i] = e < total ? checked_id(P, sh.idx[cur][e]) : -1;
-                p[i] = home_slot<HT>(id[i] >= 0 ? id[i] : 0);
-            }
+        for (int i = 0; i < EPT; ++i) {
+            const int e = tid + i * THREADS;
+            id[i] = e < total ? checked_id(P, sh.idx[cur][e]) : -1;
+            slot[i] = m[i] = 0u;
+        }
 #pragma unroll
-            for (int i = 0; i < EPT; ++i) { // (most find their place at the first try: a thread's tries are under way together)
-                seen[i] = -1;
-                if (id[i] >= kHD) seen[i] = atomicCAS(&sh.key[p[i]], -1, id[i]);
-                else if (id[i] >= 0) sh.key[p[i]] = id[i];
-            }
-#pragma unroll
-            for (int i = 0; i < EPT; ++i) {
-                const int e = tid + i * THREADS;
-                if (e >= total) break;
-                for (int t = 0; t < HT && seen[i] != -1 && seen[i] != id[i]; ++t) {
-                    p[i] = next_slot<HT>(p[i]);
-                    seen[i] = sh.key[p[i]];
-                    if (seen[i] == -1) seen[i] = atomicCAS(&sh.key[p[i]], -1, id[i]);
+        for (int i = 0; i < EPT; ++i) {
+            if ((tid & ~31) + i * THREADS >= total) break; // (whole warps)
+            uint32_t p = (uint32_t)id[i];
+            if (id[i] >= kDir) {
+                p = home_place<HT>(id[i]);
+                for (int t = 1; t <= HT; ++t) {
+                    const int32_t seen = atomicCAS(&sh.key[p], -1, id[i]);
+                    if (seen == -1 || seen == id[i]) break;
+                    p = next_place<HT>(p, t);
                 }
-                atomicOr(&sh.mask[p[i]], 1u << sh.row[cur][e]);
-                sh.slot[e] = (uint16_t)p[i];
+                p += kDir;
             }
+            const uint32_t j = sh.row[cur][tid + i * THREADS];
+            if (id[i] >= 0) atomicOr(&sh.mask[p], 1u << j);
+            slot[i] = (p & 0xffffu) | j << 16;
+        }
+        // where each coordinate's entries start in each CTA's record
+        for (int i = tid; i < (kLB + 1) << P.logC; i += THREADS) {
+            const int j = i >> P.logC, c = i & (C - 1), at = B.roff[j], ch = at >> 5;
+            sh.rc[j][c] = (uint16_t)(sh.pre[cur][ch][c] + __popc(sh.bal[cur][ch][c] & ((1u << (at & 31)) - 1u)));
         }
         __syncthreads();
         PRE_T(0);
-        // ---- the first coordinate that has an id numbers it: shared ids among their CTA's (ids in the high half of the
-        //      counter, list entries in the low half) and in lval. (The order of the numbers varies from run to run, which
-        //      moves records' contents about but changes no result: every id's own sum is taken in coordinate order, in a
-        //      shape that depends on the list's length alone.)
-        uint32_t tl[EPT];
-        {
-            uint32_t p[EPT], m[EPT], ls[EPT], rk[EPT];
-            int32_t id[EPT];
+        // ---- the first coordinate that has an id numbers it, if others have it too: its place among its CTA's lists. (The order of
+        //      the numbers varies from run to run, which moves records' contents about but changes no result: every id's own sum
+        //      is taken in coordinate order, in a shape that depends on the list's length alone.)
+        using Count = PreCount<NZ>;
+        uint32_t tl[EPT]; // of an id numbered here: where its list starts (low half), its number among the long or the short ones; else all ones
 #pragma unroll
-            for (int i = 0; i < EPT; ++i) {
-                const int e = tid + i * THREADS;
-                p[i] = e < total ? sh.slot[e] : 0u;
-                id[i] = e < total ? checked_id(P, sh.idx[cur][e]) : 0;
-                const uint32_t all = e < total ? sh.mask[p[i]] : 0u;
-                m[i] = e < total && (all & ((1u << sh.row[cur][e]) - 1u)) == 0u ? all : 0u; // 0: an earlier coordinate has the id
+        for (int i = 0; i < EPT; ++i) {
+            tl[i] = 0xffffffffu;
+            if ((tid & ~31) + i * THREADS >= total) break;
+            if (id[i] < 0) continue;
+            const uint32_t p = slot[i] & 0xffffu;
+            m[i] = sh.mask[p];
+            if ((m[i] & ((1u << (slot[i] >> 16)) - 1u)) != 0u) continue;
+            uint32_t off = (uint32_t)(tid + i * THREADS);
+            if ((m[i] & (m[i] - 1u)) != 0u) {
+                const uint32_t c = (uint32_t)id[i] & (uint32_t)(C - 1), n = (uint32_t)__popc(m[i]);
+                const uint32_t w = atomicAdd(&sh.cnt[c], n + (n > 4u ? 1u << Count::kLongBit : (Count::kOne ? 1u << 12 : 0u)));
+                const uint32_t s = !Count::kOne && n <= 4u ? atomicAdd(&sh.cntShort[c], 1u) : 0u;
+                off = Count::entries(w) | c << 12;
+                tl[i] = Count::entries(w) | (n > 4u ? Count::longs(w) : Count::shorts(w, s)) << 16;
             }
-#pragma unroll
-            for (int i = 0; i < EPT; ++i) {
-                tl[i] = 0xffffffffu;
-                ls[i] = 0u;
-                if (m[i] & (m[i] - 1u)) {
-                    const uint32_t pc = (uint32_t)__popc(m[i]);
-                    tl[i] = atomicAdd(&sh.cntTL[id[i] & (C - 1)], (1u << 16) + pc) & 0xffffu; // where its list starts
-                    rk[i] = atomicAdd(&sh.cntLong[id[i] & (C - 1)], pc > 4u ? 1u : 0x10000u); // its number among the long or the short ones
-                    tl[i] |= (pc > 4u ? rk[i] & 0xffffu : 0x8000u | (rk[i] >> 16)) << 16;
-                    ls[i] = atomicAdd(&sh.cntAll, pc);
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < EPT; ++i) {
-                if (m[i] == 0u) continue;
-                if (m[i] & (m[i] - 1u)) {
-                    sh.coff[p[i]] = (uint16_t)(tl[i] & 0xffffu);
-                    sh.soff[p[i]] = (uint16_t)(NZ + ls[i]);
-                } else sh.soff[p[i]] = (uint16_t)(tid + i * THREADS);
-            }
+            sh.lists[p] = (uint16_t)off;
         }
-        if (warp == NW - 3) { // where each coordinate's entries start in each CTA's record
-            for (int j = lane; j <= kLB; j += 32) {
-                const int s = B.roff[j], ch = s >> 5;
-                for (int c = 0; c < C; ++c)
-                    sh.rc[j][c] = (uint16_t)(sh.pre[cur][ch][c] + __popc(sh.bal[cur][ch][c] & ((1u << (s & 31)) - 1u)));
-            }
-        }
+        for (int p = tid; p < NZ / 4; p += THREADS) reinterpret_cast<int4 *>(&sh.idx[cur][0])[p] = make_int4(0, 0, 0, 0); // (from here on: the low words of the Gram matrices)
+        cp_async_wait_all(); // the next block's rows, the extents after it, the order after that
         __syncthreads();
         PRE_T(1);
         // ---- the records' places: the head has its own (one per block); the workers' records come from the pool, of which
         //      a CTA takes a piece for several blocks at a time. A block that the pool has no room for is walked in place
-        //      like one that is too long.
+        //      like one that is too long. (A warp. The others meanwhile: the next block's entries, which CTA's they are, and their
+        //      dense tile.)
         if (warp == 0) { // (a lane per CTA of the cluster)
             const bool in = lane < C;
-            const uint32_t n_c = in ? sh.rc[kLB][lane] : 0u;
-            const uint32_t len = in ? sub_bytes(n_c, sh.cntTL[lane] >> 16, sh.cntTL[lane] & 0xffffu) : 0u;
-            uint32_t incl = len;
+            const uint32_t n_c = in ? sh.rc[kLB][lane] : 0u, w = in ? sh.cnt[lane] : 0u;
+            const uint32_t lng = Count::longs(w), T_c = lng + Count::shorts(w, in ? sh.cntShort[lane] : 0u), nl_c = Count::entries(w);
+            const uint32_t len = in ? sub_bytes(n_c, T_c, nl_c) : 0u;
+            uint32_t incl = len, lists = nl_c;
 #pragma unroll
             for (int o = 1; o < kMaxC; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o), z = __shfl_up_sync(0xffffffffu, lists, o);
+                if (lane >= o) { incl += y; lists += z; }
             }
             const uint32_t need = __shfl_sync(0xffffffffu, incl, kMaxC - 1);
             // 1: longer than the arrays, or more falls to one CTA than its record holds
@@ -896,76 +958,82 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 d.offset = sl ? (unsigned long long)bid * sizeof(ChainHead) : P.pool_off + at + (incl - len);
                 d.bytes = bid == P.drop_block ? 0u : (sl ? 16u : len);
                 d.flags = sl ? 1u : 0u;
-                sh.sub_off[lane] = d.offset;
                 P.dirS[bid * C + lane] = d;
+                PreRec r;
+                r.at = d.offset;
+                r.meta = 4u * n_c;
+                r.ids = 8u * n_c;
+                r.lval = r.ids + 4u * T_c;
+                r.lst = r.lval + 4u * nl_c;
+                r.lrow = r.lst + 2u * T_c;
+                r.base = (uint16_t)(lists - nl_c);
+                r.longs = (uint16_t)lng;
+                sh.rec[lane] = r;
+                if (!sl) *reinterpret_cast<int4 *>(P.rec + d.offset) = make_int4((int)n_c, (int)T_c, (int)nl_c, cnt);
             }
             __syncwarp();
             if (lane == 0) {
                 sh.walk = sl;
                 sh.pool_at = sl ? at : at + need;
                 sh.pool_end = pool_end;
-                out.cnt = cnt;
-                out.flags = sl ? 1 : 0;
-                out.pad[0] = out.pad[1] = 0;
+                *reinterpret_cast<int4 *>(&out) = make_int4(cnt, sl ? 1 : 0, 0, 0);
             }
         }
+        const int ntotal = have_next ? N.total : 0;
+        int32_t nid[EPT];
+#pragma unroll
+        for (int i = 0; i < EPT; ++i) {
+            const int e = tid + i * THREADS;
+            nid[i] = e < ntotal ? checked_id(P, sh.idx[nxt][e]) : -1;
+        }
+#pragma unroll
+        for (int i = 0; i < EPT; ++i)
+            if (((tid + i * THREADS) & ~31) < ntotal) pre_classify(P, sh, nid[i], tid + i * THREADS, nxt, flip); // (whole warps)
         __syncthreads();
         PRE_T(2);
         const bool walk = sh.walk != 0;
         const bool carry = have_next && !walk && !N.over && P.depth >= 2 && B.k == N.k;
         if (!walk) {
             if (LOSS == CHICLE_LOSS_LOGISTIC_DUAL && P.tab_bins) write_table(P, bid, B.hdr, THREADS);
-            // ---- the workers' record heads, and the entries, row after row: place = entries of that CTA before this one; a
-            //      shared id's place in its list is the number of lower coordinates that have the id
-            if (tid < C) {
-                SubHead &h = *reinterpret_cast<SubHead *>(P.rec + sh.sub_off[tid]);
-                const int n_c = sh.rc[kLB][tid], T_c = (int)(sh.cntTL[tid] >> 16);
-                h.n = n_c;
-                h.T = T_c;
-                h.nl = (int)(sh.cntTL[tid] & 0xffffu);
-                h.cnt = cnt;
-            }
+            // ---- the workers' records: where each coordinate's entries start, and the entries, row after row: place = entries of that
+            //      CTA before this one; a shared id's place in its list is the number of lower coordinates that have the id
             for (int i = tid; i < C * (kLB + 8); i += THREADS) {
                 const int c = i / (kLB + 8), j = i - c * (kLB + 8);
-                reinterpret_cast<SubHead *>(P.rec + sh.sub_off[c])->roff[j] = sh.rc[j < kLB ? j : kLB][c];
+                reinterpret_cast<SubHead *>(P.rec + sh.rec[c].at)->roff[j] = sh.rc[j < kLB ? j : kLB][c];
             }
 #pragma unroll
             for (int i = 0; i < EPT; ++i) {
                 const int e = tid + i * THREADS;
-                const int32_t id = e < total ? checked_id(P, sh.idx[cur][e]) : 0;
-                sh.idx[cur][e] = 0; // (from here on: the low words of the Gram matrices)
-                if (e >= total) continue;
-                const int cls = id & (C - 1), j = sh.row[cur][e], p = sh.slot[e];
-                const int place = sh.pre[cur][e >> 5][cls] + __popc(sh.bal[cur][e >> 5][cls] & ((1u << lane) - 1u));
-                const uint32_t m = sh.mask[p];
-                const bool shared_id = (m & (m - 1u)) != 0u;
-                const int lower = __popc(m & ((1u << j) - 1u));
+                if ((tid & ~31) + i * THREADS >= total) break;
+                if (id[i] < 0) continue;
+                const int cls = id[i] & (C - 1), j = (int)(slot[i] >> 16);
+                const PreRec R = sh.rec[cls];
+                const uint32_t place = sh.pre[cur][e >> 5][cls] + (uint32_t)__popc(sh.bal[cur][e >> 5][cls] & ((1u << lane) - 1u));
+                const bool shared_id = (m[i] & (m[i] - 1u)) != 0u;
                 const float x = sh.val[cur][e], scaled = x * B.scl[j];
                 sh.val[cur][e] = scaled; // (the records have the value itself)
-                unsigned char *rec = P.rec + sh.sub_off[cls] + sizeof(SubHead);
-                const uint32_t n_c = sh.rc[kLB][cls], T_c = sh.cntTL[cls] >> 16, nl_c = sh.cntTL[cls] & 0xffffu;
-                const uint32_t where = (uint32_t)id < hot_total ? (uint32_t)id >> P.logC : (uint32_t)id;
+                unsigned char *rec = P.rec + R.at + sizeof(SubHead);
+                const uint32_t where = (uint32_t)id[i] < hot_total ? (uint32_t)id[i] >> P.logC : (uint32_t)id[i];
                 reinterpret_cast<float *>(rec)[place] = x;
-                reinterpret_cast<uint32_t *>(rec + 4u * n_c)[place] = where | ((uint32_t)j << kIdBits) | (shared_id ? 0x80000000u : 0u);
+                reinterpret_cast<uint32_t *>(rec + R.meta)[place] = where | ((uint32_t)j << kIdBits) | (shared_id ? 0x80000000u : 0u);
                 if (shared_id) {
-                    sh.lval[sh.soff[p] - NZ + lower] = scaled;
-                    const uint32_t at = sh.coff[p] + lower;
-                    unsigned char *lists = rec + 8u * n_c + 4u * T_c;
-                    reinterpret_cast<float *>(lists)[at] = x;
-                    (lists + 4u * nl_c + 2u * T_c)[at] = (unsigned char)j;
+                    const uint32_t start = sh.lists[slot[i] & 0xffffu] & 4095u, at = start + (uint32_t)__popc(m[i] & ((1u << j) - 1u));
+                    sh.val[2][R.base + at] = scaled;
+                    sh.row[2][R.base + at] = (uint8_t)j;
+                    reinterpret_cast<float *>(rec + R.lval)[at] = x;
+                    (rec + R.lrow)[at] = (unsigned char)j;
                     if (tl[i] != 0xffffffffu) {
-                        const uint32_t t = tl[i] >> 31 ? (sh.cntLong[cls] & 0xffffu) + ((tl[i] >> 16) & 0x7fffu) : tl[i] >> 16; // long lists first
-                        reinterpret_cast<uint32_t *>(rec + 8u * n_c)[t] = where | ((uint32_t)(__popc(m) - 1) << kIdBits);
-                        reinterpret_cast<uint16_t *>(lists + 4u * nl_c)[t] = (uint16_t)(tl[i] & 0xffffu);
+                        const uint32_t pc = (uint32_t)__popc(m[i]), t = (tl[i] >> 16) + (pc > 4u ? 0u : R.longs); // long lists first
+                        reinterpret_cast<uint32_t *>(rec + R.ids)[t] = where | ((pc - 1u) << kIdBits);
+                        reinterpret_cast<uint16_t *>(rec + R.lst)[t] = (uint16_t)start;
                     }
                 }
             }
         }
-        cp_async_wait_all(); // the next block's rows, the extents after it, the order after that
         __syncthreads();
         PRE_T(3);
-        // ---- the next block's entries: which CTA's they are, their dense tile, and (table of this block) which of this
-        //      block's coordinates have their ids; the pairs of both Gram matrices, 32 entries with some at a time
+        // ---- the next block's entries: which of this block's coordinates have their ids (table of this block); the pairs of both
+        //      Gram matrices, 32 entries with some at a time
         if (warp == NW - 1 && bid + 2 < end) pre_make_block<LOSS, NZ, HT>(P, sh, bid + 2);
         {
             uint32_t *todo = sh.work[warp];
@@ -974,48 +1042,36 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 const uint32_t b = __ballot_sync(0xffffffffu, on);
                 if (on) todo[have + __popc(b & ((1u << lane) - 1u))] = item;
                 have += __popc(b);
-                __syncwarp();
-                if (have >= 32) {
-                    have -= 32;
-                    const uint32_t mine = todo[have + lane];
-                    __syncwarp();
-                    pre_pairs<NZ>(sh, mine, true, cur, N);
-                }
             };
-            const int ntotal = have_next ? N.total : 0;
-            int32_t id[EPT], seen[EPT];
-            uint32_t p[EPT];
 #pragma unroll
             for (int i = 0; i < EPT; ++i) {
-                const int e = tid + i * THREADS;
-                id[i] = e < ntotal ? checked_id(P, sh.idx[nxt][e]) : -1;
-                p[i] = id[i] >= kHD ? home_slot<HT>(id[i]) : 0u;
-            }
-#pragma unroll
-            for (int i = 0; i < EPT; ++i) seen[i] = carry ? sh.key[p[i]] : -1;
-            if (!walk) {
-#pragma unroll 1
-                for (int e = tid; (e & ~31) < total; e += THREADS) {
-                    const uint32_t s = e < total ? sh.slot[e] : 0u;
-                    push(s >= (uint32_t)kHD && (sh.mask[s] & ((1u << sh.row[cur][e]) - 1u)) != 0u, (uint32_t)e | s << 12);
+                const uint32_t e = (uint32_t)(tid + i * THREADS);
+                if ((e & ~31u) < (uint32_t)total && !walk)
+                    push(id[i] >= kHD && (m[i] & ((1u << (slot[i] >> 16)) - 1u)) != 0u, e | (slot[i] & 0xffffu) << 12);
+                if ((e & ~31u) < (uint32_t)ntotal && carry) {
+                    uint32_t p = (uint32_t)nid[i];
+                    bool hit = nid[i] >= kHD;
+                    if (nid[i] >= kDir) {
+                        p = home_place<HT>(nid[i]);
+                        int32_t seen = sh.key[p];
+                        for (int t = 1; seen != nid[i] && seen != -1 && t <= HT; ++t) {
+                            p = next_place<HT>(p, t);
+                            seen = sh.key[p];
+                        }
+                        hit = seen == nid[i];
+                        p += kDir;
+                    } else if (hit) hit = sh.mask[p] != 0u;
+                    __syncwarp();
+                    push(hit, e | p << 12 | 1u << 25);
+                }
+                if (i + 1 < EPT && have > 32) { // (the list holds 96)
+                    __syncwarp();
+                    pre_listed_early<NZ>(sh, have, cur, N);
+                    have = 0;
                 }
             }
-#pragma unroll
-            for (int i = 0; i < EPT; ++i) {
-                const int e = tid + i * THREADS;
-                if ((e & ~31) >= ntotal) break; // (whole warps)
-                pre_classify(P, sh, id[i], e, nxt);
-                if (!carry) continue;
-                if (id[i] >= kHD)
-                    for (int t = 0; t < HT && seen[i] != id[i] && seen[i] != -1; ++t) {
-                        p[i] = next_slot<HT>(p[i]);
-                        seen[i] = sh.key[p[i]];
-                    }
-                push(id[i] >= kHD && seen[i] == id[i], (uint32_t)e | p[i] << 12 | 1u << 24);
-            }
-            const uint32_t mine = lane < have ? todo[lane] : 0u;
             __syncwarp();
-            if (have) pre_pairs<NZ>(sh, mine, lane < have, cur, N);
+            pre_listed<NZ>(sh, have, cur, N);
         }
         __syncthreads();
         PRE_T(4);
@@ -1023,9 +1079,9 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         if (have_next && warp < C) pre_prefix(sh, N.total, nxt, warp);
         {
             constexpr int R = kLB / NW;
-            float g[R], x[R];
+            float2 g2[R], x2[R]; // (the even and the odd columns)
 #pragma unroll
-            for (int r = 0; r < R; ++r) g[r] = x[r] = 0.0f;
+            for (int r = 0; r < R; ++r) g2[r] = x2[r] = make_float2(0.0f, 0.0f);
             const float4 *dj = reinterpret_cast<const float4 *>(&sh.D[cur][lane][0]), *nj = reinterpret_cast<const float4 *>(&sh.D[nxt][lane][0]);
 #pragma unroll
             for (int h = 0; h < kHD / 4; ++h) {
@@ -1033,8 +1089,10 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     const float4 c = *reinterpret_cast<const float4 *>(&sh.D[cur][warp + r * NW][4 * h]);
-                    g[r] = fmaf(a.x, c.x, g[r]); g[r] = fmaf(a.y, c.y, g[r]); g[r] = fmaf(a.z, c.z, g[r]); g[r] = fmaf(a.w, c.w, g[r]);
-                    x[r] = fmaf(b.x, c.x, x[r]); x[r] = fmaf(b.y, c.y, x[r]); x[r] = fmaf(b.z, c.z, x[r]); x[r] = fmaf(b.w, c.w, x[r]);
+                    fma2(g2[r], a.x, a.y, c.x, c.y);
+                    fma2(x2[r], b.x, b.y, c.x, c.y);
+                    fma2(g2[r], a.z, a.w, c.z, c.w);
+                    fma2(x2[r], b.z, b.w, c.z, c.w);
                 }
             }
             float qg = 0.0f, qx = 0.0f;
@@ -1045,11 +1103,12 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
             for (int r = 0; r < R; ++r) {
                 const int l = warp + r * NW;
                 const float il = B.inv[l], yl = B.ys[l], al = B.as[l];
-                float v = fmaf(fmaf((float)low[l * kLB + lane], 1.0f / 1048576.0f, (float)sh.G[0][l][lane]) * il, inv, g[r]) * (gsc * yl);
+                const int at = gram_place(l, lane);
+                float v = fmaf(fmaf((float)low[at], 1.0f / 1048576.0f, (float)(&sh.G[0][0][0])[at]) * il, inv, g2[r].x + g2[r].y) * (gsc * yl);
                 v = lane > l && !walk ? v : 0.0f;
                 out.G[l * kLB + lane] = v;
                 qg = fmaf(v, al, qg);
-                v = fmaf(fmaf((float)low[kLB * kLB + l * kLB + lane], 1.0f / 1048576.0f, (float)sh.G[1][l][lane]) * il, ninv, x[r]) * (ngsc * yl);
+                v = fmaf(fmaf((float)low[kLB * kLB + at], 1.0f / 1048576.0f, (float)(&sh.G[1][0][0])[at]) * il, ninv, x2[r].x + x2[r].y) * (ngsc * yl);
                 v = l < cnt && carry ? v : 0.0f;
                 out.X[l * kLB + lane] = v;
                 qx = fmaf(v, al, qx);
@@ -1057,12 +1116,9 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
             sh.work[warp][lane] = __float_as_uint(qg);
             sh.work[warp][32 + lane] = __float_as_uint(qx);
         }
-        for (int p = tid; p < HT / 4; p += THREADS) {
-            reinterpret_cast<int4 *>(sh.key)[p] = make_int4(-1, -1, -1, -1);
-            reinterpret_cast<uint4 *>(sh.mask)[p] = make_uint4(0u, 0u, 0u, 0u);
-        }
-        if (tid < kMaxC) sh.cntTL[tid] = sh.cntLong[tid] = 0u;
-        if (tid == 0) sh.cntAll = 0u;
+        for (int p = tid; p < HT / 4; p += THREADS) reinterpret_cast<int4 *>(sh.key)[p] = make_int4(-1, -1, -1, -1);
+        for (int p = tid; p < Shared::TS / 4; p += THREADS) reinterpret_cast<uint4 *>(sh.mask)[p] = make_uint4(0u, 0u, 0u, 0u);
+        if (tid < kMaxC) sh.cnt[tid] = sh.cntShort[tid] = 0u;
         __syncthreads();
         PRE_T(5);
     }
@@ -1378,7 +1434,7 @@ template <int LOSS, bool LONG> __device__ __forceinline__ void prepare_block_den
 // (blocks blockIdx.x, blockIdx.x + gridDim.x, ..)
 template <int LOSS, bool LONG> __global__ void __launch_bounds__(kPreThreads, LONG ? kPreDenseLongPerSm : kPreDensePerSm) k_lookahead_prepare_dense(const LookParams P)
 {
-    extern __shared__ __align__(16) unsigned char smem_pre[];
+    extern __shared__ __align__(128) unsigned char smem_pre[];
     PreDenseShared &sh = *reinterpret_cast<PreDenseShared *>(smem_pre);
     for (int64_t bid = blockIdx.x; bid < P.n_blocks; bid += gridDim.x) {
         prepare_block_dense<LOSS, LONG>(P, bid, sh);
