@@ -342,6 +342,7 @@ chicle_status_t chicle_glm_create(const chicle_matrix_t *X, const float *labels,
             h->blk_shared_ids[i] = (double)host_mass2[4 + kRankClasses + i] / 1048576.0;
             h->blk_shared[i] = (double)host_mass2[4 + 2 * kRankClasses + i] / 1048576.0;
         }
+        for (int i = 0; i < kOctaves; ++i) h->blk_octave[i] = 32.0 * (double)host_mass2[4 + 3 * kRankClasses + i] / n;
         const char *force = getenv("CHICLE_FORCE_VARIANT"); // debugging aid
         h->flat_ids = force && strcmp(force, "flat") == 0;
         if (force && strcmp(force, "flat") == 0) h->hot_variant = 0;

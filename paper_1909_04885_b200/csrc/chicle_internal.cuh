@@ -75,7 +75,8 @@ struct SolverParams;
 
 // What the ranking of the ids finds out about the data (see launch_frequency_remap).
 constexpr int kRankClasses = 8; // ids mod 8: a CTA of the largest cluster takes one class
-constexpr int kMassWords = 4 + 3 * kRankClasses;
+constexpr int kOctaves = 32;     // of ids
+constexpr int kMassWords = 4 + 3 * kRankClasses + kOctaves;
 
 // ---- handle -------------------------------------------------------------------------------------------------
 struct Glm {
@@ -112,6 +113,7 @@ struct Glm {
     // what a block of 32 random coordinates is expected to have on the ids of each class (id mod kRankClasses): entries, ids
     // that several of the 32 have, entries with such an id; and the variance of a coordinate's number of entries
     double blk_entries[kRankClasses] = {}, blk_shared_ids[kRankClasses] = {}, blk_shared[kRankClasses] = {};
+    double blk_octave[kOctaves] = {}; // and entries with ids from 2^k to 2^(k+1) - 1
     double row_variance = 0.0;
 
     // partition
@@ -145,6 +147,7 @@ struct Glm {
     uint32_t la_sub_room = 0;        // bytes of a worker record's slot in shared memory
     int la_slots = 4;                // and how many slots
     int32_t la_hotc = 0;             // entry ids per CTA kept in shared memory
+    int32_t la_far_cap = 0;          // entries of a record that the far warp's lists hold (0: no far warp)
     int32_t la_tab_bins = 0;         // logistic: bins per coordinate of the step's tables (0: none)
     size_t la_tab_off = 0;           // where they lie in a region
     size_t la_smem = 0;              // dynamic shared memory of the chain kernel

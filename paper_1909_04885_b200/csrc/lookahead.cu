@@ -60,7 +60,6 @@ constexpr int kDenseEasy = 128;    // and what it takes where the cluster may be
 // or the id itself (never below hotc, see k_lookahead_chain). Problems with more ids take the blocked solver.
 constexpr int kIdBits = 26;
 constexpr uint32_t kIdMask = (1u << kIdBits) - 1u;
-constexpr int kChainThreads = 384;
 constexpr int kSubSlots = 4;       // worker records in shared memory: blocks b .. b + 3 (three of them where long records leave no room, see lookahead_plan)
 // Recurrence records in shared memory: a record is fetched when the block that many before it is done, and takes 1 500 cycles
 // or more from memory, so two would set the pace (1 M sparse rows: 3 019 cycles a block, with three 2 600). With tables of the logistic step
@@ -75,6 +74,7 @@ constexpr int kBarWork = 1;        // named barrier of the worker warps
 constexpr int kRecordWarp = 8;     // fetches the workers' records
 constexpr int kStartWarp = 4;      // in CTA 0: the states that a block's recurrence starts from
 constexpr int kFeedWarp = 11;      // in CTA 0: what follows from a block's recurrence; fetches the recurrence records
+constexpr int kFarWarp = 13;       // (kSplit) ids beyond the model's part in shared memory; warp 12 would share warp 0's scheduler and has no role
 
 // Per-step constants for the recurrence warp (see coordinate_step for p0 .. p3).
 struct alignas(16) CHdr {
@@ -128,7 +128,9 @@ struct alignas(16) BlkDir { // where a record is
 
 // Kinds of data the chain kernel is instantiated for: sparse with the whole model in shared memory, with its most frequent
 // ids there, with none; dense rows.
-constexpr int kHot = 0, kCold = 1, kFlat = 2, kDense = 3;
+// kSplit: as kCold, with a warp of its own for the ids that are not in shared memory; kCold where there is no room for its lists.
+constexpr int kHot = 0, kCold = 1, kFlat = 2, kDense = 3, kSplit = 4;
+__host__ __device__ constexpr int chain_threads(int kind) { return kind == kSplit ? 448 : 384; }
 
 struct LookParams {
     SolverParams S;
@@ -146,6 +148,7 @@ struct LookParams {
     uint32_t sub_room;           // bytes of a worker record's slot in shared memory (sparse; a block that needs more is walked in place)
     int32_t slots;               // and how many slots there are (at least depth + 2)
     int32_t hotc;                // entry ids per CTA kept in shared memory
+    int32_t far_cap;             // entries of a worker record that the lists of kSplit have room for (a block with more is walked in place)
     int64_t n_blocks;
     int64_t drop_block;          // test aid: this block's records are left unpublished (-1: none)
     int64_t nnz;                 // entries of the matrix (what a coordinate's extent is checked against in a debug build)
@@ -280,6 +283,23 @@ __device__ __forceinline__ void fma2(float2 &acc, float ax, float ay, float bx, 
 {
     asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%0, %1};\n\tfma.rn.f32x2 c, a, b, c;\n\tmov.b64 {%0, %1}, c;\n\t}"
         : "+f"(acc.x), "+f"(acc.y) : "f"(ax), "f"(ay), "f"(bx), "f"(by));
+}
+__device__ __forceinline__ void prefetch_if(const float *p, bool on)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %1, 0;\n\t@q prefetch.global.L2 [%0];\n\t}" ::"l"(p), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void sts_u16_if(uint32_t a, uint32_t v, bool on)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.shared.u16 [%0], %1;\n\t}" ::"r"(a), "h"((uint16_t)v), "r"((uint32_t)on) : "memory");
+}
+// (the value stays where `on` does not hold)
+__device__ __forceinline__ void ldcg_again_if(float &v, const float *p, bool on)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q ld.global.cg.f32 %0, [%1];\n\t}" : "+f"(v) : "l"(p), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void red_shared_or_if(uint32_t a, uint32_t v, bool on)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q red.shared.or.b32 [%0], %1;\n\t}" ::"r"(a), "r"(v), "r"((uint32_t)on) : "memory");
 }
 __device__ __forceinline__ void red_add_if(float *p, float v, bool on)
 {
@@ -943,7 +963,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
             }
             const uint32_t need = __shfl_sync(0xffffffffu, incl, kMaxC - 1);
             // 1: longer than the arrays, or more falls to one CTA than its record holds
-            int sl = B.over || __any_sync(0xffffffffu, len > P.sub_room) ? 1 : 0;
+            int sl = B.over || __any_sync(0xffffffffu, len > P.sub_room || n_c > (uint32_t)P.far_cap) ? 1 : 0;
             unsigned long long at = sh.pool_at, pool_end = sh.pool_end;
             if (!sl && at + need > pool_end) {
                 const unsigned long long take = need > P.pool_piece ? need : P.pool_piece;
@@ -1581,6 +1601,9 @@ __device__ __noinline__ void mbar_drain(uint32_t bar, uint32_t parity)
 // The worker warps' barrier: 35 cycles when all are there (with a vote 78, by arrivals on an mbarrier 181).
 __device__ __forceinline__ void work_bar() { asm volatile("bar.sync %0, %1;" ::"n"(kBarWork), "n"(kWorkThreads) : "memory"); }
 
+// (kSplit) the worker warps and the far warp, once, behind their last block
+__device__ __forceinline__ void far_bar() { asm volatile("bar.sync %0, %1;" ::"n"(kBarWork + 1), "n"(kWorkThreads + 32) : "memory"); }
+
 struct alignas(16) ChainCtl {
     uint64_t subfull[kSubSlots];   // count the bytes of the bulk copies into the workers' record slots
     uint64_t headfull[kMaxHeadSlots]; // the same for the recurrence warp's records (CTA 0)
@@ -1592,6 +1615,7 @@ struct alignas(16) ChainCtl {
     alignas(16) float dbuf[2][kLB];
     uint64_t ready[2];             // CTA 0: the states that a block's recurrence starts from are in `start`
     uint64_t out[2];               // CTA 0: the recurrence's results are in `res`
+    uint64_t farfull[kSubSlots];   // kSplit: the slot's list of entries beyond shared memory is there
     alignas(16) float start[2][3][kLB]; // states; the scalar map's constants (p2 and lq; with tables tab_q and tab_offset)
     alignas(16) float res[2][kLB];
     float sink[32]; // where a lane's stores go that have no target
@@ -1603,9 +1627,19 @@ struct alignas(16) ChainCtl {
 // Shared-memory layout of the chain kernel (sizes fixed at launch): control, recurrence records, logistic tables,
 // worker records, the CTA's part of the model.
 struct ChainLayout {
-    uint32_t heads, tabs, subs, sub_stride, w, total;
+    uint32_t heads, tabs, subs, sub_stride, filter, far, w, total;
 };
-__host__ __device__ inline ChainLayout chain_layout(uint32_t sub_room, int slots, int hotc, bool dense, int tab_bins)
+// kSplit: partial sums of all CTAs (used in CTA 0), products of a block's entries, and per slot a list of the entries: where each
+// coordinate's start (kLB + 1 of them, and padding), and their numbers in the record.
+constexpr uint32_t kFarSums = 2u * kMaxC * kLB * 4u, kFarHead = 80u;
+__host__ __device__ constexpr uint32_t far_list_bytes(int cap) { return kFarHead + 2u * (uint32_t)cap; }
+__host__ __device__ constexpr uint32_t far_bytes(int kind, int cap, int slots) { return kind == kSplit ? kFarSums + 4u * (uint32_t)cap + (uint32_t)slots * far_list_bytes(cap) : 0u; }
+// Ids beyond the model's part in shared memory (some: kCold, all: kFlat): their model entries are gathered from L2 before the
+// block's deltas have come, and those that the block's update then changes once more. Which may have changed is kept in a bit
+// per hashed id, one set of them for even and one for odd blocks: this many bytes a set (a bit that two ids share costs a
+// second gather, nothing else).
+__host__ __device__ constexpr uint32_t filter_bytes(int kind) { return kind == kCold ? 4096u : (kind == kFlat ? 16384u : 0u); }
+__host__ __device__ inline ChainLayout chain_layout(uint32_t sub_room, int slots, int hotc, bool dense, int tab_bins, int kind, int far_cap = 0)
 {
     ChainLayout L;
     L.heads = (uint32_t)((sizeof(ChainCtl) + 127) & ~(size_t)127);
@@ -1613,22 +1647,26 @@ __host__ __device__ inline ChainLayout chain_layout(uint32_t sub_room, int slots
     L.tabs = L.heads + hs * (uint32_t)sizeof(ChainHead);
     L.subs = L.tabs + hs * tab_bytes(tab_bins);
     L.sub_stride = dense ? sub_bytes_dense(kLB, hotc) : sub_room;
-    L.w = L.subs + (uint32_t)slots * L.sub_stride;
+    L.filter = L.subs + (uint32_t)slots * L.sub_stride;
+    L.far = L.filter + 2u * filter_bytes(kind);
+    L.w = L.far + far_bytes(kind, far_cap, slots);
     L.total = L.w + 4u * (uint32_t)(hotc > 0 ? hotc : 4);
     return L;
 }
 
 template <int LOSS, int KIND, bool TAB>
-__global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const LookParams P)
+__global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(const LookParams P)
 {
-    constexpr bool DENSE = KIND == kDense;
+    constexpr bool DENSE = KIND == kDense, SPLIT = KIND == kSplit;
+    constexpr int kChainThreads = chain_threads(KIND);
+    constexpr uint32_t kRows = SPLIT ? 2u : 1u; // rows of partial sums from each CTA
     extern __shared__ __align__(128) unsigned char smem_chain[];
     const SolverParams &S = P.S;
     const int logC = P.logC, C = 1 << logC;
     const uint32_t crank = cluster_ctarank();
     const int k = (int)(blockIdx.x >> logC);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const ChainLayout L = chain_layout(P.sub_room, P.slots, P.hotc, DENSE, TAB ? P.tab_bins : 0);
+    const ChainLayout L = chain_layout(P.sub_room, P.slots, P.hotc, DENSE, TAB ? P.tab_bins : 0, KIND, P.far_cap);
     ChainCtl &ctl = *reinterpret_cast<ChainCtl *>(smem_chain);
     float *W = reinterpret_cast<float *>(smem_chain + L.w);
     volatile int *abort_flag = &ctl.abort_flag;
@@ -1653,7 +1691,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         ctl.done = 0;
         for (int i = 0; i < kSubSlots; ++i) {
             mbar_init(smem_u32(&ctl.subfull[i]), 1);
-            mbar_init(smem_u32(&ctl.subfree[i]), 1);
+            mbar_init(smem_u32(&ctl.subfree[i]), kRows); // (the worker warps, and the far warp)
+            mbar_init(smem_u32(&ctl.farfull[i]), 1);
         }
         for (int i = 0; i < kMaxHeadSlots; ++i) mbar_init(smem_u32(&ctl.headfull[i]), 1);
         for (int i = 0; i < 2; ++i) {
@@ -1662,11 +1701,11 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             mbar_init(smem_u32(&ctl.ready[i]), 1);
             mbar_init(smem_u32(&ctl.out[i]), 1);
         }
-        mbar_init(smem_u32(&ctl.ackbar), (uint32_t)(C * kWorkWarps));
+        mbar_init(smem_u32(&ctl.ackbar), (uint32_t)(C * (kWorkWarps + (SPLIT ? 1 : 0))));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // armed for the first two blocks before anybody can send
         for (int i = 0; i < 2; ++i) {
-            mbar_arrive_expect_tx(smem_u32(&ctl.pbar[i]), (uint32_t)(C * kLB * 4));
+            mbar_arrive_expect_tx(smem_u32(&ctl.pbar[i]), kRows * (uint32_t)(C * kLB * 4));
             mbar_arrive_expect_tx(smem_u32(&ctl.dbar[i]), d_bytes);
         }
     }
@@ -1685,6 +1724,9 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         for (int i = 0; i < 8; ++i)
             if (l0 + i * kChainThreads < hot_mine) W[l0 + i * kChainThreads] = P.model_in ? fmaf(sigma, u[i], v[i]) : u[i];
     }
+    constexpr bool FAR = KIND == kCold || KIND == kFlat;
+    if constexpr (FAR)
+        for (uint32_t i = (uint32_t)tid; i < 2u * filter_bytes(KIND) / 4u; i += kChainThreads) reinterpret_cast<uint32_t *>(smem_chain + L.filter)[i] = 0u;
     if (DENSE && tid < 4 && hot_mine + tid < P.hotc) W[hot_mine + tid] = 0.0f; // (the padding of the last slice)
     // the ids beyond the part in shared memory that fall to this CTA (id mod C): the model in place
     const size_t cold0 = (size_t)hot_total + (((size_t)crank - (size_t)hot_total) & (size_t)(C - 1));
@@ -1710,7 +1752,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
 
     constexpr int HS = head_slots(TAB);
     const bool is_chain = crank == 0 && warp == 0;
-    const bool is_worker = (warp & 3) != 0 && warp != kFeedWarp; // warps 1 2 3 5 6 7 9 10
+    const bool is_worker = (warp & 3) != 0 && warp < kFeedWarp; // warps 1 2 3 5 6 7 9 10
     bool aborted = false;
 
     if (is_chain && nb > 0) {
@@ -1892,6 +1934,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 if (!mbar_wait_cluster(smem_u32(&ctl.pbar[fp & 1]), (uint32_t)(fp >> 1) & 1u, abort_flag, S.status)) break;
                 float m0 = 0.0f;
                 for (int c = 0; c < C; ++c) m0 += ctl.pbuf[fp & 1][c][lane]; // the CTAs' partial sums in a fixed order
+                if (SPLIT)
+                    for (int c = 0; c < C; ++c) m0 += reinterpret_cast<const float *>(smem_chain + L.far)[((fp & 1) * kMaxC + c) * kLB + lane];
                 ++fp;
                 const float s0 = fmaf(h.B, m0, h.A);
                 ctl.start[par][0][lane] = s0;
@@ -1956,7 +2000,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 if (!in || !fine) dl = 0.0f;
                 coord = in ? h.coord : -1;
                 // armed for block fp + 2 before the deltas go out (its dot products are sent only after they arrive)
-                mbar_arrive_expect_tx_if(smem_u32(&ctl.pbar[fp & 1]), (uint32_t)(C * kLB * 4), lane == 0);
+                mbar_arrive_expect_tx_if(smem_u32(&ctl.pbar[fp & 1]), kRows * (uint32_t)(C * kLB * 4), lane == 0);
                 ++fp;
             } else fence_cluster(); // (the walk's ordinary stores go before the signal)
             float d4[4];
@@ -1990,10 +2034,50 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
         load_dir(0, d);
         int slot = 0, before = 0;     // of this block and of the one before
         int fetched = 0;
+        // The slot's block has arrived: its entries beyond the part of the model in shared memory are brought into L2 (the records
+        // that stream through it push them out) and, for the far warp, listed row after row.
+        auto list_far = [&](int at) {
+            const uint32_t rec = smem_u32(smem_chain + L.subs) + (uint32_t)at * L.sub_stride;
+            int n = ctl.walk[at] ? 0 : lds_s32(rec);
+            if (SPLIT && n > P.far_cap) n = P.far_cap; // (the prepare kernel sees to it)
+            const uint32_t meta = rec + (uint32_t)sizeof(SubHead) + 4u * (uint32_t)n;
+            const uint32_t list = smem_u32(smem_chain + L.far) + kFarSums + 4u * (uint32_t)P.far_cap + (uint32_t)at * far_list_bytes(P.far_cap);
+            const int mine = SPLIT && n > 0 ? (int)lds_u16(rec + (uint32_t)offsetof(SubHead, roff) + 2u * (uint32_t)lane) : 0;
+            int count = 0, start = 0;
+            const uint32_t hotc = (uint32_t)P.hotc, dim = (uint32_t)(S.dim <= (int64_t)kIdMask ? S.dim : (int64_t)kIdMask + 1), below = (1u << lane) - 1u;
+            uint32_t v[4];
+            for (int e0 = 0; e0 < n; e0 += 128) { // (four loads under way together: one after the other a list of 312 took 3 000 cycles)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = lds_u32_if(meta + 4u * (uint32_t)(e0 + 32 * u + lane), e0 + 32 * u + lane < n) & kIdMask; // (0: none)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool far = v[u] >= hotc && v[u] < dim && e0 + 32 * u + lane < n;
+                    prefetch_if(Uk + (far ? v[u] : 0u), far);
+                    if (!SPLIT) continue;
+                    const uint32_t all = __ballot_sync(0xffffffffu, far);
+                    const int first = mine - (e0 + 32 * u); // this lane's coordinate's first entry, from here on
+                    sts_u16_if(list + kFarHead + 2u * (uint32_t)(count + __popc(all & below)), (uint32_t)(e0 + 32 * u + lane), far);
+                    if (first >= 0) start = count + __popc(first < 32 ? all & ((1u << first) - 1u) : all);
+                    count += __popc(all);
+                }
+            }
+            if (SPLIT) {
+                asm volatile("st.shared.u16 [%0], %1;" ::"r"(list + 2u * (uint32_t)lane), "h"((uint16_t)start) : "memory");
+                if (lane == 0) asm volatile("st.shared.u16 [%0], %1;" ::"r"(list + 2u * (uint32_t)kLB), "h"((uint16_t)count) : "memory");
+                __syncwarp();
+                mbar_arrive_if(smem_u32(&ctl.farfull[at]), lane == 0);
+            }
+            __syncwarp();
+        };
         uint32_t turn = 0, tbefore = 0; // parity of how often the slots have been filled
 #pragma unroll 1
         for (int blk = 0; blk < nb; ++blk) {
             if (__any_sync(0xffffffffu, *abort_flag != 0)) break; // (no slot is refilled for workers that no longer wait for it)
+            // (the block before this one arrives while its predecessor's slot is still in use)
+            if ((KIND == kCold || KIND == kFlat || SPLIT) && blk > 0) {
+                if (!mbar_wait_cluster(smem_u32(&ctl.subfull[before]), tbefore, abort_flag, S.status)) break;
+                list_far(before);
+            }
             if (blk >= slots && !mbar_wait_cluster(smem_u32(&ctl.subfree[slot]), turn ^ 1u, abort_flag, S.status)) break;
             const unsigned long long offset = ((unsigned long long)d[1] << 32) | d[0];
             uint32_t bytes = d[2] <= L.sub_stride ? d[2] : 0u;
@@ -2013,20 +2097,6 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             bulk_g2s_if(smem_u32(smem_chain + L.subs) + (uint32_t)slot * L.sub_stride, P.rec + offset, bytes, bar, lane == 0);
             fetched = blk + 1;
             load_dir(blk + 1, d);
-            // The block before this one has arrived by now, and its dot products are a block's time away: the model entries
-            // beyond the part in shared memory that they will gather are brought into L2 (the records that stream through it
-            // push them out: with an entry or two per thread, what a block's gathers cost is one round trip to memory).
-            if ((KIND == kCold || KIND == kFlat) && blk > 0) {
-                if (!mbar_wait_cluster(smem_u32(&ctl.subfull[before]), tbefore, abort_flag, S.status)) break;
-                const uint32_t rec = smem_u32(smem_chain + L.subs) + (uint32_t)before * L.sub_stride;
-                const int n = ctl.walk[before] ? 0 : lds_s32(rec);
-                const uint32_t meta = rec + (uint32_t)sizeof(SubHead) + 4u * (uint32_t)n;
-                for (int e = lane; e < n; e += 32) {
-                    const uint32_t v = lds_u32_if(meta + 4u * (uint32_t)e, true) & kIdMask;
-                    if (v >= (uint32_t)P.hotc && (int64_t)v < S.dim) asm volatile("prefetch.global.L2 [%0];" ::"l"(Uk + v));
-                }
-                __syncwarp();
-            }
             before = slot;
             tbefore = turn;
             if (++slot == slots) {
@@ -2034,7 +2104,168 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 turn ^= 1u;
             }
         }
+        if (SPLIT && fetched == nb && mbar_wait_cluster(smem_u32(&ctl.subfull[before]), tbefore, abort_flag, S.status)) list_far(before);
         for (int i = fetched > slots ? fetched - slots : 0; i < fetched; ++i) mbar_drain(smem_u32(&ctl.subfull[i % slots]), (uint32_t)(i / slots) & 1u);
+    }
+    if (SPLIT && warp == kFarWarp) {
+        // ============================== the far warp ==============================================================
+        // What the worker warps do for the ids in shared memory, for the others, whose model entries lie in row k of the update
+        // workspace: a block's update by reductions at L2, then the gathers for the dot products that follow, in this warp's own
+        // order, beside the workers. A round trip to L2 and the reductions stood in the workers' way otherwise, block after block
+        // (45 M hashed rows, K = 16: 3 400 -> 3 060 cycles a block, step 155 -> 145 ms; with the workers' gathers in front of the
+        // deltas, as the other kinds have them, 163).
+        const uint32_t sums = smem_u32(smem_chain + L.far), prod = sums + kFarSums, lists0 = prod + 4u * (uint32_t)P.far_cap, lstride = far_list_bytes(P.far_cap);
+        const uint32_t subs0 = smem_u32(smem_chain + L.subs);
+        const uint32_t p_buf0 = mapa_u32(sums + crank * (uint32_t)(kLB * 4), 0u), p_bar0 = mapa_u32(smem_u32(&ctl.pbar[0]), 0u), ack_bar = mapa_u32(smem_u32(&ctl.ackbar), 0u);
+        const uint32_t hotc = (uint32_t)P.hotc;
+        const int depth = P.depth, slots = P.slots;
+        int fg = 0, s_upd = 0, s_dot = 0;
+        uint32_t dot_turn = 0;
+        bool ok = true, sl0 = false, sl1 = false;
+        auto in_dim = [&](uint32_t v) { return CHICLE_IN_BOUNDS(S.status, v >= hotc && (int64_t)v < S.dim); };
+        // What bounds this warp is its instructions (code that runs once a block comes from beyond the instruction caches: about four
+        // cycles each) and one round trip to L2. The first 64 entries of a block's list stay in registers from its dot products to its
+        // update; longer lists' others are looked up each time.
+        struct Entries {
+            int n;
+            float x[2];
+            uint32_t m[2]; // (0: no entry)
+        };
+        auto entry = [&](int s, int e, bool in, float &x, uint32_t &m) {
+            const uint32_t rec = subs0 + (uint32_t)s * L.sub_stride, val = rec + (uint32_t)sizeof(SubHead);
+            const uint32_t i = 4u * lds_u16_if(lists0 + (uint32_t)s * lstride + kFarHead + 2u * (uint32_t)e, in);
+            x = lds_f32_if(val + i, in);
+            m = lds_u32_if(val + 4u * (uint32_t)lds_s32(rec) + i, in);
+        };
+        auto load = [&](int s, Entries &E) {
+            E.n = (int)lds_u16(lists0 + (uint32_t)s * lstride + 2u * (uint32_t)kLB);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) entry(s, lane + 32 * u, lane + 32 * u < E.n, E.x[u], E.m[u]);
+        };
+        auto gather = [&](uint32_t m) {
+            const bool far = m != 0u && in_dim(m & kIdMask);
+            return ldcg_if(Uk + (far ? m & kIdMask : 0u), far);
+        };
+        auto send = [&](int s, const Entries &E, float w0, float w1) {
+            if (lane < E.n) sts_f32(prod + 4u * (uint32_t)lane, E.x[0] * w0);
+            if (lane + 32 < E.n) sts_f32(prod + 4u * (uint32_t)(lane + 32), E.x[1] * w1);
+#pragma unroll 1
+            for (int e = lane + 64; e < E.n; e += 32) {
+                float x;
+                uint32_t m;
+                entry(s, e, true, x, m);
+                sts_f32(prod + 4u * (uint32_t)e, x * gather(m));
+            }
+            __syncwarp();
+            float acc = 0.0f; // (a lane per coordinate)
+            const uint32_t at = lists0 + (uint32_t)s * lstride + 2u * (uint32_t)lane;
+            const int end = (int)lds_u16(at + 2u);
+#pragma unroll 1
+            for (int e = (int)lds_u16(at); e < end; ++e) acc += lds_f32(prod + 4u * (uint32_t)e);
+            __syncwarp();
+            const uint32_t slot = (uint32_t)(fg & 1);
+            ++fg;
+            st_async_f32_if(p_buf0 + (slot * (uint32_t)(kMaxC * kLB) + (uint32_t)lane) * 4u, acc, p_bar0 + slot * 8u, true);
+        };
+        Entries E0 = {0, {0.f, 0.f}, {0u, 0u}}, E1 = E0, E2 = E0; // of blocks b, b + 1, b + depth
+        // a list of block b: its id, length (0: none, or one of the worker warps'), where its values and coordinates are, the first four
+        uint32_t id = 0u, a_val = 0u, a_row = 0u, rl[4];
+        float xl[4];
+        int T = 0, len = 0; // (T: how many lists the block has)
+        auto list_of = [&](int s, int t) {
+            const uint32_t rec = subs0 + (uint32_t)s * L.sub_stride;
+            const int4 head = lds_s32x4(rec); // n, T, nl, cnt
+            const uint32_t ids = rec + (uint32_t)sizeof(SubHead) + 8u * (uint32_t)head.x, lval = ids + 4u * (uint32_t)head.y, lst = lval + 4u * (uint32_t)head.z;
+            T = head.y;
+            const uint32_t word = lds_u32_if(ids + 4u * (uint32_t)t, t < T), first = lds_u16_if(lst + 2u * (uint32_t)t, t < T);
+            id = word & kIdMask;
+            len = t < T && id >= hotc && in_dim(id) ? (int)((word >> kIdBits) & 31u) + 1 : 0;
+            if (!CHICLE_IN_BOUNDS(S.status, len == 0 || (int)first + len <= head.z)) len = 0;
+            a_val = lval + 4u * first;
+            a_row = lst + 2u * (uint32_t)head.y + first;
+        };
+#pragma unroll 1
+        for (int b = nb > 0 ? -depth : 0; b < nb; ++b) {
+            bool sl2 = false, due = b + depth < nb, late = false;
+            if (due) {
+                ok = ok && mbar_wait_cluster(smem_u32(&ctl.farfull[s_dot]), dot_turn, abort_flag, S.status);
+                sl2 = lds_s32(smem_u32(&ctl.walk[0]) + 4u * s_dot) != 0;
+                due = !sl2;
+            }
+            if (sl0 || sl1) {
+                late = depth == 2 && sl0 && !sl1 && b + 1 < nb;
+                due = due && (depth == 1 || !sl1);
+            }
+            due = due && ok;
+            if (b + depth < nb && ok) load(s_dot, E2); // (nothing where the block is walked in place)
+            if (b >= 0) {
+                const uint32_t par = (uint32_t)(b & 1), dl = smem_u32(&ctl.dbuf[0][0]) + par * (uint32_t)(kLB * 4);
+                if (sl0) { // (as the worker warps)
+                    __syncwarp();
+                    if (lane == 0 && ok) mbar_arrive_remote_release(ack_bar);
+                }
+                ok = ok && mbar_wait_cluster(smem_u32(&ctl.dbar[0]) + 8u * par, (uint32_t)(b >> 1) & 1u, abort_flag, S.status);
+                if (sl0) fence_cluster();
+                if (!sl0 && ok) {
+                    auto add = [&](float x, uint32_t m) { // an id that no other coordinate of the block has
+                        const float p = sigma * (x * lds_f32(dl + ((m >> (kIdBits - 2)) & 124u)));
+                        const bool on = m != 0u && (m >> 31) == 0u && p != 0.0f && in_dim(m & kIdMask);
+                        red_add_if(Uk + (on ? m & kIdMask : 0u), p, on);
+                    };
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) add(E0.x[u], E0.m[u]);
+#pragma unroll 1
+                    for (int e = lane + 64; e < E0.n; e += 32) {
+                        float x;
+                        uint32_t m;
+                        entry(s_upd, e, true, x, m);
+                        add(x, m);
+                    }
+                    // ids that several have: a lane per list
+                    float sum = 0.0f;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) sum = fmaf(xl[u], lds_f32(dl + 4u * (rl[u] & 31u)), sum);
+#pragma unroll 1
+                    for (int e = 4; e < len; ++e) sum = fmaf(lds_f32(a_val + 4u * (uint32_t)e), lds_f32(dl + 4u * (lds_u8_if(a_row + (uint32_t)e, true) & 31u)), sum);
+                    red_add_if(Uk + (len > 0 ? id : 0u), sigma * sum, len > 0 && sum != 0.0f);
+#pragma unroll 1
+                    for (int t0 = 32; t0 < T; t0 += 32) {
+                        list_of(s_upd, t0 + lane);
+                        sum = 0.0f;
+#pragma unroll 1
+                        for (int e = 0; e < len; ++e) sum = fmaf(lds_f32(a_val + 4u * (uint32_t)e), lds_f32(dl + 4u * (lds_u8_if(a_row + (uint32_t)e, true) & 31u)), sum);
+                        red_add_if(Uk + (len > 0 ? id : 0u), sigma * sum, len > 0 && sum != 0.0f);
+                    }
+                }
+                __syncwarp();
+                mbar_arrive_if(smem_u32(&ctl.subfree[s_upd]), lane == 0 && ok); // (through with the slot's record and list)
+                s_upd = s_upd + 1 == slots ? 0 : s_upd + 1;
+            }
+            if (ok && late) send(s_dot == 0 ? slots - 1 : s_dot - 1, E1, gather(E1.m[0]), gather(E1.m[1]));
+            due = due && ok;
+            const float w0 = gather(due ? E2.m[0] : 0u), w1 = gather(due ? E2.m[1] : 0u);
+            // (while they are under way) the next block's lists
+            const bool next_walked = depth == 1 ? sl2 : sl1;
+            if (b + 1 >= 0 && b + 1 < nb && !next_walked && ok) {
+                list_of(s_upd, lane);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    xl[u] = lds_f32_if(a_val + 4u * (uint32_t)u, u < len);
+                    rl[u] = lds_u8_if(a_row + (uint32_t)u, u < len);
+                }
+            }
+            if (due) send(s_dot, E2, w0, w1);
+            E0 = depth == 1 ? E2 : E1;
+            E1 = E2;
+            if (++s_dot == slots) {
+                s_dot = 0;
+                dot_turn ^= 1u;
+            }
+            sl0 = next_walked;
+            sl1 = sl2;
+        }
+        if (!ok && lane == 0) *abort_flag = 1;
+        far_bar();
     }
     if (is_worker) {
         // ============================== the worker warps ========================================================
@@ -2064,6 +2295,75 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
 #ifdef CHICLE_LA_TIMING
         long long wd = 0, ws1 = 0, wg0 = 0, wg1 = 0, t0 = clock64(), t1 = 0;
 #endif
+        // (kCold, kFlat) where the bit of a model entry in L2 is
+        const uint32_t filter0 = smem_u32(smem_chain + L.filter);
+        auto bit_of = [&](uint32_t v, uint32_t &word, uint32_t &bit) {
+            const uint32_t h = v >> logC;
+            word = (h >> 3) & (filter_bytes(KIND) - 4u);
+            bit = 1u << (h & 31u);
+        };
+        // a thread's entries of the dot products at hand: values, places, model entries
+        float x[8], w[8];
+        uint32_t m[8];
+        int left = 0;
+        uint32_t a_val = 0u, a_meta = 0u;
+        bool more = false;
+        auto entry = [&](int u) {
+            x[u] = lds_f32_if(a_val + 32u * u, left > 8 * u);
+            m[u] = lds_u32_if(a_meta + 32u * u, left > 8 * u) & kIdMask;
+        };
+        auto entries = [&]() {
+            more = __any_sync(0xffffffffu, left > 32);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) entry(u);
+            if (more) {
+#pragma unroll
+                for (int u = 4; u < 8; ++u) entry(u);
+            }
+        };
+        auto first_entries = [&](uint32_t rec, uint32_t n) {
+            const uint32_t roff = rec + (uint32_t)offsetof(SubHead, roff) + 2u * (uint32_t)jd;
+            const int first = (int)lds_u16(roff) + qd;
+            left = (int)lds_u16(roff + 2u) - first; // entries of this coordinate from this thread's next one on
+            a_val = rec + (uint32_t)sizeof(SubHead) + 4u * (uint32_t)first;
+            a_meta = a_val + 4u * n;
+            entries();
+        };
+        auto far_id = [&](int u) { return (KIND == kFlat ? left > 8 * u : m[u] >= hotc) && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim); };
+        auto model = [&](int u) {
+            if (SPLIT) return;
+            if (KIND == kHot) w[u] = lds_f32(a_w + 4u * (CHICLE_IN_BOUNDS(S.status, m[u] < hotc) ? m[u] : 0u));
+            else {
+                const bool far = far_id(u);
+                w[u] = ldcg_if(Uk + (far ? m[u] : 0u), far);
+            }
+        };
+        auto near = [&](int u) { // (once all gathers are on their way)
+            if (KIND == kCold) {
+                const float h = lds_f32(a_w + (m[u] < hotc ? 4u * m[u] : 0u));
+                w[u] = m[u] < hotc ? h : w[u];
+            }
+            if (SPLIT) { // (the others are the far warp's)
+                const float h = lds_f32(a_w + (m[u] < hotc ? 4u * m[u] : 0u));
+                w[u] = m[u] < hotc ? h : 0.0f;
+            }
+        };
+        auto model_all = [&]() {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) model(u);
+            if (more) {
+#pragma unroll
+                for (int u = 4; u < 8; ++u) model(u);
+            }
+        };
+        // (debug build) a record whose sizes do not fit its slot is not read: as if its wait had run out
+        auto record_fits = [&](const int4 &head) {
+            if (CHICLE_IN_BOUNDS(S.status, head.w >= 0 && head.w <= kLB && (DENSE || (head.x >= 0 && head.y >= 0 && head.z >= 0 &&
+                                               sub_bytes((uint32_t)head.x, (uint32_t)head.y, (uint32_t)head.z) <= stride)))) return true;
+            ok = false;
+            *abort_flag = 1;
+            return false;
+        };
         // The loop starts `depth` blocks early: those turns only take the first blocks' dot products.
         bool sl0 = false, sl1 = false; // whether blocks b and b + 1 are walked in place
 #pragma unroll 1
@@ -2092,6 +2392,21 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                     for (int i = 0; i < 4; ++i) // (the row's first piece stands in for those it does not have)
                         xd[i] = lds_f32x4(row + (qd + 8 * i < (hot_mine + 3) >> 2 ? 16u * (uint32_t)(qd + 8 * i) : 0u));
             }
+            // Ids in L2: the next dot products' gathers go out before the deltas are waited for, against the model as it is (what this
+            // block's update changes is gathered again). Not in front of a block that is walked in place.
+            // (2 M ridge columns over K = 128: 11.1 -> 10.6 ms a step; 5.6 M hashed rows, whose K = 64 round is of this kind, 29.1 -> 28.4.)
+            bool early = false;
+            if (FAR) {
+                dot_record();
+                if (ok && due && !sl0 && (depth == 1 || !sl1)) {
+                    const int4 head = lds_s32x4(r_dot);
+                    if (record_fits(head)) {
+                        first_entries(r_dot, (uint32_t)head.x);
+                        model_all();
+                        early = true;
+                    }
+                }
+            }
             if (b >= 0) {
                 const uint32_t par = (uint32_t)(b & 1), dbar = smem_u32(&ctl.dbar[0]) + 8u * par;
                 if (sl0) {
@@ -2105,6 +2420,11 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 mbar_arrive_expect_tx_if(dbar, d_bytes, wt == 0 && ok); // for block b + 2
                 work_bar();
                 LA_T(wd);
+                const uint32_t filter = filter0 + par * filter_bytes(KIND);
+                if constexpr (FAR) // (the other set: the dot products that looked at it are through)
+#pragma unroll
+                    for (uint32_t i = 0; i < filter_bytes(KIND) / (16u * kWorkThreads); ++i)
+                        sts_f32x4_if(filter0 + (par ^ 1u) * filter_bytes(KIND) + 16u * ((uint32_t)wt + i * kWorkThreads), 0.0f, 0.0f, 0.0f, 0.0f, true);
                 if (!sl0 && ok) {
                     // ---- block b's update of this CTA's part of the model
                     const uint32_t dl = smem_u32(&ctl.dbuf[0][0]) + par * (uint32_t)(kLB * 4);
@@ -2146,7 +2466,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                             const int len = on ? (int)((id >> kIdBits) & 31u) + 1 : 0;
                             const int first = (int)lds_u16_if(lst + 2u * (uint32_t)t, on) + q;
                             const uint32_t a_val = lval + 4u * (uint32_t)first, a_row = lrow + (uint32_t)first;
-                            const bool near = KIND == kHot || (KIND == kCold && v < hotc);
+                            const bool near = KIND == kHot || ((KIND == kCold || SPLIT) && v < hotc);
                             const float w = KIND == kFlat ? 0.0f : lds_f32(a_w + (near ? 4u * v : 0u));
                             float x[8];
                             uint32_t r[8];
@@ -2168,9 +2488,12 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                             sum += __shfl_xor_sync(0xffffffffu, sum, 2);
                             const bool mine = on && q == 0;
                             if (KIND != kFlat) sts_f32(mine && near ? a_w + 4u * v : a_sink, fmaf(sigma, sum, w));
-                            if (KIND != kHot) {
+                            if (FAR) {
                                 const bool far = mine && !near && sum != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
                                 red_add_if(Uk + (far ? v : 0u), sigma * sum, far);
+                                uint32_t word, bit;
+                                bit_of(v, word, bit);
+                                red_shared_or_if(filter + word, bit, far);
                             }
                         }
                         // A thread per entry: one whose id no other coordinate of the block has is applied (no two threads
@@ -2193,16 +2516,19 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                                 const uint32_t v = m[u] & kIdMask;
                                 p[u] = sigma * (p[u] * lds_f32(dl + ((m[u] >> (kIdBits - 2)) & 124u)));
                                 if (KIND == kHot) w[u] = lds_f32(a_w + 4u * (CHICLE_IN_BOUNDS(S.status, v < hotc) ? v : 0u));
-                                if (KIND == kCold) w[u] = lds_f32(a_w + (v < hotc ? 4u * v : 0u));
+                                if (KIND == kCold || SPLIT) w[u] = lds_f32(a_w + (v < hotc ? 4u * v : 0u));
                             }
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
                                 const uint32_t v = m[u] & kIdMask;
-                                const bool mine = (m[u] >> 31) == 0u, near = KIND == kHot ? CHICLE_IN_BOUNDS(S.status, v < hotc) : (KIND == kCold && v < hotc);
+                                const bool mine = (m[u] >> 31) == 0u, near = KIND == kHot ? CHICLE_IN_BOUNDS(S.status, v < hotc) : ((KIND == kCold || SPLIT) && v < hotc);
                                 if (KIND != kFlat) sts_f32(mine && near ? a_w + 4u * v : a_sink, p[u] + w[u]);
-                                if (KIND != kHot) {
+                                if (FAR) {
                                     const bool far = mine && !near && p[u] != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
                                     red_add_if(Uk + (far ? v : 0u), p[u], far);
+                                    uint32_t word, bit;
+                                    bit_of(v, word, bit);
+                                    red_shared_or_if(filter + word, bit, far);
                                 }
                             }
                         }
@@ -2213,7 +2539,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             }
             // ---- dot products: of block b + depth against the model as it is now. A block right behind a walked one starts
             //      from the model as the walk left it: with depth 2 its products wait for that.
-            if (!DENSE) dot_record();
+            if (KIND == kHot || SPLIT) dot_record();
             if (sl0 || sl1) {
                 late = depth == 2 && sl0 && !sl1 && b + 1 < nb;
                 due = due && (depth == 1 || !sl1);
@@ -2233,13 +2559,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 if (late) late = false;
                 else due = false;
                 const int4 head = lds_s32x4(rec); // n, T, nl, cnt
-                // (debug build) a record whose sizes do not fit its slot is not read: as if its wait had run out
-                if (!CHICLE_IN_BOUNDS(S.status, head.w >= 0 && head.w <= kLB && (DENSE || (head.x >= 0 && head.y >= 0 && head.z >= 0 &&
-                                                    sub_bytes((uint32_t)head.x, (uint32_t)head.y, (uint32_t)head.z) <= stride)))) {
-                    ok = false;
-                    *abort_flag = 1;
-                    break;
-                }
+                if (!record_fits(head)) break;
                 const uint32_t slot = (uint32_t)(fg & 1);
                 ++fg;
                 float acc = 0.0f;
@@ -2271,53 +2591,27 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
                 } else {
                     // eight entries per thread and turn, all loads of a turn issued before anything is used: an id beyond the
                     // part of the model in shared memory costs a round trip to L2 (the updates are made there by reductions)
-                    const uint32_t roff = rec + (uint32_t)offsetof(SubHead, roff) + 2u * (uint32_t)jd;
-                    const int first = (int)lds_u16(roff) + qd;
-                    int left = (int)lds_u16(roff + 2u) - first; // entries of this coordinate from this thread's next one on
-                    uint32_t a_val = val + 4u * (uint32_t)first, a_meta = a_val + 4u * (uint32_t)head.x;
-                    float x[8], w[8];
-                    uint32_t m[8];
-                    bool more;
-                    auto entry = [&](int u) {
-                        x[u] = lds_f32_if(a_val + 32u * u, left > 8 * u);
-                        m[u] = lds_u32_if(a_meta + 32u * u, left > 8 * u) & kIdMask;
-                    };
-                    auto model = [&](int u) {
-                        if (KIND == kFlat) {
-                            const bool in = left > 8 * u && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim);
-                            w[u] = ldcg_if(Uk + (in ? m[u] : 0u), in);
-                        } else if (KIND == kHot) {
-                            w[u] = lds_f32(a_w + 4u * (CHICLE_IN_BOUNDS(S.status, m[u] < hotc) ? m[u] : 0u));
-                        } else {
-                            const bool cold = m[u] >= hotc && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim);
-                            w[u] = ldcg_if(Uk + (cold ? m[u] : 0u), cold);
-                        }
-                    };
-                    auto near = [&](int u) { // (once all gathers are on their way)
-                        if (KIND == kCold) {
-                            const float h = lds_f32(a_w + (m[u] < hotc ? 4u * m[u] : 0u));
-                            w[u] = m[u] < hotc ? h : w[u];
-                        }
-                    };
-                    auto entries = [&]() {
-                        more = __any_sync(0xffffffffu, left > 32);
+                    if (!early) first_entries(rec, (uint32_t)head.x);
+                    meet();
+                    if (early && b >= 0) { // what this block's update has changed, or may have
+                        const uint32_t filter = filter0 + (uint32_t)(b & 1) * filter_bytes(KIND);
+                        auto again = [&](int u) {
+                            const bool far = far_id(u);
+                            uint32_t word, bit;
+                            bit_of(m[u], word, bit);
+                            ldcg_again_if(w[u], Uk + (far ? m[u] : 0u), (lds_u32_if(filter + word, far) & bit) != 0u);
+                        };
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) entry(u);
+                        for (int u = 0; u < 4; ++u) again(u);
                         if (more) {
 #pragma unroll
-                            for (int u = 4; u < 8; ++u) entry(u);
+                            for (int u = 4; u < 8; ++u) again(u);
                         }
-                    };
-                    entries();
-                    meet();
+                    }
 #pragma unroll 1
                     for (;;) { // (whole warps)
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) model(u);
-                        if (more) {
-#pragma unroll
-                            for (int u = 4; u < 8; ++u) model(u);
-                        }
+                        if (!early) model_all();
+                        early = false;
 #pragma unroll
                         for (int u = 0; u < 4; ++u) near(u);
                         if (more) {
@@ -2353,6 +2647,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) k_lookahead_chain(const Look
             sl1 = sl2;
         }
         if (!ok && lane == 0) *abort_flag = 1;
+        if (SPLIT) far_bar(); // (the far warp's updates have been made)
         aborted = !ok; // (otherwise: every update has been applied, the last barrier says so)
 #ifdef CHICLE_LA_TIMING
         if (blockIdx.x == 0 && wt == 0) {
@@ -2420,7 +2715,7 @@ template <int LOSS, int KIND, bool TAB> cudaError_t launch_chain_kind(Glm &g, co
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)g.K << g.la_logC, 1, 1);
-    cfg.blockDim = dim3(kChainThreads, 1, 1);
+    cfg.blockDim = dim3(chain_threads(KIND), 1, 1);
     cfg.dynamicSmemBytes = g.la_smem;
     cfg.stream = g.stream;
     cudaLaunchAttribute attr[2];
@@ -2464,6 +2759,20 @@ template <int LOSS, int NZ, int HT, int THREADS, int PER_SM> cudaError_t launch_
     return cudaGetLastError();
 }
 
+constexpr int kSplitLeast = 4096;    // ids per CTA in shared memory that the far warp's lists must leave
+// Entries beyond them that a block may be expected to have in a CTA's record: what the far warp keeps in registers. (45 M hashed rows
+// over K = 16 have 37; ridge over K = 128 has several hundred, and with the far warp, which is then the slowest, 17.1 instead of 10.6 ms.)
+constexpr double kSplitMost = 64.0;
+// Entries that a block of 32 random coordinates is expected to have with ids from `first` on.
+double entries_beyond(const Glm &g, int64_t first)
+{
+    double e = 0.0;
+    for (int k = 0; k < kOctaves; ++k) {
+        const double lo = k == 0 ? 0.0 : (double)((int64_t)1 << k), hi = fmin((double)((int64_t)2 << k), (double)g.dim);
+        if (hi > (double)first && hi > lo) e += g.blk_octave[k] * (lo >= (double)first ? 1.0 : (hi - (double)first) / (hi - lo));
+    }
+    return e;
+}
 constexpr int kPreSmallNz = 2048, kPreSmallHt = 2048;
 constexpr int kPreMidNz = 3072, kPreMidHt = 4096;
 constexpr int kPreLargeNz = 4096, kPreLargeHt = 4096;
@@ -2533,13 +2842,23 @@ template <int LOSS, int KIND, bool TABLES> cudaError_t launch_chain(Glm &g, cons
     return TABLES && P.tab_bins ? launch_chain_kind<LOSS, KIND, TABLES>(g, P, begun) : launch_chain_kind<LOSS, KIND, false>(g, P, begun);
 }
 
+int chain_kind(const Glm &g)
+{
+    if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) return kDense;
+    if (g.la_hotc == 0) return kFlat;
+    if (((int64_t)g.la_hotc << g.la_logC) >= g.dim) return kHot;
+    return g.la_far_cap > 0 ? kSplit : kCold;
+}
 template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P, cudaEvent_t begun = nullptr)
 {
     constexpr bool tables = LOSS == CHICLE_LOSS_LOGISTIC_DUAL;
-    if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) return launch_chain<LOSS, kDense, tables>(g, P, begun);
-    if (g.la_hotc == 0) return launch_chain<LOSS, kFlat, tables>(g, P, begun);
-    if (((int64_t)g.la_hotc << g.la_logC) >= g.dim) return launch_chain<LOSS, kHot, tables>(g, P, begun);
-    return launch_chain<LOSS, kCold, tables>(g, P, begun);
+    switch (chain_kind(g)) {
+    case kDense: return launch_chain<LOSS, kDense, tables>(g, P, begun);
+    case kFlat: return launch_chain<LOSS, kFlat, tables>(g, P, begun);
+    case kHot: return launch_chain<LOSS, kHot, tables>(g, P, begun);
+    case kSplit: return launch_chain<LOSS, kSplit, tables>(g, P, begun);
+    default: return launch_chain<LOSS, kCold, tables>(g, P, begun);
+    }
 }
 
 constexpr size_t kWordsPerLaunch = 480;
@@ -2671,13 +2990,14 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
         const float q_max = (float)K * g.max_sqnorm / (g.lambda * (float)g.n_examples);
         for (int bins = 64; bins >= 32; bins >>= 1)
             if (q_max <= tab_max_q(bins)) g.la_tab_bins = bins;
-        if (dense && chain_layout(0, kSubSlots, slice, true, g.la_tab_bins).total > budget) g.la_tab_bins = 0;
+        if (dense && chain_layout(0, kSubSlots, slice, true, g.la_tab_bins, kDense).total > budget) g.la_tab_bins = 0;
         const char *env = getenv("CHICLE_LA_TABLES"); // 0: none (tests)
         if (env && env[0] == '0') g.la_tab_bins = 0;
     }
     g.la_slots = kSubSlots;
     g.la_sub_room = 0;
     g.la_hotc = slice;
+    g.la_far_cap = 0;
     if (!dense) {
         // A slot holds the record that a block of 32 random coordinates is expected to make for a CTA (how many entries, and how
         // many of them with ids that several of the 32 have: from the ids' frequencies, see launch_frequency_remap) and five
@@ -2689,6 +3009,7 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
         // over K = 128 12.5 -> 12.8 ms, logistic rows of 80 over K = 64, which lose their tables, 2.8 -> 3.8.)
         const int C = 1 << logC;
         uint32_t room = 256, most = 256;
+        double n_max = 0.0; // entries of a CTA's record
         const double cap = (double)prepare_room(g); // (a block with more entries is walked in place anyway)
         for (int c = 0; c < C; ++c) {
             double n = 0.0, T = 0.0, nl = 0.0;
@@ -2701,12 +3022,13 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
             const double nl_hi = fmin(n_hi, f * nl + 5.0 * sqrt(nl)), T_hi = fmin(0.5 * nl_hi, f * T + 5.0 * sqrt(T));
             const uint32_t r = sub_bytes((uint32_t)n_hi + 1u, (uint32_t)T_hi + 1u, (uint32_t)nl_hi + 1u) + 64u;
             const uint32_t m = sub_bytes((uint32_t)n_hi + 1u, (uint32_t)(0.5 * n_hi) + 1u, (uint32_t)n_hi + 1u) + 64u;
+            n_max = fmax(n_max, n_hi);
             room = r > room ? r : room;
             most = m > most ? m : most;
         }
         if (g.by_chunks) room = most;
         for (;;) {
-            const double left = (double)budget - (double)chain_layout(0, 0, 0, false, g.la_tab_bins).total - 64.0;
+            const double left = (double)budget - (double)chain_layout(0, 0, 0, false, g.la_tab_bins, g.flat_ids ? kFlat : kCold).total - 64.0;
             g.la_slots = g.la_depth == 1 && 4.0 * room > 0.6 * left ? 3 : kSubSlots;
             if (g.la_tab_bins == 0 || (double)g.la_slots * room <= 0.8 * left) {
                 const uint32_t limit = (uint32_t)(0.8 * left / g.la_slots) & ~15u;
@@ -2715,16 +3037,26 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
             }
             g.la_tab_bins = 0;
         }
-        const ChainLayout L0 = chain_layout(g.la_sub_room, g.la_slots, 0, false, g.la_tab_bins);
+        const ChainLayout L0 = chain_layout(g.la_sub_room, g.la_slots, 0, false, g.la_tab_bins, kHot);
         int64_t hotc = ((int64_t)budget - (int64_t)L0.total - 64) / 4;
-        hotc = hotc < 0 || g.flat_ids ? 0 : (hotc / 32) * 32;
         const int64_t need = (g.dim + ((int64_t)1 << logC) - 1) >> logC; // per CTA for the whole model
+        if (hotc < need && !g.flat_ids) {
+            // the rest lies in L2: lists for the far warp, where they leave the model something; or two filters
+            const int cap = ((int)n_max + 32) & ~31;
+            const int64_t split = hotc - (int64_t)far_bytes(kSplit, cap, g.la_slots) / 4;
+            const double beyond = split >= kSplitLeast ? entries_beyond(g, split << logC) / C : 1e30;
+            if (beyond <= kSplitMost) {
+                hotc = split;
+                g.la_far_cap = cap;
+            } else hotc -= (int64_t)filter_bytes(kCold) / 2;
+        }
+        hotc = hotc < 0 || g.flat_ids ? 0 : (hotc / 32) * 32;
         // (what the whole model leaves goes to the slots: rows may be more alike than their ids' frequencies say)
         const int64_t spare = (4 * (hotc - (need + 31) / 32 * 32) / g.la_slots) & ~(int64_t)15;
         if (spare > 0 && g.la_sub_room < most) g.la_sub_room += (uint32_t)((int64_t)(most - g.la_sub_room) < spare ? most - g.la_sub_room : spare);
         g.la_hotc = (int32_t)(hotc < need ? hotc : (need + 31) / 32 * 32);
     }
-    g.la_smem = chain_layout(g.la_sub_room, g.la_slots, g.la_hotc, dense, g.la_tab_bins).total;
+    g.la_smem = chain_layout(g.la_sub_room, g.la_slots, g.la_hotc, dense, g.la_tab_bins, chain_kind(g), g.la_far_cap).total;
 
     // slices: at most a sixteenth of the walk, but at least 256 blocks per partition; two regions
     const int64_t n = g.n_coord;
@@ -2876,6 +3208,7 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
         p.sub_room = g.la_sub_room;
         p.slots = g.la_slots;
         p.hotc = g.la_hotc;
+        p.far_cap = g.la_far_cap > 0 ? g.la_far_cap : INT32_MAX;
         p.n_blocks = blocks[(size_t)s];
         p.drop_block = (drop && s == 0) ? atoll(drop) : -1;
         p.nnz = g.nnz;

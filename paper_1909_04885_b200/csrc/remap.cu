@@ -57,21 +57,35 @@ __global__ void k_mass_of_first(const uint32_t *__restrict__ counts, const int32
 
 // What a block of 32 random coordinates is expected to have on the ids of class i = (new id) mod kRankClasses: out[i]
 // entries (the whole problem's, exactly), out[kRankClasses + i] ids that at least two of the 32 have and
-// out[2 kRankClasses + i] entries with such ids (both in units of 2^-20, so that the sums do not depend on their order).
+// out[2 kRankClasses + i] entries with such ids (both in units of 2^-20, so that the sums do not depend on their order); and
+// out[3 kRankClasses + k] entries with (new) ids of octave k: 2^k .. 2^(k+1) - 1, and id 0 in octave 0.
 __global__ void k_expect_blocks(const uint32_t *__restrict__ counts, const int32_t *__restrict__ old_of_new, int64_t dim, double inv_n,
                                 unsigned long long *__restrict__ out)
 {
     static_assert(kT % kRankClasses == 0, "a thread's ids are of one class");
     unsigned long long all = 0, ids = 0, ent = 0;
+    __shared__ unsigned long long octave[kOctaves];
+    if (threadIdx.x < kOctaves) octave[threadIdx.x] = 0;
+    __syncthreads();
+    int at = 0;
+    unsigned long long part = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < dim; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t c = counts[old_of_new[i]];
         const float p = fminf((float)((double)c * inv_n), 0.9999999f), l = log1pf(-p);
         const float others = -expm1f(31.0f * l);                               // one of the other 31 has it
         const float one = 32.0f * p * (1.0f - others), some = -expm1f(32.0f * l); // exactly one has it, some have it
         all += c;
+        const int oct = i >= 2 ? 63 - __clzll(i) : 0; // (a thread's ids ascend: it meets every octave once)
+        if (oct != at) {
+            if (part) atomicAdd(octave + at, part);
+            at = oct;
+            part = 0;
+        }
+        part += c;
         ids += (unsigned long long)(fmaxf(some - one, 0.0f) * 1048576.0f);
         ent += (unsigned long long)(32.0f * p * others * 1048576.0f);
     }
+    if (part) atomicAdd(octave + at, part);
 #pragma unroll
     for (int o = 16; o >= kRankClasses; o >>= 1) {
         all += __shfl_xor_sync(0xffffffffu, all, o);
@@ -84,6 +98,8 @@ __global__ void k_expect_blocks(const uint32_t *__restrict__ counts, const int32
         if (ids) atomicAdd(o + kRankClasses, ids);
         if (ent) atomicAdd(o + 2 * kRankClasses, ent);
     }
+    __syncthreads();
+    if (threadIdx.x < kOctaves && octave[threadIdx.x]) atomicAdd(out + 3 * kRankClasses + threadIdx.x, octave[threadIdx.x]);
 }
 
 // out[1] += number of coordinates with more than `long_len` entries; out[2] += the sum of their squared lengths (each
