@@ -43,6 +43,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "solver_common.cuh"
@@ -498,7 +499,8 @@ __host__ __device__ constexpr int pre_room(int nz, int ht) { return nz < ht - kH
 // block of 1 600 non-zeros took 63 000 cycles at three CTAs per SM. Rows of 50 on 1 M coordinates, a slice of 4 096 blocks on the whole
 // GPU: 255 us; with slots without tries for frequent ids, entries' findings kept in registers, one atomic per numbered id and the
 // pairs shared out evenly 225 us (instructions a block 40 700 -> 35 200); step 4.01 -> 3.59 ms, ridge 12.5 -> 11.1 (longer blocks
-// have more tries to save). A thread's several entries together, all loads first: 46 100 instructions, 272 us. 640 or 416
+// have more tries to save). Rows fetched two pieces at a time, the dense part in front of the last barrier and without its cross half
+// where there is no cross Gram matrix, the next constants beside the records' places: 216 us; 3.60 -> 3.45 ms. A thread's several entries together, all loads first: 46 100 instructions, 272 us. 640 or 416
 // threads: 254 and 244 us; 256 us at 384.
 constexpr int kDirNew = 4; // (metadata slots: a power of two)
 
@@ -675,13 +677,19 @@ template <int NZ, int THREADS, class Shared> __device__ __forceinline__ void pre
     if (B.over) return;
     for (int j = warp; j < kLB; j += THREADS / 32) {
         const int n = B.nnz[j], r0 = B.roff[j];
-        const int32_t *ix = P.S.indices + B.rs[j];
-        const float *xv = P.S.values + B.rs[j];
-        for (int e = lane; e < n; e += 32) {
-            cp_async4(smem_u32(&sh.idx[buf][r0 + e]), ix + e);
-            cp_async4(smem_u32(&sh.val[buf][r0 + e]), xv + e);
-            sh.row[buf][r0 + e] = (uint8_t)j;
-        }
+        const int32_t *ix = P.S.indices + B.rs[j] + lane;
+        const float *xv = P.S.values + B.rs[j] + lane;
+        const uint32_t di = smem_u32(&sh.idx[buf][r0 + lane]), dv = smem_u32(&sh.val[buf][r0 + lane]);
+        uint8_t *dr = &sh.row[buf][r0 + lane];
+#pragma unroll 1
+        for (int e = 0; e < n; e += 64)
+#pragma unroll
+            for (int u = 0; u < 64; u += 32)
+                if (e + u + lane < n) {
+                    cp_async4(di + 4u * (uint32_t)(e + u), ix + e + u);
+                    cp_async4(dv + 4u * (uint32_t)(e + u), xv + e + u);
+                    dr[e + u] = (uint8_t)j;
+                }
     }
 }
 // (a warp: which of 32 consecutive entries fall to which CTA, and their part of the dense tile; id < 0: no entry. flip: per bit of a CTA's
@@ -788,9 +796,14 @@ __device__ __forceinline__ void pre_listed(Shared &sh, int have, int cur, const 
     for (int at = 0; at < have; at += 32) pre_pairs<NZ>(sh, at + lane < have ? todo[at + lane] : 0u, at + lane < have, cur, N);
     __syncwarp();
 }
-// (not inlined: for lists longer than usual, between their parts)
+// (not inlined: a list longer than usual between its parts, 32 at a time from its end; what is left)
 template <int NZ, class Shared>
-__device__ __noinline__ void pre_listed_early(Shared &sh, int have, int cur, const PreBlock &N) { pre_listed<NZ>(sh, have, cur, N); }
+__device__ __noinline__ int pre_listed_early(Shared &sh, int have, int cur, const PreBlock &N)
+{
+    for (; have > 32; have -= 32) pre_pairs<NZ>(sh, sh.work[threadIdx.x >> 5][have - 32 + (threadIdx.x & 31)], true, cur, N);
+    __syncwarp();
+    return have;
+}
 
 // What the states at round start contribute: the warps' sums (sh.work) together, off A and into q0n; the block's constants
 // go out. (A warp; one block behind the loop, so that it needs no barrier of its own.)
@@ -948,8 +961,8 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         PRE_T(1);
         // ---- the records' places: the head has its own (one per block); the workers' records come from the pool, of which
         //      a CTA takes a piece for several blocks at a time. A block that the pool has no room for is walked in place
-        //      like one that is too long. (A warp. The others meanwhile: the next block's entries, which CTA's they are, and their
-        //      dense tile.)
+        //      like one that is too long. (A warp. Meanwhile another one: the constants of the block after the next; and all: the
+        //      next block's entries, which CTA's they are, and their dense tile.)
         if (warp == 0) { // (a lane per CTA of the cluster)
             const bool in = lane < C;
             const uint32_t n_c = in ? sh.rc[kLB][lane] : 0u, w = in ? sh.cnt[lane] : 0u;
@@ -999,6 +1012,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 *reinterpret_cast<int4 *>(&out) = make_int4(cnt, sl ? 1 : 0, 0, 0);
             }
         }
+        if (warp == NW - 1 && bid + 2 < end) pre_make_block<LOSS, NZ, HT>(P, sh, bid + 2);
         const int ntotal = have_next ? N.total : 0;
         int32_t nid[EPT];
 #pragma unroll
@@ -1054,7 +1068,6 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
         PRE_T(3);
         // ---- the next block's entries: which of this block's coordinates have their ids (table of this block); the pairs of both
         //      Gram matrices, 32 entries with some at a time
-        if (warp == NW - 1 && bid + 2 < end) pre_make_block<LOSS, NZ, HT>(P, sh, bid + 2);
         {
             uint32_t *todo = sh.work[warp];
             int have = 0;
@@ -1086,35 +1099,42 @@ __global__ void __launch_bounds__(THREADS, PER_SM) k_lookahead_prepare(const Loo
                 }
                 if (i + 1 < EPT && have > 32) { // (the list holds 96)
                     __syncwarp();
-                    pre_listed_early<NZ>(sh, have, cur, N);
-                    have = 0;
+                    have = pre_listed_early<NZ>(sh, have, cur, N);
                 }
             }
             __syncwarp();
             pre_listed<NZ>(sh, have, cur, N);
         }
-        __syncthreads();
-        PRE_T(4);
-        // ---- rows l = warp, warp + NW of both matrices, lane = column: the dense part, both together, scaled
-        if (have_next && warp < C) pre_prefix(sh, N.total, nxt, warp);
+        // ---- rows l = warp, warp + NW of both matrices, lane = column: the dense part
+        constexpr int R = kLB / NW;
+        float2 g2[R], x2[R]; // (the even and the odd columns of the tiles)
         {
-            constexpr int R = kLB / NW;
-            float2 g2[R], x2[R]; // (the even and the odd columns)
 #pragma unroll
             for (int r = 0; r < R; ++r) g2[r] = x2[r] = make_float2(0.0f, 0.0f);
             const float4 *dj = reinterpret_cast<const float4 *>(&sh.D[cur][lane][0]), *nj = reinterpret_cast<const float4 *>(&sh.D[nxt][lane][0]);
+            auto part = [&](auto both_) {
+                constexpr bool both = decltype(both_)::value;
 #pragma unroll
-            for (int h = 0; h < kHD / 4; ++h) {
-                const float4 a = dj[h], b = nj[h];
+                for (int h = 0; h < kHD / 4; ++h) {
+                    const float4 a = dj[h], b = both ? nj[h] : a;
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float4 c = *reinterpret_cast<const float4 *>(&sh.D[cur][warp + r * NW][4 * h]);
-                    fma2(g2[r], a.x, a.y, c.x, c.y);
-                    fma2(x2[r], b.x, b.y, c.x, c.y);
-                    fma2(g2[r], a.z, a.w, c.z, c.w);
-                    fma2(x2[r], b.z, b.w, c.z, c.w);
+                    for (int r = 0; r < R; ++r) {
+                        const float4 c = *reinterpret_cast<const float4 *>(&sh.D[cur][warp + r * NW][4 * h]);
+                        fma2(g2[r], a.x, a.y, c.x, c.y);
+                        if (both) fma2(x2[r], b.x, b.y, c.x, c.y);
+                        fma2(g2[r], a.z, a.w, c.z, c.w);
+                        if (both) fma2(x2[r], b.z, b.w, c.z, c.w);
+                    }
                 }
-            }
+            };
+            if (carry) part(std::true_type{});
+            else part(std::false_type{});
+        }
+        __syncthreads();
+        PRE_T(4);
+        // ---- both matrices scaled and written
+        if (have_next && warp < C) pre_prefix(sh, N.total, nxt, warp);
+        {
             float qg = 0.0f, qx = 0.0f;
             // (the two inverse scales one after the other: their product is no fp32 number for two rows of norms below 1e-18)
             const float gsc = B.gsc[lane], inv = B.inv[lane], ngsc = carry ? N.gsc[lane] : 0.0f, ninv = carry ? N.inv[lane] : 0.0f;
