@@ -28,7 +28,9 @@
 //                         "wait for block b's deltas, apply them to my part of the model, take my part of block
 //                         b + 2's dot products, send the 32 partial sums to CTA 0". Deltas and partial sums travel
 //                         through distributed shared memory by asynchronous stores that complete on the receiver's
-//                         mbarrier; no multicast, every wait bounded.
+//                         mbarrier; no multicast, every wait bounded. Ids that are not in shared memory: where a block has a
+//                         few of them per CTA, a warp of its own applies their updates and takes their part of the dot products; where
+//                         it has many, the worker warps do, with the gathers sent out before the deltas have come.
 //
 // Where many partitions leave the prepare kernels few SMs (one CTA per partition on sparse data), the dot products are
 // taken one block ahead only, against the model after the block before: no cross Gram matrix (the prepare kernels are
@@ -500,8 +502,8 @@ __host__ __device__ constexpr int pre_room(int nz, int ht) { return nz < ht - kH
 // GPU: 255 us; with slots without tries for frequent ids, entries' findings kept in registers, one atomic per numbered id and the
 // pairs shared out evenly 225 us (instructions a block 40 700 -> 35 200); step 4.01 -> 3.59 ms, ridge 12.5 -> 11.1 (longer blocks
 // have more tries to save). Rows fetched two pieces at a time, the dense part in front of the last barrier and without its cross half
-// where there is no cross Gram matrix, the next constants beside the records' places: 216 us; 3.60 -> 3.45 ms. A thread's several entries together, all loads first: 46 100 instructions, 272 us. 640 or 416
-// threads: 254 and 244 us; 256 us at 384.
+// where there is no cross Gram matrix, the next constants beside the records' places: 216 us; 3.60 -> 3.45 ms. A thread's several entries together, all loads first: 46 100 instructions, 272 us. 640, 448, 416
+// or 384 threads instead of 512: 254, 241, 244 and 250 us.
 constexpr int kDirNew = 4; // (metadata slots: a power of two)
 
 // One block's coordinates as the kernel keeps them: constants of the steps and extents of the rows.
@@ -2992,9 +2994,9 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
     // the chain launches and have the whole GPU meanwhile (2 M ridge columns over K = 128: 12.5 against 584 ms a step).
     g.la_overlap = ((int64_t)K << logC) * 2 <= g.sm_count;
     // Two blocks ahead pays where the chains bound the round: dense rows (10 000 of 100, K = 4: 186 against 247 us a step) and
-    // sparse data with a cluster per partition (1 M rows of 50, K = 16: 4.0 against 5.2 ms; 45 M of 39: 156 against 278). One CTA
+    // sparse data with a cluster per partition (1 M rows of 50, K = 16, before the prepare kernel became shorter: 4.0 against 5.2 ms; 45 M of 39: 156 against 278). One CTA
     // per partition on sparse data means many partitions: there the prepare kernels bound the round, and are shorter without
-    // the cross Gram matrices (5.6 M hashed rows, a round with K = 64 and one with K = 16: 31.0 against 32.0 ms).
+    // the cross Gram matrices (5.6 M hashed rows, a round with K = 64 and one with K = 16: 28.4 against 29.3 ms).
     g.la_depth = (dense || logC >= 1) && g.la_overlap ? 2 : 1;
     {
         const char *env = getenv("CHICLE_LA_DEPTH");
