@@ -344,7 +344,6 @@ chicle_status_t chicle_glm_create(const chicle_matrix_t *X, const float *labels,
         }
         for (int i = 0; i < kOctaves; ++i) h->blk_octave[i] = 32.0 * (double)host_mass2[4 + 3 * kRankClasses + i] / n;
         const char *force = getenv("CHICLE_FORCE_VARIANT"); // debugging aid
-        h->flat_ids = force && strcmp(force, "flat") == 0;
         if (force && strcmp(force, "flat") == 0) h->hot_variant = 0;
         if (force && strcmp(force, "hot") == 0) h->hot_variant = 1;
         if (force && strcmp(force, "hot128") == 0) h->hot_variant = 2;

@@ -107,7 +107,6 @@ struct Glm {
     float *perm_tmp = nullptr;     // dim, staging for translating v at the boundary
     int hot_variant = 0;           // 1 / 2: most non-zeros fall on the first ids, the solver keeps those in a direct
                                    // array (2: with room for coordinates of up to 128 entries); 0: flat ids
-    bool flat_ids = false;         // (tests) no part of the model in shared memory
     bool by_chunks = false;        // sparse: the partitions follow the coordinates' numbers (chunks), not a random order
     double chunk_mean = 0.0;       // largest average of a partition's numbers of entries that partitions by chunks have had
     // what a block of 32 random coordinates is expected to have on the ids of each class (id mod kRankClasses): entries, ids

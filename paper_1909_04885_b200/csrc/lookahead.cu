@@ -130,9 +130,9 @@ struct alignas(16) BlkDir { // where a record is
 };
 
 // Kinds of data the chain kernel is instantiated for: sparse with the whole model in shared memory, with its most frequent
-// ids there, with none; dense rows.
+// ids there; dense rows.
 // kSplit: as kCold, with a warp of its own for the ids that are not in shared memory; kCold where there is no room for its lists.
-constexpr int kHot = 0, kCold = 1, kFlat = 2, kDense = 3, kSplit = 4;
+constexpr int kHot = 0, kCold = 1, kDense = 2, kSplit = 3;
 __host__ __device__ constexpr int chain_threads(int kind) { return kind == kSplit ? 448 : 384; }
 
 struct LookParams {
@@ -1656,11 +1656,11 @@ struct ChainLayout {
 constexpr uint32_t kFarSums = 2u * kMaxC * kLB * 4u, kFarHead = 80u;
 __host__ __device__ constexpr uint32_t far_list_bytes(int cap) { return kFarHead + 2u * (uint32_t)cap; }
 __host__ __device__ constexpr uint32_t far_bytes(int kind, int cap, int slots) { return kind == kSplit ? kFarSums + 4u * (uint32_t)cap + (uint32_t)slots * far_list_bytes(cap) : 0u; }
-// Ids beyond the model's part in shared memory (some: kCold, all: kFlat): their model entries are gathered from L2 before the
+// Ids beyond the model's part in shared memory (kCold): their model entries are gathered from L2 before the
 // block's deltas have come, and those that the block's update then changes once more. Which may have changed is kept in a bit
 // per hashed id, one set of them for even and one for odd blocks: this many bytes a set (a bit that two ids share costs a
 // second gather, nothing else).
-__host__ __device__ constexpr uint32_t filter_bytes(int kind) { return kind == kCold ? 4096u : (kind == kFlat ? 16384u : 0u); }
+__host__ __device__ constexpr uint32_t filter_bytes(int kind) { return kind == kCold ? 4096u : 0u; }
 __host__ __device__ inline ChainLayout chain_layout(uint32_t sub_room, int slots, int hotc, bool dense, int tab_bins, int kind, int far_cap = 0)
 {
     ChainLayout L;
@@ -1746,7 +1746,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
         for (int i = 0; i < 8; ++i)
             if (l0 + i * kChainThreads < hot_mine) W[l0 + i * kChainThreads] = P.model_in ? fmaf(sigma, u[i], v[i]) : u[i];
     }
-    constexpr bool FAR = KIND == kCold || KIND == kFlat;
+    constexpr bool FAR = KIND == kCold;
     if constexpr (FAR)
         for (uint32_t i = (uint32_t)tid; i < 2u * filter_bytes(KIND) / 4u; i += kChainThreads) reinterpret_cast<uint32_t *>(smem_chain + L.filter)[i] = 0u;
     if (DENSE && tid < 4 && hot_mine + tid < P.hotc) W[hot_mine + tid] = 0.0f; // (the padding of the last slice)
@@ -2096,7 +2096,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
         for (int blk = 0; blk < nb; ++blk) {
             if (__any_sync(0xffffffffu, *abort_flag != 0)) break; // (no slot is refilled for workers that no longer wait for it)
             // (the block before this one arrives while its predecessor's slot is still in use)
-            if ((KIND == kCold || KIND == kFlat || SPLIT) && blk > 0) {
+            if ((FAR || SPLIT) && blk > 0) {
                 if (!mbar_wait_cluster(smem_u32(&ctl.subfull[before]), tbefore, abort_flag, S.status)) break;
                 list_far(before);
             }
@@ -2317,7 +2317,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
 #ifdef CHICLE_LA_TIMING
         long long wd = 0, ws1 = 0, wg0 = 0, wg1 = 0, t0 = clock64(), t1 = 0;
 #endif
-        // (kCold, kFlat) where the bit of a model entry in L2 is
+        // (kCold) where the bit of a model entry in L2 is
         const uint32_t filter0 = smem_u32(smem_chain + L.filter);
         auto bit_of = [&](uint32_t v, uint32_t &word, uint32_t &bit) {
             const uint32_t h = v >> logC;
@@ -2351,7 +2351,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
             a_meta = a_val + 4u * n;
             entries();
         };
-        auto far_id = [&](int u) { return (KIND == kFlat ? left > 8 * u : m[u] >= hotc) && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim); };
+        auto far_id = [&](int u) { return m[u] >= hotc && CHICLE_IN_BOUNDS(S.status, (int64_t)m[u] < S.dim); };
         auto model = [&](int u) {
             if (SPLIT) return;
             if (KIND == kHot) w[u] = lds_f32(a_w + 4u * (CHICLE_IN_BOUNDS(S.status, m[u] < hotc) ? m[u] : 0u));
@@ -2488,8 +2488,8 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
                             const int len = on ? (int)((id >> kIdBits) & 31u) + 1 : 0;
                             const int first = (int)lds_u16_if(lst + 2u * (uint32_t)t, on) + q;
                             const uint32_t a_val = lval + 4u * (uint32_t)first, a_row = lrow + (uint32_t)first;
-                            const bool near = KIND == kHot || ((KIND == kCold || SPLIT) && v < hotc);
-                            const float w = KIND == kFlat ? 0.0f : lds_f32(a_w + (near ? 4u * v : 0u));
+                            const bool near = KIND == kHot || v < hotc;
+                            const float w = lds_f32(a_w + (near ? 4u * v : 0u));
                             float x[8];
                             uint32_t r[8];
                             auto take = [&](int u) {
@@ -2509,7 +2509,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
                             sum += __shfl_xor_sync(0xffffffffu, sum, 1);
                             sum += __shfl_xor_sync(0xffffffffu, sum, 2);
                             const bool mine = on && q == 0;
-                            if (KIND != kFlat) sts_f32(mine && near ? a_w + 4u * v : a_sink, fmaf(sigma, sum, w));
+                            sts_f32(mine && near ? a_w + 4u * v : a_sink, fmaf(sigma, sum, w));
                             if (FAR) {
                                 const bool far = mine && !near && sum != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
                                 red_add_if(Uk + (far ? v : 0u), sigma * sum, far);
@@ -2521,7 +2521,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
                         // A thread per entry: one whose id no other coordinate of the block has is applied (no two threads
                         // touch the same word). One store per entry, its address chosen without a branch: the model word, or
                         // a word that nobody reads; ids beyond the part in shared memory are added to at L2, nothing waits.
-                        constexpr int U = KIND == kFlat ? 4 : 2;
+                        constexpr int U = 2;
                         for (int e0 = wt; (e0 & ~31) < n; e0 += U * kWorkThreads) {
                             uint32_t m[U];
                             float p[U], w[U];
@@ -2538,13 +2538,13 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
                                 const uint32_t v = m[u] & kIdMask;
                                 p[u] = sigma * (p[u] * lds_f32(dl + ((m[u] >> (kIdBits - 2)) & 124u)));
                                 if (KIND == kHot) w[u] = lds_f32(a_w + 4u * (CHICLE_IN_BOUNDS(S.status, v < hotc) ? v : 0u));
-                                if (KIND == kCold || SPLIT) w[u] = lds_f32(a_w + (v < hotc ? 4u * v : 0u));
+                                else w[u] = lds_f32(a_w + (v < hotc ? 4u * v : 0u));
                             }
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
                                 const uint32_t v = m[u] & kIdMask;
-                                const bool mine = (m[u] >> 31) == 0u, near = KIND == kHot ? CHICLE_IN_BOUNDS(S.status, v < hotc) : ((KIND == kCold || SPLIT) && v < hotc);
-                                if (KIND != kFlat) sts_f32(mine && near ? a_w + 4u * v : a_sink, p[u] + w[u]);
+                                const bool mine = (m[u] >> 31) == 0u, near = KIND == kHot ? CHICLE_IN_BOUNDS(S.status, v < hotc) : v < hotc;
+                                sts_f32(mine && near ? a_w + 4u * v : a_sink, p[u] + w[u]);
                                 if (FAR) {
                                     const bool far = mine && !near && p[u] != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
                                     red_add_if(Uk + (far ? v : 0u), p[u], far);
@@ -2867,7 +2867,6 @@ template <int LOSS, int KIND, bool TABLES> cudaError_t launch_chain(Glm &g, cons
 int chain_kind(const Glm &g)
 {
     if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) return kDense;
-    if (g.la_hotc == 0) return kFlat;
     if (((int64_t)g.la_hotc << g.la_logC) >= g.dim) return kHot;
     return g.la_far_cap > 0 ? kSplit : kCold;
 }
@@ -2876,7 +2875,6 @@ template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P, cud
     constexpr bool tables = LOSS == CHICLE_LOSS_LOGISTIC_DUAL;
     switch (chain_kind(g)) {
     case kDense: return launch_chain<LOSS, kDense, tables>(g, P, begun);
-    case kFlat: return launch_chain<LOSS, kFlat, tables>(g, P, begun);
     case kHot: return launch_chain<LOSS, kHot, tables>(g, P, begun);
     case kSplit: return launch_chain<LOSS, kSplit, tables>(g, P, begun);
     default: return launch_chain<LOSS, kCold, tables>(g, P, begun);
@@ -3050,7 +3048,7 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
         }
         if (g.by_chunks) room = most;
         for (;;) {
-            const double left = (double)budget - (double)chain_layout(0, 0, 0, false, g.la_tab_bins, g.flat_ids ? kFlat : kCold).total - 64.0;
+            const double left = (double)budget - (double)chain_layout(0, 0, 0, false, g.la_tab_bins, kCold).total - 64.0;
             g.la_slots = g.la_depth == 1 && 4.0 * room > 0.6 * left ? 3 : kSubSlots;
             if (g.la_tab_bins == 0 || (double)g.la_slots * room <= 0.8 * left) {
                 const uint32_t limit = (uint32_t)(0.8 * left / g.la_slots) & ~15u;
@@ -3062,7 +3060,7 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
         const ChainLayout L0 = chain_layout(g.la_sub_room, g.la_slots, 0, false, g.la_tab_bins, kHot);
         int64_t hotc = ((int64_t)budget - (int64_t)L0.total - 64) / 4;
         const int64_t need = (g.dim + ((int64_t)1 << logC) - 1) >> logC; // per CTA for the whole model
-        if (hotc < need && !g.flat_ids) {
+        if (hotc < need) {
             // the rest lies in L2: lists for the far warp, where they leave the model something; or two filters
             const int cap = ((int)n_max + 32) & ~31;
             const int64_t split = hotc - (int64_t)far_bytes(kSplit, cap, g.la_slots) / 4;
@@ -3072,7 +3070,7 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
                 g.la_far_cap = cap;
             } else hotc -= (int64_t)filter_bytes(kCold) / 2;
         }
-        hotc = hotc < 0 || g.flat_ids ? 0 : (hotc / 32) * 32;
+        hotc = (hotc / 32) * 32;
         // (what the whole model leaves goes to the slots: rows may be more alike than their ids' frequencies say)
         const int64_t spare = (4 * (hotc - (need + 31) / 32 * 32) / g.la_slots) & ~(int64_t)15;
         if (spare > 0 && g.la_sub_room < most) g.la_sub_room += (uint32_t)((int64_t)(most - g.la_sub_room) < spare ? most - g.la_sub_room : spare);
