@@ -199,6 +199,9 @@ cudaError_t launch_gather_f32(Glm &g, const float *src, const int32_t *map, int6
 cudaError_t launch_lookahead_solver(Glm &g, const struct SolverParams &P);
 cudaError_t launch_words(Glm &g, int64_t *dst, const int64_t *src, size_t n); // small host arrays to the device
 void lookahead_plan(Glm &g, int32_t K, bool tables); // fills the la_* sizes for a partition into K (logistic: with or without tables)
+// For the log: instance of the chain kernel, ids in shared memory, entries beyond them that a block is expected to have per CTA.
+struct LookChain { const char *instance; int64_t on_chip; double beyond; };
+LookChain lookahead_chain(const Glm &g);
 int lookahead_arrays(const Glm &g, bool by_chunks, double chunk_mean); // which of the sparse prepare kernels would serve
 int lookahead_max_dense_dim();
 int lookahead_max_slices();

@@ -40,6 +40,7 @@
 // A block with more non-zeros than the shared-memory buffers hold is flagged by the prepare kernel: the pipeline
 // drains, warp 0 of CTA 0 walks the block coordinate by coordinate against the whole model, and the pipeline starts
 // again behind it. Rounds that span several local epochs run the pair of kernels once per epoch.
+#include <algorithm>
 #include <cmath>
 #include <cstddef>
 #include <cstdio>
@@ -2951,6 +2952,14 @@ cudaError_t launch_words(Glm &g, int64_t *dst, const int64_t *src, size_t n)
     return cudaGetLastError();
 }
 
+// (for the log: which instance of the chain kernel a round takes decides what a test of it has tested)
+LookChain lookahead_chain(const Glm &g)
+{
+    static const char *const names[] = {"whole", "cold", "dense", "far-warp"}; // by kind
+    const int64_t hot = std::min((int64_t)g.la_hotc << g.la_logC, g.dim);
+    const bool dense = g.fmt == CHICLE_FMT_DENSE_ROWMAJOR;
+    return {names[chain_kind(g)], dense ? g.dim : hot, dense ? 0.0 : entries_beyond(g, hot) / (1 << g.la_logC)};
+}
 int lookahead_arrays(const Glm &g, bool by_chunks, double chunk_mean) { return arrays_of(g, by_chunks, chunk_mean); }
 int lookahead_max_dense_dim() { return kMaxC * kDenseSlice; }
 int lookahead_max_slices() { return 64; }

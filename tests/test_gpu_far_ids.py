@@ -1,7 +1,7 @@
-"""Chain kernel where part of the model lies beyond shared memory: ids that fall in and out of it, ids there that several coordinates of a
-block share (their lists), many of them per block and none at all, every cluster size and both depths, rounds in several launches,
-blocks walked in place between others, and records so long that the far warp's lists find no room. Against the oracle within the
-parity tolerances, and the same bits in two runs."""
+"""Chain kernel where the model is longer than its part in shared memory. `create` numbers the ids by frequency, and these rows have fewer
+ids than shared memory holds in most cases: what lies beyond it are ids that no row has, in the others rare ones that a block rarely
+shares. Every cluster size and both depths, rounds in several launches, blocks walked in place between others, long records. Against the
+oracle within the parity tolerances, and the same bits in two runs. (Entries beyond shared memory in every block: test_gpu_far_warp.py.)"""
 import numpy as np
 import pytest
 
@@ -13,8 +13,7 @@ from paper_1909_04885_b200.datagen import Phase, Workload  # noqa: E402
 
 
 def rows(loss, n, d, per, K, far, seed):
-    """`per` ids a row: most of them Zipf-distributed, a share `far` of them among pairs of ids of the last nine tenths that the rows of a
-    block are likely to have together."""
+    """`per` ids a row: most of them Zipf-distributed, a share `far` of them from a few hundred of the last nine tenths of the numbers."""
     rng = np.random.default_rng(seed)
     ids = []
     for i in range(n):
