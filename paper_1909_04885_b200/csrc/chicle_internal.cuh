@@ -147,6 +147,7 @@ struct Glm {
     int la_slots = 4;                // and how many slots
     int32_t la_hotc = 0;             // entry ids per CTA kept in shared memory
     int32_t la_far_cap = 0;          // entries of a record that the far warp's lists hold (0: no far warp)
+    bool la_early = false;           // ids beyond shared memory are gathered before the block's deltas have come
     int32_t la_tab_bins = 0;         // logistic: bins per coordinate of the step's tables (0: none)
     size_t la_tab_off = 0;           // where they lie in a region
     size_t la_smem = 0;              // dynamic shared memory of the chain kernel

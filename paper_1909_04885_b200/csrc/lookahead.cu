@@ -30,7 +30,7 @@
 //                         through distributed shared memory by asynchronous stores that complete on the receiver's
 //                         mbarrier; no multicast, every wait bounded. Ids that are not in shared memory: where a block has a
 //                         few of them per CTA, a warp of its own applies their updates and takes their part of the dot products; where
-//                         it has many, the worker warps do, with the gathers sent out before the deltas have come.
+//                         it has many, the worker warps do, and where dot products wait for deltas in any case their gathers go out before.
 //
 // Where many partitions leave the prepare kernels few SMs (one CTA per partition on sparse data), the dot products are
 // taken one block ahead only, against the model after the block before: no cross Gram matrix (the prepare kernels are
@@ -131,9 +131,10 @@ struct alignas(16) BlkDir { // where a record is
 };
 
 // Kinds of data the chain kernel is instantiated for: sparse with the whole model in shared memory, with its most frequent
-// ids there; dense rows.
-// kSplit: as kCold, with a warp of its own for the ids that are not in shared memory; kCold where there is no room for its lists.
-constexpr int kHot = 0, kCold = 1, kDense = 2, kSplit = 3;
+// ids there (kCold, kEarly, kSplit: how the others are come by); dense rows.
+// kCold: the worker warps gather them behind the block's update. kEarly: before its deltas have come, and again what the update may
+// have changed. kSplit: a warp of its own does. Which of them: see lookahead_plan.
+constexpr int kHot = 0, kCold = 1, kDense = 2, kSplit = 3, kEarly = 4;
 __host__ __device__ constexpr int chain_threads(int kind) { return kind == kSplit ? 448 : 384; }
 
 struct LookParams {
@@ -1657,11 +1658,11 @@ struct ChainLayout {
 constexpr uint32_t kFarSums = 2u * kMaxC * kLB * 4u, kFarHead = 80u;
 __host__ __device__ constexpr uint32_t far_list_bytes(int cap) { return kFarHead + 2u * (uint32_t)cap; }
 __host__ __device__ constexpr uint32_t far_bytes(int kind, int cap, int slots) { return kind == kSplit ? kFarSums + 4u * (uint32_t)cap + (uint32_t)slots * far_list_bytes(cap) : 0u; }
-// Ids beyond the model's part in shared memory (kCold): their model entries are gathered from L2 before the
+// kEarly: the model entries of ids beyond the part in shared memory are gathered from L2 before the
 // block's deltas have come, and those that the block's update then changes once more. Which may have changed is kept in a bit
 // per hashed id, one set of them for even and one for odd blocks: this many bytes a set (a bit that two ids share costs a
 // second gather, nothing else).
-__host__ __device__ constexpr uint32_t filter_bytes(int kind) { return kind == kCold ? 4096u : 0u; }
+__host__ __device__ constexpr uint32_t filter_bytes(int kind) { return kind == kEarly ? 4096u : 0u; }
 __host__ __device__ inline ChainLayout chain_layout(uint32_t sub_room, int slots, int hotc, bool dense, int tab_bins, int kind, int far_cap = 0)
 {
     ChainLayout L;
@@ -1747,8 +1748,8 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
         for (int i = 0; i < 8; ++i)
             if (l0 + i * kChainThreads < hot_mine) W[l0 + i * kChainThreads] = P.model_in ? fmaf(sigma, u[i], v[i]) : u[i];
     }
-    constexpr bool FAR = KIND == kCold;
-    if constexpr (FAR)
+    constexpr bool EARLY = KIND == kEarly, FAR = KIND == kCold || EARLY;
+    if constexpr (EARLY)
         for (uint32_t i = (uint32_t)tid; i < 2u * filter_bytes(KIND) / 4u; i += kChainThreads) reinterpret_cast<uint32_t *>(smem_chain + L.filter)[i] = 0u;
     if (DENSE && tid < 4 && hot_mine + tid < P.hotc) W[hot_mine + tid] = 0.0f; // (the padding of the last slice)
     // the ids beyond the part in shared memory that fall to this CTA (id mod C): the model in place
@@ -2097,7 +2098,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
         for (int blk = 0; blk < nb; ++blk) {
             if (__any_sync(0xffffffffu, *abort_flag != 0)) break; // (no slot is refilled for workers that no longer wait for it)
             // (the block before this one arrives while its predecessor's slot is still in use)
-            if ((FAR || SPLIT) && blk > 0) {
+            if ((EARLY || SPLIT) && blk > 0) {
                 if (!mbar_wait_cluster(smem_u32(&ctl.subfull[before]), tbefore, abort_flag, S.status)) break;
                 list_far(before);
             }
@@ -2120,6 +2121,12 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
             bulk_g2s_if(smem_u32(smem_chain + L.subs) + (uint32_t)slot * L.sub_stride, P.rec + offset, bytes, bar, lane == 0);
             fetched = blk + 1;
             load_dir(blk + 1, d);
+            // (kCold: this block's copy goes out first. As above, the round on 0.6 M uniform rows of 39, d = 1 M, K = 9: 4.10 ms instead of
+            // 4.06, on 1 M over K = 16 4.24 instead of 4.18.)
+            if (KIND == kCold && blk > 0) {
+                if (!mbar_wait_cluster(smem_u32(&ctl.subfull[before]), tbefore, abort_flag, S.status)) break;
+                list_far(before);
+            }
             before = slot;
             tbefore = turn;
             if (++slot == slots) {
@@ -2318,7 +2325,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
 #ifdef CHICLE_LA_TIMING
         long long wd = 0, ws1 = 0, wg0 = 0, wg1 = 0, t0 = clock64(), t1 = 0;
 #endif
-        // (kCold) where the bit of a model entry in L2 is
+        // (kEarly) where the bit of a model entry in L2 is
         const uint32_t filter0 = smem_u32(smem_chain + L.filter);
         auto bit_of = [&](uint32_t v, uint32_t &word, uint32_t &bit) {
             const uint32_t h = v >> logC;
@@ -2362,7 +2369,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
             }
         };
         auto near = [&](int u) { // (once all gathers are on their way)
-            if (KIND == kCold) {
+            if (FAR) {
                 const float h = lds_f32(a_w + (m[u] < hotc ? 4u * m[u] : 0u));
                 w[u] = m[u] < hotc ? h : w[u];
             }
@@ -2419,7 +2426,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
             // block's update changes is gathered again). Not in front of a block that is walked in place.
             // (2 M ridge columns over K = 128: 11.1 -> 10.6 ms a step; 5.6 M hashed rows, whose K = 64 round is of this kind, 29.1 -> 28.4.)
             bool early = false;
-            if (FAR) {
+            if (EARLY) {
                 dot_record();
                 if (ok && due && !sl0 && (depth == 1 || !sl1)) {
                     const int4 head = lds_s32x4(r_dot);
@@ -2444,7 +2451,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
                 work_bar();
                 LA_T(wd);
                 const uint32_t filter = filter0 + par * filter_bytes(KIND);
-                if constexpr (FAR) // (the other set: the dot products that looked at it are through)
+                if constexpr (EARLY) // (the other set: the dot products that looked at it are through)
 #pragma unroll
                     for (uint32_t i = 0; i < filter_bytes(KIND) / (16u * kWorkThreads); ++i)
                         sts_f32x4_if(filter0 + (par ^ 1u) * filter_bytes(KIND) + 16u * ((uint32_t)wt + i * kWorkThreads), 0.0f, 0.0f, 0.0f, 0.0f, true);
@@ -2514,9 +2521,11 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
                             if (FAR) {
                                 const bool far = mine && !near && sum != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
                                 red_add_if(Uk + (far ? v : 0u), sigma * sum, far);
-                                uint32_t word, bit;
-                                bit_of(v, word, bit);
-                                red_shared_or_if(filter + word, bit, far);
+                                if (EARLY) {
+                                    uint32_t word, bit;
+                                    bit_of(v, word, bit);
+                                    red_shared_or_if(filter + word, bit, far);
+                                }
                             }
                         }
                         // A thread per entry: one whose id no other coordinate of the block has is applied (no two threads
@@ -2549,9 +2558,11 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
                                 if (FAR) {
                                     const bool far = mine && !near && p[u] != 0.0f && CHICLE_IN_BOUNDS(S.status, (int64_t)v < S.dim);
                                     red_add_if(Uk + (far ? v : 0u), p[u], far);
-                                    uint32_t word, bit;
-                                    bit_of(v, word, bit);
-                                    red_shared_or_if(filter + word, bit, far);
+                                    if (EARLY) {
+                                        uint32_t word, bit;
+                                        bit_of(v, word, bit);
+                                        red_shared_or_if(filter + word, bit, far);
+                                    }
                                 }
                             }
                         }
@@ -2562,7 +2573,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
             }
             // ---- dot products: of block b + depth against the model as it is now. A block right behind a walked one starts
             //      from the model as the walk left it: with depth 2 its products wait for that.
-            if (KIND == kHot || SPLIT) dot_record();
+            if (!DENSE && !EARLY) dot_record();
             if (sl0 || sl1) {
                 late = depth == 2 && sl0 && !sl1 && b + 1 < nb;
                 due = due && (depth == 1 || !sl1);
@@ -2786,6 +2797,14 @@ constexpr int kSplitLeast = 4096;    // ids per CTA in shared memory that the fa
 // Entries beyond them that a block may be expected to have in a CTA's record: what the far warp keeps in registers. (45 M hashed rows
 // over K = 16 have 37; ridge over K = 128 has several hundred, and with the far warp, which is then the slowest, 17.1 instead of 10.6 ms.)
 constexpr double kSplitMost = 64.0;
+// Two blocks ahead, a gather has a block's time as it is, and going out early costs more than it saves below this many entries a block
+// and CTA; one block ahead it pays but for rows of 80, which are alike within 2 %. Local solvers, ms, gathers early and behind the update (rows of 39 but where noted, d from
+// 250 000 to 1.25 M):
+//   two ahead: 72 entries, K = 2, C = 8: 4.49, 4.16; 61, K = 4: 4.90, 4.55; 84, K = 9: 4.13, 4.05; 85, K = 16, C = 4 (rows of 60): 4.26, 4.20;
+//   171: 4.22, 4.15; 214: 4.22, 4.18; 240 (rows of 39): 4.10, 4.19; 185, K = 30, C = 2 (rows of 15): 3.15, 3.16; 556 (rows of 39): 4.79, 4.92
+//   one ahead: 27, K = 64, C = 1: 4.71, 4.71; 77: 4.73, 4.76; 157: 4.73, 4.84; 298: 4.77, 4.95; 60 (rows of 15): 3.38, 3.51; 110, K = 100: 4.94, 5.04;
+//   158, K = 64 (rows of 80): 3.74, 3.67
+constexpr double kEarlyLeast = 180.0;
 // Entries that a block of 32 random coordinates is expected to have with ids from `first` on.
 double entries_beyond(const Glm &g, int64_t first)
 {
@@ -2869,7 +2888,7 @@ int chain_kind(const Glm &g)
 {
     if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) return kDense;
     if (((int64_t)g.la_hotc << g.la_logC) >= g.dim) return kHot;
-    return g.la_far_cap > 0 ? kSplit : kCold;
+    return g.la_far_cap > 0 ? kSplit : (g.la_early ? kEarly : kCold);
 }
 template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P, cudaEvent_t begun = nullptr)
 {
@@ -2878,6 +2897,7 @@ template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P, cud
     case kDense: return launch_chain<LOSS, kDense, tables>(g, P, begun);
     case kHot: return launch_chain<LOSS, kHot, tables>(g, P, begun);
     case kSplit: return launch_chain<LOSS, kSplit, tables>(g, P, begun);
+    case kEarly: return launch_chain<LOSS, kEarly, tables>(g, P, begun);
     default: return launch_chain<LOSS, kCold, tables>(g, P, begun);
     }
 }
@@ -2955,7 +2975,7 @@ cudaError_t launch_words(Glm &g, int64_t *dst, const int64_t *src, size_t n)
 // (for the log: which instance of the chain kernel a round takes decides what a test of it has tested)
 LookChain lookahead_chain(const Glm &g)
 {
-    static const char *const names[] = {"whole", "cold", "dense", "far-warp"}; // by kind
+    static const char *const names[] = {"whole", "cold", "dense", "far-warp", "early"}; // by kind
     const int64_t hot = std::min((int64_t)g.la_hotc << g.la_logC, g.dim);
     const bool dense = g.fmt == CHICLE_FMT_DENSE_ROWMAJOR;
     return {names[chain_kind(g)], dense ? g.dim : hot, dense ? 0.0 : entries_beyond(g, hot) / (1 << g.la_logC)};
@@ -3027,6 +3047,7 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
     g.la_sub_room = 0;
     g.la_hotc = slice;
     g.la_far_cap = 0;
+    g.la_early = false;
     if (!dense) {
         // A slot holds the record that a block of 32 random coordinates is expected to make for a CTA (how many entries, and how
         // many of them with ids that several of the 32 have: from the ids' frequencies, see launch_frequency_remap) and five
@@ -3057,7 +3078,7 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
         }
         if (g.by_chunks) room = most;
         for (;;) {
-            const double left = (double)budget - (double)chain_layout(0, 0, 0, false, g.la_tab_bins, kCold).total - 64.0;
+            const double left = (double)budget - (double)chain_layout(0, 0, 0, false, g.la_tab_bins, kEarly).total - 64.0;
             g.la_slots = g.la_depth == 1 && 4.0 * room > 0.6 * left ? 3 : kSubSlots;
             if (g.la_tab_bins == 0 || (double)g.la_slots * room <= 0.8 * left) {
                 const uint32_t limit = (uint32_t)(0.8 * left / g.la_slots) & ~15u;
@@ -3070,14 +3091,17 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
         int64_t hotc = ((int64_t)budget - (int64_t)L0.total - 64) / 4;
         const int64_t need = (g.dim + ((int64_t)1 << logC) - 1) >> logC; // per CTA for the whole model
         if (hotc < need) {
-            // the rest lies in L2: lists for the far warp, where they leave the model something; or two filters
+            // the rest lies in L2: lists for the far warp, where they leave the model something; two filters for early gathers; or nothing
             const int cap = ((int)n_max + 32) & ~31;
             const int64_t split = hotc - (int64_t)far_bytes(kSplit, cap, g.la_slots) / 4;
             const double beyond = split >= kSplitLeast ? entries_beyond(g, split << logC) / C : 1e30;
             if (beyond <= kSplitMost) {
                 hotc = split;
                 g.la_far_cap = cap;
-            } else hotc -= (int64_t)filter_bytes(kCold) / 2;
+            } else if (g.la_depth == 1 || entries_beyond(g, hotc << logC) / C > kEarlyLeast) {
+                hotc -= (int64_t)filter_bytes(kEarly) / 2;
+                g.la_early = true;
+            }
         }
         hotc = (hotc / 32) * 32;
         // (what the whole model leaves goes to the slots: rows may be more alike than their ids' frequencies say)

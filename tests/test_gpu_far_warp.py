@@ -91,11 +91,12 @@ CASES = {
     "C=4": (W4, {}, "far-warp", 4, 2),
     "C=8": (W8, {}, "far-warp", 8, 2),
     "C=8, one ahead": (W8, {"CHICLE_LA_DEPTH": "1"}, "far-warp", 8, 1),
-    "many, C=1": (("hinge", 64, 6, 36_000, 7, 1, 6, 3, ()), {}, "cold", 1, 1),
+    "many, C=1": (("hinge", 64, 6, 36_000, 7, 1, 6, 3, ()), {}, "early", 1, 1),
     "many, C=2": (("hinge", 30, 16, 82_000, 7, 2, 6, 2, ()), {}, "cold", 2, 2),
-    "many, C=2, one ahead": (("hinge", 30, 16, 82_000, 7, 2, 6, 2, ()), {"CHICLE_LA_DEPTH": "1"}, "cold", 2, 1),
+    "many, C=2, one ahead": (("hinge", 30, 16, 82_000, 7, 2, 6, 2, ()), {"CHICLE_LA_DEPTH": "1"}, "early", 2, 1),
     "many, C=2, walked": (("hinge", 30, 16, 72_000, 7, 2, 6, 2, (0, 5, 6, 9, 15)), {}, "cold", 2, 2),
-    "very many, C=2": (("hinge", 30, 16, 100_000, 7, 2, 6, 2, ()), {}, "cold", 2, 2),
+    "many, C=1, walked": (("hinge", 64, 12, 32_000, 7, 1, 6, 1, (0, 4, 5, 7)), {}, "early", 1, 1),
+    "very many, C=2": (("hinge", 30, 16, 100_000, 7, 2, 6, 2, ()), {}, "early", 2, 2),
     "many, C=4, tables": (("logistic", 16, 48, 160_000, 4, 4, 3, 1, ()), {}, "cold", 4, 2),
 }
 
