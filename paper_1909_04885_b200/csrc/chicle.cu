@@ -414,9 +414,10 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
     int32_t *d_ctask = nullptr;
     const bool by_chunks = chunks && h->fmt != CHICLE_FMT_DENSE_ROWMAJOR;
     double chunk_mean = h->chunk_mean;
+    std::vector<unsigned long long> entries;
+    unsigned long long *d_entries = nullptr;
     if (chunks) {
-        std::vector<unsigned long long> entries((size_t)K);
-        unsigned long long *d_entries = nullptr;
+        entries.resize((size_t)K);
         if (!temp.alloc(d_coff, (size_t)chunks->C + 1) || !temp.alloc(d_ctask, (size_t)chunks->C) || !temp.alloc(d_entries, (size_t)K))
             return fail(h, CHICLE_ERR_OOM, "device allocation failed (chunk placement)");
         e = cudaMemcpyAsync(d_coff, chunks->off, ((size_t)chunks->C + 1) * 8, cudaMemcpyHostToDevice, h->stream);
@@ -515,6 +516,8 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
     }
     if (fresh) { h->owner = owner; h->members = members; h->perm = perm; h->perm_epochs = 1; }
     h->U = U; h->part_off = part_off; h->h_part_off = h_off;
+    h->la_far_worst = 0.0;
+    bool far_known = false;
     h->bucket_off = part_off + K + 1;
     h->d_steps = part_off + 2 * ((size_t)K + 1);
     h->U_rows = K;
@@ -538,15 +541,25 @@ static chicle_status_t partition_impl(chicle_glm_t *h, int32_t K, uint64_t seed,
     if (e == cudaSuccess) e = cudaMemsetAsync(U, 0, (size_t)K * (size_t)h->dim * 4, h->stream);
     if (chunks && e == cudaSuccess) {
         e = launch_partition_chunks(*h, K, chunks->C, d_coff, d_ctask);
+        if (e == cudaSuccess && by_chunks && h->la_rec && h->la_far_cap > 0) {
+            far_known = true;
+            e = launch_far_sample(*h, K, (int64_t)h->la_hotc << h->la_logC, d_entries);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(entries.data(), d_entries, (size_t)K * 8, cudaMemcpyDeviceToHost, h->stream);
+        }
     } else if (e == cudaSuccess) {
         e = launch_partition(*h, K, seed);
     }
-    // the host copy of part_off is reused by later calls, so finish the upload before returning
+    // the host copy of part_off is reused by later calls, so finish the upload before returning (and the far sample is read below)
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
         h->K = 0; // the partition map is not valid: a new partition call is required
         return fail_cuda(h, e, "partition kernels");
     }
+    if (far_known)
+        for (int32_t k = 0; k < K; ++k) {
+            const double nk = (double)sizes[k], per = (double)entries[(size_t)k] / std::min(nk, (double)kFarSample);
+            h->la_far_worst = std::max(h->la_far_worst, per * std::min(nk, 32.0) / (double)(1 << h->la_logC));
+        }
     return CHICLE_OK;
 }
 

@@ -147,6 +147,7 @@ struct Glm {
     int la_slots = 4;                // and how many slots
     int32_t la_hotc = 0;             // entry ids per CTA kept in shared memory
     int32_t la_far_cap = 0;          // entries of a record that the far warp's lists hold (0: no far warp)
+    double la_far_worst = 0.0;       // partitions by chunks: entries beyond shared memory of a block of the partition with most of them, per CTA
     bool la_early = false;           // ids beyond shared memory are gathered before the block's deltas have come
     int32_t la_tab_bins = 0;         // logistic: bins per coordinate of the step's tables (0: none)
     size_t la_tab_off = 0;           // where they lie in a region
@@ -182,6 +183,8 @@ struct Glm {
 cudaError_t launch_validate(Glm &g, bool values = true, bool rest = true); // the values array; labels and structure
 cudaError_t launch_sqnorm(Glm &g);
 cudaError_t launch_partition(Glm &g, int32_t K, uint64_t seed);           // fills owner, members
+constexpr int kFarSample = 512; // coordinates of a partition that launch_far_sample looks at
+cudaError_t launch_far_sample(Glm &g, int32_t K, int64_t first, unsigned long long *far); // far: K words, written
 cudaError_t launch_partition_chunks(Glm &g, int32_t K, int64_t C, const int64_t *chunk_off, const int32_t *chunk_task); // device arrays
 cudaError_t launch_chunk_entries(Glm &g, int64_t C, const int64_t *chunk_off, const int32_t *chunk_task, unsigned long long *entries); // += per task
 cudaError_t launch_permutation(Glm &g, int64_t round, int64_t epochs, int64_t H, const int64_t *steps); // fills perm[epochs * n_coord]

@@ -2745,6 +2745,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
 template <int LOSS, int KIND, bool TAB> cudaError_t launch_chain_kind(Glm &g, const LookParams &P, cudaEvent_t begun)
 {
     auto kern = k_lookahead_chain<LOSS, KIND, TAB>;
+    if (chain_layout(P.sub_room, P.slots, P.hotc, KIND == kDense, TAB ? P.tab_bins : 0, KIND, P.far_cap).total > g.la_smem) return cudaErrorInvalidConfiguration;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.la_smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -2888,7 +2889,11 @@ int chain_kind(const Glm &g)
 {
     if (g.fmt == CHICLE_FMT_DENSE_ROWMAJOR) return kDense;
     if (((int64_t)g.la_hotc << g.la_logC) >= g.dim) return kHot;
-    return g.la_far_cap > 0 ? kSplit : (g.la_early ? kEarly : kCold);
+    // (Partitions by chunks may be sorted: one with all the rare ids has many where the average over random blocks has few, and its far
+    // warp would set the pace. 1 M rows of 39 over K = 16 by chunks, 45 entries a block on average and up to 220: 9.17 against 4.10 ms,
+    // 4.18 before there was a far warp; as many everywhere, 8: 3.60 against 3.81.)
+    if (g.la_far_cap > 0) return g.la_far_worst <= kSplitMost ? kSplit : kCold;
+    return g.la_early ? kEarly : kCold;
 }
 template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P, cudaEvent_t begun = nullptr)
 {
@@ -3047,6 +3052,7 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
     g.la_sub_room = 0;
     g.la_hotc = slice;
     g.la_far_cap = 0;
+    g.la_far_worst = 0.0; // (of the partition before; what follows sizes the shared memory for the instance that the plan allows)
     g.la_early = false;
     if (!dense) {
         // A slot holds the record that a block of 32 random coordinates is expected to make for a CTA (how many entries, and how
@@ -3261,7 +3267,7 @@ cudaError_t launch_lookahead_solver(Glm &g, const SolverParams &S)
         p.sub_room = g.la_sub_room;
         p.slots = g.la_slots;
         p.hotc = g.la_hotc;
-        p.far_cap = g.la_far_cap > 0 ? g.la_far_cap : INT32_MAX;
+        p.far_cap = chain_kind(g) == kSplit ? g.la_far_cap : INT32_MAX;
         p.n_blocks = blocks[(size_t)s];
         p.drop_block = (drop && s == 0) ? atoll(drop) : -1;
         p.nnz = g.nnz;

@@ -812,6 +812,31 @@ cudaError_t launch_chunk_entries(Glm &g, int64_t C, const int64_t *chunk_off, co
     return cudaGetLastError();
 }
 
+// far[k] = entries with ids from `first` on in up to kFarSample of partition k's coordinates, evenly spaced (a CTA per partition)
+__global__ void k_far_sample(const int32_t *__restrict__ members, const int64_t *__restrict__ part_off, const int64_t *__restrict__ indptr,
+                             const int32_t *__restrict__ indices, int64_t first, unsigned long long *__restrict__ far)
+{
+    __shared__ uint32_t sum;
+    if (threadIdx.x == 0) sum = 0u;
+    __syncthreads();
+    const int64_t off = part_off[blockIdx.x], nk = part_off[blockIdx.x + 1] - off, m = nk < kFarSample ? nk : kFarSample;
+    uint32_t n = 0u;
+    for (int64_t i = threadIdx.x >> 5; i < m; i += blockDim.x >> 5) {
+        const int32_t c = members[off + i * nk / m];
+        for (int64_t e = indptr[c] + (threadIdx.x & 31); e < indptr[c + 1]; e += 32) n += indices[e] >= first ? 1u : 0u;
+    }
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(&sum, n);
+    __syncthreads();
+    if (threadIdx.x == 0) far[blockIdx.x] = sum;
+}
+
+cudaError_t launch_far_sample(Glm &g, int32_t K, int64_t first, unsigned long long *far)
+{
+    k_far_sample<<<K, 256, 0, g.stream>>>(g.members, g.part_off, g.indptr, g.indices, first, far);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_partition_chunks(Glm &g, int32_t K, int64_t C, const int64_t *chunk_off, const int32_t *chunk_task)
 {
     const int64_t n = g.n_coord;

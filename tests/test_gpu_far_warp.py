@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 import oracle  # noqa: E402
 from paper_1909_04885_b200 import binding  # noqa: E402
 from paper_1909_04885_b200.datagen import Phase, Workload  # noqa: E402
-from parity_util import run_parity  # noqa: E402
+from parity_util import REL_TOL, make_pair, rel_l2, run_parity  # noqa: E402
 
 HEAD = 40  # ids that three rows in ten have: lists of many entries
 
@@ -101,6 +101,35 @@ CASES = {
 }
 
 
+@functools.lru_cache(maxsize=None)
+def by_topic(together):
+    """36 000 ids in two rows each; `together`: of the first sixth of the rows."""
+    rng = np.random.default_rng(2)
+    n, near, rare = 34_560, 57_000, 36_000
+    row, ids = np.nonzero(rng.random((n, HEAD)) < 0.3)
+    row = np.concatenate([row, np.arange(near * 7) % n, rng.integers(0, n // 6 if together else n, 2 * rare)])
+    ids = np.concatenate([ids, HEAD + rng.permutation(np.repeat(np.arange(near), 7)), HEAD + near + np.arange(2 * rare) % rare])
+    key = np.unique(row.astype(np.int64) * (HEAD + near + rare) + ids)
+    row, ids = key // (HEAD + near + rare), key % (HEAD + near + rare)
+    count = np.bincount(row, minlength=n)
+    return Workload("topics", "hinge", "csr", n, HEAD + near + rare, (rng.standard_normal(ids.size) / np.sqrt(count[row])).astype(np.float32),
+                    np.where(rng.random(n) < 0.5, 1.0, -1.0).astype(np.float32), 5.0 / n, 4, [Phase(0, 30, 1, 30.0)],
+                    indptr=np.concatenate([[0], np.cumsum(count)]).astype(np.int64), indices=ids.astype(np.int32))
+
+
+def run_chunks(w, K=30):
+    orc, glm = make_pair(w)
+    with glm:
+        for chunks in (False, True, False, True):
+            for x in (orc, glm):
+                if chunks:
+                    x.partition_chunks(K, 7, np.linspace(0, w.n_rows, K + 1).astype(np.int64), np.arange(K, dtype=np.int32))
+                else:
+                    x.partition(K, 5)
+                x.cocoa_round(0, float(K))
+            assert rel_l2(glm.get_alpha(), orc.state) <= REL_TOL and rel_l2(glm.get_v(), orc.v) <= REL_TOL
+
+
 def run_all():
     """(a process of its own: the library looks once whether it is to write a log)"""
     for name, (args, env, *_) in CASES.items():
@@ -121,6 +150,9 @@ def run_all():
             print("failed: %s" % e, file=sys.stderr, flush=True)
         for k in env:
             del os.environ[k]
+    for together in (False, True):
+        print("case %s" % together, file=sys.stderr, flush=True)
+        run_chunks(by_topic(together))
 
 
 @pytest.fixture(scope="module")
@@ -149,3 +181,10 @@ def test_entries_beyond_shared_memory(logs, name):
     # more than the far warp keeps in registers, few and none; lists longer than it keeps, lists beyond the first 32
     assert far.max() > 64 and (far > 64).sum() >= 0.03 * far.size and (far < 24).sum() >= (0.1 * far.size if instance == "far-warp" else 0)
     assert most.max() >= longest and (instance != "far-warp" or lists.max() > 32), (far.mean(), most.max(), lists.max())
+
+
+@pytest.mark.parametrize("together,instance", [(False, "far-warp"), (True, "cold")])
+def test_partitions_by_chunks(logs, together, instance):
+    """Rows sorted by topic: the partitions that have all the rare ids have six times the average, more than a far warp keeps up with."""
+    found = re.findall(r"ctas/partition=2 .*chain=(\S+) .*walked in place: 0\n", logs[str(together)])
+    assert found == ["far-warp", instance, "far-warp", instance], logs[str(together)]
