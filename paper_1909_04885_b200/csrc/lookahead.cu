@@ -2802,6 +2802,9 @@ template <int LOSS, int NZ, int HT, int THREADS, int PER_SM> cudaError_t launch_
     return cudaGetLastError();
 }
 
+// Not for the logistic loss: its recurrence is what a block takes, and the record warp, which lists the far warp's entries, shares its
+// scheduler. Rows of 39 with tables, 6 to 30 entries a block, local solvers with the far warp and without, ms: 50 000, K = 2: 2.36, 2.25;
+// 200 000, K = 9: 2.18, 2.13; 400 000, K = 16: 2.24, 2.18; 500 000, K = 30: 1.95, 1.93; 750 000, K = 64: 2.43, 2.44 (early gathers).
 constexpr int kSplitLeast = 4096;    // ids per CTA in shared memory that the far warp's lists must leave
 // Entries beyond them that a block may be expected to have in a CTA's record: what the far warp keeps in registers. (45 M hashed rows
 // over K = 16 have 37; ridge over K = 128 has several hundred, and with the far warp, which is then the slowest, 17.1 instead of 10.6 ms.)
@@ -2909,7 +2912,9 @@ template <int LOSS> cudaError_t launch_chain_on(Glm &g, const LookParams &P, cud
     switch (chain_kind(g)) {
     case kDense: return launch_chain<LOSS, kDense, tables>(g, P, begun);
     case kHot: return launch_chain<LOSS, kHot, tables>(g, P, begun);
-    case kSplit: return launch_chain<LOSS, kSplit, tables>(g, P, begun);
+    case kSplit:
+        if constexpr (LOSS != CHICLE_LOSS_LOGISTIC_DUAL) return launch_chain<LOSS, kSplit, tables>(g, P, begun);
+        else return cudaErrorInvalidConfiguration; // (never planned)
     case kEarly: return launch_chain<LOSS, kEarly, tables>(g, P, begun);
     default: return launch_chain<LOSS, kCold, tables>(g, P, begun);
     }
@@ -3108,7 +3113,8 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
             // the rest lies in L2: lists for the far warp, where they leave the model something; two filters for early gathers; or nothing
             const int cap = ((int)n_max + 32) & ~31;
             const int64_t split = hotc - (int64_t)far_bytes(kSplit, cap, g.la_slots) / 4;
-            const double beyond = split >= kSplitLeast ? entries_beyond(g, split << logC) / C : 1e30;
+            const bool far_warp = split >= kSplitLeast && g.loss != CHICLE_LOSS_LOGISTIC_DUAL;
+            const double beyond = far_warp ? entries_beyond(g, split << logC) / C : 1e30;
             if (beyond <= kSplitMost) {
                 hotc = split;
                 g.la_far_cap = cap;

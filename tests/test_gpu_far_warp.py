@@ -81,12 +81,13 @@ W1, W2, W4, W8 = ("hinge", 64, 12, 36_600, 7, 1, 6, 1, ()), ("hinge", 30, 24, 79
 CASES = {
     "C=1": (W1, {}, "far-warp", 1, 1),
     "C=1, two ahead": (W1, {"CHICLE_LA_DEPTH": "2"}, "far-warp", 1, 2),
-    "C=1, tables": (("logistic", 64, 12, 23_700, 7, 1, 6, 1, ()), {}, "far-warp", 1, 1),
+    "C=1, tables": (("logistic", 64, 12, 26_000, 7, 1, 6, 1, ()), {}, "early", 1, 1),
     "C=1, walked": (("hinge", 64, 12, 23_900, 7, 1, 6, 1, (0, 4, 5, 7)), {}, "far-warp", 1, 1),
     "C=2": (W2, {}, "far-warp", 2, 2),
     "C=2, one ahead": (W2, {"CHICLE_LA_DEPTH": "1"}, "far-warp", 2, 1),
     "C=2, three launches": (W2, {"CHICLE_LA_SLICES": "3"}, "far-warp", 2, 2),
-    "C=2, tables": (("logistic", 30, 24, 54_400, 7, 2, 6, 1, ()), {}, "far-warp", 2, 2),
+    "C=2, tables": (("logistic", 30, 24, 58_500, 7, 2, 6, 1, ()), {}, "cold", 2, 2),
+    "C=2, no tables": (("logistic", 30, 24, 84_000, 7, 2, 6, 1, ()), {"CHICLE_LA_TABLES": "0"}, "cold", 2, 2),
     "C=2, walked": (("hinge", 30, 24, 68_000, 7, 2, 6, 1, (0, 5, 6, 9, 23)), {}, "far-warp", 2, 2),
     "C=4": (W4, {}, "far-warp", 4, 2),
     "C=8": (W8, {}, "far-warp", 8, 2),
