@@ -2806,9 +2806,14 @@ template <int LOSS, int NZ, int HT, int THREADS, int PER_SM> cudaError_t launch_
 // scheduler. Rows of 39 with tables, 6 to 30 entries a block, local solvers with the far warp and without, ms: 50 000, K = 2: 2.36, 2.25;
 // 200 000, K = 9: 2.18, 2.13; 400 000, K = 16: 2.24, 2.18; 500 000, K = 30: 1.95, 1.93; 750 000, K = 64: 2.43, 2.44 (early gathers).
 constexpr int kSplitLeast = 4096;    // ids per CTA in shared memory that the far warp's lists must leave
-// Entries beyond them that a block may be expected to have in a CTA's record: what the far warp keeps in registers. (45 M hashed rows
-// over K = 16 have 37; ridge over K = 128 has several hundred, and with the far warp, which is then the slowest, 17.1 instead of 10.6 ms.)
-constexpr double kSplitMost = 64.0;
+// Entries beyond them that a block may be expected to have in a CTA's record: few blocks then have more than the 64 that the far warp
+// keeps in registers; with more of those it is the slowest of all roles. Local solvers, ms, with the far warp and without:
+//   two ahead: 47 entries, K = 2, C = 8 (rows of 39): 4.10, 4.37; 58: 4.36, 4.38; 50, K = 4: 4.38, 4.56; 57 (rows of 60): 4.73, 4.70; 62 (rows of
+//   39): 4.87, 4.55; 59, K = 9 (rows of 60): 4.63, 4.46; 54, K = 16, C = 4 (rows of 39): 3.76, 3.85; 61 (rows of 15): 4.01, 3.63; 85: 4.96, 3.84;
+//   50, K = 30, C = 2 (rows of 15): 2.96, 3.07; 67: 3.58, 3.08; 10 to 40 (rows of 39): 3.96, 3.85
+//   one ahead: 36, K = 64, C = 1 (rows of 39): 4.61, 4.72; 77: 4.70, 4.73; 47 (rows of 15): 3.44, 3.38; 62: 3.60, 3.38; 55, K = 100: 4.65, 4.92;
+//   several hundred, ridge over K = 128: 17.1, 10.6 (the step)
+constexpr double kSplitMost = 56.0;
 // Two blocks ahead, a gather has a block's time as it is, and going out early costs more than it saves below this many entries a block
 // and CTA; one block ahead it pays but for rows of 80, which are alike within 2 %. Local solvers, ms, gathers early and behind the update (rows of 39 but where noted, d from
 // 250 000 to 1.25 M):

@@ -77,7 +77,7 @@ def far_entries(w, K, C, on_chip):
 
 
 # name: (workload, environment, instance, CTAs, depth)
-W1, W2, W4, W8 = ("hinge", 64, 12, 36_600, 7, 1, 6, 1, ()), ("hinge", 30, 24, 79_800, 7, 2, 6, 1, ()), ("hinge", 16, 48, 176_000, 4, 4, 3, 1, ()), ("hinge", 9, 120, 366_000, 3, 8, 2, 1, ())
+W1, W2, W4, W8 = ("hinge", 64, 12, 36_600, 7, 1, 6, 1, ()), ("hinge", 30, 26, 79_000, 7, 2, 6, 1, ()), ("hinge", 16, 48, 176_000, 4, 4, 3, 1, ()), ("hinge", 9, 120, 366_000, 3, 8, 2, 1, ())
 CASES = {
     "C=1": (W1, {}, "far-warp", 1, 1),
     "C=1, two ahead": (W1, {"CHICLE_LA_DEPTH": "2"}, "far-warp", 1, 2),
@@ -92,6 +92,7 @@ CASES = {
     "C=4": (W4, {}, "far-warp", 4, 2),
     "C=8": (W8, {}, "far-warp", 8, 2),
     "C=8, one ahead": (W8, {"CHICLE_LA_DEPTH": "1"}, "far-warp", 8, 1),
+    "some more, C=4": (("hinge", 16, 48, 204_000, 4, 4, 3, 1, ()), {}, "cold", 4, 2),
     "many, C=1": (("hinge", 64, 6, 36_000, 7, 1, 6, 3, ()), {}, "early", 1, 1),
     "many, C=2": (("hinge", 30, 16, 82_000, 7, 2, 6, 2, ()), {}, "cold", 2, 2),
     "many, C=2, one ahead": (("hinge", 30, 16, 82_000, 7, 2, 6, 2, ()), {"CHICLE_LA_DEPTH": "1"}, "early", 2, 1),
@@ -106,7 +107,7 @@ CASES = {
 def by_topic(together):
     """36 000 ids in two rows each; `together`: of the first sixth of the rows."""
     rng = np.random.default_rng(2)
-    n, near, rare = 34_560, 57_000, 36_000
+    n, near, rare = 36_480, 57_000, 36_000
     row, ids = np.nonzero(rng.random((n, HEAD)) < 0.3)
     row = np.concatenate([row, np.arange(near * 7) % n, rng.integers(0, n // 6 if together else n, 2 * rare)])
     ids = np.concatenate([ids, HEAD + rng.permutation(np.repeat(np.arange(near), 7)), HEAD + near + np.arange(2 * rare) % rare])
