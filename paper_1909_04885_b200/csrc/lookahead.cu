@@ -2094,13 +2094,18 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
             __syncwarp();
         };
         uint32_t turn = 0, tbefore = 0; // parity of how often the slots have been filled
+#ifdef CHICLE_LA_TIMING
+        long long ra = 0, rl = 0, rs = 0, t0 = clock64(), t1 = 0;
+#endif
 #pragma unroll 1
         for (int blk = 0; blk < nb; ++blk) {
             if (__any_sync(0xffffffffu, *abort_flag != 0)) break; // (no slot is refilled for workers that no longer wait for it)
             // (the block before this one arrives while its predecessor's slot is still in use)
             if ((EARLY || SPLIT) && blk > 0) {
                 if (!mbar_wait_cluster(smem_u32(&ctl.subfull[before]), tbefore, abort_flag, S.status)) break;
+                LA_T(ra);
                 list_far(before);
+                LA_T(rl);
             }
             if (blk >= slots && !mbar_wait_cluster(smem_u32(&ctl.subfree[slot]), turn ^ 1u, abort_flag, S.status)) break;
             const unsigned long long offset = ((unsigned long long)d[1] << 32) | d[0];
@@ -2141,7 +2146,14 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
                 slot = 0;
                 turn ^= 1u;
             }
+            LA_T(rs);
         }
+#ifdef CHICLE_LA_TIMING
+        if (blockIdx.x == 0 && lane == 0) {
+            unsigned long long *d = P.timing + 24;
+            d[0] = ra; d[1] = rl; d[2] = rs;
+        }
+#endif
         if (SPLIT && fetched == nb && mbar_wait_cluster(smem_u32(&ctl.subfull[before]), tbefore, abort_flag, S.status)) list_far(before);
         for (int i = fetched > slots ? fetched - slots : 0; i < fetched; ++i) mbar_drain(smem_u32(&ctl.subfull[i % slots]), (uint32_t)(i / slots) & 1u);
     }
@@ -2222,6 +2234,9 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
             a_val = lval + 4u * first;
             a_row = lst + 2u * (uint32_t)head.y + first;
         };
+#ifdef CHICLE_LA_TIMING
+        long long fe = 0, fd = 0, fu = 0, fl = 0, fs = 0, t0 = clock64(), t1 = 0;
+#endif
 #pragma unroll 1
         for (int b = nb > 0 ? -depth : 0; b < nb; ++b) {
             bool sl2 = false, due = b + depth < nb, late = false;
@@ -2236,6 +2251,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
             }
             due = due && ok;
             if (b + depth < nb && ok) load(s_dot, E2); // (nothing where the block is walked in place)
+            LA_T(fe);
             if (b >= 0) {
                 const uint32_t par = (uint32_t)(b & 1), dl = smem_u32(&ctl.dbuf[0][0]) + par * (uint32_t)(kLB * 4);
                 if (sl0) { // (as the worker warps)
@@ -2244,6 +2260,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
                 }
                 ok = ok && mbar_wait_cluster(smem_u32(&ctl.dbar[0]) + 8u * par, (uint32_t)(b >> 1) & 1u, abort_flag, S.status);
                 if (sl0) fence_cluster();
+                LA_T(fd);
                 if (!sl0 && ok) {
                     auto add = [&](float x, uint32_t m) { // an id that no other coordinate of the block has
                         const float p = sigma * (x * lds_f32(dl + ((m >> (kIdBits - 2)) & 124u)));
@@ -2278,6 +2295,7 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
                 __syncwarp();
                 mbar_arrive_if(smem_u32(&ctl.subfree[s_upd]), lane == 0 && ok); // (through with the slot's record and list)
                 s_upd = s_upd + 1 == slots ? 0 : s_upd + 1;
+                LA_T(fu);
             }
             if (ok && late) send(s_dot == 0 ? slots - 1 : s_dot - 1, E1, gather(E1.m[0]), gather(E1.m[1]));
             due = due && ok;
@@ -2292,7 +2310,9 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
                     rl[u] = lds_u8_if(a_row + (uint32_t)u, u < len);
                 }
             }
+            LA_T(fl);
             if (due) send(s_dot, E2, w0, w1);
+            LA_T(fs);
             E0 = depth == 1 ? E2 : E1;
             E1 = E2;
             if (++s_dot == slots) {
@@ -2302,6 +2322,12 @@ __global__ void __launch_bounds__(chain_threads(KIND), 1) k_lookahead_chain(cons
             sl0 = next_walked;
             sl1 = sl2;
         }
+#ifdef CHICLE_LA_TIMING
+        if (blockIdx.x == 0 && lane == 0) {
+            unsigned long long *d = P.timing + 28;
+            d[0] = fe; d[1] = fd; d[2] = fu; d[3] = fl; d[4] = fs;
+        }
+#endif
         if (!ok && lane == 0) *abort_flag = 1;
         far_bar();
     }
@@ -2777,13 +2803,16 @@ template <int LOSS, int KIND, bool TAB> cudaError_t launch_chain_kind(Glm &g, co
     e = cudaLaunchKernelEx(&cfg, kern, P);
 #ifdef CHICLE_LA_TIMING
     if (e == cudaSuccess) {
-        unsigned long long t[12] = {0};
+        unsigned long long t[33] = {0};
         (void)cudaStreamSynchronize(g.stream);
         (void)cudaMemcpy(t, P.timing, sizeof(t), cudaMemcpyDeviceToHost);
         const double nb = t[3] ? (double)t[3] : 1.0;
         fprintf(stderr, "lookahead chain, cycles per block (partition 0): waiting for dot products %.0f, recurrence %.0f, deltas %.0f; "
                 "workers of CTA 0: waiting for deltas %.0f, update %.0f, record wait %.0f, products %.0f (%llu blocks)\n",
                 t[0] / nb, t[1] / nb, t[2] / nb, t[4] / nb, t[7] / nb, t[8] / nb, t[9] / nb, t[3]);
+        if (KIND == kEarly || KIND == kSplit) fprintf(stderr, "  record warp of CTA 0: waiting for the record %.0f, entries beyond shared memory %.0f, slot and copy %.0f\n", t[24] / nb, t[25] / nb, t[26] / nb);
+        if (KIND == kSplit) fprintf(stderr, "  far warp of CTA 0: entries %.0f, waiting for deltas %.0f, update %.0f, gathers out and next lists %.0f, gathers back and sums %.0f\n",
+                                    t[28] / nb, t[29] / nb, t[30] / nb, t[31] / nb, t[32] / nb);
     }
 #endif
     return e;
@@ -2890,7 +2919,7 @@ template <int LOSS> cudaError_t launch_prepare_on(Glm &g, const LookParams &P, c
         (void)cudaMemcpy(t, P.timing + 16, sizeof(t), cudaMemcpyDeviceToHost);
         (void)cudaMemset(P.timing + 16, 0, sizeof(t));
         const double n = (double)nb;
-        fprintf(stderr, "lookahead prepare, cycles per block: insert %.0f, number %.0f, place %.0f, entries %.0f, scan and pairs %.0f, dense and write %.0f\n", t[0] / n, t[1] / n, t[2] / n, t[3] / n, t[4] / n, t[5] / n);
+        fprintf(stderr, "lookahead prepare, cycles per block: insert %.0f, number %.0f, place and next entries %.0f, entries %.0f, pairs and dense part %.0f, write %.0f\n", t[0] / n, t[1] / n, t[2] / n, t[3] / n, t[4] / n, t[5] / n);
     }
 #endif
     return e;
