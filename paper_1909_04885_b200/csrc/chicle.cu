@@ -669,10 +669,10 @@ static chicle_status_t round_impl(chicle_glm_t *h, int64_t H, const int64_t *hos
             (void)cudaMemsetAsync(h->d_status + kStatusWalked, 0, sizeof(uint32_t), s);
             (void)cudaStreamSynchronize(s);
             const LookChain c = variant >= 4 ? lookahead_chain(*h) : LookChain{"none", 0, 0.0};
-            fprintf(stderr, "[chicle] round %lld: K=%d steps=%lld solver=%d slices=%d ctas/partition=%d depth=%d chain=%s on-chip=%lld beyond=%.1f launches=%d; ms: orders %.3f, "
+            fprintf(stderr, "[chicle] round %lld: K=%d steps=%lld solver=%d slices=%d ctas/partition=%d depth=%d chain=%s on-chip=%lld beyond=%.1f table-bins=%d launches=%d; ms: orders %.3f, "
                     "local solvers %.3f (first prepare %.3f), aggregation %.3f; blocks walked in place: %u\n", (long long)(h->round - 1), (int)h->K,
                     (long long)r.steps, (int)r.solver_variant, (int)r.solver_slices, (int)r.cluster_ctas,
-                    variant >= 4 ? (int)h->la_depth : 0, c.instance, (long long)c.on_chip, c.beyond,
+                    variant >= 4 ? (int)h->la_depth : 0, c.instance, (long long)c.on_chip, c.beyond, variant >= 4 ? (int)h->la_tab_bins : 0,
                     (int)(r.solver_launches + r.order_launches + 1), r.ms_permutation, r.ms_local, r.ms_prepare, r.ms_reduce, *walked);
         }
     }

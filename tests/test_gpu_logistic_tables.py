@@ -73,3 +73,34 @@ def test_no_memory_for_tables(fmt, monkeypatch):
         assert glm.cocoa_round(0, 4.0, stats=True)["solver_variant"] in (4, 5)
     finally:
         glm.close()
+
+
+def long_rows_by_chunks():
+    """Rows of 80 ids, 20 partitions by chunks: record slots as long as the arrays for 3 072 entries take, and tables of 32 bins beside them,
+    leave little of shared memory (a process of its own: the library looks once whether it is to write a log)."""
+    import numpy as np
+    from paper_1909_04885_b200.datagen import Phase, Workload
+    from parity_util import make_pair, rel_l2
+    n, d, K = 4000, 160, 20
+    rng = np.random.default_rng(5)
+    ids = 2 * np.arange(80) + rng.integers(0, 2, (n, 80))
+    w = Workload("long", "logistic", "csr", n, d, (rng.standard_normal(n * 80) / 9.0).astype(np.float32), np.where(rng.random(n) < 0.5, 1.0, -1.0).astype(np.float32),
+                 10.0 / n, 1, [Phase(0, K, 1, float(K))], np.arange(n + 1, dtype=np.int64) * 80, ids.reshape(-1).astype(np.int32))
+    orc, glm = make_pair(w)
+    with glm:
+        for x in (orc, glm):
+            x.partition_chunks(K, 7, np.linspace(0, n, K + 1).astype(np.int64), np.arange(K, dtype=np.int32))
+            x.cocoa_round(0, float(K))
+        assert rel_l2(glm.get_alpha(), orc.state) <= 1e-4 and rel_l2(glm.get_v(), orc.v) <= 1e-4
+
+
+def test_long_slots_leave_room_for_tables():
+    import os
+    import subprocess
+    import sys
+    here = os.path.dirname(os.path.abspath(__file__))
+    root = os.path.dirname(here)
+    r = subprocess.run([sys.executable, "-c", "import sys; sys.path.insert(0, %r); import test_gpu_logistic_tables as t; t.long_rows_by_chunks()" % here],
+                       env=dict(os.environ, CHICLE_LOG="1", PYTHONPATH=root), cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-3000:]
+    assert "table-bins=32 " in r.stderr, r.stderr[-1000:]
