@@ -2843,13 +2843,21 @@ constexpr int kSplitLeast = 4096;    // ids per CTA in shared memory that the fa
 //   one ahead: 36, K = 64, C = 1 (rows of 39): 4.61, 4.72; 77: 4.70, 4.73; 47 (rows of 15): 3.44, 3.38; 62: 3.60, 3.38; 55, K = 100: 4.65, 4.92;
 //   several hundred, ridge over K = 128: 17.1, 10.6 (the step)
 constexpr double kSplitMost = 56.0;
-// Two blocks ahead, a gather has a block's time as it is, and going out early costs more than it saves below this many entries a block
-// and CTA; one block ahead it pays but for rows of 80, which are alike within 2 %. Local solvers, ms, gathers early and behind the update (rows of 39 but where noted, d from
-// 250 000 to 1.25 M):
-//   two ahead: 72 entries, K = 2, C = 8: 4.49, 4.16; 61, K = 4: 4.90, 4.55; 84, K = 9: 4.13, 4.05; 85, K = 16, C = 4 (rows of 60): 4.26, 4.20;
-//   171: 4.22, 4.15; 214: 4.22, 4.18; 240 (rows of 39): 4.10, 4.19; 185, K = 30, C = 2 (rows of 15): 3.15, 3.16; 556 (rows of 39): 4.79, 4.92
-//   one ahead: 27, K = 64, C = 1: 4.71, 4.71; 77: 4.73, 4.76; 157: 4.73, 4.84; 298: 4.77, 4.95; 60 (rows of 15): 3.38, 3.51; 110, K = 100: 4.94, 5.04;
-//   158, K = 64 (rows of 80): 3.74, 3.67
+// Two blocks ahead, a gather has a block's time as it is, and the record warp, which must look at every entry, sets the pace where records
+// are long: the far warp only up to this many entries a record. Local solvers, ms, with the far warp and without, 10 to 30 entries beyond shared
+// memory: 800 (rows of 50, K = 20, C = 2): 2.55, 1.99; 1 024: 2.87, 2.38; 624 (K = 30): 3.96, 3.85; 240: 2.83, 3.03; 360 (K = 16, C = 4): 2.62, 2.75;
+// 400: 2.81, 2.80; 480: 3.11, 3.08; 320 (K = 9, C = 8): 2.75, 2.85; 400: 3.32, 3.32; 480: 3.98, 3.96. (One ahead, K = 64, 1 920: 1.91, 1.92; 2 560: 2.31, 2.31.)
+constexpr double kSplitLongest = 380.0;
+// Gathers early and behind the update, ms (rows of 39 but where noted).
+// Two ahead, going out early costs more than it saves unless most of a record's entries, and at least this many, lie beyond shared memory:
+//   72 of 156 entries, K = 2, C = 8: 4.49, 4.16; 84, K = 9: 4.13, 4.05; 133: 5.23, 5.20; 85 of 480, K = 16, C = 4 (rows of 60): 4.26, 4.20; 214: 4.22, 4.18;
+//   109 of 120 (rows of 15): 5.07, 4.97; 215 of 240 (rows of 30): 4.71, 4.83; 240 of 312: 4.10, 4.19; 185 of 240, K = 30, C = 2 (rows of 15): 3.15, 3.16;
+//   300 of 320 (rows of 20): 3.52, 3.59; 590 of 1 024 (rows of 64): 4.03, 3.94; 919 of 960 (rows of 60): 5.29, 5.63
+// One ahead it pays while records are not longer than that:
+//   27 of 1 248, K = 64, C = 1: 4.71, 4.71; 77: 4.73, 4.76; 157: 4.73, 4.84; 298: 4.77, 4.95; 60 of 480 (rows of 15): 3.38, 3.51; 110 of 1 248, K = 100:
+//   4.94, 5.04; 1 161 of 1 280, C = 2 (rows of 80): 5.31, 5.55; 871 of 1 920 (rows of 60): 3.02, 3.00; 158 of 2 560 (rows of 80): 3.74, 3.67; 7 of 3 520 (rows
+//   of 110): 3.14, 3.08; 229 of 1 600, logistic with tables (rows of 50): 2.99, 2.90
+constexpr double kEarlyShare = 0.7, kEarlyLongest = 1400.0;
 constexpr double kEarlyLeast = 180.0;
 // Entries that a block of 32 random coordinates is expected to have with ids from `first` on.
 double entries_beyond(const Glm &g, int64_t first)
@@ -3112,7 +3120,7 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
         // over K = 128 12.5 -> 12.8 ms, logistic rows of 80 over K = 64, which lose their tables, 2.8 -> 3.8.)
         const int C = 1 << logC;
         uint32_t room = 256, most = 256;
-        double n_max = 0.0; // entries of a CTA's record
+        double n_max = 0.0, n_mean = 0.0; // entries of a CTA's record: at most, on average
         const double cap = (double)prepare_room(g); // (a block with more entries is walked in place anyway)
         for (int c = 0; c < C; ++c) {
             double n = 0.0, T = 0.0, nl = 0.0;
@@ -3126,6 +3134,7 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
             const uint32_t r = sub_bytes((uint32_t)n_hi + 1u, (uint32_t)T_hi + 1u, (uint32_t)nl_hi + 1u) + 64u;
             const uint32_t m = sub_bytes((uint32_t)n_hi + 1u, (uint32_t)(0.5 * n_hi) + 1u, (uint32_t)n_hi + 1u) + 64u;
             n_max = fmax(n_max, n_hi);
+            n_mean = fmax(n_mean, n);
             room = r > room ? r : room;
             most = m > most ? m : most;
         }
@@ -3149,12 +3158,13 @@ void lookahead_plan(Glm &g, int32_t K, bool want_tables)
             // the rest lies in L2: lists for the far warp, where they leave the model something; two filters for early gathers; or nothing
             const int cap = ((int)n_max + 32) & ~31;
             const int64_t split = hotc - (int64_t)far_bytes(kSplit, cap, g.la_slots) / 4;
-            const bool far_warp = split >= kSplitLeast && g.loss != CHICLE_LOSS_LOGISTIC_DUAL;
+            const bool far_warp = split >= kSplitLeast && g.loss != CHICLE_LOSS_LOGISTIC_DUAL && (g.la_depth == 1 || n_mean <= kSplitLongest);
             const double beyond = far_warp ? entries_beyond(g, split << logC) / C : 1e30;
             if (beyond <= kSplitMost) {
                 hotc = split;
                 g.la_far_cap = cap;
-            } else if (hotc > (int64_t)filter_bytes(kEarly) && (g.la_depth == 1 || entries_beyond(g, hotc << logC) / C > kEarlyLeast)) {
+            } else if (hotc > (int64_t)filter_bytes(kEarly) &&
+                       (g.la_depth == 1 ? n_mean <= kEarlyLongest : entries_beyond(g, hotc << logC) / C > fmax(kEarlyLeast, kEarlyShare * n_mean))) {
                 hotc -= (int64_t)filter_bytes(kEarly) / 2;
                 g.la_early = true;
             }
